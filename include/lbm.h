@@ -75,8 +75,8 @@ enum { LBM_BGK = 0, LBM_MRT = 1 };
  * with M = 6 w_i rho_w (e_i . v) and v the disk's velocity at the cut (the
  * half-way value where x + e_i is not a fluid node).  The Eq. 4/5 forces use
  * the same returned population, and v and the torque lever at the cut.  The
- * channel walls stay half-way.  With it, BGK runs the per-node path in the
- * deferred pass (kernel variants 0-2 act as 3-5).  Batches take LBM_HALFWAY
+ * channel walls stay half-way.  With it, BGK in FP16 runs the per-node path in
+ * the deferred pass (kernel variants 0-2 act as 3-5).  Batches take LBM_HALFWAY
  * only. */
 enum { LBM_HALFWAY = 0, LBM_INTERPOLATED = 1 };
 /* force form: Eq. 4 (conventional) or Eq. 5 (Galilean invariant) */
@@ -285,25 +285,25 @@ int64_t lbm_launch_count(const lbm_ctx *ctx);
 
 /* Launch variant of the advection-collision kernel.  Nodes per thread, as
  * the width of one population word: 0 = 16 bytes (default), 1 = 8 bytes,
- * 2 = 4 bytes; 3, 4, 5 = the same widths with the nodes next to solids and
- * edges (the per-node path) computed by a second kernel after the first
- * instead of inline.  Every variant evaluates the same expressions; the
- * compiler may fuse multiply-adds differently in each, so results agree to
- * the storage precision's rounding (not always bit for bit).  LBM_EINVAL for
- * other values. */
+ * 2 = 4 bytes (FP64: 8); 3, 4, 5 = the same widths, in FP16 with the nodes next
+ * to solids and edges (the per-node path) computed by a second kernel after the
+ * first instead of inline (FP64 and FP32 have no per-node path: 3-5 act as 0-2).
+ * Every variant evaluates the same expressions; the compiler may fuse
+ * multiply-adds differently in each, so results agree to the storage precision's
+ * rounding (not always bit for bit).  LBM_EINVAL for other values. */
 lbm_status lbm_set_kernel_variant(lbm_ctx *ctx, int32_t variant);
 int32_t lbm_kernel_variant(const lbm_ctx *ctx);
 
-/* Where the force kernel of a step (force record of time t, motion) runs:
- * 1 = on a second stream of the context, beside the advection-collision
- * kernel, which reads the same state (default); 0 = before it, on the
- * context's stream.  Results do not depend on it.  LBM_EINVAL for other
- * values. */
+/* Where the per-solid work of a step that the advection-collision kernel does not
+ * wait for runs (force record of time t, motion, the moving solids' node changes;
+ * in FP16 the link sums too): 1 = on a second stream of the context, beside that
+ * kernel, which reads the same state (default); 0 = before it, on the context's
+ * stream.  Results do not depend on it.  LBM_EINVAL for other values. */
 lbm_status lbm_set_force_overlap(lbm_ctx *ctx, int32_t on);
 int32_t lbm_force_overlap(const lbm_ctx *ctx);
 
 /* Autotuner: run 1 + steps real steps with each of the 6 variants of the
- * advection-collision kernel, with the force kernel beside it and before it,
+ * advection-collision kernel, with the per-solid work beside it and before it,
  * timing whole steps with CUDA events, and keep the fastest pair (the variant
  * stored in *best when not NULL; lbm_force_overlap tells the other).  The
  * simulation advances by 12 (1 + steps) steps; results do not depend on the

@@ -1,17 +1,17 @@
-// Per-solid work of one step t -> t+1, in three launches.
+// Per-solid work of one step t -> t+1.
 //
-// k_forces, one block per solid, and then k_ring run beside the
-// advection-collision kernel of the step: they read the populations of time
-// t, the owner map and the node flags (which that kernel also only reads),
-// and write nothing that it reads.
-//   k_forces: the momentum booked by the node-type changes of the previous
-//      step (the solid's segment of the event list), the link sums of Eq. 4
-//      and Eq. 5 over every fluid-solid link of time t (Eq. 6 and Eq. 7) ->
-//      the force record of t; the motion t -> t+1 (prescribed, or
-//      Newton-Euler on the Eq. 5 force; Eq. 4 when the context selects it for
-//      comparison); the largest displacement of any solid since the last
-//      pair test.
-//   k_ring, one warp per moving solid:
+// k_forces, one block per solid (or k_links, one or several blocks per solid, and
+// k_record, one warp per solid), comes first:
+//   the link sums of Eq. 4 and Eq. 5 over every fluid-solid link of time t (Eq. 6
+//   and Eq. 7), and in the FP64 and FP32 modes the population each link returns,
+//   left in the solid node's slot for the advection-collision kernel to pull;
+//   the momentum booked by the node-type changes of the previous step (the
+//   solid's segment of the event list) -> the force record of t; the motion
+//   t -> t+1 (prescribed, or Newton-Euler on the Eq. 5 force; Eq. 4 when the
+//   context selects it for comparison); the largest displacement of any solid
+//   since the last pair test.
+// k_ring, one warp per moving solid, reads no population and writes nothing that
+// the advection-collision kernel reads: it may run beside it.
 //   P  only when some solid may have come within reach of another one since
 //      the last test: the solid's near list, the solids whose centres are
 //      closer than r_s + r_q + NEAR_REACH + NEAR_MARGIN at t or t+1
@@ -32,9 +32,8 @@
 //      clock advances.
 //
 // Work per solid follows its perimeter: the nodes near the ends of the disk's
-// chord in every row (FP32 bounds with a one-node margin) are dealt out to
-// the warp's lanes, each lane fetching several nodes before it processes
-// them; every decision is taken by the exact test.
+// chord in every row (FP32 bounds with a one-node margin) are dealt out to the
+// threads; every decision is taken by the exact test.
 //
 // Precision: per-link products and each lane's running sum over its links
 // (a handful) are in the arithmetic precision of the storage mode (FP32 in the
@@ -138,17 +137,6 @@ struct Centre {
         b = xi + (int)floorf(fx + h);
         return true;
     }
-    // Unwrapped x-range [a, b] containing every node of row j within rr of
-    // the centre (one node of margin on each side); false if none can be.
-    __device__ __forceinline__ bool span(int j, float rr, int &a, int &b) const {
-        const float dy = (float)(j - yi) - fy;
-        const float h2 = rr * rr - dy * dy;
-        if (h2 < 0.f) return false;
-        const float h = sqrtf(h2);
-        a = xi + (int)floorf(fx - h) - 1;
-        b = xi + (int)ceilf(fx + h) + 1;
-        return true;
-    }
 };
 
 // Cell of the neighbour (x + dx, y + dy) of an in-domain node (|dx|, |dy|
@@ -237,30 +225,6 @@ __device__ __forceinline__ bool ring_ranges(const Centre &c0, const Centre &c1, 
     R.a1 = min(q0, q1) + 1;  // right: after the inner chords .. last of the outer
     R.b1 = max(b0, b1);
     if (R.a1 <= R.b0 + 1) {  // the two ends meet: one range
-        R.b0 = R.b1;
-        R.a1 = 1;
-        R.b1 = 0;
-    }
-    return true;
-}
-
-// Nodes of row j that can be fluid nodes linked to a disk of radius r:
-// r < distance <= r + sqrt(2), bounded by the chords of radius r and r + 1.5.
-__device__ __forceinline__ bool annulus_ranges(const Centre &c, float r, int j, Ranges &R) {
-    int ao, bo, ai, bi;
-    if (!c.span(j, r + 1.5f, ao, bo)) return false;
-    if (!c.span(j, r - 0.01f, ai, bi)) {
-        R.a0 = ao;
-        R.b0 = bo;
-        R.a1 = 1;
-        R.b1 = 0;
-        return true;
-    }
-    R.a0 = ao;
-    R.b0 = ai + 2;
-    R.a1 = bi - 2;
-    R.b1 = bo;
-    if (R.a1 <= R.b0 + 1) {
         R.b0 = R.b1;
         R.a1 = 1;
         R.b1 = 0;
@@ -382,9 +346,17 @@ __device__ void move_solid(const StepParams &p, int s, int lane, long long t, co
     double fl[2] = {0.0, 0.0};
     if (p.lub > 0.0) {
         const double ka = net_weight(p, b);
+        const float zf = (float)p.lub + 0.01f * (float)b.r + 1.f;
         for (int q = lane; q < p.nsolid; q += 32) {
             if (q == s) continue;
             const DSolid &B = p.S[q];
+            // FP32 first, with a slack far above its rounding: out of range for most
+            float ddx = (float)(b.ix0 - B.ix0) + (b.fx0 - B.fx0);
+            float ddy = (float)(b.iy0 - B.iy0) + (b.fy0 - B.fy0);
+            if (L.bc_x == LBM_PERIODIC) ddx -= (float)L.nx * rintf(ddx / (float)L.nx);
+            if (L.bc_y == LBM_PERIODIC) ddy -= (float)L.ny * rintf(ddy / (float)L.ny);
+            const float reach = (sqrtf(b.r2f) + sqrtf(B.r2f)) * 1.001f + zf;
+            if (ddx * ddx + ddy * ddy > reach * reach) continue;
             const double dx = min_image(b.x - B.x, L.nx, L.bc_x == LBM_PERIODIC);
             const double dy = min_image(b.y - B.y, L.ny, L.bc_y == LBM_PERIODIC);
             const double d = sqrt(dx * dx + dy * dy);
@@ -422,142 +394,6 @@ __device__ void move_solid(const StepParams &p, int s, int lane, long long t, co
     b.omn = b.om + fg[2] / I;
 }
 
-// Link sums of solid s at time t (populations f of time t), acc = Eq. 4
-// force and torque, then Eq. 5, summed over the warp (warp wi of nw sharing
-// the disk's rows).  Per link (x_f fluid, x_f + e_i owned by s): f_i =
-// f~_i(x_f), the bounced f_bb = f_i - 6 w_i rho_w (e_i . v) with v the
-// solid's velocity at x_s = x_f + e_i / 2; Eq. 4 = e_i f_i - e_opp f_bb,
-// Eq. 5 = (e_i - v) f_i - (e_opp - v) f_bb, torque (x_s - R) x F (Eq. 7).
-// (The batch's disks take the half-way boundary.)  A candidate node's flags
-// and its 9 populations are loaded together, with its 8
-// neighbours' owners unless lists_ok and the solid has no other solid within
-// reach (then every solid neighbour of the annulus is the solid's own: a
-// solid q holding a node within r_s + 4 of s's centre is in s's near list).
-template <int P, bool LOCAL>
-__device__ void forces_sum(const StepParams &p, int s, int lane, const void *f, int wi, int nw,
-                           bool lists_ok, double (&acc)[6]) {
-    using C = typename Prec<P>::C;
-    using S = typename Prec<P>::S;
-    constexpr int UF = 2;  // candidates a lane takes at once
-    // with rho_w = rho0 and the half-way boundary a link needs only f_i of its
-    // own direction: the flags come first and only the bounced directions'
-    // populations (and owners) are read; otherwise all nine with the flags
-    constexpr bool SPARSE = !LOCAL;
-    const DSolid &b = p.S[s];
-    const Lattice &L = p.L;
-    const S *fs = static_cast<const S *>(f);
-    const double X = b.x, Y = b.y;
-    const Centre c(b.ix0, b.iy0, b.fx0, b.fy0);
-    const C vx = pick<C>(b.vx, b.vxf), vy = pick<C>(b.vy, b.vyf), om = pick<C>(b.om, b.omf);
-    const C rho0 = pick<C>(p.rho0, p.rho0_f);
-    const int plane = (int)L.plane;
-    const float r = sqrtf(b.r2f);
-    const bool owners = !lists_ok || b.near_n != 0;
-    const bool px = L.bc_x == LBM_PERIODIC, py = L.bc_y == LBM_PERIODIC;
-    const Wrap wrap(L, b.ix0, b.iy0, b.rc);
-    int j0, j1;
-    rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
-    C lacc[6] = {0, 0, 0, 0, 0, 0};  // this lane's links
-    int ii[UF], jj[UF], kk[UF];
-    uint16_t fl[UF];
-    uint16_t own[UF][9];
-    S fv[UF][9];
-    // is x_f + e_i (in the domain) a node of solid s?  own holds the owners
-    // when they were read; else the flag bit suffices (no other solid in reach)
-    auto linked = [&](int u, int i) -> bool {
-        if (!((fl[u] >> opp(i)) & 1u)) return false;  // x_f + e_i is not solid
-        if (owners) return own[u][i] == (uint16_t)s;
-        return (px || (unsigned)(ii[u] + cx(i)) < (unsigned)L.nx) &&
-               (py || (unsigned)(jj[u] + cy(i)) < (unsigned)L.ny);  // not beyond a wall
-    };
-    warp_nodes_n<UF, 16>(
-        j0, j1, lane, [&](int j, Ranges &R) { return annulus_ranges(c, r, j, R); },
-        [&](int iu, int j, int u) {
-            int x, y;
-            if (!wrap(iu, j, x, y)) return false;
-            const int k = (int)cell_of(L, x, y);
-            ii[u] = iu;
-            jj[u] = j;
-            kk[u] = k;
-            fl[u] = p.flags[k];
-            if (!SPARSE) {
-#pragma unroll
-                for (int q = 0; q < 9; q++) fv[u][q] = fs[q * plane + k];
-                if (owners) {
-#pragma unroll
-                    for (int i = 1; i < 9; i++) {
-                        const int kb = neighbour(L, x, y, cx(i), cy(i));
-                        own[u][i] = kb >= 0 ? p.owner[kb] : FLUID;
-                    }
-                }
-            }
-            return true;
-        },
-        [&](int u, bool ok) {
-            const uint16_t m = fl[u];
-            if (!ok || (m & 1u) || !(m & 0x1FEu)) return;
-            const int iu = ii[u], j = jj[u];
-            C rho_w = rho0;
-            if (LOCAL) {
-                C a = 0;
-#pragma unroll
-                for (int q = 0; q < 9; q++) a += (C)cvt_s(fv[u][q]);
-                rho_w = Prec<P>::dev ? (C)1 + a : a;
-            }
-#pragma unroll
-            for (int i = 1; i < 9; i++) {
-                if (!linked(u, i)) continue;
-                C dx, dy;
-                C fi = (C)cvt_s(fv[u][i]);
-                if (Prec<P>::dev) fi += wgt<C>(i);
-                // x_s = x_f + e_i / 2 relative to R, from the unwrapped coordinate
-                if (Prec<P>::dev) {
-                    dx = (C)(iu - c.xi) + (C)(0.5f * cx(i)) - (C)c.fx;
-                    dy = (C)(j - c.yi) + (C)(0.5f * cy(i)) - (C)c.fy;
-                } else {
-                    dx = (C)(((double)iu + 0.5 * cx(i)) - X);
-                    dy = (C)(((double)j + 0.5 * cy(i)) - Y);
-                }
-                const C ux = vx - om * dy, uy = vy + om * dx;
-                const C fbb = fi - (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * ux + (C)cy(i) * uy);
-                const C cmx = (C)cx(i) * fi - (C)cx(opp(i)) * fbb;
-                const C cmy = (C)cy(i) * fi - (C)cy(opp(i)) * fbb;
-                const C gmx = ((C)cx(i) - ux) * fi - ((C)cx(opp(i)) - ux) * fbb;
-                const C gmy = ((C)cy(i) - uy) * fi - ((C)cy(opp(i)) - uy) * fbb;
-                lacc[0] += cmx;
-                lacc[1] += cmy;
-                lacc[2] += dx * cmy - dy * cmx;
-                lacc[3] += gmx;
-                lacc[4] += gmy;
-                lacc[5] += dx * gmy - dy * gmx;
-            }
-        },
-        wi, nw,
-        [&](const bool (&ok)[UF]) {
-            if (!SPARSE) return;
-            // the bounced directions of every fluid candidate, for all of them together
-#pragma unroll
-            for (int u = 0; u < UF; u++) {
-                const uint16_t m = fl[u];
-                if (!ok[u] || (m & 1u) || !(m & 0x1FEu)) continue;
-                int x = 0, y = 0;
-                if (owners) wrap(ii[u], jj[u], x, y);
-#pragma unroll
-                for (int i = 1; i < 9; i++) {
-                    if (!((m >> opp(i)) & 1u)) continue;
-                    fv[u][i] = fs[i * plane + kk[u]];
-                    if (owners) {
-                        const int kb = neighbour(L, x, y, cx(i), cy(i));
-                        own[u][i] = kb >= 0 ? p.owner[kb] : FLUID;
-                    }
-                }
-            }
-        });
-#pragma unroll
-    for (int q = 0; q < 6; q++) acc[q] = (double)lacc[q];
-    warp_sum(acc);
-}
-
 // Force record of time t of solid s from its link sums acc and the momentum
 // booked into t by the node-type changes of the previous step (lane 0: Eq. 4
 // force and torque, then Eq. 5); then its motion to t+1.
@@ -577,258 +413,409 @@ __device__ void record_forces(const StepParams &p, int s, int lane, long long t,
     move_solid(p, s, lane, t, fg);
 }
 
-// ------------------------------------------------- force kernel (block)
+// ------------------------------------------------- fluid-solid links
 
-// One block per solid: thread t takes the annulus candidates t, t + FB, ...
-// (a candidate node x_f can have a link into the disk when r - eps < |x_f - R|
-// <= r + sqrt 2 + eps: between the outer chord of each row and the inner one).
-// A candidate's flags are read first, then only the populations of its
-// bounced directions (all nine when rho_w is local or the boundary is
-// interpolated) and, unless the solid's near list is empty, the owners of
-// those directions.  Sums: per thread and over each warp's tree in the
+// A block of FB threads walks the links of one solid in two stages.  Candidates:
+// a node x_f can have a link into the disk when r - eps < |x_f - R| <= r +
+// sqrt 2 + eps, between the outer chord of each row and the inner one; thread t
+// reads the flags of candidate t, t + FB ... and lists its links (direction i
+// with x_f + e_i solid) in shared memory, in candidate order.  Links: every thread
+// takes links t, t + FB ... of that list, so that all lanes work: with a thread
+// per candidate, the lanes of a warp had one to five links each in different
+// directions, and the warp went through the link's arithmetic up to eight times
+// (which in FP64, two lanes per clock and SM, was most of the kernel's time).
+// A link reads its own population, its solid's owner only when the near list is
+// not empty, and with the interpolated boundary one population more.  Sums: a
+// link's six terms go through shared memory to its candidate's thread, which adds
+// them in the order of the directions; then over each warp's tree, both in the
 // arithmetic precision of the storage mode, then across the block's warps in
-// FP64, in warp order.  Warp 0 then records the force and moves the solid.
+// FP64, in warp order.  (A force is a small difference of large link terms, so
+// another order of the FP32 sums would change it in the fifth digit.)
 constexpr int FB = 128;                  // threads per solid
 constexpr int FW = FB / 32;
+constexpr int LU = 2;                    // links a thread loads before it works on them
 constexpr float ANN_EPS = 0.05f;         // above the FP32 rounding of a chord end
 
-template <int P, bool LOCAL, bool BND>
-__global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
+template <int P> struct LinkShared {
+    using C = typename Prec<P>::C;
+    int wsum[FW];
+    int cnt[FB];                  // the chunk's rows: exclusive prefix of their candidates
+    int lo[FB], i0[FB], i1[FB];   // row: [lo, hi] minus the inner chord [i0, i1]
+    int4 cand[FB];                // candidate: {cell, x - floor X, y - floor Y, flags}
+    uint16_t link[8 * FB];        // direction | candidate << 4
+    C rho[FB];                    // local density of the candidates (rho_w local)
+    C term[6][LU * FB];           // the terms of the links in hand
+    double part[FW][6];
+};
+
+// Exclusive prefix of n over the block, and its total (whole blocks call it).
+template <int P>
+__device__ __forceinline__ int block_scan(int n, LinkShared<P> &sh, int &total) {
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    int inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(FULL, inc, o);
+        if (lane >= o) inc += v;
+    }
+    __syncthreads();  // wsum's last use, and the tables' the caller rewrites after this
+    if (lane == 31) sh.wsum[wib] = inc;
+    __syncthreads();
+    int before = 0;
+    total = 0;
+#pragma unroll
+    for (int w = 0; w < FW; w++) {
+        if (w < wib) before += sh.wsum[w];
+        total += sh.wsum[w];
+    }
+    return before + inc - n;
+}
+
+// The links of solid s: their sums into lacc (this thread's share; Eq. 4 force
+// and torque, then Eq. 5) and, with GHOST, the returned populations into the solid
+// nodes' slots of fs.  The solid's candidates are taken chunk by chunk of `chunk`
+// <= FB; this block takes the chunks part, part + nparts ...
+//   per link  f_i = f~_i(x_f), the returned f_bb = f_i - 6 w_i rho_w (e_i . v) with
+//   v the solid's velocity at x_s = x_f + e_i / 2 (BND: interpolated from the cut
+//   of the link, v and the lever there); Eq. 4 = e_i f_i - e_opp f_bb, Eq. 5 =
+//   (e_i - v) f_i - (e_opp - v) f_bb, torque (x_s - R) x F (Eq. 7).
+template <int P, bool LOCAL, bool BND, bool GHOST>
+__device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b, int s,
+                                            typename Prec<P>::S *fs, bool owners, bool list,
+                                            long long t, int chunk, int part, int nparts,
+                                            LinkShared<P> &sh, typename Prec<P>::C (&lacc)[6]) {
     using C = typename Prec<P>::C;
     using S = typename Prec<P>::S;
-    constexpr bool SPARSE = !LOCAL && !BND;
-    __shared__ int s_cnt[FB];          // the chunk's rows: exclusive prefix of their candidates
-    __shared__ int s_lo[FB], s_i0[FB], s_i1[FB];  // row: [lo, hi] minus the inner chord [i0, i1]
-    __shared__ double s_part[FW][6];
-    __shared__ float s_disp;
-    const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
     const Lattice &L = p.L;
-    const long long t = *p.t;
-    const S *fs = static_cast<const S *>((t & 1) ? p.f1 : p.f0);  // populations of time t
     const int plane = (int)L.plane;
-    const bool px = L.bc_x == LBM_PERIODIC, py = L.bc_y == LBM_PERIODIC;
-    // the near lists hold at t unless a solid was added or changed since the
-    // last pair test
+    const Centre c(b.ix0, b.iy0, b.fx0, b.fy0);
+    const Wrap wrap(L, b.ix0, b.iy0, b.rc);
+    const float r = sqrtf(b.r2f);
+    const C vx = pick<C>(b.vx, b.vxf), vy = pick<C>(b.vy, b.vyf), om = pick<C>(b.om, b.omf);
+    const C rho0 = pick<C>(p.rho0, p.rho0_f);
+    int j0, j1;
+    rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
+    for (int jc = j0; jc <= j1; jc += FB) {  // rows in chunks of FB
+        // candidates of row jc + tid
+        int lo = 1, hi = 0, i0 = 1, i1 = 0, n = 0;
+        const int j = jc + tid;
+        if (j <= j1 && c.chord(j, r + 1.4143f + ANN_EPS, lo, hi) && lo <= hi) {
+            n = hi - lo + 1;
+            if (c.chord(j, r - ANN_EPS, i0, i1) && i0 <= i1) n -= i1 - i0 + 1;
+        }
+        int total;
+        const int excl = block_scan(n, sh, total);
+        sh.cnt[tid] = excl;
+        sh.lo[tid] = lo;
+        sh.i0[tid] = i0 <= i1 ? i0 : 1;  // an empty inner chord: i0 > i1
+        sh.i1[tid] = i0 <= i1 ? i1 : 0;
+        __syncthreads();
+        for (int base = part * chunk; base < total; base += nparts * chunk) {
+            // candidate e -> row (binary search over the prefix) and column
+            const int e = base + tid;
+            int q = 0;
+#pragma unroll
+            for (int step = FB / 2; step > 0; step >>= 1)
+                if (q + step < FB && sh.cnt[q + step] <= e) q += step;
+            const int jj = jc + q;
+            int iu = sh.lo[q] + (e - sh.cnt[q]);
+            const int a = sh.i0[q], bb = sh.i1[q];
+            if (a <= bb && iu >= a) iu += bb - a + 1;  // step over the inner chord
+            int x = 0, y = 0;
+            const bool here = tid < chunk && e < total && wrap(iu, jj, x, y);
+            const int k = here ? (int)cell_of(L, x, y) : 0;
+            const unsigned m = here ? p.flags[k] : 1u;
+            const bool bounced_node = !(m & 1u) && (m & 0x1FEu);
+            if (!GHOST && list) {
+                // FP16: the node goes to the deferred per-node path's list of step t
+                const unsigned want = __ballot_sync(FULL, bounced_node);
+                if (want) {
+                    int at = 0;
+                    if (lane == 0) at = atomicAdd(p.bnd + (t & 1), __popc(want));
+                    at = __shfl_sync(FULL, at, 0) + __popc(want & ((1u << lane) - 1u));
+                    if (bounced_node) {
+                        if (at < p.bnd_cap) p.bnd[2 + at] = k;
+                        else atomicOr(p.status, 16);
+                    }
+                }
+            }
+            // bit i: x_f + e_i is solid or beyond a wall (bit opp(i) of the flags)
+            unsigned dirs = bounced_node ? ((m & 0x66u) << 2 | (m >> 2 & 0x66u)) : 0u;
+            int nlink;
+            const int mine0 = block_scan(__popc(dirs), sh, nlink), mine1 = mine0 + __popc(dirs);
+            if (LOCAL) {
+                C a9 = 0;
+                if (dirs) {
+                    S fv[9];
+#pragma unroll
+                    for (int q9 = 0; q9 < 9; q9++) fv[q9] = fs[q9 * plane + k];
+#pragma unroll
+                    for (int q9 = 0; q9 < 9; q9++) a9 += (C)cvt_s(fv[q9]);
+                }
+                sh.rho[tid] = Prec<P>::dev ? (C)1 + a9 : a9;
+            }
+            sh.cand[tid] = make_int4(k, iu - c.xi, jj - c.yi, (int)m);
+            for (int at = mine0; dirs; dirs &= dirs - 1)
+                sh.link[at++] = (uint16_t)((__ffs(dirs) - 1) | tid << 4);
+            __syncthreads();
+            for (int l0 = 0; l0 < nlink; l0 += LU * FB) {
+                int4 cd[LU];
+                int kb[LU], dir[LU];
+                S fi_s[LU], fo_s[LU], fn_s[LU];
+                C rho_w[LU];
+                uint16_t own[LU];
+                bool inner[LU];  // BND: x_f - e_i is a fluid node of the domain
+#pragma unroll
+                for (int u = 0; u < LU; u++) {
+                    kb[u] = -1;
+                    const int l = l0 + u * FB + tid;
+                    if (l >= nlink) continue;
+                    const int lk = sh.link[l], i = lk & 15;
+                    const int4 cc = cd[u] = sh.cand[lk >> 4];
+                    dir[u] = i;
+                    rho_w[u] = LOCAL ? sh.rho[lk >> 4] : rho0;
+                    int xb, yb;
+                    if (!wrap(c.xi + cc.y + cx(i), c.yi + cc.z + cy(i), xb, yb)) continue;
+                    kb[u] = (int)cell_of(L, xb, yb);  // else beyond a wall
+                    fi_s[u] = fs[i * plane + cc.x];
+                    if (owners) own[u] = p.owner[kb[u]];
+                    if (BND) {
+                        inner[u] = !((cc.w >> i) & 1);
+                        fo_s[u] = fs[opp(i) * plane + cc.x];
+                        fn_s[u] = fi_s[u];
+                        int xn, yn;
+                        if (inner[u] && wrap(c.xi + cc.y - cx(i), c.yi + cc.z - cy(i), xn, yn))
+                            fn_s[u] = fs[i * plane + (int)cell_of(L, xn, yn)];
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < LU; u++) {
+                    C v[6] = {0, 0, 0, 0, 0, 0};
+                    if (kb[u] >= 0 && !(owners && own[u] != (uint16_t)s)) {
+                        const int i = dir[u], di = cd[u].y, dj = cd[u].z;
+                        const C ex = (C)cx(i), ey = (C)cy(i), w = wgt<C>(i);
+                        const C back = (C)cvt_s(fi_s[u]);  // as stored
+                        const C fi = Prec<P>::dev ? back + w : back;
+                        C dx, dy, ux, uy, fbb, ret = 0;  // ret: f_bb as stored
+                        if (BND) {
+                            C q;  // the link is cut at this fraction
+                            if (Prec<P>::dev) {
+                                q = (C)link_fraction_split(di, dj, c.fx, c.fy, b.r, cx(i), cy(i));
+                                dx = ((C)di - (C)c.fx) + q * ex;
+                                dy = ((C)dj - (C)c.fy) + q * ey;
+                            } else {
+                                // the unwrapped node is at the centre's nearest image
+                                const double px = (double)(c.xi + di) - b.x;
+                                const double py = (double)(c.yi + dj) - b.y;
+                                q = (C)link_fraction_at(px, py, b.r, cx(i), cy(i));
+                                dx = (C)px + q * ex;
+                                dy = (C)py + q * ey;
+                            }
+                            ux = vx - om * dy;
+                            uy = vy + om * dx;
+                            const C mw = -(C)6 * w * rho_w[u] * (ex * ux + ey * uy);
+                            const C q2 = (C)2 * q;
+                            const C fo = (C)cvt_s(fo_s[u]), fn = (C)cvt_s(fn_s[u]);
+                            auto returned = [&](C f, C o, C nb) {
+                                if (q2 >= (C)1) return (f + mw) / q2 + ((q2 - (C)1) / q2) * o;
+                                if (inner[u]) return q2 * f + ((C)1 - q2) * nb + mw;
+                                return f + mw;
+                            };
+                            // full populations for the force; as stored for the pull
+                            // (the interpolation's weights sum to one)
+                            if (Prec<P>::dev) fbb = returned(fi, fo + w, fn + w);
+                            if (GHOST || !Prec<P>::dev) ret = returned(back, fo, fn);
+                            if (!Prec<P>::dev) fbb = ret;
+                        } else {
+                            // x_s = x_f + e_i / 2 relative to R, from the unwrapped coordinate
+                            if (Prec<P>::dev) {
+                                dx = (C)di + (C)0.5 * ex - (C)c.fx;
+                                dy = (C)dj + (C)0.5 * ey - (C)c.fy;
+                            } else {
+                                dx = (C)(((double)(c.xi + di) + 0.5 * (double)ex) - b.x);
+                                dy = (C)(((double)(c.yi + dj) + 0.5 * (double)ey) - b.y);
+                            }
+                            ux = vx - om * dy;
+                            uy = vy + om * dx;
+                            const C a6 = (C)6 * w * rho_w[u], eu = ex * ux + ey * uy;
+                            fbb = fma(-a6, eu, fi);
+                            ret = fma(-a6, eu, back);
+                        }
+                        if (GHOST) st(fs + opp(i) * plane + kb[u], ret);
+                        const C cmx = ex * fi + ex * fbb, cmy = ey * fi + ey * fbb;
+                        const C gmx = (ex - ux) * fi - (-ex - ux) * fbb;
+                        const C gmy = (ey - uy) * fi - (-ey - uy) * fbb;
+                        v[0] = cmx;
+                        v[1] = cmy;
+                        v[2] = dx * cmy - dy * cmx;
+                        v[3] = gmx;
+                        v[4] = gmy;
+                        v[5] = dx * gmy - dy * gmx;
+                    }
+#pragma unroll
+                    for (int q6 = 0; q6 < 6; q6++) sh.term[q6][u * FB + tid] = v[q6];
+                }
+                __syncthreads();
+                // the candidate's thread adds its links' terms
+                for (int l = max(mine0, l0); l < min(mine1, l0 + LU * FB); l++)
+#pragma unroll
+                    for (int q6 = 0; q6 < 6; q6++) lacc[q6] += sh.term[q6][l - l0];
+                __syncthreads();  // the terms (and the list) are reused
+            }
+        }
+    }
+}
+
+// Lane 0's sums over the block of every thread's lacc, in warp order, plus one
+// term per component (acc[q] of lane q < 6), to all lanes of warp 0.
+template <int P>
+__device__ __forceinline__ void block_sums(typename Prec<P>::C (&lacc)[6], LinkShared<P> &sh,
+                                           double (&acc)[6]) {
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    warp_sum(lacc);
+    if (lane == 0)
+        for (int q = 0; q < 6; q++) sh.part[wib][q] = (double)lacc[q];
+    __syncthreads();
+    if (wib != 0) return;
+    double aq = 0.0;
+    if (lane < 6)
+        for (int w = 0; w < FW; w++) aq += sh.part[w][lane];
+#pragma unroll
+    for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
+}
+
+// The momenta booked into the record of t by the node-type changes of the step
+// before: component q of the solid's event segment, in order, in lane q < 6.
+__device__ __forceinline__ void booked_events(const StepParams &p, const DSolid &b, long long t,
+                                              int lane, double (&booked)[6]) {
+    double bq = 0.0;
+    if (lane < 6 && b.ev_t == t)
+        for (int e0 = 0; e0 < b.ev_n; e0 += 8) {  // eight loads in flight, added in order
+            double v[8];
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                v[k] = e0 + k < b.ev_n ? p.ev_mom[6 * (b.ev_off + e0 + k) + lane] : 0.0;
+#pragma unroll
+            for (int k = 0; k < 8; k++)
+                if (e0 + k < b.ev_n) bq += v[k];
+        }
+#pragma unroll
+    for (int q = 0; q < 6; q++) booked[q] = __shfl_sync(FULL, bq, q);
+}
+
+// Distance of the solid's centre at t and t+1 from that at the last pair test
+// (FP32 from the split centres, with a slack above its rounding).
+__device__ __forceinline__ float displacement(const DSolid &b) {
+    const float d0 = hypotf((float)(b.ix0 - b.ixt) + (b.fx0 - b.fxt),
+                            (float)(b.iy0 - b.iyt) + (b.fy0 - b.fyt));
+    const float d1 = hypotf((float)(b.ix1 - b.ixt) + (b.fx1 - b.fxt),
+                            (float)(b.iy1 - b.iyt) + (b.fy1 - b.fyt));
+    return fmaxf(d0, d1) + 1e-3f;
+}
+
+// FP16 rounds a returned population: it stays in registers there (sc_tile).
+template <int P>
+__host__ __device__ constexpr bool ghosts() {
+    return P != LBM_FP16_DEV;
+}
+
+// The near lists hold at t unless a solid was added or changed since the last
+// pair test; without them (or with solids in reach) a link's owner is read.
+__device__ __forceinline__ bool need_owners(const StepParams &p, const DSolid &b) {
     const bool lists_ok = p.near_id && ((volatile unsigned int *)p.bar)[3] == 0u;
+    return !lists_ok || b.near_n != 0;
+}
+
+// The half-way boundary: links, record and motion of one solid per block.
+template <int P, bool LOCAL>
+__global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
+    using S = typename Prec<P>::S;
+    __shared__ LinkShared<P> sh;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const long long t = *p.t;
+    S *fs = static_cast<S *>((t & 1) ? p.f1 : p.f0);  // populations of time t
     // the previous step's events are reached through the solids' segments;
     // the list fills again in this step's re-rasterisation
     if (blockIdx.x == 0 && tid == 0 && p.ev_len) {
         *p.ev_len = 0;
         *p.chg_len = 0;
     }
-    if (tid == 0) s_disp = 0.f;
+    float disp = 0.f;
     for (int s = blockIdx.x; s < p.nsolid; s += gridDim.x) {
         DSolid &b = p.S[s];
         if (!solid_ok(b)) {
             if (tid == 0) atomicOr(p.status, 2);
             continue;
         }
-        const Centre c(b.ix0, b.iy0, b.fx0, b.fy0);
-        const Wrap wrap(L, b.ix0, b.iy0, b.rc);
-        const float r = sqrtf(b.r2f);
-        const bool owners = !lists_ok || b.near_n != 0;
-        const C vx = pick<C>(b.vx, b.vxf), vy = pick<C>(b.vy, b.vyf), om = pick<C>(b.om, b.omf);
-        const C rho0 = pick<C>(p.rho0, p.rho0_f);
-        int j0, j1;
-        rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
-        C lacc[6] = {0, 0, 0, 0, 0, 0};
-        for (int jc = j0; jc <= j1; jc += FB) {  // rows in chunks of FB
-            // candidates of row jc + tid
-            int lo = 1, hi = 0, i0 = 1, i1 = 0, n = 0;
-            const int j = jc + tid;
-            if (j <= j1 && c.chord(j, r + 1.4143f + ANN_EPS, lo, hi) && lo <= hi) {
-                n = hi - lo + 1;
-                if (c.chord(j, r - ANN_EPS, i0, i1) && i0 <= i1) n -= i1 - i0 + 1;
-            }
-            // exclusive prefix over the block
-            int inc = n;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(FULL, inc, o);
-                if (lane >= o) inc += v;
-            }
-            if (lane == 31) s_cnt[wib] = inc;
-            __syncthreads();
-            if (tid < 32) {
-                int w = tid < FW ? s_cnt[tid] : 0;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int v = __shfl_up_sync(FULL, w, o);
-                    if (lane >= o) w += v;
-                }
-                if (tid < FW) s_cnt[tid] = w;  // inclusive over warps
-            }
-            __syncthreads();
-            const int excl = (wib ? s_cnt[wib - 1] : 0) + inc - n;
-            const int total = s_cnt[FW - 1];
-            __syncthreads();
-            s_cnt[tid] = excl;
-            s_lo[tid] = lo;
-            s_i0[tid] = i0 <= i1 ? i0 : 1;  // an empty inner chord: i0 > i1
-            s_i1[tid] = i0 <= i1 ? i1 : 0;
-            __syncthreads();
-            // candidate e -> row (binary search over the prefix) and column; every
-            // thread runs the same iterations (the list append is warp-wide)
-            for (int base = 0; base < total; base += FB) {
-                const int e = base + tid;
-                int q = 0;
-#pragma unroll
-                for (int step = FB / 2; step > 0; step >>= 1)
-                    if (q + step < FB && s_cnt[q + step] <= e) q += step;
-                const int jj = jc + q;
-                int iu = s_lo[q] + (e - s_cnt[q]);
-                const int a = s_i0[q], bb = s_i1[q];
-                if (a <= bb && iu >= a) iu += bb - a + 1;  // step over the inner chord
-                int x = 0, y = 0;
-                const bool here = e < total && wrap(iu, jj, x, y);
-                const int k = here ? (int)cell_of(L, x, y) : 0;
-                const uint16_t m = here ? p.flags[k] : (uint16_t)1u;
-                const bool bounced_node = !(m & 1u) && (m & 0x1FEu);
-                if (p.list_by_forces) {
-                    // the node goes to the deferred per-node path's list of step t
-                    const unsigned want = __ballot_sync(FULL, bounced_node);
-                    if (want) {
-                        int at = 0;
-                        if (lane == 0) at = atomicAdd(p.bnd + (t & 1), __popc(want));
-                        at = __shfl_sync(FULL, at, 0) + __popc(want & ((1u << lane) - 1u));
-                        if (bounced_node) {
-                            if (at < p.bnd_cap) p.bnd[2 + at] = k;
-                            else atomicOr(p.status, 16);
-                        }
-                    }
-                }
-                if (!bounced_node) continue;  // solid, or no bounced population
-                S fv[9];
-                uint16_t own[9];
-#pragma unroll
-                for (int i = 1; i < 9; i++) {
-                    const bool bounced = (m >> opp(i)) & 1u;  // x_f + e_i is solid
-                    if (!SPARSE || bounced) fv[i] = fs[i * plane + k];
-                    if (owners && bounced) {
-                        const int kb = neighbour(L, x, y, cx(i), cy(i));
-                        own[i] = kb >= 0 ? p.owner[kb] : FLUID;
-                    }
-                }
-                if (!SPARSE) fv[0] = fs[k];
-                C rho_w = rho0;
-                if (LOCAL) {
-                    C a9 = 0;
-#pragma unroll
-                    for (int q9 = 0; q9 < 9; q9++) a9 += (C)cvt_s(fv[q9]);
-                    rho_w = Prec<P>::dev ? (C)1 + a9 : a9;
-                }
-#pragma unroll
-                for (int i = 1; i < 9; i++) {
-                    if (!((m >> opp(i)) & 1u)) continue;  // x_f + e_i is not solid
-                    if (owners) {
-                        if (own[i] != (uint16_t)s) continue;
-                    } else if ((!px && (unsigned)(iu + cx(i)) >= (unsigned)L.nx) ||
-                               (!py && (unsigned)(jj + cy(i)) >= (unsigned)L.ny)) {
-                        continue;  // beyond a wall, not a solid
-                    }
-                    C dx, dy, ux, uy, fbb;
-                    C fi = (C)cvt_s(fv[i]);
-                    if (Prec<P>::dev) fi += wgt<C>(i);
-                    if (BND) {
-                        // the cut at fraction q of the link, and the population that
-                        // returns to x_f along e_opp by the fused kernel's
-                        // interpolation (full populations; M = 6 w rho_w (e_opp . v))
-                        C qf;
-                        if (Prec<P>::dev) {  // FP32 from the unwrapped offset, split
-                            qf = (C)link_fraction_split(iu - c.xi, jj - c.yi, c.fx, c.fy, b.r,
-                                                        cx(i), cy(i));
-                            dx = ((C)(iu - c.xi) - (C)c.fx) + qf * (C)cx(i);
-                            dy = ((C)(jj - c.yi) - (C)c.fy) + qf * (C)cy(i);
-                            ux = (C)b.vxf - (C)b.omf * dy;
-                            uy = (C)b.vyf + (C)b.omf * dx;
-                        } else {
-                            const double qd = link_fraction(L, b, x, y, i);
-                            double vxd, vyd, ddx, ddy;
-                            point_velocity(L, b.x, b.y, b.vx, b.vy, b.om, (double)x + qd * cx(i),
-                                           (double)y + qd * cy(i), vxd, vyd, ddx, ddy);
-                            qf = (C)qd;
-                            dx = (C)ddx;
-                            dy = (C)ddy;
-                            ux = (C)vxd;
-                            uy = (C)vyd;
-                        }
-                        const C mw =
-                            -(C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * ux + (C)cy(i) * uy);
-                        C fo = (C)cvt_s(fv[opp(i)]);
-                        if (Prec<P>::dev) fo += wgt<C>(i);
-                        const C q2 = (C)2 * qf;
-                        if (q2 >= (C)1) {
-                            fbb = (fi + mw) / q2 + ((q2 - (C)1) / q2) * fo;
-                        } else if (!((m >> i) & 1u)) {  // x_f - e_i is a fluid node
-                            int xn, yn;
-                            locate(L, x - cx(i), y - cy(i), xn, yn);
-                            C fn = (C)cvt_s(fs[i * plane + (int)cell_of(L, xn, yn)]);
-                            if (Prec<P>::dev) fn += wgt<C>(i);
-                            fbb = q2 * fi + ((C)1 - q2) * fn + mw;
-                        } else {
-                            fbb = fi + mw;
-                        }
-                    } else {
-                        // x_s = x_f + e_i / 2 relative to R, from the unwrapped coordinate
-                        if (Prec<P>::dev) {
-                            dx = (C)(iu - c.xi) + (C)(0.5f * cx(i)) - (C)c.fx;
-                            dy = (C)(jj - c.yi) + (C)(0.5f * cy(i)) - (C)c.fy;
-                        } else {
-                            dx = (C)(((double)iu + 0.5 * cx(i)) - b.x);
-                            dy = (C)(((double)jj + 0.5 * cy(i)) - b.y);
-                        }
-                        ux = vx - om * dy;
-                        uy = vy + om * dx;
-                        fbb = fi - (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * ux + (C)cy(i) * uy);
-                    }
-                    const C cmx = (C)cx(i) * fi - (C)cx(opp(i)) * fbb;
-                    const C cmy = (C)cy(i) * fi - (C)cy(opp(i)) * fbb;
-                    const C gmx = ((C)cx(i) - ux) * fi - ((C)cx(opp(i)) - ux) * fbb;
-                    const C gmy = ((C)cy(i) - uy) * fi - ((C)cy(opp(i)) - uy) * fbb;
-                    lacc[0] += cmx;
-                    lacc[1] += cmy;
-                    lacc[2] += dx * cmy - dy * cmx;
-                    lacc[3] += gmx;
-                    lacc[4] += gmy;
-                    lacc[5] += dx * gmy - dy * gmx;
-                }
-            }
-            __syncthreads();  // the chunk's tables are reused
-        }
-        warp_sum(lacc);
-        if (lane == 0)
-            for (int q = 0; q < 6; q++) s_part[wib][q] = (double)lacc[q];
-        __syncthreads();
-        if (wib == 0) {
-            // lane q < 6 sums component q over the warps and over the booked
-            // events, each in order; lane 0 gathers them
-            double aq = 0.0, bq = 0.0;
-            if (lane < 6) {
-                for (int w = 0; w < FW; w++) aq += s_part[w][lane];
-                if (b.ev_t == t)
-                    for (int e = b.ev_off; e < b.ev_off + b.ev_n; e++) bq += p.ev_mom[6 * e + lane];
-            }
-            double acc[6], booked[6];
-#pragma unroll
-            for (int q = 0; q < 6; q++) {
-                acc[q] = __shfl_sync(FULL, aq, q);
-                booked[q] = __shfl_sync(FULL, bq, q);
-            }
+        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
+        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
+                                                 FB, 0, 1, sh, lacc);
+        double acc[6];
+        block_sums(lacc, sh, acc);
+        if (tid < 32) {
+            double booked[6];
+            booked_events(p, b, t, lane, booked);
             record_forces(p, s, lane, t, acc, booked);
-            if (lane == 0) {
-                // distance from the centre at the last pair test, at t and t+1 (FP32
-                // from the split centres, with a slack above its rounding)
-                const float d0 = hypotf((float)(b.ix0 - b.ixt) + (b.fx0 - b.fxt),
-                                        (float)(b.iy0 - b.iyt) + (b.fy0 - b.fyt));
-                const float d1 = hypotf((float)(b.ix1 - b.ixt) + (b.fx1 - b.fxt),
-                                        (float)(b.iy1 - b.iyt) + (b.fy1 - b.fyt));
-                s_disp = fmaxf(s_disp, fmaxf(d0, d1) + 1e-3f);
-            }
+            if (lane == 0) disp = fmaxf(disp, displacement(b));
         }
-        __syncthreads();  // s_part is reused
+        __syncthreads();  // sh.part is reused
     }
-    if (tid == 0 && s_disp > 0.f)  // non-negative: bits order as values
-        atomicMax(p.bar + 2, __float_as_uint(s_disp));
+    if (tid == 0 && disp > 0.f)  // non-negative: bits order as values
+        atomicMax(p.bar + 2, __float_as_uint(disp));
+}
+
+// The same in two kernels: k_links, after which the advection-collision kernel can
+// run, and k_record (records and motion), beside it.  A solid's links go to
+// gridDim.y blocks: one, or LINK_PARTS that take its candidates 32 at a time in
+// turn, each the share of one warp of the single block, so that the sums are the
+// same bit for bit.  (With the interpolated boundary one 30-node disk in FP64 took
+// 68 us in one block with a thread per candidate: one SM's FP64 unit.)
+constexpr int LINK_CHUNK = FB / LINK_PARTS;
+
+template <int P, bool LOCAL, bool BND>
+__global__ void __launch_bounds__(FB) k_links(const StepParams p) {
+    using S = typename Prec<P>::S;
+    __shared__ LinkShared<P> sh;
+    const long long t = *p.t;
+    S *fs = static_cast<S *>((t & 1) ? p.f1 : p.f0);
+    for (int s = blockIdx.x; s < p.nsolid; s += gridDim.x) {
+        const DSolid &b = p.S[s];
+        if (!solid_ok(b)) continue;  // k_record reports it
+        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
+        solid_links<P, LOCAL, BND, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
+                                                gridDim.y > 1 ? LINK_CHUNK : FB, blockIdx.y,
+                                                gridDim.y, sh, lacc);
+        double acc[6];
+        block_sums(lacc, sh, acc);
+        if (threadIdx.x == 0)
+            for (int q = 0; q < 6; q++) p.part[((long long)s * LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
+    const int lane = threadIdx.x & 31;
+    const long long t = *p.t;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.ev_len) {
+        *p.ev_len = 0;
+        *p.chg_len = 0;
+    }
+    const int s = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    if (s >= p.nsolid) return;
+    DSolid &b = p.S[s];
+    if (!solid_ok(b)) {
+        if (lane == 0) atomicOr(p.status, 2);
+        return;
+    }
+    double aq = 0.0, acc[6], booked[6];
+    if (lane < 6)
+        for (int c = 0; c < p.link_parts; c++) aq += p.part[((long long)s * LINK_PARTS + c) * 6 + lane];
+#pragma unroll
+    for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
+    booked_events(p, b, t, lane, booked);
+    record_forces(p, s, lane, t, acc, booked);
+    if (lane == 0) atomicMax(p.bar + 2, __float_as_uint(displacement(b)));
 }
 
 // ----------------------------------------------------- re-rasterisation
@@ -1309,7 +1296,7 @@ __global__ void __launch_bounds__(SW_BLOCK, 4) k_remask(const StepParams p) {
     for (int m = gt; m < p.nmoving; m += nt) advance_solid(L, p.S[p.moving[m]]);
 }
 
-template <int P, bool LOCAL, bool BND>
+template <int P, bool LOCAL>
 cudaError_t launch_f(const StepParams &p, cudaStream_t st) {
     static int per_sm = -1, sms = 0;
     if (per_sm < 0) {
@@ -1317,14 +1304,19 @@ cudaError_t launch_f(const StepParams &p, cudaStream_t st) {
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forces<P, LOCAL, BND>,
-                                                              FB, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forces<P, LOCAL>, FB, 0);
         if (e != cudaSuccess) return e;
     }
     int blocks = p.nsolid;  // one solid per block, looped beyond the resident blocks
     if (blocks > 8 * per_sm * sms) blocks = 8 * per_sm * sms;
     if (blocks < 1) blocks = 1;
-    k_forces<P, LOCAL, BND><<<blocks, FB, 0, st>>>(p);
+    if (!p.link_parts) {
+        k_forces<P, LOCAL><<<blocks, FB, 0, st>>>(p);
+        return cudaGetLastError();
+    }
+    const dim3 grid(blocks, p.link_parts);
+    if (p.boundary == LBM_INTERPOLATED) k_links<P, LOCAL, true><<<grid, FB, 0, st>>>(p);
+    else k_links<P, LOCAL, false><<<grid, FB, 0, st>>>(p);
     return cudaGetLastError();
 }
 
@@ -1339,9 +1331,11 @@ cudaError_t launch_r(const StepParams &p, cudaStream_t st) {
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_remask<P>, SW_BLOCK, 0);
         if (e != cudaSuccess) return e;
     }
-    // every resident block: the changes go to every thread, the events to
-    // every warp
+    // the changes go to every thread, the events to every warp: up to every
+    // resident block, but not many more warps than a step has events (tens per
+    // moving solid), for the barrier waits for all of them
     int blocks = per_sm * sms;
+    if (blocks > 4LL * p.nmoving) blocks = 4 * p.nmoving;
     if (blocks < 1) blocks = 1;
     StepParams pp = p;
     void *args[] = {&pp};
@@ -1351,45 +1345,41 @@ cudaError_t launch_r(const StepParams &p, cudaStream_t st) {
 
 // ------------------------------------------------------------- batch
 
-// Force records of a batch of independent domains whose solids rest: one
-// block per (case, solid) item of the active list, phase F only.  The last
-// block to finish (a ticket, no waiting) advances the step counter of every
-// active case and swaps its population buffers (batch convention: f0 holds
-// the current time), after every block has read them.
+// Force records of a batch of independent domains whose solids rest, the first
+// kernel of a step: one block per (case, solid) item of the active list (the links
+// and the record, as k_forces).  The last block to finish (a ticket, no waiting)
+// advances the step counter of every active case and swaps its population
+// buffers, after every block has read them.  Batch convention: between steps f0
+// holds the current populations; the fused kernel, which comes after this swap,
+// reads f1 and writes f0.
 template <int P, bool LOCAL>
-__global__ void __launch_bounds__(SW_BLOCK, 2)
+__global__ void __launch_bounds__(FB, 8)
     k_solids_batch(StepParams *cases, const int2 *__restrict__ items,
                    const int *__restrict__ nitems, const int *__restrict__ active,
                    const int *__restrict__ nactive, unsigned int *ticket) {
+    using S = typename Prec<P>::S;
     __shared__ bool last;
-    __shared__ double part[WARPS][6];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    __shared__ LinkShared<P> sh;
     const int n = *nitems;
-    // one block per item: the warps share the disk's rows, then warp 0 adds
-    // their sums in warp order
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         const int2 it = items[k];
         const StepParams &p = cases[it.x];
         const long long t = *p.t;
-        const void *fcur = p.f0;  // batch convention: f0 holds time t
-        if (!solid_ok(p.S[it.y])) {
+        const DSolid &b = p.S[it.y];
+        if (!solid_ok(b)) {
             if (threadIdx.x == 0) atomicOr(p.status, 2);
             continue;
         }
+        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
+        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, FB,
+                                                 0, 1, sh, lacc);
         double acc[6];
-        forces_sum<P, LOCAL>(p, it.y, lane, fcur, wib, WARPS, false, acc);
-        if (lane == 0)
-            for (int q = 0; q < 6; q++) part[wib][q] = acc[q];
-        __syncthreads();
-        if (wib == 0) {
-            double tot[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-            if (lane == 0)
-                for (int w = 0; w < WARPS; w++)
-                    for (int q = 0; q < 6; q++) tot[q] += part[w][q];
+        block_sums(lacc, sh, acc);
+        if (threadIdx.x < 32) {
             const double none[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // resting: no node changes type
-            record_forces(p, it.y, lane, t, tot, none);
+            record_forces(p, it.y, threadIdx.x, t, acc, none);
         }
-        __syncthreads();
+        __syncthreads();  // sh.part is reused
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1403,7 +1393,7 @@ __global__ void __launch_bounds__(SW_BLOCK, 2)
     for (int a = threadIdx.x; a < na; a += blockDim.x) {
         StepParams &p = cases[active[a]];
         *p.t += 1;
-        void *f = p.f0;  // the populations of t+1 become the current ones
+        void *f = p.f0;  // the buffer that the step fills becomes the current one
         p.f0 = p.f1;
         p.f1 = f;
     }
@@ -1419,13 +1409,13 @@ cudaError_t launch_sb(const BatchLaunch &b, cudaStream_t st) {
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solids_batch<P, LOCAL>,
-                                                              SW_BLOCK, 0);
+                                                              FB, 0);
         if (e != cudaSuccess) return e;
     }
     int blocks = b.max_items;
     if (blocks > per_sm * sms) blocks = per_sm * sms;
     if (blocks < 1) blocks = 1;
-    k_solids_batch<P, LOCAL><<<blocks, SW_BLOCK, 0, st>>>(b.cases, b.items, b.nitems, b.active,
+    k_solids_batch<P, LOCAL><<<blocks, FB, 0, st>>>(b.cases, b.items, b.nitems, b.active,
                                                           b.nactive, b.ticket);
     return cudaGetLastError();
 }
@@ -1580,16 +1570,19 @@ cudaError_t launch_batch_converge(const BatchLaunch &b, const BatchState &s, int
 
 cudaError_t launch_forces(const StepParams &p, cudaStream_t st) {
     if (p.nsolid == 0) return cudaSuccess;
-    const bool local = p.rho_w_mode == LBM_RHOW_LOCAL, bnd = p.boundary == LBM_INTERPOLATED;
-#define GBM_F(P)                                                                            \
-    return local ? (bnd ? launch_f<P, true, true>(p, st) : launch_f<P, true, false>(p, st)) \
-                 : (bnd ? launch_f<P, false, true>(p, st) : launch_f<P, false, false>(p, st))
+    const bool local = p.rho_w_mode == LBM_RHOW_LOCAL;
     switch (p.precision) {
-        case LBM_FP64: GBM_F(LBM_FP64);
-        case LBM_FP32_DEV: GBM_F(LBM_FP32_DEV);
-        default: GBM_F(LBM_FP16_DEV);
+        case LBM_FP64: return local ? launch_f<LBM_FP64, true>(p, st) : launch_f<LBM_FP64, false>(p, st);
+        case LBM_FP32_DEV:
+            return local ? launch_f<LBM_FP32_DEV, true>(p, st) : launch_f<LBM_FP32_DEV, false>(p, st);
+        default: return local ? launch_f<LBM_FP16_DEV, true>(p, st) : launch_f<LBM_FP16_DEV, false>(p, st);
     }
-#undef GBM_F
+}
+
+cudaError_t launch_record(const StepParams &p, cudaStream_t st) {
+    if (p.nsolid == 0 || !p.link_parts) return cudaSuccess;
+    k_record<<<(p.nsolid + WARPS - 1) / WARPS, SW_BLOCK, 0, st>>>(p);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_ring(const StepParams &p, cudaStream_t st) {

@@ -1,49 +1,63 @@
-// Fused pull-advection + half-way bounce-back + BGK collision (Eq. 1-3, Eq. 8)
-// on one domain: one block per tile (row y, SC_BLOCK_X * V nodes); and the
-// open-channel columns pass.  The device code is in k_stream_collide.cuh.
+// Fused pull-advection + bounce-back + collision (Eq. 1-3, Eq. 8) on one domain.
+// The device code is in k_stream_collide.cuh: sc_row for FP64 and FP32 storage
+// (after the force kernel, which leaves the returned populations in the solid
+// nodes' slots), sc_tile for FP16.
 #include "k_stream_collide.cuh"
 
 namespace gbm {
 
 namespace {
 
-template <int P, int V, bool FORCE, bool LOCAL, bool WALLS, bool DEFER, int COLL = 0,
-          bool BND = false>
+// One block per SC_BLOCK_X * V nodes of a row.
+template <int P, int V, bool FORCE, bool OPEN, int COLL>
 __global__ void __launch_bounds__(SC_BLOCK_X) k_stream_collide(const StepParams p) {
-    sc_tile<P, V, FORCE, LOCAL, false, WALLS, DEFER, COLL, BND>(p, blockIdx.x, blockIdx.y);
+    using R = typename Raw<P>::R;
+    const long long t = *p.t;
+    sc_row<P, V, FORCE, OPEN, COLL>(p, static_cast<const R *>((t & 1) ? p.f1 : p.f0),
+                                    static_cast<R *>((t & 1) ? p.f0 : p.f1),
+                                    (blockIdx.x * SC_BLOCK_X + threadIdx.x) * V, blockIdx.y);
 }
 
-// With the per-node path deferred (variants 3-5), the nodes k_stream_collide
-// leaves to the per-node update (update_node) are computed from the same
-// populations after it, by k_boundary_update: one thread per node of the
-// step's list of fluid nodes next to solids, then of the first and last
-// columns and, where the vector path does not take them, of the wall rows.
-// The force kernel of the step fills the list: it visits every fluid node
-// with a link into its solid (one atomic per warp and list chunk).  The
-// list's length is kept per step parity; the update kernel of step t clears
-// the slot of step t + 1.  A node next to two disks is computed twice, with
-// identical results.  Inline in the vector path these nodes run with one or
-// two active lanes per warp; which way is faster depends on the workload (the
-// autotuner measures both).
+template <int V, bool FORCE, bool LOCAL, bool DEFER, int COLL = 0, bool BND = false>
+__global__ void __launch_bounds__(SC_BLOCK_X) k_stream_collide16(const StepParams p) {
+    constexpr int P = LBM_FP16_DEV;
+    using R = Raw<P>::R;
+    const long long t = *p.t;
+    sc_tile<P, V, FORCE, LOCAL, false, DEFER, COLL, BND>(
+        p, static_cast<const R *>((t & 1) ? p.f1 : p.f0), static_cast<R *>((t & 1) ? p.f0 : p.f1),
+        (blockIdx.x * SC_BLOCK_X + threadIdx.x) * V, blockIdx.y);
+}
+
+// FP16 with the per-node path deferred (variants 3-5): the nodes that
+// k_stream_collide16 leaves to the per-node update (update_node) are computed
+// from the same populations after it, by k_boundary_update: one thread per node
+// of the step's list of fluid nodes next to solids, then of the first and last
+// columns and of the wall rows.  The force kernel of the step fills the list: it
+// visits every fluid node with a link into its solid (one atomic per warp and
+// list chunk).  The list's length is kept per step parity; the update kernel of
+// step t clears the slot of step t + 1.  A node next to two disks is computed
+// twice, with identical results.  Inline in the vector path these nodes run with
+// one or two active lanes per warp; which way is faster depends on the workload
+// (the autotuner measures both).
 constexpr int BN_BLOCK = 256;
 
-template <int P, bool FORCE, bool LOCAL>
-__host__ __device__ long long boundary_edge_nodes(const Lattice &L) {
+__host__ __device__ inline long long boundary_edge_nodes(const Lattice &L) {
     long long n = L.nx > 1 ? 2LL * L.ny : (long long)L.ny;
-    if (!walls_on_vector_path<P, LOCAL>() && L.bc_y == LBM_WALL && L.nx > 2) n += 2LL * (L.nx - 2);
+    if (L.bc_y == LBM_WALL && L.nx > 2) n += 2LL * (L.nx - 2);
     return n;
 }
 
-template <int P, bool FORCE, bool LOCAL, bool BND>
+template <bool FORCE, bool LOCAL, bool BND>
 __global__ void __launch_bounds__(BN_BLOCK) k_boundary_update(const StepParams p) {
-    using R = typename Raw<P>::R;
+    constexpr int P = LBM_FP16_DEV;
+    using R = Raw<P>::R;
     const Lattice &L = p.L;
     const long long t = *p.t;
     const R *fin = static_cast<const R *>((t & 1) ? p.f1 : p.f0);
     R *fout = static_cast<R *>((t & 1) ? p.f0 : p.f1);
     const int nlist = (p.nsolid > 0 && p.bnd) ? min(p.bnd[t & 1], p.bnd_cap) : 0;
     const int ncol = L.nx > 1 ? 2 * L.ny : L.ny;
-    const long long total = nlist + boundary_edge_nodes<P, FORCE, LOCAL>(L);
+    const long long total = nlist + boundary_edge_nodes(L);
     for (long long e = (long long)blockIdx.x * BN_BLOCK + threadIdx.x; e < total;
          e += (long long)gridDim.x * BN_BLOCK) {
         int x, y;
@@ -66,38 +80,52 @@ __global__ void __launch_bounds__(BN_BLOCK) k_boundary_update(const StepParams p
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.bnd) p.bnd[(t + 1) & 1] = 0;
 }
 
-// Open-channel columns of every row, on the populations of t+1.
-template <int P, bool FORCE>
+// FP16: open-channel columns of every row, on the populations of t+1.
+template <bool FORCE>
 __global__ void k_open_columns(const StepParams p) {
-    using R = typename Raw<P>::R;
+    using R = Raw<LBM_FP16_DEV>::R;
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= p.L.ny) return;
     const long long t = *p.t;
-    open_row<P, FORCE>(p, static_cast<R *>((t & 1) ? p.f0 : p.f1), y);
+    open_row<LBM_FP16_DEV, FORCE>(p, static_cast<R *>((t & 1) ? p.f0 : p.f1), y);
 }
 
-template <int P, bool FORCE, bool LOCAL>
-cudaError_t launch_update(const StepParams &p, cudaStream_t st);
+// ------------------------------------------------------------ FP64, FP32
 
-// Walled domains (y walls) with rho_w = rho0 in FP32/FP64 take the kernel
-// whose vector path also covers the wall rows.
-template <int P, int V, bool FORCE, bool LOCAL, bool DEFER>
-cudaError_t launch_sc(const StepParams &p, cudaStream_t st) {
-    dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
-    if (walls_on_vector_path<P, LOCAL>() && p.L.bc_y == LBM_WALL)
-        k_stream_collide<P, V, FORCE, LOCAL, walls_on_vector_path<P, LOCAL>(), DEFER>
-            <<<grid, SC_BLOCK_X, 0, st>>>(p);
+template <int P, int V, bool FORCE, int COLL>
+cudaError_t launch_row(const StepParams &p, cudaStream_t st) {
+    const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
+    if (p.L.bc_x == LBM_OPEN)
+        k_stream_collide<P, V, FORCE, true, COLL><<<grid, SC_BLOCK_X, 0, st>>>(p);
     else
-        k_stream_collide<P, V, FORCE, LOCAL, false, DEFER><<<grid, SC_BLOCK_X, 0, st>>>(p);
-    cudaError_t e = cudaGetLastError();
-    // with solids, the force kernel lists the nodes next to them and the
-    // host launches the update after it (launch_deferred_update)
-    if (e != cudaSuccess || !DEFER || p.list_by_forces) return e;
-    return launch_update<P, FORCE, LOCAL>(p, st);
+        k_stream_collide<P, V, FORCE, false, COLL><<<grid, SC_BLOCK_X, 0, st>>>(p);
+    return cudaGetLastError();
 }
+
+template <int P, int V>
+cudaError_t launch_row_v(const StepParams &p, cudaStream_t st) {
+    if (p.body_x != 0.0 || p.body_y != 0.0) return launch_row<P, V, true, 0>(p, st);
+    return launch_row<P, V, false, 0>(p, st);
+}
+
+// Node widths per thread: variants 0 and 3 one 16-byte word per population,
+// 1 and 4 8 bytes, 2 and 5 4 bytes (FP64: one node).  MRT: 8-byte words.
+template <int P>
+cudaError_t launch_row_p(const StepParams &p, cudaStream_t st) {
+    constexpr int V16 = 16 / (int)sizeof(typename Raw<P>::R);
+    constexpr int V4 = V16 / 4 > 0 ? V16 / 4 : 1;
+    if (p.collision == LBM_MRT) return launch_row<P, V16 / 2, false, 1>(p, st);
+    switch (p.sc_variant % 3) {
+        case 1: return launch_row_v<P, V16 / 2>(p, st);
+        case 2: return launch_row_v<P, V4>(p, st);
+        default: return launch_row_v<P, V16>(p, st);
+    }
+}
+
+// ------------------------------------------------------------------ FP16
 
 // The update kernel of the deferred per-node path, over the list of step t.
-template <int P, bool FORCE, bool LOCAL>
+template <bool FORCE, bool LOCAL>
 cudaError_t launch_update(const StepParams &p, cudaStream_t st) {
     cudaError_t e = cudaSuccess;
     static int sms = 0;
@@ -107,64 +135,62 @@ cudaError_t launch_update(const StepParams &p, cudaStream_t st) {
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
     }
-    const long long most = (p.nsolid > 0 ? p.bnd_cap : 0) + boundary_edge_nodes<P, FORCE, LOCAL>(p.L);
+    const long long most = (p.nsolid > 0 ? p.bnd_cap : 0) + boundary_edge_nodes(p.L);
     long long blocks = (most + BN_BLOCK - 1) / BN_BLOCK;
     if (blocks > 8LL * sms) blocks = 8LL * sms;
     if (blocks < 1) blocks = 1;
     if (p.boundary == LBM_INTERPOLATED)
-        k_boundary_update<P, FORCE, LOCAL, true><<<(unsigned)blocks, BN_BLOCK, 0, st>>>(p);
+        k_boundary_update<FORCE, LOCAL, true><<<(unsigned)blocks, BN_BLOCK, 0, st>>>(p);
     else
-        k_boundary_update<P, FORCE, LOCAL, false><<<(unsigned)blocks, BN_BLOCK, 0, st>>>(p);
+        k_boundary_update<FORCE, LOCAL, false><<<(unsigned)blocks, BN_BLOCK, 0, st>>>(p);
     return cudaGetLastError();
 }
 
-template <int P, int V, bool DEFER>
+template <int V, bool FORCE, bool LOCAL, bool DEFER>
+cudaError_t launch_sc(const StepParams &p, cudaStream_t st) {
+    const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
+    k_stream_collide16<V, FORCE, LOCAL, DEFER><<<grid, SC_BLOCK_X, 0, st>>>(p);
+    cudaError_t e = cudaGetLastError();
+    // with solids, the force kernel lists the nodes next to them and the
+    // host launches the update after it (launch_deferred_update)
+    if (e != cudaSuccess || !DEFER || p.list_by_forces) return e;
+    return launch_update<FORCE, LOCAL>(p, st);
+}
+
+template <int V, bool DEFER>
 cudaError_t launch_sc_v(const StepParams &p, cudaStream_t st) {
     const bool force = p.body_x != 0.0 || p.body_y != 0.0;
     const bool local = p.rho_w_mode == LBM_RHOW_LOCAL;
     if (force)
-        return local ? launch_sc<P, V, true, true, DEFER>(p, st)
-                     : launch_sc<P, V, true, false, DEFER>(p, st);
-    return local ? launch_sc<P, V, false, true, DEFER>(p, st)
-                 : launch_sc<P, V, false, false, DEFER>(p, st);
+        return local ? launch_sc<V, true, true, DEFER>(p, st) : launch_sc<V, true, false, DEFER>(p, st);
+    return local ? launch_sc<V, false, true, DEFER>(p, st) : launch_sc<V, false, false, DEFER>(p, st);
 }
 
-// Node widths per thread: variant 0 = one 16-byte word per population,
-// variant 1 = 8 bytes, variant 2 = 4 bytes; variants 3-5 the same widths
-// with the per-node path deferred to k_boundary_update.
 // MRT: one launch shape, 8-byte words per population plane, slow nodes inline.
-template <int P, bool LOCAL, bool BND>
-cudaError_t launch_mrt_b(const StepParams &p, cudaStream_t st) {
-    constexpr int V = 8 / (int)sizeof(typename Raw<P>::R) > 0 ? 8 / (int)sizeof(typename Raw<P>::R) : 1;
-    dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
-    if (walls_on_vector_path<P, LOCAL>() && p.L.bc_y == LBM_WALL)
-        k_stream_collide<P, V, false, LOCAL, walls_on_vector_path<P, LOCAL>(), false, 1, BND>
-            <<<grid, SC_BLOCK_X, 0, st>>>(p);
-    else
-        k_stream_collide<P, V, false, LOCAL, false, false, 1, BND><<<grid, SC_BLOCK_X, 0, st>>>(p);
+template <bool LOCAL, bool BND>
+cudaError_t launch_mrt16(const StepParams &p, cudaStream_t st) {
+    constexpr int V = 4;
+    const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
+    k_stream_collide16<V, false, LOCAL, false, 1, BND><<<grid, SC_BLOCK_X, 0, st>>>(p);
     return cudaGetLastError();
 }
 
-template <int P, bool LOCAL>
-cudaError_t launch_mrt(const StepParams &p, cudaStream_t st) {
-    return p.boundary == LBM_INTERPOLATED ? launch_mrt_b<P, LOCAL, true>(p, st)
-                                          : launch_mrt_b<P, LOCAL, false>(p, st);
-}
-
-template <int P>
-cudaError_t launch_sc_p(const StepParams &p, cudaStream_t st) {
-    if (p.collision == LBM_MRT)
-        return p.rho_w_mode == LBM_RHOW_LOCAL ? launch_mrt<P, true>(p, st) : launch_mrt<P, false>(p, st);
-    constexpr int V16 = 16 / (int)sizeof(typename Raw<P>::R);
-    constexpr int V4 = V16 / 4 > 0 ? V16 / 4 : 1;
-    // the interpolated boundary runs the per-node path in the deferred pass only
+// Node widths as for FP32; variants 3-5 with the per-node path deferred to
+// k_boundary_update (always, with the interpolated boundary).
+cudaError_t launch_sc16(const StepParams &p, cudaStream_t st) {
+    if (p.collision == LBM_MRT) {
+        const bool local = p.rho_w_mode == LBM_RHOW_LOCAL;
+        if (p.boundary == LBM_INTERPOLATED)
+            return local ? launch_mrt16<true, true>(p, st) : launch_mrt16<false, true>(p, st);
+        return local ? launch_mrt16<true, false>(p, st) : launch_mrt16<false, false>(p, st);
+    }
     switch (p.boundary == LBM_INTERPOLATED && p.sc_variant < 3 ? p.sc_variant + 3 : p.sc_variant) {
-        case 1: return launch_sc_v<P, V16 / 2, false>(p, st);
-        case 2: return launch_sc_v<P, V4, false>(p, st);
-        case 3: return launch_sc_v<P, V16, true>(p, st);
-        case 4: return launch_sc_v<P, V16 / 2, true>(p, st);
-        case 5: return launch_sc_v<P, V4, true>(p, st);
-        default: return launch_sc_v<P, V16, false>(p, st);
+        case 1: return launch_sc_v<4, false>(p, st);
+        case 2: return launch_sc_v<2, false>(p, st);
+        case 3: return launch_sc_v<8, true>(p, st);
+        case 4: return launch_sc_v<4, true>(p, st);
+        case 5: return launch_sc_v<2, true>(p, st);
+        default: return launch_sc_v<8, false>(p, st);
     }
 }
 
@@ -172,43 +198,23 @@ cudaError_t launch_sc_p(const StepParams &p, cudaStream_t st) {
 
 cudaError_t launch_stream_collide(const StepParams &p, cudaStream_t st) {
     switch (p.precision) {
-        case LBM_FP64: return launch_sc_p<LBM_FP64>(p, st);
-        case LBM_FP32_DEV: return launch_sc_p<LBM_FP32_DEV>(p, st);
-        default: return launch_sc_p<LBM_FP16_DEV>(p, st);
+        case LBM_FP64: return launch_row_p<LBM_FP64>(p, st);
+        case LBM_FP32_DEV: return launch_row_p<LBM_FP32_DEV>(p, st);
+        default: return launch_sc16(p, st);
     }
 }
 
 cudaError_t launch_deferred_update(const StepParams &p, cudaStream_t st) {
     const bool force = p.body_x != 0.0 || p.body_y != 0.0;
     const bool local = p.rho_w_mode == LBM_RHOW_LOCAL;
-#define GBM_U(P)                                                                            \
-    return force ? (local ? launch_update<P, true, true>(p, st) : launch_update<P, true, false>(p, st)) \
-                 : (local ? launch_update<P, false, true>(p, st) : launch_update<P, false, false>(p, st))
-    switch (p.precision) {
-        case LBM_FP64: GBM_U(LBM_FP64);
-        case LBM_FP32_DEV: GBM_U(LBM_FP32_DEV);
-        default: GBM_U(LBM_FP16_DEV);
-    }
-#undef GBM_U
+    if (force) return local ? launch_update<true, true>(p, st) : launch_update<true, false>(p, st);
+    return local ? launch_update<false, true>(p, st) : launch_update<false, false>(p, st);
 }
 
 cudaError_t launch_open_columns(const StepParams &p, cudaStream_t st) {
-    if (p.L.bc_x != LBM_OPEN) return cudaSuccess;
-    const bool force = p.body_x != 0.0 || p.body_y != 0.0;
     const dim3 grid((p.L.ny + 127) / 128);
-    switch (p.precision) {
-        case LBM_FP64:
-            if (force) k_open_columns<LBM_FP64, true><<<grid, 128, 0, st>>>(p);
-            else k_open_columns<LBM_FP64, false><<<grid, 128, 0, st>>>(p);
-            break;
-        case LBM_FP32_DEV:
-            if (force) k_open_columns<LBM_FP32_DEV, true><<<grid, 128, 0, st>>>(p);
-            else k_open_columns<LBM_FP32_DEV, false><<<grid, 128, 0, st>>>(p);
-            break;
-        default:
-            if (force) k_open_columns<LBM_FP16_DEV, true><<<grid, 128, 0, st>>>(p);
-            else k_open_columns<LBM_FP16_DEV, false><<<grid, 128, 0, st>>>(p);
-    }
+    if (p.body_x != 0.0 || p.body_y != 0.0) k_open_columns<true><<<grid, 128, 0, st>>>(p);
+    else k_open_columns<false><<<grid, 128, 0, st>>>(p);
     return cudaGetLastError();
 }
 

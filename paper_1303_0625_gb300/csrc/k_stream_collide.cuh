@@ -6,20 +6,29 @@
 //
 // Layout: SoA planes f_i[ny][pitch], x fastest, pitch a multiple of 64.
 // Every thread owns V consecutive nodes of one row, V chosen so that one
-// population of those nodes is 16 bytes (FP64: 2, FP32: 4, FP16: 8).  Each of
-// the nine pulls is one aligned 128-bit load from the source row (y - c_y);
-// the x-shifted pulls (c_x = +-1) take the missing neighbour element from the
-// adjacent lane with a warp shuffle (lanes 0 and 31 load it directly, wrapped
-// at the row ends), so DRAM sees each population plane read once, fully
-// coalesced.  Results go out as nine 128-bit stores (nodes in the row padding
-// store zeros).  Nodes next to a solid or a wall and the first and last
-// column take a per-node path, which in the batch kernels (OPEN) also
-// computes the columns of an open channel; the single-domain kernel leaves
-// those to a separate pass (open_row), to keep its per-node path small.
+// population of those nodes is 16, 8 or 4 bytes.  Each of the nine pulls is one
+// aligned vector load from the source row (y - c_y); the x-shifted pulls (c_x =
+// +-1) take the missing neighbour element from the adjacent lane with a warp
+// shuffle (lanes 0 and 31 load it directly), so DRAM sees each population plane
+// read once, fully coalesced.  Results go out as nine vector stores (solid nodes
+// and nodes in the row padding store zeros).
 //
-// Bounce-back: a node whose flags word has bit i set (x - e_i solid or
-// outside) replaces population i by f~_opp(x) + 6 w_i rho_w (e_i . v), v the
-// velocity of the wall or solid at x - e_i / 2.  Solid nodes store zeros.
+// Bounce-back in the FP64 and FP32 modes (sc_row): a population that comes back
+// from a solid, f~_opp(x) + 6 w_i rho_w (e_i . v), is found by the force kernel
+// of the step, which visits every fluid-solid link anyway, and left where the
+// pull reads it: in slot i of the solid node x - e_i, which holds no state.  So
+// the vector path treats a node next to a solid as any other.  Walls, periodic
+// edges and open columns are put in place in registers by the threads that hold
+// them.  No node takes a per-node path: next to the solids one ran with one or
+// two active lanes per warp through a chain of dependent loads (flags, owner,
+// solid record), which cost 0.05 ms of 0.41 on 8192 x 4096 nodes with 2000 disks
+// in FP32 (and held the MRT kernel with the interpolated boundary at 0.31 ms on
+// a quarter of that).
+//
+// FP16 storage (sc_tile) would round such a value once more than arithmetic in
+// registers does, so there the nodes next to a solid or a wall and the first and
+// last column take a per-node path (update_node), in the vector kernel itself or
+// in a pass after it.
 //
 // Storage: FP64 stores f_i; the deviation modes store f_i - w_i (FP32 or
 // FP16) and compute in FP32 entirely in deviation form, so that the small
@@ -205,8 +214,9 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
     }
 }
 
-// BGK collision (with Guo forcing when FORCE) of one node in place.
-template <int P, bool FORCE>
+// BGK collision (with Guo forcing when FORCE) of one node in place.  CHECK:
+// flag a non-physical state (sc_row checks its fluid nodes itself).
+template <int P, bool FORCE, bool CHECK = true>
 __device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C (&g)[9]) {
     using C = typename Prec<P>::C;
     C s0 = 0, jx = 0, jy = 0;
@@ -223,7 +233,8 @@ __device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C
     const C uy = FORCE ? (jy + (C)0.5 * Fy) * inv : jy * inv;
     const C uu = ux * ux + uy * uy;
     const C om = pick<C>(p.omega, p.omega_f);
-    if (!(rho > (C)0) || !(fabs(ux) < (C)1e30) || !(fabs(uy) < (C)1e30)) atomicOr(p.status, 1);
+    if (CHECK && (!(rho > (C)0) || !(fabs(ux) < (C)1e30) || !(fabs(uy) < (C)1e30)))
+        atomicOr(p.status, 1);
 #pragma unroll
     for (int i = 0; i < 9; i++) {
         const C eu = (C)cx(i) * ux + (C)cy(i) * uy;
@@ -413,32 +424,21 @@ __device__ __noinline__ void update_node(const StepParams &p, const typename Raw
     }
 }
 
-// One tile: row y, nodes bx * SC_BLOCK_X * V .. + SC_BLOCK_X * V - 1 (the
-// whole block works on the same tile).
-// WALLS: bounce-back from the y walls on the vector path (FP32 and FP64 with
-// rho_w = rho0 only; FP16 storage would round the bounced values).
-template <int P, bool LOCAL>
-__host__ __device__ constexpr bool walls_on_vector_path() { return !LOCAL && P != LBM_FP16_DEV; }
-
-// DEFER: the per-node path is left to a later pass over the nodes next to
-// solids and edges (the single-domain kernel); otherwise each thread runs it
-// for its own nodes at the end of the tile.
+// FP16: one row segment, V nodes a lane from x0 on (the whole warp works on the
+// same row), nodes next to a solid or a wall and the first and last column left
+// to the per-node path.
+// DEFER: the per-node path is a later pass over those nodes (k_boundary_update);
+// otherwise each thread runs it for its own nodes at the end of the segment.
 // COLL: 0 = BGK, 1 = MRT (no body force, slow nodes inline).
-template <int P, int V, bool FORCE, bool LOCAL, bool OPEN, bool WALLS = false, bool DEFER = false,
-          int COLL = 0, bool BND = false>
-__device__ __forceinline__ void sc_tile(const StepParams &p, int bx, int y) {
-    static_assert(!WALLS || walls_on_vector_path<P, LOCAL>(), "wall rows need rho0 and R == C");
+template <int P, int V, bool FORCE, bool LOCAL, bool OPEN, bool DEFER = false, int COLL = 0,
+          bool BND = false>
+__device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<P>::R *__restrict__ fin,
+                                        typename Raw<P>::R *__restrict__ fout, int x0, int y) {
+    static_assert(P == LBM_FP16_DEV, "FP64 and FP32 take sc_row");
     using R = typename Raw<P>::R;
     using C = typename Prec<P>::C;
     const Lattice &L = p.L;
     const int lane = threadIdx.x & 31;
-    const int x0 = (bx * SC_BLOCK_X + threadIdx.x) * V;
-    // OPEN marks the batch kernels, whose case parameters keep the current
-    // populations in f0 and the next in f1 (swapped as the clock advances);
-    // a single domain selects by the parity of its step counter
-    const long long t = OPEN ? 0 : *p.t;
-    const R *__restrict__ fin = static_cast<const R *>((t & 1) ? p.f1 : p.f0);
-    R *__restrict__ fout = static_cast<R *>((t & 1) ? p.f0 : p.f1);
     const int plane = (int)L.plane;
     const int xl = min(x0, L.pitch - V);  // in-bounds load position for every lane
     int ym = y - 1, yp = y + 1;
@@ -486,38 +486,6 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, int bx, int y) {
         halo[6] = hl[1];
         halo[7] = hl[2];
     }
-    // Wall rows (WALLS): the populations that arrive from the wall (y = -1/2
-    // or ny - 1/2) are the node's own opposite populations plus the moving-wall
-    // term, 6 w_i rho0 (e_i . u_wall) (Sec. III.A, rho_w = rho0).  They are
-    // written where the pulls below read them, so the row stays on the vector
-    // path; nodes with any other bounced population still take the per-node path.
-    uint16_t wall_bits = 0;
-    if (WALLS && L.bc_y == LBM_WALL && (y == 0 || y == L.ny - 1)) {
-        const bool lo = y == 0;
-        wall_bits = lo ? 0x64 : 0x190;  // {2, 5, 6} at y = 0, {4, 7, 8} at y = ny - 1
-        const C uw = lo ? pick<C>(p.wall_ux0, p.wall_ux0_f) : pick<C>(p.wall_ux1, p.wall_ux1_f);
-        const C rho_w = pick<C>(p.rho0, p.rho0_f);
-#pragma unroll
-        for (int i = 1; i < 9; i++) {
-            if (!((wall_bits >> i) & 1u)) continue;
-            Pack<R, V> own;  // the node's own population opp(i), row y
-            own.u = __ldg(reinterpret_cast<const typename Word<sizeof(R) * V>::T *>(
-                fin + opp(i) * plane + r0 + xl));
-            const C term = (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * uw);
-#pragma unroll
-            for (int j = 0; j < V; j++) {
-                const R b = (R)(cvt(own.r[j]) + term);
-                if (cx(i) == 0) raw[i].r[j] = b;
-                else if (cx(i) == 1) {
-                    if (j == 0) halo[i] = b;
-                    else raw[i].r[j - 1] = b;
-                } else {
-                    if (j == V - 1) halo[i] = b;
-                    else raw[i].r[j + 1] = b;
-                }
-            }
-        }
-    }
 #define PULL(i, j) \
     cvt(cx(i) == 0 ? raw[i].r[j] \
                    : (cx(i) == 1 ? ((j) == 0 ? halo[i] : raw[i].r[(j) - 1]) \
@@ -527,7 +495,7 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, int bx, int y) {
     auto classify = [&](int j, C r, C vx, C vy) {
         const uint16_t f = fl.f[j];
         const int x = x0 + j;
-        if (!(f & 1u) && ((f & 0x1FEu & ~wall_bits) || x == 0 || x == L.nx - 1)) slow |= 1u << j;
+        if (!(f & 1u) && ((f & 0x1FEu) || x == 0 || x == L.nx - 1)) slow |= 1u << j;
         else if (!(f & 1u) && x < L.nx &&
                  (!(r > (C)0) || !(fabs(vx) < (C)1e30) || !(fabs(vy) < (C)1e30)))
             atomicOr(p.status, 1);
@@ -693,6 +661,325 @@ template <int P, bool FORCE>
 __device__ __forceinline__ void open_row(const StepParams &p, typename Raw<P>::R *f, int y) {
     open_col<P, FORCE>(p, f, y, true);
     open_col<P, FORCE>(p, f, y, false);
+}
+
+
+// ------------------------------------------------ FP64 and FP32: sc_row
+
+// Is (rho, ux, uy) not a physical state?
+__device__ __forceinline__ bool unphysical(float r, float vx, float vy) {
+    return !(r > 0.f) || !(fabsf(vx) < 1e30f) || !(fabsf(vy) < 1e30f);
+}
+__device__ __forceinline__ bool unphysical(double r, double vx, double vy) {
+    return !(r > 0.0) || !(fabs(vx) < 1e30) || !(fabs(vy) < 1e30);
+}
+
+// Two FP32 nodes per instruction: the deviation form of BGK.  With E_i = s0 +
+// rho (3 e_i.u + 4.5 (e_i.u)^2 - 1.5 u.u) the equilibrium deviation is w_i E_i,
+// and BGK gives (1 - omega) g_i + omega w_i E_i.  Opposite populations share
+// A = s0 - 1.5 rho u.u and the even part 4.5 rho (e.u)^2; the odd part 3 rho e.u
+// changes sign.
+__device__ __forceinline__ void bgk32x2(float om, float2 (&g)[9], float2 &rho, float2 &ux,
+                                        float2 &uy) {
+    const float2 omc = dup2(1.f - om);
+    const float2 s0 = add2(add2(add2(g[0], g[1]), add2(g[2], g[3])),
+                           add2(add2(g[4], g[5]), add2(add2(g[6], g[7]), g[8])));
+    const float2 jx = sub2(add2(add2(g[1], g[5]), g[8]), add2(add2(g[3], g[6]), g[7]));
+    const float2 jy = sub2(add2(add2(g[2], g[5]), g[6]), add2(add2(g[4], g[7]), g[8]));
+    rho = add2(dup2(1.f), s0);
+    const float2 inv = make_float2(1.f / rho.x, 1.f / rho.y);
+    ux = mul2(jx, inv);
+    uy = mul2(jy, inv);
+    const float2 A = fma2(mul2(dup2(-1.5f), rho), fma2(ux, ux, mul2(uy, uy)), s0);
+    g[0] = fma2(dup2(om * wgt<float>(0)), A, mul2(omc, g[0]));
+    // (i, opp(i)) with e_i.u = eu: (1, 3) ux, (2, 4) uy, (5, 7) ux + uy, (6, 8) uy - ux
+    auto pair = [&](int i, int k, float2 eu) {
+        const float2 q = mul2(rho, eu);
+        const float2 sym = fma2(q, mul2(dup2(4.5f), eu), A);
+        const float2 ow = dup2(om * wgt<float>(i));
+        g[i] = fma2(ow, fma2(dup2(3.f), q, sym), mul2(omc, g[i]));
+        g[k] = fma2(ow, fma2(dup2(-3.f), q, sym), mul2(omc, g[k]));
+    };
+    pair(1, 3, ux);
+    pair(2, 4, uy);
+    pair(5, 7, add2(ux, uy));
+    pair(6, 8, sub2(uy, ux));
+}
+
+// Density and velocity of one node from its pulled populations.
+template <int P, bool FORCE>
+__device__ __forceinline__ void node_state(const StepParams &p, const typename Prec<P>::C (&g)[9],
+                                           typename Prec<P>::C &rho, typename Prec<P>::C &ux,
+                                           typename Prec<P>::C &uy) {
+    using C = typename Prec<P>::C;
+    C s0 = 0, jx = 0, jy = 0;
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        s0 += g[i];
+        jx += (C)cx(i) * g[i];
+        jy += (C)cy(i) * g[i];
+    }
+    rho = Prec<P>::dev ? (C)1 + s0 : s0;
+    const C inv = (C)1 / rho;
+    ux = FORCE ? (jx + (C)0.5 * pick<C>(p.body_x, p.body_xf)) * inv : jx * inv;
+    uy = FORCE ? (jy + (C)0.5 * pick<C>(p.body_y, p.body_yf)) * inv : jy * inv;
+}
+
+// Collision of V nodes in place; check(j, rho, ux, uy) for each of them.
+template <int P, int V, bool FORCE, int COLL, class Check>
+__device__ __forceinline__ void collide_nodes(const StepParams &p, typename Prec<P>::C (&g)[V][9],
+                                              Check &&check) {
+    using C = typename Prec<P>::C;
+    if constexpr (COLL == 0 && !FORCE && P == LBM_FP32_DEV && V % 2 == 0) {
+#pragma unroll
+        for (int j = 0; j < V; j += 2) {
+            float2 h[9], r, ux, uy;
+#pragma unroll
+            for (int i = 0; i < 9; i++) h[i] = make_float2(g[j][i], g[j + 1][i]);
+            bgk32x2(p.omega_f, h, r, ux, uy);
+            check(j, r.x, ux.x, uy.x);
+            check(j + 1, r.y, ux.y, uy.y);
+#pragma unroll
+            for (int i = 0; i < 9; i++) {
+                g[j][i] = h[i].x;
+                g[j + 1][i] = h[i].y;
+            }
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < V; j++) {
+            C rho, ux, uy;
+            node_state<P, FORCE>(p, g[j], rho, ux, uy);
+            check(j, rho, ux, uy);
+            if constexpr (COLL == 1) collide_mrt<P, false>(p, g[j]);
+            else collide<P, FORCE, false>(p, g[j]);
+        }
+    }
+}
+
+// Update (advection, walls, collision) of the inner node (x, y) of an open
+// channel, 0 < x < nx - 1, into g: for the outlet column's lane when the node
+// before it belongs to another warp.  Returned populations come from the solid
+// nodes' slots, as in sc_row.
+template <int P, bool FORCE, int COLL>
+__device__ __noinline__ void inner_update(const StepParams &p, const typename Raw<P>::R *fin, int x,
+                                          int y, typename Prec<P>::C (&g)[9]) {
+    using C = typename Prec<P>::C;
+    const Lattice &L = p.L;
+    const int plane = (int)L.plane, k = y * L.pitch + x;
+    C rho_w = pick<C>(p.rho0, p.rho0_f);
+    if (p.rho_w_mode == LBM_RHOW_LOCAL) {
+        C s = 0;
+#pragma unroll
+        for (int i = 0; i < 9; i++) s += cvt(fin[i * plane + k]);
+        rho_w = Prec<P>::dev ? (C)1 + s : s;
+    }
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        const int ys = y - cy(i);
+        if (ys < 0 || ys >= L.ny) {  // open channels are walled in y
+            const C uw = ys < 0 ? pick<C>(p.wall_ux0, p.wall_ux0_f) : pick<C>(p.wall_ux1, p.wall_ux1_f);
+            g[i] = cvt(fin[opp(i) * plane + k]) + (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * uw);
+        } else {
+            g[i] = cvt(fin[i * plane + ys * L.pitch + x - cx(i)]);
+        }
+    }
+    if constexpr (COLL == 1) collide_mrt<P, false>(p, g);
+    else collide<P, FORCE, false>(p, g);
+}
+
+// One row segment: nodes x0 .. x0 + V - 1 of row y in each lane, x0 = 32 V times
+// the segment's index plus V times the lane (whole warps call it, with the same
+// y in every lane).  fin: populations of t with the returned populations in the
+// solid nodes' slots; fout: of t + 1.
+//   edges  periodic: the first column's pulls from column nx - 1 come through
+//          lane 0's halo load, the last column's from column 0 through one
+//          predicated load in the lane that holds it;
+//          walls (half-way, at rest in x): the node's own opposite populations;
+//          y walls (first and last row): the same plus the moving-wall term
+//          6 w_i rho_w (e_i . u_wall), over whichever is there already;
+//          open columns (OPEN): the collided inner neighbour extrapolated
+//          (extrapolate_open), from this lane's registers or the lane before.
+template <int P, int V, bool FORCE, bool OPEN, int COLL>
+__device__ __forceinline__ void sc_row(const StepParams &p, const typename Raw<P>::R *__restrict__ fin,
+                                       typename Raw<P>::R *__restrict__ fout, int x0, int y) {
+    using R = typename Raw<P>::R;
+    using C = typename Prec<P>::C;
+    using W = typename Word<sizeof(R) * V>::T;
+    static_assert(P != LBM_FP16_DEV, "FP16 rounds the returned populations: sc_tile");
+    const Lattice &L = p.L;
+    const int lane = threadIdx.x & 31;
+    const int plane = (int)L.plane;
+    const int xl = min(x0, L.pitch - V);  // in-bounds load position for every lane
+    const bool per_x = L.bc_x == LBM_PERIODIC;
+    int ym = y - 1, yp = y + 1;
+    if (ym < 0) ym = L.bc_y == LBM_PERIODIC ? L.ny - 1 : 0;
+    if (yp >= L.ny) yp = L.bc_y == LBM_PERIODIC ? 0 : L.ny - 1;
+    const int rm = ym * L.pitch, r0 = y * L.pitch, rp = yp * L.pitch;
+#define SROW(i) (cy(i) == 1 ? rm : (cy(i) == -1 ? rp : r0))
+    Pack<R, V> raw[9];
+#pragma unroll
+    for (int i = 0; i < 9; i++)
+        raw[i].u = __ldg(reinterpret_cast<const W *>(fin + i * plane + SROW(i) + xl));
+    FlagPack<V> fl;
+    fl.u = *reinterpret_cast<const typename Word<2 * V>::T *>(p.flags + r0 + xl);
+    R hl[3] = {R(0), R(0), R(0)};
+    if (lane == 0) {
+        const int xh = x0 > 0 ? min(x0, L.pitch) - 1 : (per_x ? L.nx - 1 : 0);
+        hl[0] = fin[1 * plane + SROW(1) + xh];
+        hl[1] = fin[5 * plane + SROW(5) + xh];
+        hl[2] = fin[8 * plane + SROW(8) + xh];
+    } else if (lane == 31) {
+        const int xh = min(x0 + V, L.pitch - 1);
+        hl[0] = fin[3 * plane + SROW(3) + xh];
+        hl[1] = fin[6 * plane + SROW(6) + xh];
+        hl[2] = fin[7 * plane + SROW(7) + xh];
+    }
+    R halo[9];
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        halo[i] = R(0);
+        if (cx(i) == 1) halo[i] = shfl_up1(raw[i].r[V - 1]);
+        else if (cx(i) == -1) halo[i] = shfl_dn1(raw[i].r[0]);
+    }
+    if (lane == 0) {
+        halo[1] = hl[0];
+        halo[5] = hl[1];
+        halo[8] = hl[2];
+    } else if (lane == 31) {
+        halo[3] = hl[0];
+        halo[6] = hl[1];
+        halo[7] = hl[2];
+    }
+    // pulled populations of every node
+    C g[V][9];
+#pragma unroll
+    for (int j = 0; j < V; j++)
+#pragma unroll
+        for (int i = 0; i < 9; i++)
+            g[j][i] = cvt(cx(i) == 0 ? raw[i].r[j]
+                                     : (cx(i) == 1 ? (j == 0 ? halo[i] : raw[i].r[j == 0 ? 0 : j - 1])
+                                                   : (j == V - 1 ? halo[i]
+                                                                 : raw[i].r[j == V - 1 ? j : j + 1])));
+    const int jl = L.nx - 1 - x0;  // this lane's node in the last column, if 0 <= jl < V
+    if (jl >= 0 && jl < V) {
+        C e[3];
+        if (per_x) {
+            e[0] = cvt(fin[3 * plane + SROW(3)]);
+            e[1] = cvt(fin[6 * plane + SROW(6)]);
+            e[2] = cvt(fin[7 * plane + SROW(7)]);
+        } else {
+            const int k = r0 + L.nx - 1;
+            e[0] = cvt(fin[1 * plane + k]);
+            e[1] = cvt(fin[8 * plane + k]);
+            e[2] = cvt(fin[5 * plane + k]);
+        }
+#pragma unroll
+        for (int j = 0; j < V; j++)
+            if (j == jl) {
+                g[j][3] = e[0];
+                g[j][6] = e[1];
+                g[j][7] = e[2];
+            }
+    }
+    if (x0 == 0 && !per_x) {
+        g[0][1] = cvt(fin[3 * plane + r0]);
+        g[0][5] = cvt(fin[7 * plane + r0]);
+        g[0][8] = cvt(fin[6 * plane + r0]);
+    }
+#undef SROW
+    if (L.bc_y == LBM_WALL && (y == 0 || y == L.ny - 1)) {
+        const bool lo = y == 0;
+        const C uw = lo ? pick<C>(p.wall_ux0, p.wall_ux0_f) : pick<C>(p.wall_ux1, p.wall_ux1_f);
+        Pack<R, V> own[9];  // the node's own populations (rho_w = rho0 needs three of them)
+#pragma unroll
+        for (int i = 0; i < 9; i++) {
+            own[i].u = W{};
+            if (p.rho_w_mode == LBM_RHOW_LOCAL || cy(i) == (lo ? -1 : 1))
+                own[i].u = __ldg(reinterpret_cast<const W *>(fin + i * plane + r0 + xl));
+        }
+#pragma unroll
+        for (int j = 0; j < V; j++) {
+            C rho_w = pick<C>(p.rho0, p.rho0_f);
+            if (p.rho_w_mode == LBM_RHOW_LOCAL) {
+                C s = 0;
+#pragma unroll
+                for (int i = 0; i < 9; i++) s += cvt(own[i].r[j]);
+                rho_w = Prec<P>::dev ? (C)1 + s : s;
+            }
+#pragma unroll
+            for (int i = 1; i < 9; i++)
+                if (cy(i) != 0 && (cy(i) == 1) == lo)
+                    g[j][i] = cvt(own[opp(i)].r[j]) + (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * uw);
+        }
+    }
+    collide_nodes<P, V, FORCE, COLL>(p, g, [&](int j, C r, C vx, C vy) {
+        if (!(fl.f[j] & 1u) && x0 + j < L.nx && unphysical(r, vx, vy)) atomicOr(p.status, 1);
+    });
+    if constexpr (OPEN) {
+        // whole warps, uniform branches: the collided inner neighbour of column 0 is
+        // node 1 (this lane, or the next with one node per lane), of column nx - 1
+        // node nx - 2 (this lane, the lane before, or the warp before: recomputed)
+        const bool first = x0 == 0, last = jl >= 0 && jl < V;
+        if (__any_sync(0xffffffffu, first)) {
+            C n[9];
+            uint16_t fn = 1u;
+            if constexpr (V > 1) {
+#pragma unroll
+                for (int i = 0; i < 9; i++) n[i] = g[1][i];
+                fn = fl.f[1];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 9; i++) n[i] = __shfl_down_sync(0xffffffffu, g[0][i], 1);
+                fn = (uint16_t)__shfl_down_sync(0xffffffffu, (int)fl.f[0], 1);
+            }
+            if (first) {
+                const C u_in = inlet_ux<C>(p, y);
+                if (fn & 1u) inlet_equilibrium<P>(p, u_in, n);
+                else extrapolate_open<P, FORCE>(p, true, u_in, n);
+#pragma unroll
+                for (int i = 0; i < 9; i++) g[0][i] = n[i];
+            }
+        }
+        if (__any_sync(0xffffffffu, last)) {
+            C n[9];
+            uint16_t fn;
+#pragma unroll
+            for (int i = 0; i < 9; i++) n[i] = __shfl_up_sync(0xffffffffu, g[V - 1][i], 1);
+            fn = (uint16_t)__shfl_up_sync(0xffffffffu, (int)fl.f[V - 1], 1);
+            if (last) {
+                if (jl > 0) {
+#pragma unroll
+                    for (int j = 1; j < V; j++)
+                        if (j == jl) {
+#pragma unroll
+                            for (int i = 0; i < 9; i++) n[i] = g[j - 1][i];
+                            fn = fl.f[j - 1];
+                        }
+                } else if (lane == 0) {
+                    fn = p.flags[r0 + L.nx - 2];
+                    if (!(fn & 1u)) inner_update<P, FORCE, COLL>(p, fin, L.nx - 2, y, n);
+                }
+                if (!(fn & 1u)) {
+                    extrapolate_open<P, FORCE>(p, false, (C)0, n);
+#pragma unroll
+                    for (int j = 0; j < V; j++)
+                        if (j == jl) {
+#pragma unroll
+                            for (int i = 0; i < 9; i++) g[j][i] = n[i];
+                        }
+                }
+            }
+        }
+    }
+    if (x0 >= L.nx) return;
+#pragma unroll
+    for (int i = 0; i < 9; i++) {
+        Pack<R, V> o;
+#pragma unroll
+        for (int j = 0; j < V; j++) put(o.r[j], (fl.f[j] & 1u) ? (C)0 : g[j][i]);
+        *reinterpret_cast<W *>(fout + i * plane + r0 + x0) = o.u;
+    }
 }
 
 }  // namespace

@@ -8,10 +8,22 @@ namespace gbm {
 
 namespace {
 
+// One row of one tile.  The force kernel of the step has swapped the buffers: f1
+// holds the current populations, f0 takes the next.
+template <int P, int V, bool FORCE, bool LOCAL>
+__device__ __forceinline__ void tile_row(const StepParams &p, int bx, int y) {
+    using R = typename Raw<P>::R;
+    const R *fin = static_cast<const R *>(p.f1);
+    R *fout = static_cast<R *>(p.f0);
+    const int x0 = (bx * SC_BLOCK_X + threadIdx.x) * V;
+    if constexpr (P == LBM_FP16_DEV) sc_tile<P, V, FORCE, LOCAL, true>(p, fin, fout, x0, y);
+    else if (p.L.bc_x == LBM_OPEN) sc_row<P, V, FORCE, true, 0>(p, fin, fout, x0, y);
+    else sc_row<P, V, FORCE, false, 0>(p, fin, fout, x0, y);
+}
+
 // Batch of independent domains: persistent blocks walk the list of active
 // tiles {case, x block, first row} of all cases (case-major), each tile
-// (tile_h rows of SC_BLOCK_X * V nodes) with its own case's parameters and
-// step counter.
+// (tile_h rows of SC_BLOCK_X * V nodes) with its own case's parameters.
 template <int P, int V, bool FORCE, bool LOCAL>
 __global__ void __launch_bounds__(SC_BLOCK_X, 6)
     k_stream_collide_batch(const StepParams *__restrict__ cases, const int4 *__restrict__ tiles,
@@ -21,13 +33,13 @@ __global__ void __launch_bounds__(SC_BLOCK_X, 6)
         const int4 tl = tiles[k];
         const StepParams &p = cases[tl.x];
         const int y1 = min(tl.z + tile_h, p.L.ny);
-        for (int y = tl.z; y < y1; y++) sc_tile<P, V, FORCE, LOCAL, true, walls_on_vector_path<P, LOCAL>()>(p, tl.y, y);
+        for (int y = tl.z; y < y1; y++) tile_row<P, V, FORCE, LOCAL>(p, tl.y, y);
     }
 }
 
 // The same tiles with one block per tile (grid = capacity of the list).
-// FP32 with 4- or 8-byte words: at most 48 registers (10 blocks per SM, as
-// the single-domain kernel), at the cost of a few bytes of spills.
+// FP32 with 4- or 8-byte words: at most 48 registers (10 blocks per SM), at the
+// cost of a few bytes of spills.
 template <int P, int V>
 constexpr int tiles_min_blocks() { return (P == LBM_FP32_DEV && V <= 2) ? 10 : 6; }
 
@@ -39,11 +51,11 @@ __global__ void __launch_bounds__(SC_BLOCK_X, (tiles_min_blocks<P, V>()))
     const int4 tl = tiles[blockIdx.x];
     const StepParams &p = cases[tl.x];
     if (!ROWS) {
-        sc_tile<P, V, FORCE, LOCAL, true, walls_on_vector_path<P, LOCAL>()>(p, tl.y, tl.z);
+        tile_row<P, V, FORCE, LOCAL>(p, tl.y, tl.z);
         return;
     }
     const int y1 = min(tl.z + tile_h, p.L.ny);
-    for (int y = tl.z; y < y1; y++) sc_tile<P, V, FORCE, LOCAL, true, walls_on_vector_path<P, LOCAL>()>(p, tl.y, y);
+    for (int y = tl.z; y < y1; y++) tile_row<P, V, FORCE, LOCAL>(p, tl.y, y);
 }
 
 template <int P, int V, bool FORCE, bool LOCAL>
@@ -72,9 +84,11 @@ cudaError_t launch_scb(const BatchLaunch &b, cudaStream_t st) {
 
 template <int P, int V>
 cudaError_t launch_scb_v(const BatchLaunch &b, cudaStream_t st) {
+    // FP64 and FP32 need rho_w only in wall rows (a run-time branch of sc_row)
+    const bool local = P == LBM_FP16_DEV && b.local;
     if (b.force)
-        return b.local ? launch_scb<P, V, true, true>(b, st) : launch_scb<P, V, true, false>(b, st);
-    return b.local ? launch_scb<P, V, false, true>(b, st) : launch_scb<P, V, false, false>(b, st);
+        return local ? launch_scb<P, V, true, P == LBM_FP16_DEV>(b, st) : launch_scb<P, V, true, false>(b, st);
+    return local ? launch_scb<P, V, false, P == LBM_FP16_DEV>(b, st) : launch_scb<P, V, false, false>(b, st);
 }
 
 template <int P>

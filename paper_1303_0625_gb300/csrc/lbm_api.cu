@@ -42,6 +42,7 @@ struct lbm_ctx {
     int *status_d = nullptr;
     unsigned int *bar_d = nullptr;  // per-solid control words (barrier, displacement, pair test)
     uint16_t *near_d = nullptr;     // near lists, [solid_cap][NEAR_CAP]
+    double *part_d = nullptr;       // link sums by block, [solid_cap][LINK_PARTS][6]
     long long spin_limit = 1ll << 24;  // polls of a bounded device wait (about one second)
     // the force kernel runs on a second stream beside the advection-collision
     // kernel: fork after the previous step, join before the re-rasterisation
@@ -95,6 +96,22 @@ lbm_status fail(lbm_ctx *c, lbm_status st, const char *fmt, ...) {
     } while (0)
 
 size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DEV ? 4 : 2); }
+
+// Does work go to the side stream, beside the advection-collision kernel?
+bool forks(const lbm_ctx *c) {
+    if (!c->overlap || c->nsolid == 0) return false;
+    return c->cfg.precision == LBM_FP16_DEV || !c->moving.empty();
+}
+
+// Blocks per solid of the link kernel, or 0 for links, record and motion in one
+// kernel.  The record and the motion are a kernel of their own where they can run
+// beside the advection-collision kernel, and with the interpolated boundary, whose
+// links are worth several blocks where the solids alone would not fill the SMs.
+int link_parts(const lbm_ctx *c) {
+    const bool cut = c->cfg.boundary == LBM_INTERPOLATED;
+    if (!cut && (c->cfg.precision == LBM_FP16_DEV || !forks(c))) return 0;
+    return cut && c->nsolid < 256 ? gbm::LINK_PARTS : 1;
+}
 
 StepParams params(const lbm_ctx *c) {
     StepParams p{};
@@ -165,6 +182,8 @@ StepParams params(const lbm_ctx *c) {
     p.bar = c->bar_d;
     p.spin_limit = c->spin_limit;
     p.near_id = c->near_d;
+    p.part = c->part_d;
+    p.link_parts = link_parts(c);
     return p;
 }
 
@@ -178,7 +197,8 @@ void release(lbm_ctx *c) {
     drop_graph(c);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     void *bufs[] = {c->f[0], c->f[1], c->owner, c->flags, c->solids, c->moving_d, c->ring,
-                    c->t_d, c->status_d, c->bar_d, c->scratch, c->bnd_d, c->ev_d, c->near_d};
+                    c->t_d, c->status_d, c->bar_d, c->scratch, c->bnd_d, c->ev_d, c->near_d,
+                    c->part_d};
     for (void *b : bufs)
         if (b) cudaFree(b);
     if (c->fork) cudaEventDestroy(c->fork);
@@ -248,26 +268,27 @@ lbm_status upload_moving(lbm_ctx *c) {
     return LBM_OK;
 }
 
-// One step t -> t+1: the force kernel (force record of time t, motion) and
-// the ring kernel (the moving solids' owner changes and covered/fresh nodes,
-// listed) on the side stream beside the advection-collision kernel, all after
-// the previous step; then the re-rasterisation of the moving solids (the
+// One step t -> t+1: the links (force sums of time t, and in FP64 and FP32 the
+// populations the solids return, which the advection-collision kernel pulls); the
+// force record and the motion, and the ring kernel (the moving solids' owner
+// changes and covered/fresh nodes, listed), on the side stream beside the
+// advection-collision kernel; then the re-rasterisation of the moving solids (the
 // changes applied, refill), which advances t (or a clock tick when no solid
-// moves).
+// moves).  FP16: the links too are the side stream's.
 lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
-    const bool fork = p.nsolid > 0 && c->overlap;
+    const bool half = p.precision == LBM_FP16_DEV, fork = forks(c);
+    if (!(half && fork)) CK(c, gbm::launch_forces(p, c->stream));
+    cudaStream_t rest = c->stream;
     if (fork) {
         CK(c, cudaEventRecord(c->fork, c->stream));
         CK(c, cudaStreamWaitEvent(c->side, c->fork, 0));
-        CK(c, gbm::launch_forces(p, c->side));
-        CK(c, gbm::launch_ring(p, c->side));
-        CK(c, cudaEventRecord(c->join, c->side));
-        c->launches += p.nmoving > 0 ? 2 : 1;
-    } else if (p.nsolid > 0) {
-        CK(c, gbm::launch_forces(p, c->stream));
-        CK(c, gbm::launch_ring(p, c->stream));
-        c->launches += p.nmoving > 0 ? 2 : 1;
+        rest = c->side;
+        if (half) CK(c, gbm::launch_forces(p, rest));
     }
+    CK(c, gbm::launch_record(p, rest));
+    CK(c, gbm::launch_ring(p, rest));
+    if (fork) CK(c, cudaEventRecord(c->join, rest));
+    c->launches += (p.nsolid > 0 ? (p.link_parts ? 2 : 1) : 0) + (p.nmoving > 0 ? 1 : 0);
     if (timed) {
         if (c->ev_used + 2 > c->ev.size()) {
             for (int k = 0; k < 2; k++) {
@@ -287,7 +308,7 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
         CK(c, cudaEventRecord(c->ev[c->ev_used + 1], c->stream));
         c->ev_used += 2;
     }
-    if (p.L.bc_x == LBM_OPEN) {
+    if (half && p.L.bc_x == LBM_OPEN) {
         CK(c, gbm::launch_open_columns(p, c->stream));
         c->launches++;
     }
@@ -481,6 +502,9 @@ lbm_status lbm_add_solid(lbm_ctx *c, const lbm_disk *d, int32_t *id_out) {
         if (c->near_d) CK(c, cudaFree(c->near_d));  // rebuilt by the next pair test
         c->near_d = nullptr;
         CK(c, cudaMalloc(&c->near_d, (size_t)cap * gbm::NEAR_CAP * sizeof(uint16_t)));
+        if (c->part_d) CK(c, cudaFree(c->part_d));
+        c->part_d = nullptr;
+        CK(c, cudaMalloc(&c->part_d, (size_t)cap * gbm::LINK_PARTS * 6 * sizeof(double)));
         c->solid_cap = cap;
     }
     if (c->nsolid + 1 > c->ring_cap) {
@@ -1367,6 +1391,7 @@ lbm_status bprepare(lbm_batch *b) {
 }
 
 lbm_status benqueue_step(lbm_batch *b, const gbm::BatchLaunch &l, bool timed) {
+    BCK(b, gbm::launch_solids_batch(l, b->stream));
     if (timed) {
         if (b->ev_used + 2 > b->ev.size()) {
             for (int k = 0; k < 2; k++) {
@@ -1382,7 +1407,6 @@ lbm_status benqueue_step(lbm_batch *b, const gbm::BatchLaunch &l, bool timed) {
         BCK(b, cudaEventRecord(b->ev[b->ev_used + 1], b->stream));
         b->ev_used += 2;
     }
-    BCK(b, gbm::launch_solids_batch(l, b->stream));
     b->launches += 2;
     return LBM_OK;
 }

@@ -82,6 +82,9 @@ constexpr int NEAR_CAP = 32;
 constexpr float NEAR_REACH = 4.5f;
 constexpr float NEAR_MARGIN = 4.0f;
 
+// blocks that can share one solid's links
+constexpr int LINK_PARTS = 4;
+
 // covered/fresh nodes one solid can queue per step
 constexpr int SOLID_EVENTS = 256;
 
@@ -133,7 +136,9 @@ struct StepParams {
     int chg_cap;
     int *bnd;                 // deferred per-node path: {length at even t, at odd t, list...}
     int bnd_cap;              // capacity of the list
-    int list_by_forces;       // the force kernel fills the deferred list; the fused pass
+    double *part;             // [nsolid][LINK_PARTS][6] link sums of a solid's blocks
+    int link_parts;           // blocks per solid of k_links, which k_record follows; 0: k_forces
+    int list_by_forces;       // FP16: the force kernel fills the deferred list; the fused pass
                               // leaves the update to launch_deferred_update
 };
 
@@ -324,6 +329,17 @@ __device__ __forceinline__ double link_fraction(const Lattice &L, const DSolid &
     return q;
 }
 
+// The same from the node's offset (px, py) from the centre's nearest image, known
+// already (a is 1 or 2: the division by it is exact).
+__device__ __forceinline__ double link_fraction_at(double px, double py, double r, int ex, int ey) {
+    const double a = (double)(ex * ex + ey * ey), h = px * ex + py * ey;
+    const double disc = h * h - a * (px * px + py * py - r * r);
+    double q = disc > 0.0 ? (-h - sqrt(disc)) * (ex * ey ? 0.5 : 1.0) : 0.5;
+    if (!(q > 0.0)) q = 0.0;
+    if (q > 1.0) q = 1.0;
+    return q;
+}
+
 // The same fraction for the FP32 kernels, from the node's offset from the
 // centre split as an integer part minus an FP32 remainder, (di - fx, dj - fy),
 // along (ex, ey): the offset and c = |p - R|^2 - r^2 in FP64 without a
@@ -388,11 +404,11 @@ struct BatchState {
 };
 
 // k_stream_collide.cu
-// the fused advection-collision kernel, and with variants 3-5 the pass over
-// the nodes it leaves to the per-node update
+// the fused advection-collision kernel, and in FP16 with variants 3-5 the pass
+// over the nodes it leaves to the per-node update
 constexpr int KERNEL_VARIANTS = 6;
 inline bool deferred_path(const StepParams &p) {
-    return p.collision != LBM_MRT && (p.sc_variant >= 3 || p.boundary == LBM_INTERPOLATED);
+    return p.precision == LBM_FP16_DEV && p.collision != LBM_MRT && (p.sc_variant >= 3 || p.boundary == LBM_INTERPOLATED);
 }
 inline int stream_collide_launches(const StepParams &p) {
     return deferred_path(p) ? 2 : 1;  // MRT keeps the slow nodes inline
@@ -400,20 +416,23 @@ inline int stream_collide_launches(const StepParams &p) {
 cudaError_t launch_stream_collide(const StepParams &p, cudaStream_t st);
 // the update of the deferred per-node path, when list_by_forces
 cudaError_t launch_deferred_update(const StepParams &p, cudaStream_t st);
-// open channel: columns 0 and nx-1 of the populations just written (t+1)
+// FP16 open channel: columns 0 and nx-1 of the populations just written (t+1)
 cudaError_t launch_open_columns(const StepParams &p, cudaStream_t st);
 
 // k_stream_collide_batch.cu
 cudaError_t launch_stream_collide_batch(const BatchLaunch &b, cudaStream_t st);
 int tile_nodes(int precision, int variant);  // nodes along x of one tile
-// k_solid_step.cu: per-solid work of a step t -> t+1.  launch_forces: force
-// record of time t and motion t -> t+1 of every solid; launch_ring after it:
-// near lists when due, the moving solids' owner changes and covered/fresh
-// nodes, listed (both only read what the advection-collision kernel of the
-// step reads and write nothing it reads, so they may run beside it);
-// launch_remask, after all three: the owner changes applied, refill, t += 1
-// (one cooperative launch).
+// k_solid_step.cu: per-solid work of a step t -> t+1.  launch_forces, before the
+// advection-collision kernel (FP16: before or beside it): force record of time t
+// and motion t -> t+1 of every solid, and in FP64 and FP32 the populations that
+// the solids return, left in the solid nodes' slots (with link_parts the record
+// and the motion are launch_record's, after it); launch_ring after them: near
+// lists when due, the moving solids' owner changes and covered/fresh nodes, listed
+// (it writes nothing that the advection-collision kernel reads, so it may run
+// beside it); launch_remask, after all three: the owner changes applied, refill,
+// t += 1 (one cooperative launch).
 cudaError_t launch_forces(const StepParams &p, cudaStream_t st);
+cudaError_t launch_record(const StepParams &p, cudaStream_t st);
 cudaError_t launch_ring(const StepParams &p, cudaStream_t st);
 cudaError_t launch_remask(const StepParams &p, cudaStream_t st);
 // batch: force record of every resting solid of every active case, t += 1
