@@ -270,7 +270,7 @@ __device__ __forceinline__ void collide_mrt(const StepParams &p, typename Prec<P
     const C jx = g[1] - g[3] + g[5] - g[6] - g[7] + g[8];
     const C jy = g[2] - g[4] + g[5] + g[6] - g[7] - g[8];
     const C rho = Prec<P>::dev ? (C)1 + s0 : s0;
-    const C inv = (C)1 / rho;
+    const C inv = reciprocal(rho);
     if (CHECK && (!(rho > (C)0) || !(fabs(jx * inv) < (C)1e30) || !(fabs(jy * inv) < (C)1e30)))
         atomicOr(p.status, 1);
     const C jj = (jx * jx + jy * jy) * inv;
@@ -666,12 +666,51 @@ __device__ __forceinline__ void open_row(const StepParams &p, typename Raw<P>::R
 
 // ------------------------------------------------ FP64 and FP32: sc_row
 
-// Is (rho, ux, uy) not a physical state?
+// Is (rho, ux, uy) not a physical state?  FP64: from the high words (the FP64
+// unit is what bounds the FP64 kernel, and a comparison occupies it too).
 __device__ __forceinline__ bool unphysical(float r, float vx, float vy) {
     return !(r > 0.f) || !(fabsf(vx) < 1e30f) || !(fabsf(vy) < 1e30f);
 }
 __device__ __forceinline__ bool unphysical(double r, double vx, double vy) {
-    return !(r > 0.0) || !(fabs(vx) < 1e30) || !(fabs(vy) < 1e30);
+    constexpr int BIG = 0x46293E59;  // high word of 1e30
+    const int h = __double2hiint(r);
+    return h <= 0 || h >= 0x7FF00000 || (__double2hiint(vx) & 0x7FFFFFFF) > BIG ||
+           (__double2hiint(vy) & 0x7FFFFFFF) > BIG;
+}
+
+// BGK collision of one FP64 node, no body force.  GB300 issues about two FP64
+// lanes per clock and SM, so the number of FP64 operations is the kernel's time:
+// about 60 here, against about 154 with nine separate equilibria and a division
+// (2048 x 1024 nodes: 259 us a launch against 550).
+// With h_i = (f_i + f_opp) / 2 and d_i = (f_i - f_opp) / 2 the even and the odd
+// part of the equilibrium relax on their own:
+//   E_i = rho - 1.5 j.u + 4.5 (e_i.j)(e_i.u)   (rho u = j)
+//   f_i, f_opp  <-  [(1 - omega) h_i + omega w_i E_i] +- [(1 - omega) d_i + 3 omega w_i (e_i.j)]
+__device__ __forceinline__ void bgk64(double om, double (&g)[9], double &rho, double &ux,
+                                      double &uy) {
+    const double a1 = g[1] + g[3], d1 = g[1] - g[3], a2 = g[2] + g[4], d2 = g[2] - g[4];
+    const double a5 = g[5] + g[7], d5 = g[5] - g[7], a6 = g[6] + g[8], d6 = g[6] - g[8];
+    rho = (g[0] + (a1 + a2)) + (a5 + a6);
+    const double jx = d1 + (d5 - d6), jy = d2 + (d5 + d6);
+    const double inv = reciprocal(rho);
+    ux = jx * inv;
+    uy = jy * inv;
+    const double pxx = jx * ux, pyy = jy * uy, pxy = jx * uy, t = pxx + pyy;
+    // omega E_i: omega goes into rho, not into the weights, whose sum is then as
+    // close to one as 9 fl(1/9) is (omega w_i rounded one by one let the mass drift)
+    const double o4 = 4.5 * om, A = fma(-1.5 * om, t, om * rho), B = fma(o4, t, A);
+    const double c = 1.0 - om, ch = 0.5 * c;  // uniform over the launch
+    g[0] = fma(wgt<double>(0), A, c * g[0]);
+    auto pair = [&](int i, int k, double E, double ej, double a, double d) {
+        const double hs = fma(wgt<double>(i), E, ch * a);
+        const double hd = fma(3.0 * wgt<double>(i) * om, ej, ch * d);
+        g[i] = hs + hd;
+        g[k] = hs - hd;
+    };
+    pair(1, 3, fma(o4, pxx, A), jx, a1, d1);
+    pair(2, 4, fma(o4, pyy, A), jy, a2, d2);
+    pair(5, 7, fma(2.0 * o4, pxy, B), jx + jy, a5, d5);
+    pair(6, 8, fma(-2.0 * o4, pxy, B), jy - jx, a6, d6);
 }
 
 // Two FP32 nodes per instruction: the deviation form of BGK.  With E_i = s0 +
@@ -720,7 +759,7 @@ __device__ __forceinline__ void node_state(const StepParams &p, const typename P
         jy += (C)cy(i) * g[i];
     }
     rho = Prec<P>::dev ? (C)1 + s0 : s0;
-    const C inv = (C)1 / rho;
+    const C inv = reciprocal(rho);
     ux = FORCE ? (jx + (C)0.5 * pick<C>(p.body_x, p.body_xf)) * inv : jx * inv;
     uy = FORCE ? (jy + (C)0.5 * pick<C>(p.body_y, p.body_yf)) * inv : jy * inv;
 }
@@ -749,10 +788,15 @@ __device__ __forceinline__ void collide_nodes(const StepParams &p, typename Prec
 #pragma unroll
         for (int j = 0; j < V; j++) {
             C rho, ux, uy;
-            node_state<P, FORCE>(p, g[j], rho, ux, uy);
-            check(j, rho, ux, uy);
-            if constexpr (COLL == 1) collide_mrt<P, false>(p, g[j]);
-            else collide<P, FORCE, false>(p, g[j]);
+            if constexpr (COLL == 0 && !FORCE && P == LBM_FP64) {
+                bgk64(p.omega, g[j], rho, ux, uy);
+                check(j, rho, ux, uy);
+            } else {
+                node_state<P, FORCE>(p, g[j], rho, ux, uy);
+                check(j, rho, ux, uy);
+                if constexpr (COLL == 1) collide_mrt<P, false>(p, g[j]);
+                else collide<P, FORCE, false>(p, g[j]);
+            }
         }
     }
 }

@@ -368,6 +368,19 @@ __device__ __forceinline__ long long cell_of(const Lattice &L, int x, int y) {
     return (long long)y * L.pitch + x;
 }
 
+// ------------------------------------------------------------- arithmetic
+
+// 1 / r for r of the order of one, without the divide instruction sequence:
+// the hardware's approximation (about 20 bits) and two Newton-Raphson steps
+// y += y (1 - r y), each of which doubles the bits.
+__device__ __forceinline__ double reciprocal(double r) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(r));
+    y = fma(fma(-r, y, 1.0), y, y);
+    return fma(fma(-r, y, 1.0), y, y);
+}
+__device__ __forceinline__ float reciprocal(float r) { return 1.f / r; }
+
 // ----------------------------------------------------------- launchers
 
 // Device tables of a batch of independent domains (k_stream_collide.cu and
