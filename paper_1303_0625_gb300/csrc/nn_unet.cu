@@ -1,28 +1,36 @@
-// The warm-start U-Net on the GPU: forward, backward and Adam, with every
-// 3x3 convolution an implicit GEMM on the tensor cores (BF16 operands, FP32
-// accumulation) with tcgen05 and the accumulator in tensor memory: forward
-// and data gradient with K-major operands, the weight gradient with MN-major
-// ones read straight from the NHWC tensors.  The remaining layers (pooling,
-// upsampling with concatenation, the 1x1 head, the loss, Adam) are small
-// kernels of their own.
+// The warm-start U-Net on the GPU: forward, backward and Adam, with every 3x3
+// convolution an implicit GEMM on the tensor cores (tcgen05, BF16 operands, FP32
+// accumulation in tensor memory).  The remaining layers (pooling, the 1x1 head, the
+// loss, Adam) are small kernels of their own.
 //
-// Layout: activations NHWC in BF16 (channels innermost, every channel count
-// a multiple of 8, so that 8 channels are one 16-byte load); conv weights
-// [Cout][tap][Cin] (tap = 3 ky + kx) in BF16, with a transposed copy
-// [Cin][tap][Cout] for the backward pass over the data; FP32 master weights,
-// gradients and Adam moments in the same layout.
+// Layout: activations and their gradients are planes of 8 channels,
+// X[C / 8][B][H + 2][W + 2][8] in BF16, with a border of zeros that is written once
+// (a plane's image stride is rounded up to 128 pixels).  A pixel of a plane is 16
+// bytes and pixels are consecutive, so a run of pixels is one bulk copy, and in
+// shared memory it is, as it stands, the no-swizzle core-matrix layout of
+// tcgen05.mma: 8 pixels x 8 channels = 128 bytes, the next 8 pixels behind them.  A
+// tap's displacement is then a shift of the operand's start address by (dy (W + 2)
+// + dx) pixels of 16 bytes, borders included, and no operand is gathered: the
+// convolutions copy each input pixel once per output tile instead of once per tap
+// (with NHWC and one 16-byte cp.async per pixel, tap and 8 channels, they ran at 6%
+// of the tensor cores' rate).
 //
-// Convolutions as GEMMs (P = B H W pixels, s(tap) = (ky - 1, kx - 1)):
-//   forward      out[p][co]  = sum_{tap,ci} x[p + s][ci] w[co][tap][ci]        M=P  N=Cout K=9 Cin
-//   data grad    dx[p][ci]   = sum_{tap,co} dz[p - s][co] w[co][tap][ci]       M=P  N=Cin  K=9 Cout
-//   weight grad  dw[co][tap][ci] = sum_p dz[p][co] x[p + s][ci]                M=Cout N=9 Cin K=P
-// (zero outside the image).  The weight gradient splits K over blocks and
+// Convolutions as GEMMs over the padded pixels Q = (b, y, x) of all images (rows
+// that are border pixels are computed and not stored):
+//   forward      out[Q][co]  = sum_{tap,ci} x[Q + s(tap)][ci] w[co][tap][ci]      M=Q  N=Cout K=9 Cin
+//   data grad    dx[Q][ci]   = sum_{tap,co} dz[Q - s(tap)][co] w[co][tap][ci]     M=Q  N=Cin  K=9 Cout
+//   weight grad  dw[tap][ci][co] = sum_Q x[Q + s(tap)][ci] dz[Q][co]  M=(dy, ci)  N=Cout K=Q, one per dx
+// s(tap) = (tap / 3 - 1, tap % 3 - 1).  The weight gradient splits K over blocks and
 // adds FP32 partial sums atomically.
+//
+// Weights: FP32 masters, gradients and Adam moments [tap][Cin][Cout]; BF16 copies
+// packed as the B operands of the forward and data-gradient convolutions (packed_at).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <random>
@@ -35,632 +43,45 @@ namespace nn {
 
 using bf16 = __nv_bfloat16;
 
-// ------------------------------------------------------------ GEMM core
+// ------------------------------------------------------------- layout
 
-constexpr int BM = 64, BN = 64, BK = 32, LDS = BK + 8;  // smem rows padded by 16 bytes
-constexpr int GEMM_THREADS = 128;                       // 2 x 2 warps of 32 x 32
-
-struct alignas(16) Tiles {
-    bf16 a[BM][LDS];
-    bf16 b[BN][LDS];
-};
-
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4],
-                                         const uint32_t (&b)[2]) {
-    asm volatile(
-        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, "
-        "{%8,%9}, {%0,%1,%2,%3};\n"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void *p) {
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-                 : "r"(a));
-}
-
-__device__ __forceinline__ void ldsm_x2(uint32_t (&r)[2], const void *p) {
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-    asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n"
-                 : "=r"(r[0]), "=r"(r[1])
-                 : "r"(a));
-}
-
-// C[M][N] = sum_k A[m][k] B[n][k] over this block's K range; the operation
-// Op gathers the tiles (load_a, load_b) and consumes the result (store).
-template <class Op>
-__global__ void __launch_bounds__(GEMM_THREADS) k_gemm(const Op op) {
-    __shared__ Tiles t;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wm = warp >> 1, wn = warp & 1;
-    const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    int kb = 0, ke = op.K;
-    if (gridDim.z > 1) {
-        kb = blockIdx.z * op.kchunk;
-        ke = min(op.K, kb + op.kchunk);
+// One level's images: H x W pixels with a border of one, PSI pixels per image.
+struct Geo {
+    int H, W, Wp, PSI;
+    __host__ __device__ Geo() : H(0), W(0), Wp(0), PSI(0) {}
+    __host__ __device__ Geo(int h, int w) : H(h), W(w), Wp(w + 2), PSI(((h + 2) * (w + 2) + 127) / 128 * 128) {}
+    // pixel (n, y, x)
+    __host__ __device__ long long at(int n, int y, int x) const {
+        return (long long)n * PSI + (long long)(y + 1) * Wp + x + 1;
     }
-    float c[2][4][4] = {};
-    for (int k0 = kb; k0 < ke; k0 += BK) {
-        op.load_a(t.a, m0, k0, ke, tid);
-        op.load_b(t.b, n0, k0, ke, tid);
-        __syncthreads();
-#pragma unroll
-        for (int ks = 0; ks < BK; ks += 16) {
-            uint32_t af[2][4], bfr[4][2];
-#pragma unroll
-            for (int mi = 0; mi < 2; mi++)
-                ldsm_x4(af[mi], &t.a[wm * 32 + mi * 16 + (lane & 15)][ks + (lane >> 4) * 8]);
-#pragma unroll
-            for (int ni = 0; ni < 4; ni++)
-                ldsm_x2(bfr[ni], &t.b[wn * 32 + ni * 8 + (lane & 7)][ks + ((lane >> 3) & 1) * 8]);
-#pragma unroll
-            for (int mi = 0; mi < 2; mi++)
-#pragma unroll
-                for (int ni = 0; ni < 4; ni++) mma_bf16(c[mi][ni], af[mi], bfr[ni]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int mi = 0; mi < 2; mi++)
-#pragma unroll
-        for (int ni = 0; ni < 4; ni++) {
-            const int r = m0 + wm * 32 + mi * 16 + (lane >> 2);
-            const int col = n0 + wn * 32 + ni * 8 + (lane & 3) * 2;
-            op.store(r, col, c[mi][ni][0], c[mi][ni][1]);
-            op.store(r + 8, col, c[mi][ni][2], c[mi][ni][3]);
-        }
-}
-
-// Geometry of an NHWC image batch.
-struct Img {
-    int B, H, W;
-    __device__ __forceinline__ bool shift(int p, int dy, int dx, int &q) const {
-        const int hw = H * W;
-        const int n = p / hw, r = p - n * hw, y = r / W, x = r - y * W;
-        const int ys = y + dy, xs = x + dx;
-        if (ys < 0 || ys >= H || xs < 0 || xs >= W) return false;
-        q = (n * H + ys) * W + xs;
-        return true;
+    // interior pixel of Q, or false
+    __device__ __forceinline__ bool where(int Q, int B, int &n, int &y, int &x) const {
+        n = Q / PSI;
+        const int r = Q - n * PSI;
+        y = r / Wp - 1;
+        x = r - (y + 1) * Wp - 1;
+        return n < B && (unsigned)y < (unsigned)H && (unsigned)x < (unsigned)W;
     }
 };
 
-// Forward convolution (sign = +1) or the gradient with respect to its input
-// (sign = -1, w the transposed weights): out[p][n] = act(bias + sum over taps
-// and source channels of src[p + sign s(tap)][c] w[n][tap][c]), times
-// (mask > 0) when a mask is given.
-struct ConvOp {
-    const bf16 *src;   // [P][Cs]
-    const bf16 *w;     // [N][taps][Cs]
-    const float *bias; // [N] or null
-    const bf16 *mask;  // [P][N] or null
-    bf16 *out;         // [P][N]
-    Img img;
-    int Cs, taps, sign, relu;
-    int M, N, K, kchunk;
-
-    // 8 consecutive K elements of row p of A (source channels of one tap)
-    __device__ __forceinline__ uint4 gather_a(int p, int k, int ke) const {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (p < M && k < ke) {
-            const int tap = k / Cs, c = k - tap * Cs;
-            int qp = p;
-            bool ok = true;
-            if (taps == 9) ok = img.shift(p, sign * (tap / 3 - 1), sign * (tap % 3 - 1), qp);
-            if (ok) v = *reinterpret_cast<const uint4 *>(src + (size_t)qp * Cs + c);
-        }
-        return v;
-    }
-    // address of the 8 K elements of row p of A, or null where they are zero
-    __device__ __forceinline__ const bf16 *addr_a(int p, int k, int ke) const {
-        if (p >= M || k >= ke) return nullptr;
-        const int tap = k / Cs, c = k - tap * Cs;
-        int qp = p;
-        if (taps == 9 && !img.shift(p, sign * (tap / 3 - 1), sign * (tap % 3 - 1), qp)) return nullptr;
-        return src + (size_t)qp * Cs + c;
-    }
-    __device__ __forceinline__ const bf16 *addr_b(int n, int k, int ke) const {
-        return (n < N && k < ke) ? w + (size_t)n * K + k : nullptr;
-    }
-    // 8 consecutive K elements of row n of B (the weights of one output)
-    __device__ __forceinline__ uint4 gather_b(int n, int k, int ke) const {
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (n < N && k < ke) v = *reinterpret_cast<const uint4 *>(w + (size_t)n * K + k);
-        return v;
-    }
-    __device__ __forceinline__ void load_a(bf16 (&a)[BM][LDS], int m0, int k0, int ke, int tid) const {
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int q = tid + i * GEMM_THREADS, r = q >> 2, cc = q & 3;
-            *reinterpret_cast<uint4 *>(&a[r][cc * 8]) = gather_a(m0 + r, k0 + cc * 8, ke);
-        }
-    }
-    __device__ __forceinline__ void load_b(bf16 (&b)[BN][LDS], int n0, int k0, int ke, int tid) const {
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int q = tid + i * GEMM_THREADS, r = q >> 2, cc = q & 3;
-            *reinterpret_cast<uint4 *>(&b[r][cc * 8]) = gather_b(n0 + r, k0 + cc * 8, ke);
-        }
-    }
-    // epilogue of 16 consecutive outputs (n multiple of 8, N a multiple of 8)
-    __device__ __forceinline__ void store16(int m, int n, const float *v) const {
-        if (m >= M) return;
-#pragma unroll
-        for (int h = 0; h < 2; h++) {
-            const int nh = n + 8 * h;
-            if (nh >= N) return;
-            float o[8];
-#pragma unroll
-            for (int j = 0; j < 8; j++) {
-                o[j] = v[8 * h + j];
-                if (bias) o[j] += bias[nh + j];
-                if (relu) o[j] = fmaxf(o[j], 0.f);
-            }
-            const size_t off = (size_t)m * N + nh;
-            if (mask) {
-                const uint4 mk = *reinterpret_cast<const uint4 *>(mask + off);
-                const bf16 *me = reinterpret_cast<const bf16 *>(&mk);
-#pragma unroll
-                for (int j = 0; j < 8; j++)
-                    if (!(__bfloat162float(me[j]) > 0.f)) o[j] = 0.f;
-            }
-            uint4 pk;
-            __nv_bfloat162 *pp = reinterpret_cast<__nv_bfloat162 *>(&pk);
-#pragma unroll
-            for (int j = 0; j < 4; j++) pp[j] = __floats2bfloat162_rn(o[2 * j], o[2 * j + 1]);
-            *reinterpret_cast<uint4 *>(out + off) = pk;
-        }
-    }
-    __device__ __forceinline__ void store(int m, int n, float v0, float v1) const {
-        if (m >= M || n >= N) return;
-        if (bias) {
-            v0 += bias[n];
-            v1 += bias[n + 1];
-        }
-        if (relu) {
-            v0 = fmaxf(v0, 0.f);
-            v1 = fmaxf(v1, 0.f);
-        }
-        const size_t o = (size_t)m * N + n;
-        if (mask) {
-            const __nv_bfloat162 mk = *reinterpret_cast<const __nv_bfloat162 *>(mask + o);
-            if (!(__bfloat162float(mk.x) > 0.f)) v0 = 0.f;
-            if (!(__bfloat162float(mk.y) > 0.f)) v1 = 0.f;
-        }
-        *reinterpret_cast<__nv_bfloat162 *>(out + o) = __floats2bfloat162_rn(v0, v1);
-    }
-};
-
-// Weight gradient: dw[co][tap][c] += sum_p dz[p][co] x[p + s(tap)][c] over
-// this block's pixel range (K = pixels).
-struct WgradOp {
-    const bf16 *dz;  // [P][Co]
-    const bf16 *x;   // [P][Ci]
-    float *dw;       // [Co][taps][Ci]
-    Img img;
-    int Co, Ci, taps;
-    int M, N, K, kchunk;  // M = Co, N = taps Ci, K = P
-
-    __device__ __forceinline__ void load_a(bf16 (&a)[BM][LDS], int m0, int k0, int ke, int tid) const {
-        // 32 pixels x 64 output channels: chunk (pixel, 8 channels), transposed into a[co][pixel]
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int q = tid + i * GEMM_THREADS, pl = q >> 3, cc = q & 7;
-            const int p = k0 + pl, co = m0 + cc * 8;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (p < ke && co < M) v = *reinterpret_cast<const uint4 *>(dz + (size_t)p * Co + co);
-            const bf16 *e = reinterpret_cast<const bf16 *>(&v);
-#pragma unroll
-            for (int j = 0; j < 8; j++) a[cc * 8 + j][pl] = e[j];
-        }
-    }
-    __device__ __forceinline__ void load_b(bf16 (&b)[BN][LDS], int n0, int k0, int ke, int tid) const {
-#pragma unroll
-        for (int i = 0; i < 2; i++) {
-            const int q = tid + i * GEMM_THREADS, pl = q >> 3, cc = q & 7;
-            const int p = k0 + pl, n = n0 + cc * 8;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (p < ke && n < N) {
-                const int tap = n / Ci, c = n - tap * Ci;
-                int qp = p;
-                bool ok = true;
-                if (taps == 9) ok = img.shift(p, tap / 3 - 1, tap % 3 - 1, qp);
-                if (ok) v = *reinterpret_cast<const uint4 *>(x + (size_t)qp * Ci + c);
-            }
-            const bf16 *e = reinterpret_cast<const bf16 *>(&v);
-#pragma unroll
-            for (int j = 0; j < 8; j++) b[cc * 8 + j][pl] = e[j];
-        }
-    }
-    __device__ __forceinline__ void store(int m, int n, float v0, float v1) const {
-        if (m >= M || n >= N) return;
-        atomicAdd(dw + (size_t)m * N + n, v0);
-        atomicAdd(dw + (size_t)m * N + n + 1, v1);
-    }
-};
-
-// ------------------------------------------------ tcgen05 convolution
-//
-// The forward and data-gradient convolutions (ConvOp) on the 5th-generation
-// tensor cores: a CTA of 128 threads owns a 128 x BN output tile whose FP32
-// accumulator lives in tensor memory (BN columns allocated per CTA).  Each K
-// block of 64 is gathered into shared memory with cp.async (16 bytes per
-// copy, zero-filled outside the image) in the K-major no-swizzle layout of
-// 8 x 16-byte core matrices (core matrix (row group g, K group j) at
-// g * 1024 + j * 128 bytes); one thread then issues four
-// tcgen05.mma.kind::f16 (M = 128, N = BN, K = 16; BF16 in, FP32 accumulate)
-// and commits them to the stage's mbarrier.  TC_STAGES stages: the copies of
-// the next blocks are in flight while the tensor cores work.  Every mbarrier
-// wait is bounded (by the network's wait limit, a number of polls); a wait
-// that runs out stops the pipeline, the CTA waits (bounded by TC_SPIN) for the
-// MMAs it has issued, frees its tensor memory, sets *err and stores nothing.
-constexpr int TC_M = 128, TC_K = 64, TC_THREADS = 256, TC_STAGES = 3;
-constexpr int TC_TABLE_MAX = 8192;  // bytes of the A operand's K table (K up to 8192)
-constexpr long long TC_SPIN = 1 << 24;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-    return (uint32_t)__cvta_generic_to_shared(p);
+// 8-channel groups of the K axis of a convolution with G source groups: taps come in
+// pairs of groups (K = 16 an instruction), so an odd G gets one more group of zero
+// weights, unless one group is all (the input layer): there two taps share a pair.
+__host__ __device__ inline int k_groups(int G, bool pair_taps) {
+    return pair_taps ? 10 : 9 * (G + (G & 1));
+}
+// N tile of a convolution with N outputs, and their number
+__host__ __device__ inline int n_tiles(int N) { return (N + 127) / 128; }
+__host__ __device__ inline int n_tile(int N) {
+    return ((N + n_tiles(N) - 1) / n_tiles(N) + 31) / 32 * 32;
+}
+// Element of the packed B operand [N tile][K group][n][8]: output n, tap, source
+// channel c; KG groups, Ge of them per tap.
+__host__ __device__ inline long long packed_at(int n, int tap, int c, int BN, int KG, int Ge) {
+    return (((long long)(n / BN) * KG + tap * Ge + c / 8) * BN + n % BN) * 8 + c % 8;
 }
 
-// shared-memory matrix descriptor: K-major, no swizzle, 128 B between K
-// groups (leading), 1024 B between 8-row groups (stride)
-__device__ __forceinline__ uint64_t tc_desc(uint32_t addr) {
-    uint64_t d = (uint64_t)((addr >> 4) & 0x3FFF);
-    d |= (uint64_t)(128 >> 4) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    return d;
-}
-
-__device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity, long long limit) {
-    uint32_t done = 0;
-    for (long long it = 0; it < limit && !done; it++)
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            "selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(mbar), "r"(parity)
-            : "memory");
-    return done != 0;
-}
-
-// 16-byte global -> shared copy; a null source fills zeros
-__device__ __forceinline__ void cp16(uint32_t dst, const void *src, const void *dummy) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(dst),
-                 "l"(src ? src : dummy), "r"(src ? 16 : 0)
-                 : "memory");
-}
-
-// The MMA pipeline of the tcgen05 kernels: TC_STAGES shared-memory stages
-// filled with cp.async by every thread (stage(i, addr) copies K block i; it is
-// called for i = 0, 1, 2, ... in order), one thread issuing a block's four
-// K = 16 MMAs (mma(addr, accumulate)) and committing them to the stage's
-// mbarrier, which is waited for (at most `limit` polls) before the stage is
-// refilled.  The block of iteration j completes phase j / TC_STAGES of barrier
-// j % TC_STAGES, and every barrier has at most one phase outstanding when it
-// is waited for.  A wait that gives up in any thread ends the pipeline before
-// the next MMA (no stage is refilled while the tensor cores may read it);
-// the issuing thread then commits once more to the drain barrier
-// mbar[TC_STAGES], which completes when every MMA it issued has, and the CTA
-// waits for that (at most TC_SPIN polls) before its tensor memory is read or
-// freed.  Returns false, in every thread, when a wait gave up.
-template <int STAGE, class StageFn, class MmaFn>
-__device__ __forceinline__ bool tc_pipeline(int nk, uint32_t base, uint64_t *mbar, int tid,
-                                            long long limit, StageFn &&stage, MmaFn &&mma) {
-    bool ok = true;
-    int issued = 0;  // K blocks whose MMAs were issued (the same in every thread)
-#pragma unroll
-    for (int st = 0; st < TC_STAGES - 1; st++) {
-        if (st < nk) stage(st, base + st * STAGE);
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    for (int kt = 0; kt < nk; kt++) {
-        const int s = kt % TC_STAGES;
-        asm volatile("cp.async.wait_group %0;\n" ::"n"(TC_STAGES - 2) : "memory");
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        if (__syncthreads_or(!ok)) break;
-        if (tid == 0) {
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            mma(base + s * STAGE, kt > 0);
-            asm volatile(
-                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                    smem_u32(&mbar[s])));
-        }
-        issued = kt + 1;
-        // refill the stage of block kt - 1 once its MMAs are done
-        const int nxt = kt + TC_STAGES - 1;
-        if (nxt < nk) {
-            if (kt > 0)
-                ok &= tc_wait(smem_u32(&mbar[(kt - 1) % TC_STAGES]), ((kt - 1) / TC_STAGES) & 1,
-                              limit);
-            if (ok) stage(nxt, base + (nxt % TC_STAGES) * STAGE);
-        }
-        asm volatile("cp.async.commit_group;\n" ::: "memory");
-    }
-    // blocks max(nk - TC_STAGES, 0) .. nk - 1 have not been waited for
-    if (issued == nk)
-        for (int j = nk > TC_STAGES ? nk - TC_STAGES : 0; j < nk; j++)
-            ok &= tc_wait(smem_u32(&mbar[j % TC_STAGES]), (j / TC_STAGES) & 1, limit);
-    ok = __syncthreads_and(ok);
-    if (!ok) {
-        if (tid == 0)
-            asm volatile(
-                "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
-                    smem_u32(&mbar[TC_STAGES])));
-        tc_wait(smem_u32(&mbar[TC_STAGES]), 0, TC_SPIN);
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    asm volatile("tcgen05.fence::after_thread_sync;\n");
-    return ok;
-}
-
-__device__ __forceinline__ void tc_alloc(uint32_t *slot, uint64_t *mbar, int ncols, int warp, int tid) {
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                         smem_u32(slot)),
-                     "r"(ncols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
-    }
-    if (tid == 0) {
-        for (int s = 0; s <= TC_STAGES; s++)
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mbar[s])));
-        asm volatile("fence.mbarrier_init.release.cluster;\n");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n");
-}
-
-__device__ __forceinline__ void tc_free(uint32_t tmem, int ncols, int warp) {
-    asm volatile("tcgen05.fence::before_thread_sync;\n");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(ncols));
-}
-
-// 16 consecutive FP32 accumulator columns of this warp's 32 TMEM lanes
-__device__ __forceinline__ void tc_ld16(uint32_t addr, float (&f)[16]) {
-    uint32_t v[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-        "%14,%15}, [%16];\n"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-          "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-          "=r"(v[14]), "=r"(v[15])
-        : "r"(addr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-    for (int j = 0; j < 16; j++) f[j] = __uint_as_float(v[j]);
-}
-
-__device__ __forceinline__ void tc_mma(uint32_t tmem, uint64_t ad, uint64_t bd, uint32_t idesc,
-                                       uint32_t acc) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.u32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-        "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
-}
-
-// Shared-memory table of the K axis of a convolution's A operand, one entry
-// per 8 consecutive K elements: the element offset of the 8 source channels
-// from the row's own pixel, and the index 3 dy + dx + 4 of the displacement
-// (31 beyond K, which no row's bounds mask has).
-__device__ __forceinline__ void conv_table(const ConvOp &op, int2 *tab, int nent, int tid) {
-    for (int e = tid; e < nent; e += TC_THREADS) {
-        int2 v = make_int2(0, 31);
-        if (8 * e < op.K) {
-            const int k = 8 * e, tap = k / op.Cs, c = k - tap * op.Cs;
-            const int dy = op.taps == 9 ? op.sign * (tap / 3 - 1) : 0;
-            const int dx = op.taps == 9 ? op.sign * (tap % 3 - 1) : 0;
-            v = make_int2((dy * op.img.W + dx) * op.Cs + c, 3 * dy + dx + 4);
-        }
-        tab[e] = v;
-    }
-}
-
-template <int BN>
-__global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long long limit, int *err) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint32_t tmem_base;
-    __shared__ __align__(8) uint64_t mbar[TC_STAGES + 1];  // the stages' and the drain barrier
-    constexpr int STAGE = TC_M * TC_K * 2 + BN * TC_K * 2;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * BN;
-    const uint32_t base = smem_u32(smem);
-    const int nk = (op.K + TC_K - 1) / TC_K, nkk = op.K >> 3;
-    int2 *tab = reinterpret_cast<int2 *>(smem + TC_STAGES * STAGE);
-    conv_table(op, tab, nk * (TC_K / 8), tid);
-    // Copies: lanes l and l + 16 of a warp take 8-channel chunks 2j and 2j + 1
-    // of one row, so a warp reads 16 rows x 32 contiguous bytes (whole
-    // sectors) and each 8-lane phase writes 8 rows of one core matrix.
-    // This thread's A row (a pixel) and its 3x3 neighbours inside the image:
-    const int r = 16 * warp + (lane & 15), p = m0 + r;
-    uint32_t inb = 0;
-    const bf16 *arow = op.src;
-    if (p < op.M) {
-        const int hw = op.img.H * op.img.W, q = p % hw, y = q / op.img.W, x = q - y * op.img.W;
-#pragma unroll
-        for (int b = 0; b < 9; b++) {
-            const int ys = y + b / 3 - 1, xs = x + b % 3 - 1;
-            if (ys >= 0 && ys < op.img.H && xs >= 0 && xs < op.img.W) inb |= 1u << b;
-        }
-        arow = op.src + (size_t)p * op.Cs;
-    }
-    // this thread's B row (an output channel) and first chunk pair
-    const int rb = 16 * (warp % (BN / 16)) + (lane & 15), nb = n0 + rb, kpb = warp / (BN / 16);
-    const bf16 *brow = op.w + (size_t)(nb < op.N ? nb : 0) * op.K;
-    tc_alloc(&tmem_base, mbar, BN, warp, tid);  // its barrier also publishes the table
-    const uint32_t tmem = tmem_base;
-    // kind::f16: D FP32, A and B BF16, both K-major, N = BN, M = 128
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                           ((uint32_t)(TC_M >> 4) << 24);
-    auto stage = [&](int kt, uint32_t sa) {
-        const uint32_t sb = sa + TC_M * TC_K * 2;
-        const int kk0 = kt * (TC_K / 8);
-#pragma unroll
-        for (int i = 0; i < TC_M * 8 / TC_THREADS; i++) {
-            const int kg = 2 * i + (lane >> 4);
-            const int2 e = tab[kk0 + kg];
-            cp16(sa + (r >> 3) * 1024 + kg * 128 + (r & 7) * 16,
-                 ((inb >> e.y) & 1u) ? arow + e.x : nullptr, op.src);
-        }
-#pragma unroll
-        for (int i = 0; i < BN * 8 / TC_THREADS; i++) {
-            const int kg = 2 * (kpb + (TC_M / BN) * i) + (lane >> 4), kk = kk0 + kg;
-            cp16(sb + (rb >> 3) * 1024 + kg * 128 + (rb & 7) * 16,
-                 (nb < op.N && kk < nkk) ? brow + 8 * kk : nullptr, op.w);
-        }
-    };
-    auto mma = [&](uint32_t sa, bool accumulate) {
-        const uint32_t sb = sa + TC_M * TC_K * 2;
-#pragma unroll
-        for (int ks = 0; ks < TC_K / 16; ks++)
-            tc_mma(tmem, tc_desc(sa + ks * 256), tc_desc(sb + ks * 256), idesc,
-                   (accumulate || ks > 0) ? 1u : 0u);
-    };
-    const bool ok = tc_pipeline<STAGE>(nk, base, mbar, tid, limit, stage, mma);
-    if (!ok) atomicOr(err, 1);
-    // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, columns of half w / 4
-    const int row = m0 + (warp & 3) * 32 + lane, cb = (warp >> 2) * (BN / 2);
-#pragma unroll
-    for (int c0 = 0; c0 < BN / 2; c0 += 16) {
-        float f[16];
-        tc_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb + c0, f);
-        if (ok && n0 + cb + c0 < op.N) op.store16(row, n0 + cb + c0, f);
-    }
-    tc_free(tmem, BN, warp);
-}
-
-// Weight gradient on tcgen05: dw[co][tap][ci] += sum_p x[p + s(tap)][ci] dz[p][co],
-// i.e. D[m][n] with m = (tap, ci) (M = taps Cin), n = co, K = pixels.  Both
-// operands are MN-major in shared memory (8 consecutive channels of one
-// pixel form a 16-byte core-matrix row), so they are copied straight from the
-// NHWC tensors: core matrix (MN group g, K group j) at j * LBO + g * 128
-// bytes, LBO = (rows / 8) * 128.  The pixel range of a block is one split of
-// K (gridDim.z); results are added to dw with FP32 atomics.
-struct WgradTc {
-    const bf16 *dz;  // [P][Co]
-    const bf16 *x;   // [P][Ci]
-    float *dw;       // [Co][taps][Ci]
-    Img img;
-    int Co, Ci, taps, M, N, K, kchunk;  // M = taps Ci, N = Co, K = P
-};
-
-template <int BN>
-__global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const WgradTc op, long long limit, int *err) {
-    extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint32_t tmem_base;
-    __shared__ __align__(8) uint64_t mbar[TC_STAGES + 1];  // the stages' and the drain barrier
-    constexpr int STAGE = TC_M * TC_K * 2 + BN * TC_K * 2;
-    constexpr int AG = TC_M * TC_K / 8 / TC_THREADS, BG = BN * TC_K / 8 / TC_THREADS;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * TC_M, n0 = blockIdx.y * BN;
-    const int kb = blockIdx.z * op.kchunk, ke = min(op.K, kb + op.kchunk);
-    const int nk = ke > kb ? (ke - kb + TC_K - 1) / TC_K : 0;
-    const uint32_t base = smem_u32(smem);
-    // This thread copies pixel pl of every K block, channel groups
-    // g = 2 (w / 4 + 2 i) + l / 16 (warp w, lane l): lanes l and l + 16 take
-    // adjacent groups of one pixel (32 contiguous bytes), and each 8-lane
-    // phase writes 8 pixels of one core matrix.  The (tap, channel) of each A
-    // group is fixed: its offset from the pixel and displacement (dy, dx).
-    const int pl = 16 * (warp & 3) + (lane & 15), g0 = 2 * (warp >> 2) + (lane >> 4);
-    int aoff[AG], ady[AG], adx[AG];
-#pragma unroll
-    for (int i = 0; i < AG; i++) {
-        const int m = m0 + 8 * (g0 + 4 * i);
-        aoff[i] = 0;
-        ady[i] = 1 << 20;  // never inside the image
-        adx[i] = 0;
-        if (m < op.M) {
-            const int tap = m / op.Ci, c = m - tap * op.Ci;
-            ady[i] = op.taps == 9 ? tap / 3 - 1 : 0;
-            adx[i] = op.taps == 9 ? tap % 3 - 1 : 0;
-            aoff[i] = (ady[i] * op.img.W + adx[i]) * op.Ci + c;
-        }
-    }
-    // coordinates of this thread's pixel, advanced by TC_K per block
-    int p = kb + pl, xx = p % op.img.W, yy = (p / op.img.W) % op.img.H;
-    tc_alloc(&tmem_base, mbar, BN < 32 ? 32 : BN, warp, tid);
-    const uint32_t tmem = tmem_base;
-    // kind::f16: D FP32, A and B BF16, both MN-major, N = BN, M = 128
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
-                           ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
-    auto stage = [&](int, uint32_t sa) {
-        const uint32_t sb = sa + TC_M * TC_K * 2;
-        const bool pv = p < ke;
-#pragma unroll
-        for (int i = 0; i < AG; i++) {
-            const int g = g0 + 4 * i;
-            const bool in = pv && (unsigned)(yy + ady[i]) < (unsigned)op.img.H &&
-                            (unsigned)(xx + adx[i]) < (unsigned)op.img.W;
-            cp16(sa + (pl >> 3) * (TC_M / 8 * 128) + g * 128 + (pl & 7) * 16,
-                 in ? op.x + (size_t)p * op.Ci + aoff[i] : nullptr, op.x);
-        }
-#pragma unroll
-        for (int i = 0; i < BG; i++) {
-            const int g = g0 + 4 * i, n = n0 + 8 * g;
-            cp16(sb + (pl >> 3) * (BN / 8 * 128) + g * 128 + (pl & 7) * 16,
-                 (pv && n < op.N) ? op.dz + (size_t)p * op.Co + n : nullptr, op.dz);
-        }
-        p += TC_K;
-        xx += TC_K;
-        while (xx >= op.img.W) {
-            xx -= op.img.W;
-            if (++yy == op.img.H) yy = 0;
-        }
-    };
-    auto mma = [&](uint32_t sa, bool accumulate) {
-        const uint32_t sb = sa + TC_M * TC_K * 2;
-#pragma unroll
-        for (int ks = 0; ks < TC_K / 16; ks++) {
-            // two K groups per MMA; leading offset = K-group stride, stride offset = 128
-            uint64_t ad = (uint64_t)(((sa + ks * 2 * (TC_M / 8 * 128)) >> 4) & 0x3FFF);
-            ad |= (uint64_t)((TC_M / 8 * 128) >> 4) << 16;
-            ad |= (uint64_t)(128 >> 4) << 32;
-            ad |= (uint64_t)1 << 46;
-            uint64_t bd = (uint64_t)(((sb + ks * 2 * (BN / 8 * 128)) >> 4) & 0x3FFF);
-            bd |= (uint64_t)((BN / 8 * 128) >> 4) << 16;
-            bd |= (uint64_t)(128 >> 4) << 32;
-            bd |= (uint64_t)1 << 46;
-            tc_mma(tmem, ad, bd, idesc, (accumulate || ks > 0) ? 1u : 0u);
-        }
-    };
-    const bool ok = tc_pipeline<STAGE>(nk, base, mbar, tid, limit, stage, mma);
-    if (!ok) atomicOr(err, 1);
-    const int m = m0 + (warp & 3) * 32 + lane, cb = (warp >> 2) * (BN / 2);
-#pragma unroll
-    for (int c0 = 0; c0 < BN / 2; c0 += 16) {
-        float f[16];
-        tc_ld16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + cb + c0, f);
-        if (ok && m < op.M && nk > 0) {
-#pragma unroll
-            for (int j = 0; j < 16; j++) {
-                const int n = n0 + cb + c0 + j;
-                if (n < op.N) atomicAdd(op.dw + (size_t)n * op.M + m, f[j]);
-            }
-        }
-    }
-    tc_free(tmem, BN < 32 ? 32 : BN, warp);
-}
-
-// ------------------------------------------------------ other layers
-
-constexpr int EW = 256;  // threads of the elementwise kernels
-
-inline unsigned blocks(long long n) { return (unsigned)((n + EW - 1) / EW); }
-
-// NCHW float input [B][8][H][W] -> NHWC BF16 [P][8]
-__global__ void k_pack_input(const float *in, bf16 *x, int B, int HW) {
-    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)B * HW * 8) return;
-    const int c = (int)(i & 7);
-    const long long p = i >> 3, n = p / HW, r = p - n * HW;
-    x[i] = __float2bfloat16(in[(n * 8 + c) * HW + r]);
-}
-
-// The NHWC layers below work on groups of 8 channels (one 16-byte word);
-// every channel count is a multiple of 8.
+// 8 channels of a pixel
 __device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
     const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
 #pragma unroll
@@ -678,110 +99,679 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
     return v;
 }
 
-// 2x2 average pooling of NHWC [B][H][W][C] into [B][H/2][W/2][C]
-__global__ void k_pool(const bf16 *in, bf16 *out, int B, int H, int W, int C) {
-    const int G = C / 8, Ho = H / 2, Wo = W / 2;
-    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)B * Ho * Wo * G) return;
-    const int g = (int)(i % G);
-    const long long p = i / G;
-    const int x = (int)(p % Wo), y = (int)((p / Wo) % Ho);
-    const long long n = p / ((long long)Wo * Ho);
-    const long long b0 = ((n * H + 2 * y) * W + 2 * x) * C + 8 * g;
-    float a[8], t[8];
-    unpack8(*reinterpret_cast<const uint4 *>(in + b0), a);
-    const long long offs[3] = {C, (long long)W * C, (long long)W * C + C};
+// ------------------------------------------------ tcgen05 convolution
+
+constexpr int TC_M = 128, TC_THREADS = 192;  // producer warp, MMA warp, four epilogue warps
+constexpr int TC_MAX_STAGES = 10, TC_MAX_A = 4;
+constexpr int TC_KB = 16;                // K groups of 8 channels per stage of B, at most
+constexpr long long TC_SPIN = 1 << 24;
+
+__device__ __forceinline__ uint32_t smem_u32(const void *p) {
+    return (uint32_t)__cvta_generic_to_shared(p);
+}
+
+// Shared-memory matrix descriptor without swizzle: `lead` bytes between K groups
+// (8 channels, or 8 pixels when K is the pixels), `stride` bytes between groups of 8
+// rows (pixels, outputs, or channels).
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr, uint32_t lead) { return addr >> 4 | lead >> 4 << 16; }
+__host__ __device__ constexpr uint32_t desc_hi(uint32_t stride) { return stride >> 4 | 1u << 14; }
+
+// Waits for phase `parity` of an mbarrier, at most `limit` polls.
+__device__ __forceinline__ bool tc_wait(uint32_t mbar, uint32_t parity, long long limit) {
+    uint32_t done = 0;
+    for (long long it = 0; it < limit && !done; it++)
+        asm volatile(
+            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(mbar), "r"(parity)
+            : "memory");
+    return done != 0;
+}
+
+__device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(mbar), "r"(count));
+}
+__device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(mbar), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_arrive(uint32_t mbar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(mbar) : "memory");
+}
+// contiguous global -> shared copy (16-byte aligned, a multiple of 16 bytes)
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+        "l"(src), "r"(bytes), "r"(mbar)
+        : "memory");
+}
+// the mbarrier completes a phase when every MMA this thread issued has
+__device__ __forceinline__ void tc_commit(uint32_t mbar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(mbar)
+        : "memory");
+}
+__device__ __forceinline__ void tc_alloc(uint32_t *slot, int ncols) {  // one warp
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(slot)),
+                 "r"(ncols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
+}
+__device__ __forceinline__ void tc_free(uint32_t tmem, int ncols, int warp) {
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(ncols));
+}
+
+// 32 consecutive FP32 accumulator columns of this warp's 32 TMEM lanes
+__device__ __forceinline__ void tc_ld32(uint32_t addr, float (&f)[32]) {
+    uint32_t v[32];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
+          "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]),
+          "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]),
+          "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(addr));
 #pragma unroll
-    for (int k = 0; k < 3; k++) {
-        unpack8(*reinterpret_cast<const uint4 *>(in + b0 + offs[k]), t);
+    for (int j = 0; j < 32; j++) f[j] = __uint_as_float(v[j]);
+}
+
+// one lane of the calling warp
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+    return p != 0;
+}
+
+// One MMA from the low words of its descriptors (address and leading stride) and their
+// common high words (stride between row groups).  The issuing warp's own instructions
+// are in series, and the MMA takes its operands from uniform registers: the whole warp
+// runs the loops, on values that are uniform by construction, and one lane issues.
+// (One thread, with tap offsets from shared memory, issued an MMA in 200 cycles, where
+// one takes 50 to 64.)
+__device__ __forceinline__ void tc_mma(uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                       uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n.reg .pred p;\n.reg .b64 a, b;\nsetp.ne.u32 p, %6, 0;\nmov.b64 a, {%1, %2};\nmov.b64 b, {%3, %4};\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(tmem),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc));
+}
+
+// The barriers and flags of a kernel's pipeline.  A producer warp fills shared-memory
+// stages with bulk copies, one thread issues MMAs, further warps read.  full[s]
+// completes when a fill's bytes have arrived, empty[s] when the stage's readers are
+// done.  A wait that gives up (`limit` polls) in any role raises `abort`: the other
+// roles stop at their next wait, and before the CTA frees its tensor memory the
+// producer waits for the copies it has in flight and the issuer for its MMAs (at most
+// TC_SPIN polls each).
+struct Pipe {
+    uint64_t full[TC_MAX_STAGES], empty[TC_MAX_STAGES];    // the stages
+    uint64_t afull[TC_MAX_A], aempty[TC_MAX_A];            // convolution: tiles of A
+    uint64_t tfull[2], tempty[2];                          // accumulators
+    uint64_t once, drain;
+    uint32_t tmem;
+    int abort;
+};
+
+__device__ __forceinline__ void pipe_init(Pipe &pp, int readers, int ncols, int warp, int tid) {
+    if (warp == 0) tc_alloc(&pp.tmem, ncols);
+    if (warp == 1) {
+        constexpr int N = offsetof(Pipe, tmem) / 8;  // all barriers, a lane each
+        static_assert(N <= 64, "two per lane");
+        for (int k = tid & 31; k < N; k += 32) {
+            uint64_t *b = pp.full + k;
+            mbar_init(smem_u32(b), b >= pp.empty && b < pp.afull ? readers : (b >= pp.tempty && b < &pp.once ? 4 : 1));
+        }
+        if ((tid & 31) == 0) pp.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;\n");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;\n");
+}
+
+// Wait of one role; raises abort when it gives up, and stops when another role has.
+__device__ __forceinline__ bool pipe_wait(Pipe &pp, uint64_t &bar, uint32_t parity, long long limit) {
+    for (long long it = 0; it < limit; it++) {
+        if (tc_wait(smem_u32(&bar), parity, 1)) return true;
+        if (*(volatile int *)&pp.abort) return false;
+    }
+    *(volatile int *)&pp.abort = 1;
+    return false;
+}
+// The same for a whole warp; every lane sees the completed phase.
+__device__ __forceinline__ bool pipe_wait_warp(Pipe &pp, uint64_t &bar, uint32_t parity, long long limit) {
+    const bool go = pipe_wait(pp, bar, parity, limit);
+    return __all_sync(0xffffffffu, go);
+}
+// Position in a ring of n stages: the stage, and the parity of its phase (no divisions:
+// the roles' own instructions are in series, and a division is as long as an MMA).
+struct Ring {
+    int s = 0;
+    uint32_t phase = 0;
+    bool first = true;  // not all stages used yet
+    __device__ __forceinline__ void next(int n) {
+        if (++s == n) {
+            s = 0;
+            phase ^= 1;
+            first = false;
+        }
+    }
+};
+// After an abort: the last fills of a ring of n stages, `fills` of them issued.
+__device__ __forceinline__ void drain_fills(uint64_t *full, int n, int fills) {
+    for (int c = max(fills - n, 0); c < fills; c++) tc_wait(smem_u32(&full[c % n]), (c / n) & 1, TC_SPIN);
+}
+// After an abort: the MMAs this thread has issued.
+__device__ __forceinline__ void drain_mmas(Pipe &pp) {
+    tc_commit(smem_u32(&pp.drain));
+    tc_wait(smem_u32(&pp.drain), 0, TC_SPIN);
+}
+
+// Forward convolution (sign = +1), or the gradient with respect to its input (sign =
+// -1, w the transposed weights): out[Q][n] = act(bias + sum over taps and source
+// channels of src[Q + sign s(tap)][c] w[n][tap][c]), times (mask > 0) when a mask is
+// given; with up, stored to the 2 x 2 pixels of the next finer level.
+struct ConvOp {
+    const bf16 *src;    // planes, sstr pixels each
+    const bf16 *w;      // packed, [N tile][KG][BN][8]
+    const float *bias;  // [N] or null
+    const bf16 *mask;   // planes as out, or null
+    bf16 *out;          // planes, ostr pixels each
+    long long sstr, ostr;
+    Geo geo, fine;
+    int B, G, N, Ge, KG, sign, relu, up;
+    // A in shared memory: a tile's pixels with their neighbours, once for all taps
+    // (nseg row segments of segpx pixels per plane, rowpx between rows), na buffers; or
+    // nseg = 0: too large, each stage brings its taps' A along
+    int nseg, segpx, rowpx, na;
+    int stages;  // of kb K groups of B (kb divides Ge); 0: all of B stays in shared memory
+    int kb;
+    int ntile;   // tiles of 128 padded pixels
+};
+
+// Persistent CTAs, tiles of 128 consecutive padded pixels x BN outputs.  Warp 0 copies
+// (a tile's A once for all taps; the weights once, where they fit beside it, else in
+// stages), a thread of warp 1 issues the MMAs in the order of K (tap by tap, channels
+// ascending) into one of two accumulators, warps 2 to 5 store the other.  What bounds
+// it: the operands' shared-memory reads at N = 32 and 64 (4 KB of A for 16 or 32 cycles
+// of tensor work), the streamed weights' way through L2 on the coarse levels.  One CTA
+// per tile, with everything in turn, left each CTA waiting for its own copies (8 to 14
+// us per tile, tensor pipe 6 to 17% active).
+template <int BN>
+__global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long long limit, int *err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) Pipe pp;
+    __shared__ __align__(16) float bias[BN];
+    constexpr uint32_t HI = desc_hi(128);
+    constexpr int ACC = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128), NCOLS = 2 * ACC;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockIdx.y;
+    const bool resident = op.nseg > 0, bstays = op.stages == 0;
+    const int S = op.stages, nkb = bstays ? 0 : op.KG / op.kb;
+    const uint32_t gs = resident ? (uint32_t)(op.nseg * op.segpx * 16) : TC_M * 16;  // K group stride
+    const uint32_t abytes = resident ? op.Ge * gs : 0;
+    const uint32_t a0 = smem_u32(smem), b0 = a0 + op.na * abytes;
+    const uint32_t stage = op.kb * (BN + (resident ? 0 : TC_M)) * 16;  // B, then A
+    const bf16 *w = op.w + (long long)nt * op.KG * BN * 8;
+    // displacement of tap t in pixels of the padded image
+    auto shift = [&](int t, int row) { return op.sign * ((t / 3 - 1) * row + t % 3 - 1); };
+    if (tid < BN) bias[tid] = op.bias && nt * BN + tid < op.N ? op.bias[nt * BN + tid] : 0.f;
+    pipe_init(pp, 1, NCOLS, warp, tid);
+    const uint32_t tmem = pp.tmem;
+    if (warp == 0) {
+        int fills = 0, afills = 0;
+        Ring br, ar;  // an empty[] of an earlier use: the other parity
+        bool go = true;
+        if (bstays && lane == 0) {
+            mbar_expect(smem_u32(&pp.once), op.KG * BN * 16);
+            for (int k = 0; k < op.KG; k += TC_KB)
+                bulk_copy(b0 + k * BN * 16, w + (long long)k * BN * 8, min(TC_KB, op.KG - k) * BN * 16,
+                          smem_u32(&pp.once));
+        }
+        const int ncopy = op.Ge * op.nseg;
+        for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x) {
+            const int q0 = op.geo.Wp + tile * TC_M;
+            if (resident) {
+                if (!ar.first) go = pipe_wait_warp(pp, pp.aempty[ar.s], ar.phase ^ 1, limit);
+                if (!go) break;
+                const uint32_t bar = smem_u32(&pp.afull[ar.s]), to = a0 + ar.s * abytes;
+                if (lane == 0) mbar_expect(bar, abytes);
+                __syncwarp();
+                for (int c = lane; c < ncopy; c += 32) {
+                    const int g = op.nseg == 3 ? c / 3 : c, sg = c - g * op.nseg;
+                    const long long from =
+                        (g < op.G ? g : 0) * op.sstr + q0 - 1 + (op.nseg == 3 ? (sg - 1) * op.geo.Wp : -op.geo.Wp);
+                    bulk_copy(to + c * op.segpx * 16, op.src + from * 8, op.segpx * 16, bar);
+                }
+                ar.next(op.na);
+                afills++;
+            }
+            for (int kb = 0; kb < nkb; kb++) {
+                const int n = op.kb;
+                if (!br.first) go = pipe_wait_warp(pp, pp.empty[br.s], br.phase ^ 1, limit);
+                if (!go) break;
+                const uint32_t at = b0 + br.s * stage, bar = smem_u32(&pp.full[br.s]);
+                if (lane == 0) {
+                    mbar_expect(bar, n * (BN + (resident ? 0 : TC_M)) * 16);
+                    bulk_copy(at, w + (long long)kb * n * BN * 8, n * BN * 16, bar);
+                }
+                __syncwarp();
+                if (!resident && lane < n) {
+                    const int kg = kb * n + lane, t = kg / op.Ge, g = kg % op.Ge;
+                    bulk_copy(at + n * BN * 16 + lane * TC_M * 16,
+                              op.src + ((g < op.G ? g : 0) * op.sstr + q0 + shift(t, op.geo.Wp)) * 8, TC_M * 16, bar);
+                }
+                br.next(S);
+                fills++;
+            }
+        }
+        __syncwarp();
+        if (lane == 0 && *(volatile int *)&pp.abort) {
+            if (bstays) tc_wait(smem_u32(&pp.once), 0, TC_SPIN);
+            else drain_fills(pp.full, S, fills);
+            drain_fills(pp.afull, op.na, afills);
+        }
+    } else if (warp == 1) {
+        // kind::f16: D FP32, A and B BF16, both K-major, M = 128, N = BN
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) |
+                                   ((uint32_t)(TC_M >> 4) << 24);
+        const bool leader = elect_one();
+        bool go = !bstays || pipe_wait_warp(pp, pp.once, 0, limit), issued = false;
+        Ring br, ar, acr;  // stages, tiles of A, accumulators
+        for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x) {
+            if (!acr.first) go = pipe_wait_warp(pp, pp.tempty[acr.s], acr.phase ^ 1, limit);
+            if (go && resident) go = pipe_wait_warp(pp, pp.afull[ar.s], ar.phase, limit);
+            if (!go) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const uint32_t d = tmem + acr.s * ACC, abuf = a0 + ar.s * abytes;
+            uint32_t blo = desc_lo(b0, BN * 16), acc = 0;
+            if (op.Ge == 1) {
+                // one group (all of B stays): two taps each, the distance between them
+                // the stride of K groups; the last one's partner (the next pixel) has
+                // zero weights
+#pragma unroll
+                for (int t = 0; t < 10; t += 2) {
+                    const uint32_t o0 = t / 3 * op.rowpx + t % 3, o1 = t < 8 ? (t + 1) / 3 * op.rowpx + (t + 1) % 3 : o0 + 1;
+                    if (leader) tc_mma(d, desc_lo(abuf, (o1 - o0) * 16) + o0, HI, blo, HI, idesc, t > 0);
+                    blo += 2 * BN;
+                }
+            } else if (bstays) {
+                const uint32_t alo = desc_lo(abuf, gs) + (op.sign > 0 ? 0 : 2 * op.rowpx + 2);
+                for (int dy = 0; dy < 3; dy++)
+                    for (int dx = 0; dx < 3; dx++) {
+                        uint32_t an = alo + op.sign * (dy * op.rowpx + dx);
+#pragma unroll 2
+                        for (int g = 0; g < op.Ge; g += 2) {
+                            if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
+                            acc = 1;
+                            an += gs >> 3;
+                            blo += 2 * BN;
+                        }
+                    }
+            } else if (resident) {
+                const uint32_t alo = desc_lo(abuf, gs) + (op.sign > 0 ? 0 : 2 * op.rowpx + 2);
+                for (int dy = 0; dy < 3 && go; dy++)
+                    for (int dx = 0; dx < 3 && go; dx++) {
+                        uint32_t an = alo + op.sign * (dy * op.rowpx + dx);
+                        for (int g0 = 0; g0 < op.Ge; g0 += op.kb) {  // a stage each
+                            if (!(go = pipe_wait_warp(pp, pp.full[br.s], br.phase, limit))) break;
+                            asm volatile("tcgen05.fence::after_thread_sync;\n");
+                            blo = desc_lo(b0 + br.s * stage, BN * 16);
+#pragma unroll 2
+                            for (int k = 0; k < op.kb; k += 2) {
+                                if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
+                                acc = 1;
+                                an += gs >> 3;
+                                blo += 2 * BN;
+                            }
+                            issued = true;
+                            if (leader) tc_commit(smem_u32(&pp.empty[br.s]));
+                            br.next(S);
+                        }
+                    }
+            } else {
+                for (int kb = 0; kb < nkb; kb++) {
+                    if (!(go = pipe_wait_warp(pp, pp.full[br.s], br.phase, limit))) break;
+                    asm volatile("tcgen05.fence::after_thread_sync;\n");
+                    const uint32_t at = b0 + br.s * stage;
+                    uint32_t an = desc_lo(at + op.kb * BN * 16, TC_M * 16);
+                    blo = desc_lo(at, BN * 16);
+#pragma unroll 2
+                    for (int k = 0; k < op.kb; k += 2) {
+                        if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
+                        acc = 1;
+                        an += 2 * TC_M;
+                        blo += 2 * BN;
+                    }
+                    issued = true;
+                    if (leader) tc_commit(smem_u32(&pp.empty[br.s]));
+                    br.next(S);
+                }
+            }
+            issued = true;
+            if (go && leader) {
+                if (resident) tc_commit(smem_u32(&pp.aempty[ar.s]));
+                tc_commit(smem_u32(&pp.tfull[acr.s]));
+            }
+            ar.next(op.na);
+            acr.next(2);
+        }
+        if (issued && leader && *(volatile int *)&pp.abort) drain_mmas(pp);
+        __syncwarp();
+    } else {
+        // epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31, a pixel per lane; the
+        // mask (one bit per channel) is fetched while the MMAs run
+        const int part = warp & 3, ng = (min(BN, op.N - nt * BN) + 7) >> 3;
+        const uint4 *mask = reinterpret_cast<const uint4 *>(op.mask) + (long long)(nt * BN >> 3) * op.ostr;
+        uint4 *out = reinterpret_cast<uint4 *>(op.out) + (long long)(nt * BN >> 3) * op.ostr;
+        int i = 0;
+        for (int tile = blockIdx.x; tile < op.ntile; tile += gridDim.x, i++) {
+            const int Q = op.geo.Wp + tile * TC_M + part * 32 + lane;
+            int n_, y, x;
+            const bool in = op.geo.where(Q, op.B, n_, y, x);
+            uint32_t keep[BN / 32];
+#pragma unroll
+            for (int c = 0; c < BN / 32; c++) {
+                keep[c] = 0xffffffffu;
+                if (!op.mask) continue;
+                uint4 mk[4];
+#pragma unroll
+                for (int h = 0; h < 4; h++)
+                    mk[h] = in && 4 * c + h < ng ? mask[(4 * c + h) * op.ostr + Q] : make_uint4(0, 0, 0, 0);
+                keep[c] = 0;
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    float m[8];
+                    unpack8(mk[h], m);
+#pragma unroll
+                    for (int j = 0; j < 8; j++) keep[c] |= m[j] > 0.f ? 1u << (8 * h + j) : 0u;
+                }
+            }
+            long long at = Q;
+            if (op.up && in) at = op.fine.at(n_, 2 * y, 2 * x);
+            if (!pipe_wait_warp(pp, pp.tfull[i & 1], (i / 2) & 1, limit)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+#pragma unroll
+            for (int c = 0; c < BN / 32; c++) {
+                float f[32];
+                __syncwarp();
+                tc_ld32(tmem + ((uint32_t)(part * 32) << 16) + (i & 1) * ACC + 32 * c, f);
+                if (c == BN / 32 - 1) {  // the accumulator is read
+                    asm volatile("tcgen05.fence::before_thread_sync;\n");
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&pp.tempty[i & 1]));
+                }
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    float o[8];
+#pragma unroll
+                    for (int j = 0; j < 8; j++) {
+                        o[j] = f[8 * h + j] + bias[32 * c + 8 * h + j];
+                        if (op.relu) o[j] = fmaxf(o[j], 0.f);
+                        if (!(keep[c] >> (8 * h + j) & 1u)) o[j] = 0.f;
+                    }
+                    if (!in || 4 * c + h >= ng) continue;
+                    const uint4 pk = pack8(o);
+                    uint4 *to = out + (4 * c + h) * op.ostr + at;
+                    to[0] = pk;
+                    if (op.up) {
+                        to[1] = pk;
+                        to[op.fine.Wp] = pk;
+                        to[op.fine.Wp + 1] = pk;
+                    }
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (tid == 0 && pp.abort) atomicOr(err, 1);
+    tc_free(tmem, NCOLS, warp);
+}
+
+// Weight gradient: for each dx a GEMM D[(dy, ci)][co] over the padded pixels, both
+// operands MN-major (8 consecutive channels of a pixel are a core-matrix row), so the
+// planes are copied as they are: 8-channel groups (dy, g) of 130 pixels, from (dy, -1)
+// on, and dz's groups of 128.  dx shifts A's start address by a pixel.  The border's
+// dz is zero, so its pixels add nothing.  A CTA takes 16 groups (128 rows) x BN outputs
+// and a run of chunks of 128 pixels; the result goes to dw with FP32 atomics, four outputs at a time.  The bias gradient, the sum of dz, is taken from the
+// staged dz by the epilogue warps.
+struct WgradOp {
+    const bf16 *x, *dz;  // planes, xstr and zstr pixels each
+    float *dw, *db;      // [tap][Ci][Co], [Co]
+    long long xstr, zstr;
+    int Wp, Ci, Co, G, stages;
+    int nchunk, perz;    // chunks of 128 pixels, and those of one CTA
+};
+constexpr int WG_PX = 128, WG_APX = WG_PX + 2;
+
+template <int BN>
+__global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const WgradOp op, long long limit, int *err) {
+    extern __shared__ __align__(1024) unsigned char smem[];
+    __shared__ __align__(8) Pipe pp;
+    __shared__ float bsum[BN];
+    constexpr int COLS = 3 * BN, NCOLS = COLS <= 128 ? 128 : (COLS <= 256 ? 256 : 512);
+    constexpr uint32_t AG = WG_APX * 16, ZG = WG_PX * 16;  // bytes of a group of A, of dz
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int m0 = blockIdx.x * 16;                       // first (dy, g) group
+    const int ng = min(16, 3 * op.G - m0);                // groups that exist
+    const int n0 = blockIdx.y * BN, zg = min(BN, op.Co - n0) / 8;
+    const int S = op.stages;
+    const uint32_t base = smem_u32(smem), stage = 16 * AG + BN / 8 * ZG;
+    const bool bias = blockIdx.x == 0;
+    const int first = blockIdx.z * op.perz, nmine = min(op.perz, op.nchunk - first);  // chunks
+    if (tid < BN) bsum[tid] = 0.f;
+    pipe_init(pp, bias ? 5 : 1, NCOLS, warp, tid);
+    const uint32_t tmem = pp.tmem;
+    if (warp == 0) {
+        int fills = 0;
+        Ring r;
+        for (int i = 0; i < nmine; i++, r.next(S)) {
+            if (!r.first && !pipe_wait_warp(pp, pp.empty[r.s], r.phase ^ 1, limit)) break;
+            const uint32_t at = base + r.s * stage, bar = smem_u32(&pp.full[r.s]);
+            if (lane == 0) mbar_expect(bar, ng * AG + zg * ZG);
+            __syncwarp();
+            const long long q = (long long)(first + i) * WG_PX;
+            for (int c = lane; c < ng + zg; c += 32) {
+                if (c < ng) {
+                    const int m = m0 + c, dy = m / op.G, g = m - dy * op.G;
+                    bulk_copy(at + c * AG, op.x + (g * op.xstr + q + (dy - 1) * op.Wp - 1) * 8, AG, bar);
+                } else {
+                    bulk_copy(at + 16 * AG + (c - ng) * ZG,
+                              op.dz + ((long long)(n0 / 8 + c - ng) * op.zstr + q) * 8, ZG, bar);
+                }
+            }
+            fills = i + 1;
+        }
+        __syncwarp();
+        if (lane == 0 && *(volatile int *)&pp.abort) drain_fills(pp.full, S, fills);
+    } else if (warp == 1) {
+        // kind::f16: D FP32, A and B BF16, both MN-major, M = 128, N = BN
+        constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                                   ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
+        const bool leader = elect_one();
+        bool go = true, issued = false;
+        Ring r;
+        for (int i = 0; i < nmine; i++, r.next(S)) {
+            if (!(go = pipe_wait_warp(pp, pp.full[r.s], r.phase, limit))) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const uint32_t at = base + r.s * stage, acc = i > 0;
+            const uint32_t alo = desc_lo(at, 128), zlo = desc_lo(at + 16 * AG, 128);
+            if (leader) {
+#pragma unroll
+                for (int dx = 0; dx < 3; dx++)
+#pragma unroll
+                    for (int ks = 0; ks < WG_PX / 16; ks++)
+                        tc_mma(tmem + dx * BN, alo + dx + ks * 16, desc_hi(AG), zlo + ks * 16, desc_hi(ZG), idesc,
+                               ks > 0 ? 1u : acc);
+                tc_commit(smem_u32(&pp.empty[r.s]));
+            }
+            issued = true;
+        }
+        if (go && leader) tc_commit(smem_u32(&pp.tfull[0]));
+        if (issued && leader && *(volatile int *)&pp.abort) drain_mmas(pp);
+        __syncwarp();
+    } else {
+        if (bias) {
+            // 128 threads: channel group g, every np-th pixel
+            const int t = tid - 64, g = t % zg, np = 128 / zg, p0 = t / zg;
+            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            Ring r;
+            for (int i = 0; i < nmine; i++, r.next(S)) {
+                if (!pipe_wait_warp(pp, pp.full[r.s], r.phase, limit)) break;
+                const uint4 *z = reinterpret_cast<const uint4 *>(smem + r.s * stage + 16 * AG + g * ZG);
+                if (p0 < np)
+                    for (int px = p0; px < WG_PX; px += np) {
+                        const uint4 v = z[px];
+                        const __nv_bfloat162 *h = reinterpret_cast<const __nv_bfloat162 *>(&v);
+#pragma unroll
+                        for (int j = 0; j < 4; j++) {
+                            const float2 f = __bfloat1622float2(h[j]);
+                            a[2 * j] += f.x;
+                            a[2 * j + 1] += f.y;
+                        }
+                    }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&pp.empty[r.s]));
+            }
+            if (p0 < np)
+#pragma unroll
+                for (int j = 0; j < 8; j++) atomicAdd(&bsum[g * 8 + j], a[j]);
+        }
+        if (pipe_wait_warp(pp, pp.tfull[0], 0, limit)) {
+            asm volatile("tcgen05.fence::after_thread_sync;\n");
+            const int part = warp & 3;
+            const int m = m0 + part * 4 + (lane >> 3);  // this lane's (dy, g)
+            const bool mine = m < 3 * op.G;
+            const int dy = m / op.G, ci = (m - dy * op.G) * 8 + (lane & 7);
+#pragma unroll
+            for (int dx = 0; dx < 3; dx++) {
+                float *row = op.dw + ((long long)(dy * 3 + dx) * op.Ci + ci) * op.Co + n0;
+#pragma unroll
+                for (int c0 = 0; c0 < BN; c0 += 32) {
+                    float f[32];
+                    __syncwarp();
+                    tc_ld32(tmem + ((uint32_t)(part * 32) << 16) + dx * BN + c0, f);
+#pragma unroll
+                    for (int j = 0; j < 32; j += 4)
+                        if (mine && n0 + c0 + j < op.Co)
+                            atomicAdd(reinterpret_cast<float4 *>(row + c0 + j),
+                                      make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]));
+                }
+            }
+        }
+    }
+    __syncthreads();
+    if (pp.abort) {
+        if (tid == 0) atomicOr(err, 1);
+    } else if (bias && tid < BN && n0 + tid < op.Co) {
+        atomicAdd(op.db + n0 + tid, bsum[tid]);
+    }
+    tc_free(tmem, NCOLS, warp);
+}
+
+// ------------------------------------------------------ other layers
+
+constexpr int EW = 256;  // threads of the elementwise kernels
+
+inline unsigned blocks(long long n) { return (unsigned)((n + EW - 1) / EW); }
+
+// NCHW float input [B][8][H][W] -> one plane
+__global__ void k_pack_input(const float *in, bf16 *x, int B, Geo geo) {
+    const int HW = geo.H * geo.W;
+    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
+    if (i >= (long long)B * HW) return;
+    const int n = (int)(i / HW), r = (int)(i - (long long)n * HW), y = r / geo.W;
+    float f[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) f[c] = in[((long long)n * 8 + c) * HW + r];
+    reinterpret_cast<uint4 *>(x)[geo.at(n, y, r - y * geo.W)] = pack8(f);
+}
+
+// The layers below take a group of 8 channels (blockIdx.y) of one pixel per thread:
+// neighbouring threads have neighbouring pixels, 16 bytes each.
+__device__ __forceinline__ bool pixel_of(long long i, int B, const Geo &geo, int &n, int &y, int &x) {
+    const int HW = geo.H * geo.W;
+    if (i >= (long long)B * HW) return false;
+    n = (int)(i / HW);
+    const int r = (int)(i - (long long)n * HW);
+    y = r / geo.W;
+    x = r - y * geo.W;
+    return true;
+}
+
+// 2x2 average pooling of planes on `fine` into planes on `geo`
+__global__ void k_pool(const bf16 *in, long long istr, bf16 *out, long long ostr, int B, Geo fine, Geo geo) {
+    int n, y, x;
+    if (!pixel_of((long long)blockIdx.x * EW + threadIdx.x, B, geo, n, y, x)) return;
+    const uint4 *p = reinterpret_cast<const uint4 *>(in) + blockIdx.y * istr + fine.at(n, 2 * y, 2 * x);
+    const uint4 v[4] = {p[0], p[1], p[fine.Wp], p[fine.Wp + 1]};
+    float a[8], t[8];
+    unpack8(v[0], a);
+#pragma unroll
+    for (int k = 1; k < 4; k++) {
+        unpack8(v[k], t);
 #pragma unroll
         for (int j = 0; j < 8; j++) a[j] += t[j];
     }
 #pragma unroll
     for (int j = 0; j < 8; j++) a[j] *= 0.25f;
-    *reinterpret_cast<uint4 *>(out + p * C + 8 * g) = pack8(a);
+    reinterpret_cast<uint4 *>(out)[blockIdx.y * ostr + geo.at(n, y, x)] = pack8(a);
 }
 
-// de[p][c] = (e[p][c] > 0) * dpool[p/2][c] / 4 + dskip[p][c] (dskip: a
-// channel slice of stride Cs at offset off, already masked)
-__global__ void k_pool_back(const bf16 *dpool, const bf16 *e, const bf16 *dskip, int Cs, int off,
-                            bf16 *de, int B, int H, int W, int C) {
-    const int G = C / 8;
-    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)B * H * W * G) return;
-    const int g = (int)(i % G);
-    const long long p = i / G;
-    const int x = (int)(p % W), y = (int)((p / W) % H);
-    const long long n = p / ((long long)W * H);
-    const long long q = (n * (H / 2) + y / 2) * (W / 2) + x / 2;
-    float dp[8], ev[8], ds[8] = {0, 0, 0, 0, 0, 0, 0, 0}, o[8];
-    unpack8(*reinterpret_cast<const uint4 *>(dpool + q * C + 8 * g), dp);
-    unpack8(*reinterpret_cast<const uint4 *>(e + p * C + 8 * g), ev);
-    if (dskip) unpack8(*reinterpret_cast<const uint4 *>(dskip + p * Cs + off + 8 * g), ds);
+// de = (e > 0) * dpool / 4 + dskip on `geo`, dpool on the next coarser level (dskip:
+// already masked)
+__global__ void k_pool_back(const bf16 *dpool, long long pstr, const bf16 *e, const bf16 *dskip, bf16 *de,
+                            long long str, int B, Geo coarse, Geo geo) {
+    int n, y, x;
+    if (!pixel_of((long long)blockIdx.x * EW + threadIdx.x, B, geo, n, y, x)) return;
+    const long long q = blockIdx.y * str + geo.at(n, y, x);
+    float dp[8], ev[8], ds[8], o[8];
+    unpack8(reinterpret_cast<const uint4 *>(dpool)[blockIdx.y * pstr + coarse.at(n, y / 2, x / 2)], dp);
+    unpack8(reinterpret_cast<const uint4 *>(e)[q], ev);
+    unpack8(reinterpret_cast<const uint4 *>(dskip)[q], ds);
 #pragma unroll
     for (int j = 0; j < 8; j++) o[j] = (ev[j] > 0.f ? 0.25f * dp[j] : 0.f) + ds[j];
-    *reinterpret_cast<uint4 *>(de + p * C + 8 * g) = pack8(o);
+    reinterpret_cast<uint4 *>(de)[q] = pack8(o);
 }
 
-// cat[p] = [up(d)[p] (Cu channels), e[p] (Ce channels)]
-__global__ void k_upcat(const bf16 *d, const bf16 *e, bf16 *cat, int B, int H, int W, int Cu,
-                        int Ce) {
-    const int Gc = (Cu + Ce) / 8, Gu = Cu / 8;
-    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)B * H * W * Gc) return;
-    const int g = (int)(i % Gc);
-    const long long p = i / Gc;
-    uint4 v;
-    if (g < Gu) {
-        const int x = (int)(p % W), y = (int)((p / W) % H);
-        const long long n = p / ((long long)W * H);
-        const long long q = (n * (H / 2) + y / 2) * (W / 2) + x / 2;
-        v = *reinterpret_cast<const uint4 *>(d + q * Cu + 8 * g);
-    } else {
-        v = *reinterpret_cast<const uint4 *>(e + p * Ce + 8 * (g - Gu));
-    }
-    *reinterpret_cast<uint4 *>(cat + p * (Cu + Ce) + 8 * g) = v;
-}
-
-// dd[q][c] = sum over the 2x2 children p of q of dcat[p][c], c < Cu
-__global__ void k_up_back(const bf16 *dcat, int Cc, bf16 *dd, int B, int Hc, int Wc, int Cu) {
-    const int G = Cu / 8;
-    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)B * Hc * Wc * G) return;
-    const int g = (int)(i % G);
-    const long long q = i / G;
-    const int x = (int)(q % Wc), y = (int)((q / Wc) % Hc);
-    const long long n = q / ((long long)Wc * Hc);
-    const int H = 2 * Hc, W = 2 * Wc;
-    const long long p0 = (n * H + 2 * y) * W + 2 * x;
-    const long long ps[4] = {p0, p0 + 1, p0 + W, p0 + W + 1};
+// dd on `geo` = sum over the 2x2 children of dcat on `fine`
+__global__ void k_up_back(const bf16 *dcat, long long cstr, bf16 *dd, long long str, int B, Geo fine, Geo geo) {
+    int n, y, x;
+    if (!pixel_of((long long)blockIdx.x * EW + threadIdx.x, B, geo, n, y, x)) return;
+    const uint4 *p = reinterpret_cast<const uint4 *>(dcat) + blockIdx.y * cstr + fine.at(n, 2 * y, 2 * x);
+    const uint4 v[4] = {p[0], p[1], p[fine.Wp], p[fine.Wp + 1]};
     float a[8] = {0, 0, 0, 0, 0, 0, 0, 0}, t[8];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        unpack8(*reinterpret_cast<const uint4 *>(dcat + ps[k] * Cc + 8 * g), t);
+        unpack8(v[k], t);
 #pragma unroll
         for (int j = 0; j < 8; j++) a[j] += t[j];
     }
-    *reinterpret_cast<uint4 *>(dd + q * Cu + 8 * g) = pack8(a);
+    reinterpret_cast<uint4 *>(dd)[blockIdx.y * str + geo.at(n, y, x)] = pack8(a);
 }
 
-// 1x1 head: out[n][o][y][x] = b[o] + sum_c w[o][c] d[p][c] (FP32), NCHW output
-__global__ void k_head(const bf16 *d, const float *w, const float *b, float *out, int B, int HW,
-                       int C) {
-    const long long p = (long long)blockIdx.x * EW + threadIdx.x;
-    if (p >= (long long)B * HW) return;
+// 1x1 head: out[n][o][y][x] = b[o] + sum_c w[o][c] d[c] (FP32), NCHW output
+__global__ void k_head(const bf16 *d, long long dstr, const float *w, const float *b, float *out, int B,
+                       Geo geo, int C) {
+    const long long i = (long long)blockIdx.x * EW + threadIdx.x;
+    int n, y, x;
+    if (!pixel_of(i, B, geo, n, y, x)) return;
+    const uint4 *p = reinterpret_cast<const uint4 *>(d) + geo.at(n, y, x);
     float acc[3] = {b[0], b[1], b[2]};
     for (int c = 0; c < C; c += 8) {
-        const uint4 v = *reinterpret_cast<const uint4 *>(d + p * C + c);
-        const bf16 *e = reinterpret_cast<const bf16 *>(&v);
+        float v[8];
+        unpack8(p[(c >> 3) * dstr], v);
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            const float x = __bfloat162float(e[j]);
+        for (int j = 0; j < 8; j++)
 #pragma unroll
-            for (int o = 0; o < 3; o++) acc[o] += w[o * C + c + j] * x;
-        }
+            for (int o = 0; o < 3; o++) acc[o] += w[o * C + c + j] * v[j];
     }
-    const long long n = p / HW, r = p - n * HW;
+    const long long HW = (long long)geo.H * geo.W, r = i - n * HW;
 #pragma unroll
     for (int o = 0; o < 3; o++) out[(n * 3 + o) * HW + r] = acc[o];
 }
@@ -824,73 +814,106 @@ __global__ void k_loss(const float *out, const float *tgt, const float *fluid, c
     if (threadIdx.x == 0) atomicAdd(loss, (double)(s[0] * inv));
 }
 
-// head backward: dd[p][c] = (d[p][c] > 0) sum_o dout[o][p] w[o][c];
-// dw[o][c] += sum_p dout[o][p] d[p][c]; db[o] += sum_p dout[o][p]
-template <int C>
-__global__ void k_head_back(const float *dout, const bf16 *d, const float *w, bf16 *dd, float *dw,
-                            float *db, int B, int HW) {
-    __shared__ float red[4 * C];
-    for (int i = threadIdx.x; i < 4 * C; i += blockDim.x) red[i] = 0.f;
+// head backward: dd[c] = (d[c] > 0) sum_o dout[o] w[o][c]; dw[o][c] += sum over the
+// pixels of dout[o] d[c]; db[o] += sum of dout[o].  A thread takes every
+// gridDim.x EW-th pixel of one group of 8 channels and keeps its 24 sums in registers
+// to the end (one pixel per thread and 96 warp sums for it took 220 us at 0.5 M
+// pixels, the memory traffic 12).
+__global__ void __launch_bounds__(EW) k_head_back(const float *dout, const bf16 *d, long long dstr,
+                                                  const float *w, bf16 *dd, float *dw, float *db, int B,
+                                                  Geo geo, int C) {
+    __shared__ float red[27];
+    if (threadIdx.x < 27) red[threadIdx.x] = 0.f;
     __syncthreads();
-    const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    float g[3] = {0.f, 0.f, 0.f};
-    float lw[3][C];
-    if (p < (long long)B * HW) {
-        const long long n = p / HW, r = p - n * HW;
+    const int c0 = blockIdx.y * 8;
+    const long long HW = (long long)geo.H * geo.W;
+    float wv[3][8], s[3][8], sb[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int o = 0; o < 3; o++)
+#pragma unroll
+        for (int j = 0; j < 8; j++) {
+            wv[o][j] = w[o * C + c0 + j];
+            s[o][j] = 0.f;
+        }
+    for (long long i = (long long)blockIdx.x * EW + threadIdx.x; i < B * HW; i += (long long)gridDim.x * EW) {
+        int n, y, x;
+        pixel_of(i, B, geo, n, y, x);
+        const long long q = blockIdx.y * dstr + geo.at(n, y, x), r = i - n * HW;
+        float g[3], v[8], o8[8];
 #pragma unroll
         for (int o = 0; o < 3; o++) g[o] = dout[(n * 3 + o) * HW + r];
+        unpack8(reinterpret_cast<const uint4 *>(d)[q], v);
 #pragma unroll
-        for (int c = 0; c < C; c++) {
-            const float x = __bfloat162float(d[p * C + c]);
-            const float v = g[0] * w[c] + g[1] * w[C + c] + g[2] * w[2 * C + c];
-            dd[p * C + c] = __float2bfloat16(x > 0.f ? v : 0.f);
+        for (int j = 0; j < 8; j++) {
+            const float t = g[0] * wv[0][j] + g[1] * wv[1][j] + g[2] * wv[2][j];
+            o8[j] = v[j] > 0.f ? t : 0.f;
 #pragma unroll
-            for (int o = 0; o < 3; o++) lw[o][c] = g[o] * x;
+            for (int o = 0; o < 3; o++) s[o][j] += g[o] * v[j];
         }
-    } else {
 #pragma unroll
-        for (int o = 0; o < 3; o++)
-#pragma unroll
-            for (int c = 0; c < C; c++) lw[o][c] = 0.f;
+        for (int o = 0; o < 3; o++) sb[o] += g[o];
+        reinterpret_cast<uint4 *>(dd)[q] = pack8(o8);
     }
-    // warp sums, then one shared atomic per warp and value
+    auto sum = [&](float v, int k) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(&red[k], v);
+    };
 #pragma unroll
     for (int o = 0; o < 3; o++) {
 #pragma unroll
-        for (int c = 0; c < C; c++) {
-            float v = lw[o][c];
-            for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
-            if ((threadIdx.x & 31) == 0) atomicAdd(&red[o * C + c], v);
-        }
-        float v = g[o];
-        for (int s = 16; s > 0; s >>= 1) v += __shfl_down_sync(0xffffffffu, v, s);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&red[3 * C + o], v);
+        for (int j = 0; j < 8; j++) sum(s[o][j], o * 8 + j);
+        sum(sb[o], 24 + o);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 3 * C; i += blockDim.x) atomicAdd(dw + i, red[i]);
-    if (threadIdx.x < 3) atomicAdd(db + threadIdx.x, red[3 * C + threadIdx.x]);
+    if (threadIdx.x < 24) atomicAdd(dw + (threadIdx.x >> 3) * C + c0 + (threadIdx.x & 7), red[threadIdx.x]);
+    if (blockIdx.y == 0 && threadIdx.x >= 24 && threadIdx.x < 27) atomicAdd(db + threadIdx.x - 24, red[threadIdx.x]);
 }
 
-// db[c] += sum_p dz[p][c] (NHWC BF16), C <= 256
-__global__ void k_colsum(const bf16 *dz, long long P, int C, float *db) {
-    __shared__ float s[EW];
-    const int c = threadIdx.x % C, rows = EW / C;
-    const int r0 = threadIdx.x / C;
-    float a = 0.f;
-    if (r0 < rows)
-        for (long long p = (long long)blockIdx.x * rows + r0; p < P; p += (long long)gridDim.x * rows)
-            a += __bfloat162float(dz[p * C + c]);
-    s[threadIdx.x] = a;
-    __syncthreads();
-    if (threadIdx.x < C) {
-        float t = 0.f;
-        for (int r = 0; r < rows; r++) t += s[r * C + threadIdx.x];
-        atomicAdd(db + threadIdx.x, t);
+// Where a parameter sits: the vector of all convolutions, weights [tap][Cin][Cout] (the
+// 1x1 head: [Cout][Cin]) then biases, both padded to 8; in the caller's order
+// [Cout][Cin][k][k] then biases, from abi; and the packed BF16 copies.
+constexpr int MAX_CONVS = 16;
+struct ConvTab {
+    struct E {
+        int w_off, b_off, abi, ci, co, taps;
+        bf16 *fwd, *bwd;  // null: none
+        int fBN, fKG, fGe, bBN, bKG, bGe;
+    } e[MAX_CONVS];
+    int n;
+    // caller's index of parameter i, or -1 (padding); the weight's (co, tap, ci) or co = -1
+    __device__ __forceinline__ long long abi_of(long long i, int &k, int &co, int &tap, int &ci) const {
+        k = 0;
+        while (k + 1 < n && i >= e[k + 1].w_off) k++;
+        const E &c = e[k];
+        co = -1;
+        if (i >= c.b_off) {
+            const int j = (int)(i - c.b_off);
+            return j < c.co ? c.abi + (long long)c.co * c.ci * c.taps + j : -1;
+        }
+        const int j = (int)(i - c.w_off);
+        if (j >= c.co * c.ci * c.taps) return -1;
+        if (c.taps == 1) {
+            co = j / c.ci;
+            ci = j - co * c.ci;
+            tap = 0;
+        } else {
+            co = j % c.co;
+            const int r = j / c.co;
+            tap = r / c.ci;
+            ci = r - tap * c.ci;
+        }
+        return c.abi + ((long long)co * c.ci + ci) * c.taps + tap;
     }
-}
+    __device__ __forceinline__ void pack(int k, int co, int tap, int ci, float v) const {
+        const E &c = e[k];
+        const bf16 b = __float2bfloat16(v);
+        if (c.fwd) c.fwd[packed_at(co, tap, ci, c.fBN, c.fKG, c.fGe)] = b;
+        if (c.bwd) c.bwd[packed_at(ci, tap, co, c.bBN, c.bKG, c.bGe)] = b;
+    }
+};
 
 // Adam on the flat FP32 master vector; refreshes the BF16 copies.
-__global__ void k_adam(float *w, const float *g, float *m, float *v, bf16 *wb, long long n, float lr,
+__global__ void k_adam(ConvTab tab, float *w, const float *g, float *m, float *v, long long n, float lr,
                        float c1, float c2) {
     const long long i = (long long)blockIdx.x * EW + threadIdx.x;
     if (i >= n) return;
@@ -900,20 +923,28 @@ __global__ void k_adam(float *w, const float *g, float *m, float *v, bf16 *wb, l
     v[i] = vi;
     const float wi = w[i] - lr * (mi / c1) / (sqrtf(vi / c2) + 1e-8f);
     w[i] = wi;
-    wb[i] = __float2bfloat16(wi);
+    int k, co, tap, ci;
+    if (tab.abi_of(i, k, co, tap, ci) >= 0 && co >= 0) tab.pack(k, co, tap, ci, wi);
 }
 
-__global__ void k_to_bf16(const float *w, bf16 *wb, long long n) {
+// The caller's parameter vector into the masters and BF16 copies
+__global__ void k_from_abi(ConvTab tab, const float *abi, float *w, long long n) {
     const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i < n) wb[i] = __float2bfloat16(w[i]);
+    if (i >= n) return;
+    int k, co, tap, ci;
+    const long long a = tab.abi_of(i, k, co, tap, ci);
+    const float v = a >= 0 ? abi[a] : 0.f;
+    w[i] = v;
+    if (a >= 0 && co >= 0) tab.pack(k, co, tap, ci, v);
 }
 
-// wt[ci][tap][co] = w[co][tap][ci]
-__global__ void k_transpose_w(const bf16 *w, bf16 *wt, int Co, int taps, int Ci) {
+// A vector in the masters' layout into the caller's order
+__global__ void k_to_abi(ConvTab tab, const float *w, float *abi, long long n) {
     const long long i = (long long)blockIdx.x * EW + threadIdx.x;
-    if (i >= (long long)Co * taps * Ci) return;
-    const int ci = (int)(i % Ci), tap = (int)((i / Ci) % taps), co = (int)(i / ((long long)Ci * taps));
-    wt[((long long)ci * taps + tap) * Co + co] = w[i];
+    if (i >= n) return;
+    int k, co, tap, ci;
+    const long long a = tab.abi_of(i, k, co, tap, ci);
+    if (a >= 0) abi[a] = w[i];
 }
 
 // network input of one case: mask (owner >= 0) and Re / 100, zero elsewhere
@@ -934,17 +965,28 @@ using nn::bf16;
 namespace {
 
 struct Conv {
-    int ci, co, k;           // k = 3 or 1
-    size_t w_off, b_off;     // into the flat parameter vector (internal layout)
-    bf16 *wt = nullptr;      // transposed BF16 weights [ci][tap][co]
+    int ci, co, k;            // k = 3 or 1
+    size_t w_off, b_off;      // into the flat parameter vector
+    bf16 *fwd = nullptr;      // packed BF16 weights of the forward convolution
+    bf16 *bwd = nullptr;      // and of the data gradient
+};
+
+// planes of 8 channels on one level's pixels
+struct Planes {
+    bf16 *p = nullptr;        // pixel 0 of the first plane
+    long long str = 0;        // pixels per plane
+    Planes group(int g) const { return Planes{p + (long long)g * str * 8, str}; }
 };
 
 struct Level {
-    int H, W, C;
-    bf16 *inp = nullptr;  // pooled input (l > 0)
-    bf16 *ea = nullptr, *e = nullptr;              // encoder: relu(conv a), level output
-    bf16 *cat = nullptr, *da = nullptr, *d = nullptr;  // decoder (l < L-1)
-    bf16 *g1 = nullptr, *g2 = nullptr, *gcat = nullptr, *gin = nullptr;  // gradients
+    nn::Geo geo;
+    int C;
+    Planes inp;               // pooled input (l > 0)
+    Planes ea;                // encoder: relu(conv a)
+    Planes cat;               // decoder (l < L-1): {upsampled output of level l + 1, e}
+    Planes e;                 // level output: the last C channels of cat (l < L-1)
+    Planes da, d;             // decoder: relu(conv a); relu(conv b) (l = 0: for the head)
+    Planes g1, g2, gcat, gin; // gradients
 };
 
 }  // namespace
@@ -955,13 +997,13 @@ struct lbm_unet {
     bool own_stream = false;
     std::vector<Conv> convs;  // parameter order
     std::vector<Level> lv;
-    long long nparam = 0;
+    nn::ConvTab tab{};
+    long long nparam = 0, nabi = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
-    bf16 *wb = nullptr;      // BF16 copy of the whole vector (biases unused)
-    bf16 *x = nullptr;       // packed input [P0][8]
+    Planes x;                // packed input
     float *out = nullptr, *dout = nullptr;
-    float *io_in = nullptr, *io_out = nullptr, *io_tgt = nullptr, *io_fl = nullptr;  // staging
-    float *grad_abi = nullptr;
+    float *io_in = nullptr, *io_tgt = nullptr, *io_fl = nullptr;  // staging
+    float *abi = nullptr;    // parameters or gradients in the caller's order
     float *cnt = nullptr;
     double *loss = nullptr;
     int *err_d = nullptr;    // bit 0: a bounded wait of a tensor-core kernel ran out
@@ -1015,6 +1057,19 @@ cudaError_t nalloc(lbm_unet *n, T **p, size_t count) {
     return e;
 }
 
+// C channels of planes for max_batch images, all zero, with room before and after
+// them that the convolutions' halos may read (zero as well)
+cudaError_t palloc(lbm_unet *n, Planes *q, const nn::Geo &geo, int C) {
+    const size_t front = (size_t)(geo.Wp + 16) / 8 * 8 + 8, back = nn::TC_M + geo.Wp + 32;
+    q->str = (long long)n->cfg.max_batch * geo.PSI;
+    const size_t px = front + (size_t)(C / 8) * q->str + back;
+    bf16 *base = nullptr;
+    cudaError_t e = nalloc(n, &base, px * 8);
+    if (e == cudaSuccess) e = cudaMemsetAsync(base, 0, px * 8 * sizeof(bf16), n->stream);
+    q->p = base + front * 8;
+    return e;
+}
+
 void nrelease(lbm_unet *n) {
     if (!n) return;
     for (void *p : n->allocs) cudaFree(p);
@@ -1030,201 +1085,178 @@ int conv_index(const lbm_unet *n, const char kind, int l, int ab) {
     return 2 * L + 2 * (L - 1);
 }
 
+constexpr int SMEM_MAX = 225 * 1024, SMEM_TWO = 111 * 1024;  // of one CTA; of each of two on an SM
+
 template <int BN>
-cudaError_t launch_tc(lbm_unet *n, const nn::ConvOp &op) {
-    constexpr int stages = nn::TC_STAGES * (nn::TC_M * nn::TC_K * 2 + BN * nn::TC_K * 2);
-    const int table = ((op.K + nn::TC_K - 1) / nn::TC_K) * nn::TC_K;  // 8 bytes per 8 K elements
-    if (table > nn::TC_TABLE_MAX) return cudaErrorInvalidValue;
+cudaError_t launch_tc(lbm_unet *n, nn::ConvOp &op) {
+    using namespace nn;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(nn::k_conv_tc<BN>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             stages + nn::TC_TABLE_MAX);
+        cudaError_t e = cudaFuncSetAttribute(k_conv_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const dim3 grid((op.M + nn::TC_M - 1) / nn::TC_M, (op.N + BN - 1) / BN);
-    nn::k_conv_tc<BN><<<grid, nn::TC_THREADS, stages + table, n->stream>>>(op, n->wait_limit, n->err_d);
+    // A once for all taps: three row segments where a tile is shorter than a row, else
+    // the run of pixels from the row above to the row below; in the stages, tap by tap,
+    // where it does not fit beside two stages of weights
+    op.kb = op.Ge < TC_KB ? op.Ge : TC_KB;
+    while (op.Ge % op.kb) op.kb -= 2;
+    const int wstage = op.kb * BN * 16, wall = op.KG * BN * 16;
+    op.nseg = op.geo.Wp >= TC_M + 2 ? 3 : 1;
+    // (pairs of taps: a pixel more, for the partner of the last tap)
+    op.segpx = (op.nseg == 3 ? TC_M + 2 : TC_M + 2 * op.geo.Wp + 2) + (op.Ge == 1);
+    op.rowpx = op.nseg == 3 ? op.segpx : op.geo.Wp;
+    int a = op.Ge * op.nseg * op.segpx * 16, smem = 0;
+    if (2 * a + wall <= SMEM_MAX) {  // all weights
+        op.stages = 0;
+        op.na = 2 * a + wall <= SMEM_TWO ? (SMEM_TWO - wall) / a : (SMEM_MAX - wall) / a;
+        if (op.na > TC_MAX_A) op.na = TC_MAX_A;
+        smem = op.na * a + wall;
+    } else if (a + 2 * wstage <= SMEM_MAX) {
+        op.na = 2 * a + 3 * wstage <= SMEM_MAX ? 2 : 1;
+        op.stages = (SMEM_MAX - op.na * a) / wstage;
+        if (op.stages > TC_MAX_STAGES) op.stages = TC_MAX_STAGES;
+        smem = op.na * a + op.stages * wstage;
+    } else {
+        op.nseg = 0;
+        op.na = 1;
+        const int both = wstage + op.kb * nn::TC_M * 16;
+        op.stages = SMEM_MAX / both < TC_MAX_STAGES ? SMEM_MAX / both : TC_MAX_STAGES;
+        smem = op.stages * both;
+    }
+    const long long rows = (long long)op.B * op.geo.PSI - op.geo.Wp;
+    op.ntile = (int)((rows + TC_M - 1) / TC_M);
+    const int ny = n_tiles(op.N);
+    int ctas = (smem <= SMEM_TWO ? 2 : 1) * n->sms / ny;
+    if (ctas > op.ntile) ctas = op.ntile;
+    if (ctas < 1) ctas = 1;
+    k_conv_tc<BN><<<dim3(ctas, ny), TC_THREADS, smem, n->stream>>>(op, n->wait_limit, n->err_d);
     return cudaGetLastError();
 }
 
-// N tile: the output channels rounded up to 32 or 64, else 128 unless that
-// leaves fewer than two tiles per SM
-cudaError_t launch_conv_tc(lbm_unet *n, const nn::ConvOp &op) {
-    const int mt = (op.M + nn::TC_M - 1) / nn::TC_M;
-    if (op.N <= 32) return launch_tc<32>(n, op);
-    if (op.N <= 64 || (long long)mt * ((op.N + 127) / 128) < 2LL * n->sms) return launch_tc<64>(n, op);
-    return launch_tc<128>(n, op);
+// src, out, mask: planes on geo (up: out on fine)
+cudaError_t conv(lbm_unet *n, const bf16 *w, int Cs, int N, int sign, const float *bias, bool relu,
+                 const Planes &src, const Planes *mask, const Planes &out, const nn::Geo &geo,
+                 const nn::Geo *fine, int B) {
+    nn::ConvOp op{};
+    op.src = src.p;
+    op.sstr = src.str;
+    op.w = w;
+    op.bias = bias;
+    op.mask = mask ? mask->p : nullptr;
+    op.out = out.p;
+    op.ostr = out.str;
+    op.geo = geo;
+    op.up = fine ? 1 : 0;
+    if (fine) op.fine = *fine;
+    op.B = B;
+    op.G = Cs / 8;
+    op.N = N;
+    const bool pairs = op.G == 1 && sign > 0;
+    op.Ge = pairs ? 1 : op.G + (op.G & 1);
+    op.KG = nn::k_groups(op.G, pairs);
+    op.sign = sign;
+    op.relu = relu;
+    switch (nn::n_tile(N)) {
+        case 32: return launch_tc<32>(n, op);
+        case 64: return launch_tc<64>(n, op);
+        case 96: return launch_tc<96>(n, op);
+        default: return launch_tc<128>(n, op);
+    }
 }
 
-cudaError_t conv_fwd(lbm_unet *n, const Conv &cv, const bf16 *src, bf16 *dst, int B, int H, int W,
-                     bool relu) {
-    nn::ConvOp op{};
-    op.src = src;
-    op.w = n->wb + cv.w_off;
-    op.bias = n->w + cv.b_off;
-    op.mask = nullptr;
-    op.out = dst;
-    op.img = {B, H, W};
-    op.Cs = cv.ci;
-    op.taps = cv.k * cv.k;
-    op.sign = 1;
-    op.relu = relu;
-    op.M = B * H * W;
-    op.N = cv.co;
-    op.K = op.taps * cv.ci;
-    op.kchunk = op.K;
-    return launch_conv_tc(n, op);
+cudaError_t conv_fwd(lbm_unet *n, const Conv &cv, const Planes &src, const Planes &out, const nn::Geo &geo,
+                     const nn::Geo *fine, int B) {
+    return conv(n, cv.fwd, cv.ci, cv.co, 1, n->w + cv.b_off, true, src, nullptr, out, geo, fine, B);
 }
 
 // gradient with respect to the conv's input (masked by mask > 0 when given)
-cudaError_t conv_dgrad(lbm_unet *n, const Conv &cv, const bf16 *dz, const bf16 *mask, bf16 *dx,
-                       int B, int H, int W) {
-    nn::ConvOp op{};
-    op.src = dz;
-    op.w = cv.wt;
-    op.bias = nullptr;
-    op.mask = mask;
-    op.out = dx;
-    op.img = {B, H, W};
-    op.Cs = cv.co;
-    op.taps = cv.k * cv.k;
-    op.sign = -1;
-    op.relu = 0;
-    op.M = B * H * W;
-    op.N = cv.ci;
-    op.K = op.taps * cv.co;
-    op.kchunk = op.K;
-    return launch_conv_tc(n, op);
+cudaError_t conv_dgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Planes *mask, const Planes &dx,
+                       const nn::Geo &geo, int B) {
+    return conv(n, cv.bwd, cv.co, cv.ci, -1, nullptr, false, dz, mask, dx, geo, nullptr, B);
 }
 
 template <int BN>
-cudaError_t launch_wg(lbm_unet *n, const nn::WgradTc &op, int z) {
-    constexpr int smem = nn::TC_STAGES * (nn::TC_M * nn::TC_K * 2 + BN * nn::TC_K * 2);
+cudaError_t launch_wg(lbm_unet *n, nn::WgradOp &op) {
+    using namespace nn;
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(nn::k_wgrad_tc<BN>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(k_wgrad_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_MAX);
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    const dim3 grid((op.M + nn::TC_M - 1) / nn::TC_M, (op.N + BN - 1) / BN, z);
-    nn::k_wgrad_tc<BN><<<grid, nn::TC_THREADS, smem, n->stream>>>(op, n->wait_limit, n->err_d);
-    return cudaGetLastError();
-}
-
-cudaError_t conv_wgrad(lbm_unet *n, const Conv &cv, const bf16 *dz, const bf16 *x, int B, int H,
-                       int W) {
-    if (cv.k == 3) {
-        nn::WgradTc op{};
-        op.dz = dz;
-        op.x = x;
-        op.dw = n->g + cv.w_off;
-        op.img = {B, H, W};
-        op.Co = cv.co;
-        op.Ci = cv.ci;
-        op.taps = 9;
-        op.M = 9 * cv.ci;
-        op.N = cv.co;
-        op.K = B * H * W;
-        const int bn = cv.co <= 32 ? 32 : (cv.co <= 64 ? 64 : 128);
-        const int mt = (op.M + nn::TC_M - 1) / nn::TC_M, nt = (op.N + bn - 1) / bn;
-        const int kt = (op.K + nn::TC_K - 1) / nn::TC_K;
-        int z = 4 * n->sms / (mt * nt);
-        if (z < 1) z = 1;
-        if (z > kt) z = kt;
-        op.kchunk = ((kt + z - 1) / z) * nn::TC_K;
-        z = (op.K + op.kchunk - 1) / op.kchunk;
-        cudaError_t e = bn == 32 ? launch_wg<32>(n, op, z)
-                                 : (bn == 64 ? launch_wg<64>(n, op, z) : launch_wg<128>(n, op, z));
-        if (e != cudaSuccess) return e;
-        const long long P = op.K;
-        int nb = (int)((P * cv.co + nn::EW - 1) / nn::EW);
-        if (nb > 1024) nb = 1024;
-        nn::k_colsum<<<nb, nn::EW, 0, n->stream>>>(dz, P, cv.co, n->g + cv.b_off);
-        return cudaGetLastError();
-    }
-    nn::WgradOp op{};
-    op.dz = dz;
-    op.x = x;
-    op.dw = n->g + cv.w_off;
-    op.img = {B, H, W};
-    op.Co = cv.co;
-    op.Ci = cv.ci;
-    op.taps = cv.k * cv.k;
-    op.M = cv.co;
-    op.N = op.taps * cv.ci;
-    op.K = B * H * W;
-    const int mt = (op.M + nn::BM - 1) / nn::BM, nt = (op.N + nn::BN - 1) / nn::BN;
-    int z = 1200 / (mt * nt);
-    const int kt = (op.K + nn::BK - 1) / nn::BK;
+    constexpr int stage = 16 * WG_APX * 16 + BN / 8 * WG_PX * 16;
+    constexpr bool two = 2 * stage <= SMEM_TWO && 3 * BN <= 256;  // CTAs on an SM
+    op.stages = (two ? SMEM_TWO : SMEM_MAX) / stage;
+    if (op.stages > 4) op.stages = 4;
+    const int gx = (3 * op.G + 15) / 16, gy = (op.Co + BN - 1) / BN;
+    // K splits: four per SM and tile of 128 (tap, ci) rows.  An accumulator adds one
+    // split's pixels in series, each addition rounded towards zero in the tensor core,
+    // so the length of a split is part of the gradient's rounding, not only of its time
+    int z = 4 * n->sms / ((9 * op.Ci + 127) / 128 * gy);
     if (z < 1) z = 1;
-    if (z > kt) z = kt;
-    op.kchunk = ((kt + z - 1) / z) * nn::BK;
-    z = (op.K + op.kchunk - 1) / op.kchunk;
-    const dim3 grid(mt, nt, z);
-    nn::k_gemm<nn::WgradOp><<<grid, nn::GEMM_THREADS, 0, n->stream>>>(op);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const long long P = op.K;
-    int nb = (int)((P * cv.co + nn::EW - 1) / nn::EW);
-    if (nb > 1024) nb = 1024;
-    nn::k_colsum<<<nb, nn::EW, 0, n->stream>>>(dz, P, cv.co, n->g + cv.b_off);
+    if (z > op.nchunk) z = op.nchunk;
+    op.perz = (op.nchunk + z - 1) / z;
+    z = (op.nchunk + op.perz - 1) / op.perz;
+    k_wgrad_tc<BN><<<dim3(gx, gy, z), TC_THREADS, op.stages * stage, n->stream>>>(op, n->wait_limit, n->err_d);
     return cudaGetLastError();
 }
 
-cudaError_t refresh_weights(lbm_unet *n) {
-    nn::k_to_bf16<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->w, n->wb, n->nparam);
-    cudaError_t e = cudaGetLastError();
-    for (const Conv &cv : n->convs) {
-        if (e != cudaSuccess) return e;
-        const long long cnt = (long long)cv.co * cv.k * cv.k * cv.ci;
-        nn::k_transpose_w<<<nn::blocks(cnt), nn::EW, 0, n->stream>>>(n->wb + cv.w_off, cv.wt, cv.co,
-                                                                   cv.k * cv.k, cv.ci);
-        e = cudaGetLastError();
-    }
-    return e;
+cudaError_t conv_wgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Planes &x, const nn::Geo &geo, int B) {
+    nn::WgradOp op{};
+    op.x = x.p;
+    op.xstr = x.str;
+    op.dz = dz.p;
+    op.zstr = dz.str;
+    op.dw = n->g + cv.w_off;
+    op.db = n->g + cv.b_off;
+    op.Wp = geo.Wp;
+    op.nchunk = (int)((long long)B * geo.PSI / nn::WG_PX);
+    op.Ci = cv.ci;
+    op.Co = cv.co;
+    op.G = cv.ci / 8;
+    return cv.co <= 32 ? launch_wg<32>(n, op) : (cv.co <= 64 ? launch_wg<64>(n, op) : launch_wg<128>(n, op));
 }
 
-lbm_status forward(lbm_unet *n, const float *in_dev, int B) {
-    const int L = n->cfg.levels, H = n->cfg.height, W = n->cfg.width;
-    NCK(n, (nn::k_pack_input<<<nn::blocks((long long)B * H * W * 8), nn::EW, 0, n->stream>>>(
-               in_dev, n->x, B, H * W),
-           cudaGetLastError()));
+lbm_status forward(lbm_unet *n, const float *in_dev, float *out_dev, int B) {
+    const int L = n->cfg.levels;
+    const nn::Geo &g0 = n->lv[0].geo;
+    const unsigned pixels = nn::blocks((long long)B * g0.H * g0.W);
+    NCK(n, (nn::k_pack_input<<<pixels, nn::EW, 0, n->stream>>>(in_dev, n->x.p, B, g0), cudaGetLastError()));
     for (int l = 0; l < L; l++) {
         Level &v = n->lv[l];
-        const bf16 *inp = n->x;
         if (l > 0) {
             const Level &u = n->lv[l - 1];
-            NCK(n, (nn::k_pool<<<nn::blocks((long long)B * v.H * v.W * u.C / 8), nn::EW, 0, n->stream>>>(
-                       u.e, v.inp, B, u.H, u.W, u.C),
-                   cudaGetLastError()));
-            inp = v.inp;
+            const dim3 grid(nn::blocks((long long)B * v.geo.H * v.geo.W), u.C / 8);
+            NCK(n, (nn::k_pool<<<grid, nn::EW, 0, n->stream>>>(u.e.p, u.e.str, v.inp.p, v.inp.str, B, u.geo, v.geo),
+                    cudaGetLastError()));
         }
-        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'e', l, 0)], inp, v.ea, B, v.H, v.W, true));
-        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'e', l, 1)], v.ea, v.e, B, v.H, v.W, true));
+        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'e', l, 0)], l > 0 ? v.inp : n->x, v.ea, v.geo, nullptr, B));
+        // the deepest level's output is only used upsampled, as the channels before
+        // the skip's in the level above
+        const Level *u = l == L - 1 ? &n->lv[l - 1] : nullptr;
+        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'e', l, 1)], v.ea, u ? u->cat : v.e, v.geo,
+                        u ? &u->geo : nullptr, B));
     }
-    const bf16 *d = n->lv[L - 1].e;
     for (int l = L - 2; l >= 0; l--) {
         Level &v = n->lv[l];
-        const int Cu = n->lv[l + 1].C;
-        NCK(n, (nn::k_upcat<<<nn::blocks((long long)B * v.H * v.W * (Cu + v.C) / 8), nn::EW, 0,
-                              n->stream>>>(d, v.e, v.cat, B, v.H, v.W, Cu, v.C),
-               cudaGetLastError()));
-        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'd', l, 0)], v.cat, v.da, B, v.H, v.W, true));
-        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'd', l, 1)], v.da, v.d, B, v.H, v.W, true));
-        d = v.d;
+        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'd', l, 0)], v.cat, v.da, v.geo, nullptr, B));
+        const Level *u = l > 0 ? &n->lv[l - 1] : nullptr;
+        NCK(n, conv_fwd(n, n->convs[conv_index(n, 'd', l, 1)], v.da, u ? u->cat : v.d, v.geo,
+                        u ? &u->geo : nullptr, B));
     }
     const Conv &hd = n->convs[conv_index(n, 'h', 0, 0)];
-    NCK(n, (nn::k_head<<<nn::blocks((long long)B * H * W), nn::EW, 0, n->stream>>>(
-               d, n->w + hd.w_off, n->w + hd.b_off, n->out, B, H * W, n->lv[0].C),
-           cudaGetLastError()));
+    const Planes &d = n->lv[0].d;
+    NCK(n, (nn::k_head<<<pixels, nn::EW, 0, n->stream>>>(d.p, d.str, n->w + hd.w_off, n->w + hd.b_off, out_dev, B,
+                                                         g0, n->lv[0].C),
+            cudaGetLastError()));
     return LBM_OK;
 }
 
 lbm_status backward(lbm_unet *n, const float *tgt_dev, const float *fl_dev, int B) {
-    const int L = n->cfg.levels, H = n->cfg.height, W = n->cfg.width;
-    const long long HW = (long long)H * W;
+    const int L = n->cfg.levels;
+    const nn::Geo &g0 = n->lv[0].geo;
+    const long long HW = (long long)g0.H * g0.W;
     NCK(n, cudaMemsetAsync(n->g, 0, n->nparam * sizeof(float), n->stream));
     NCK(n, cudaMemsetAsync(n->cnt, 0, sizeof(float), n->stream));
     NCK(n, cudaMemsetAsync(n->loss, 0, sizeof(double), n->stream));
@@ -1234,79 +1266,42 @@ lbm_status backward(lbm_unet *n, const float *tgt_dev, const float *fl_dev, int 
            cudaGetLastError()));
     // head: gradient of d0 (masked by d0 > 0) into lv[0].g1
     Level &v0 = n->lv[0];
-    const bf16 *d0 = L > 1 ? v0.d : v0.e;
     const Conv &hd = n->convs[conv_index(n, 'h', 0, 0)];
-    const unsigned hb = nn::blocks(B * HW);
-    if (v0.C == 32)
-        nn::k_head_back<32><<<hb, nn::EW, 0, n->stream>>>(n->dout, d0, n->w + hd.w_off, v0.g1,
-                                                          n->g + hd.w_off, n->g + hd.b_off, B, (int)HW);
-    else if (v0.C == 16)
-        nn::k_head_back<16><<<hb, nn::EW, 0, n->stream>>>(n->dout, d0, n->w + hd.w_off, v0.g1,
-                                                          n->g + hd.w_off, n->g + hd.b_off, B, (int)HW);
-    else
-        nn::k_head_back<8><<<hb, nn::EW, 0, n->stream>>>(n->dout, d0, n->w + hd.w_off, v0.g1,
-                                                         n->g + hd.w_off, n->g + hd.b_off, B, (int)HW);
-    NCK(n, cudaGetLastError());
+    unsigned hb = nn::blocks(B * HW);
+    if (hb > 2u * n->sms) hb = 2u * n->sms;
+    NCK(n, (nn::k_head_back<<<dim3(hb, v0.C / 8), nn::EW, 0, n->stream>>>(
+               n->dout, v0.d.p, v0.d.str, n->w + hd.w_off, v0.g1.p, n->g + hd.w_off, n->g + hd.b_off, B, g0, v0.C),
+            cudaGetLastError()));
     // decoder: g1 of level l holds d(d_l) (masked)
     for (int l = 0; l < L - 1; l++) {
         Level &v = n->lv[l];
         const Conv &cb = n->convs[conv_index(n, 'd', l, 1)], &ca = n->convs[conv_index(n, 'd', l, 0)];
-        NCK(n, conv_wgrad(n, cb, v.g1, v.da, B, v.H, v.W));
-        NCK(n, conv_dgrad(n, cb, v.g1, v.da, v.g2, B, v.H, v.W));
-        NCK(n, conv_wgrad(n, ca, v.g2, v.cat, B, v.H, v.W));
-        NCK(n, conv_dgrad(n, ca, v.g2, v.cat, v.gcat, B, v.H, v.W));
+        NCK(n, conv_wgrad(n, cb, v.g1, v.da, v.geo, B));
+        NCK(n, conv_dgrad(n, cb, v.g1, &v.da, v.g2, v.geo, B));
+        NCK(n, conv_wgrad(n, ca, v.g2, v.cat, v.geo, B));
+        NCK(n, conv_dgrad(n, ca, v.g2, &v.cat, v.gcat, v.geo, B));
         Level &u = n->lv[l + 1];
-        NCK(n, (nn::k_up_back<<<nn::blocks((long long)B * u.H * u.W * u.C / 8), nn::EW, 0, n->stream>>>(
-                   v.gcat, u.C + v.C, u.g1, B, u.H, u.W, u.C),
-               cudaGetLastError()));
+        const dim3 grid(nn::blocks((long long)B * u.geo.H * u.geo.W), u.C / 8);
+        NCK(n, (nn::k_up_back<<<grid, nn::EW, 0, n->stream>>>(v.gcat.p, v.gcat.str, u.g1.p, u.g1.str, B, v.geo, u.geo),
+                cudaGetLastError()));
     }
     // encoder: g1 of level l holds d(e_l) (masked)
     for (int l = L - 1; l >= 0; l--) {
         Level &v = n->lv[l];
         const Conv &cb = n->convs[conv_index(n, 'e', l, 1)], &ca = n->convs[conv_index(n, 'e', l, 0)];
-        const bf16 *inp = l > 0 ? v.inp : n->x;
-        NCK(n, conv_wgrad(n, cb, v.g1, v.ea, B, v.H, v.W));
-        NCK(n, conv_dgrad(n, cb, v.g1, v.ea, v.g2, B, v.H, v.W));
-        NCK(n, conv_wgrad(n, ca, v.g2, inp, B, v.H, v.W));
+        NCK(n, conv_wgrad(n, cb, v.g1, v.ea, v.geo, B));
+        NCK(n, conv_dgrad(n, cb, v.g1, &v.ea, v.g2, v.geo, B));
+        NCK(n, conv_wgrad(n, ca, v.g2, l > 0 ? v.inp : n->x, v.geo, B));
         if (l == 0) break;
-        NCK(n, conv_dgrad(n, ca, v.g2, nullptr, v.gin, B, v.H, v.W));
+        NCK(n, conv_dgrad(n, ca, v.g2, nullptr, v.gin, v.geo, B));
         Level &u = n->lv[l - 1];
-        NCK(n, (nn::k_pool_back<<<nn::blocks((long long)B * u.H * u.W * u.C / 8), nn::EW, 0, n->stream>>>(
-                   v.gin, u.e, u.gcat, v.C + u.C, v.C, u.g1, B, u.H, u.W, u.C),
-               cudaGetLastError()));
+        const Planes skip = u.gcat.group(v.C / 8);
+        const dim3 grid(nn::blocks((long long)B * u.geo.H * u.geo.W), u.C / 8);
+        NCK(n, (nn::k_pool_back<<<grid, nn::EW, 0, n->stream>>>(v.gin.p, v.gin.str, u.e.p, skip.p, u.g1.p, u.g1.str, B,
+                                                                v.geo, u.geo),
+                cudaGetLastError()));
     }
     return LBM_OK;
-}
-
-// host permutation between the ABI layout [co][ci][k][k] and the internal
-// [co][tap][ci]
-void abi_to_internal(const lbm_unet *n, const float *a, std::vector<float> &w) {
-    w.assign(n->nparam, 0.f);
-    size_t o = 0;
-    for (const Conv &cv : n->convs) {
-        const int t = cv.k * cv.k;
-        for (int co = 0; co < cv.co; co++)
-            for (int ci = 0; ci < cv.ci; ci++)
-                for (int tap = 0; tap < t; tap++)
-                    w[cv.w_off + ((size_t)co * t + tap) * cv.ci + ci] = a[o + ((size_t)co * cv.ci + ci) * t + tap];
-        o += (size_t)cv.co * cv.ci * t;
-        for (int co = 0; co < cv.co; co++) w[cv.b_off + co] = a[o + co];
-        o += cv.co;
-    }
-}
-
-void internal_to_abi(const lbm_unet *n, const float *w, float *a) {
-    size_t o = 0;
-    for (const Conv &cv : n->convs) {
-        const int t = cv.k * cv.k;
-        for (int co = 0; co < cv.co; co++)
-            for (int ci = 0; ci < cv.ci; ci++)
-                for (int tap = 0; tap < t; tap++)
-                    a[o + ((size_t)co * cv.ci + ci) * t + tap] = w[cv.w_off + ((size_t)co * t + tap) * cv.ci + ci];
-        o += (size_t)cv.co * cv.ci * t;
-        for (int co = 0; co < cv.co; co++) a[o + co] = w[cv.b_off + co];
-        o += cv.co;
-    }
 }
 
 lbm_status stage_inputs(lbm_unet *n, const float *in, const float *tgt, const float *fl, int B,
@@ -1383,6 +1378,7 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
         off = (off + 7) & ~size_t(7);  // keep every weight block 16-byte aligned in BF16
         cv.b_off = off;
         off += (co + 7) & ~7;
+        n->nabi += (long long)co * ci * k * k + co;
         n->convs.push_back(cv);
     };
     int cin = 8;
@@ -1403,15 +1399,34 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
     if (e == cudaSuccess) e = nalloc(n, &n->g, off);
     if (e == cudaSuccess) e = nalloc(n, &n->m, off);
     if (e == cudaSuccess) e = nalloc(n, &n->v, off);
-    if (e == cudaSuccess) e = nalloc(n, &n->wb, off);
-    for (Conv &cv : n->convs)
-        if (e == cudaSuccess) e = nalloc(n, &cv.wt, (size_t)cv.co * cv.ci * cv.k * cv.k);
+    // packed BF16 weights (zero where a tile or a pair of groups is padded) and the
+    // table of the parameters' places
+    long long abi = 0;
+    for (Conv &cv : n->convs) {
+        nn::ConvTab::E &t = n->tab.e[n->tab.n++];
+        t = {(int)cv.w_off, (int)cv.b_off, (int)abi, cv.ci, cv.co, cv.k * cv.k, nullptr, nullptr, 0, 0, 0, 0, 0, 0};
+        abi += (long long)cv.co * cv.ci * cv.k * cv.k + cv.co;
+        if (cv.k == 1) continue;
+        auto pack = [&](int N, int Cs, bool pairs, bf16 **p, int &BN, int &KG, int &Ge) {
+            const int G = Cs / 8;
+            BN = nn::n_tile(N);
+            KG = nn::k_groups(G, pairs);
+            Ge = pairs ? 1 : G + (G & 1);
+            const size_t cnt = (size_t)nn::n_tiles(N) * KG * BN * 8;
+            if (e == cudaSuccess) e = nalloc(n, p, cnt);
+            if (e == cudaSuccess) e = cudaMemsetAsync(*p, 0, cnt * sizeof(bf16), n->stream);
+        };
+        pack(cv.co, cv.ci, cv.ci == 8, &cv.fwd, t.fBN, t.fKG, t.fGe);
+        pack(cv.ci, cv.co, false, &cv.bwd, t.bBN, t.bKG, t.bGe);
+        t.fwd = cv.fwd;
+        t.bwd = cv.bwd;
+    }
     const size_t HW = (size_t)c.height * c.width;
-    if (e == cudaSuccess) e = nalloc(n, &n->x, B * HW * 8);
+    if (e == cudaSuccess) e = palloc(n, &n->x, nn::Geo(c.height, c.width), 8);
+    if (e == cudaSuccess) e = nalloc(n, &n->abi, (size_t)n->nabi);
     if (e == cudaSuccess) e = nalloc(n, &n->out, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->dout, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->io_in, B * HW * 8);
-    if (e == cudaSuccess) e = nalloc(n, &n->io_out, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->io_tgt, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->io_fl, B * HW);
     if (e == cudaSuccess) e = nalloc(n, &n->cnt, 1);
@@ -1421,22 +1436,21 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
     n->lv.resize(L);
     for (int l = 0; l < L && e == cudaSuccess; l++) {
         Level &v = n->lv[l];
-        v.H = c.height >> l;
-        v.W = c.width >> l;
+        v.geo = nn::Geo(c.height >> l, c.width >> l);
         v.C = ch[l];
-        const size_t P = B * v.H * v.W;
-        const int cprev = l > 0 ? ch[l - 1] : 8;
-        const int cnext = l + 1 < L ? ch[l + 1] : 0;
-        if (l > 0) e = nalloc(n, &v.inp, P * cprev);
-        if (e == cudaSuccess) e = nalloc(n, &v.ea, P * v.C);
-        if (e == cudaSuccess) e = nalloc(n, &v.e, P * v.C);
-        if (e == cudaSuccess && l < L - 1) e = nalloc(n, &v.cat, P * (v.C + cnext));
-        if (e == cudaSuccess && l < L - 1) e = nalloc(n, &v.da, P * v.C);
-        if (e == cudaSuccess && l < L - 1) e = nalloc(n, &v.d, P * v.C);
-        if (e == cudaSuccess) e = nalloc(n, &v.g1, P * v.C);
-        if (e == cudaSuccess) e = nalloc(n, &v.g2, P * v.C);
-        if (e == cudaSuccess && l < L - 1) e = nalloc(n, &v.gcat, P * (v.C + cnext));
-        if (e == cudaSuccess && l > 0) e = nalloc(n, &v.gin, P * cprev);
+        const int cprev = l > 0 ? ch[l - 1] : 8, cnext = l + 1 < L ? ch[l + 1] : 0;
+        if (l > 0) e = palloc(n, &v.inp, v.geo, cprev);
+        if (e == cudaSuccess) e = palloc(n, &v.ea, v.geo, v.C);
+        if (l < L - 1) {
+            if (e == cudaSuccess) e = palloc(n, &v.cat, v.geo, v.C + cnext);
+            v.e = v.cat.group(cnext / 8);
+            if (e == cudaSuccess) e = palloc(n, &v.da, v.geo, v.C);
+            if (e == cudaSuccess && l == 0) e = palloc(n, &v.d, v.geo, v.C);
+            if (e == cudaSuccess) e = palloc(n, &v.gcat, v.geo, v.C + cnext);
+        }
+        if (e == cudaSuccess) e = palloc(n, &v.g1, v.geo, v.C);
+        if (e == cudaSuccess) e = palloc(n, &v.g2, v.geo, v.C);
+        if (e == cudaSuccess && l > 0) e = palloc(n, &v.gin, v.geo, cprev);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(n->m, 0, off * sizeof(float), n->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->v, 0, off * sizeof(float), n->stream);
@@ -1446,16 +1460,24 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
         nrelease(n);
         return st;
     }
-    // He-normal weights (std sqrt(2 / fan_in)), zero biases, seeded
-    std::vector<float> w(off, 0.f);
+    // He-normal weights (std sqrt(2 / fan_in)), zero biases, seeded: drawn in the order
+    // [Cout][tap][Cin] of each convolution
+    std::vector<float> w(n->nabi, 0.f);
     std::mt19937_64 rng(c.seed);
     std::normal_distribution<double> nd(0.0, 1.0);
-    for (const Conv &cv : n->convs) {
-        const double sd = std::sqrt(2.0 / (cv.ci * cv.k * cv.k));
-        for (size_t i = 0; i < (size_t)cv.co * cv.ci * cv.k * cv.k; i++) w[cv.w_off + i] = (float)(sd * nd(rng));
+    for (int k = 0; k < n->tab.n; k++) {
+        const nn::ConvTab::E &t = n->tab.e[k];
+        const double sd = std::sqrt(2.0 / (t.ci * t.taps));
+        for (int co = 0; co < t.co; co++)
+            for (int tap = 0; tap < t.taps; tap++)
+                for (int ci = 0; ci < t.ci; ci++)
+                    w[t.abi + ((size_t)co * t.ci + ci) * t.taps + tap] = (float)(sd * nd(rng));
     }
-    e = cudaMemcpyAsync(n->w, w.data(), off * sizeof(float), cudaMemcpyHostToDevice, n->stream);
-    if (e == cudaSuccess) e = refresh_weights(n);
+    e = cudaMemcpyAsync(n->abi, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice, n->stream);
+    if (e == cudaSuccess) {
+        nn::k_from_abi<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->tab, n->abi, n->w, n->nparam);
+        e = cudaGetLastError();
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
     if (e != cudaSuccess) {
         nfail(nullptr, LBM_ECUDA, "lbm_unet_create: %s", cudaGetErrorString(e));
@@ -1482,44 +1504,40 @@ lbm_status lbm_unet_set_wait_limit(lbm_unet *n, int64_t polls) {
     return LBM_OK;
 }
 
-int64_t lbm_unet_param_count(const lbm_unet *n) {
-    if (!n) return -1;
-    int64_t s = 0;
-    for (const Conv &cv : n->convs) s += (int64_t)cv.co * cv.ci * cv.k * cv.k + cv.co;
-    return s;
+int64_t lbm_unet_param_count(const lbm_unet *n) { return n ? n->nabi : -1; }
+
+// a vector in the masters' layout to the caller, in the caller's order
+static lbm_status export_abi(lbm_unet *n, const float *w, float *a, int32_t on_device) {
+    float *to = on_device ? a : n->abi;
+    NCK(n, (nn::k_to_abi<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->tab, w, to, n->nparam),
+            cudaGetLastError()));
+    if (!on_device)
+        NCK(n, cudaMemcpyAsync(a, to, n->nabi * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
+    NCK(n, cudaStreamSynchronize(n->stream));
+    return LBM_OK;
 }
 
 lbm_status lbm_unet_get_params(lbm_unet *n, float *a, int32_t on_device) {
     if (!n || !a) return LBM_EINVAL;
     NCK(n, cudaSetDevice(n->cfg.device));
-    std::vector<float> w(n->nparam), h(lbm_unet_param_count(n));
-    NCK(n, cudaMemcpyAsync(w.data(), n->w, w.size() * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
-    NCK(n, cudaStreamSynchronize(n->stream));
-    internal_to_abi(n, w.data(), h.data());
-    if (on_device) {
-        NCK(n, cudaMemcpyAsync(a, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, n->stream));
-        NCK(n, cudaStreamSynchronize(n->stream));
-    } else {
-        std::memcpy(a, h.data(), h.size() * sizeof(float));
-    }
-    return LBM_OK;
+    return export_abi(n, n->w, a, on_device);
 }
 
 lbm_status lbm_unet_set_params(lbm_unet *n, const float *a, int32_t on_device) {
     if (!n || !a) return LBM_EINVAL;
     NCK(n, cudaSetDevice(n->cfg.device));
-    std::vector<float> h(lbm_unet_param_count(n)), w;
+    std::vector<float> h;
     if (on_device) {
+        h.resize(n->nabi);
         NCK(n, cudaMemcpyAsync(h.data(), a, h.size() * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
         NCK(n, cudaStreamSynchronize(n->stream));
-    } else {
-        std::memcpy(h.data(), a, h.size() * sizeof(float));
     }
-    for (float x : h)
-        if (!std::isfinite(x)) return nfail(n, LBM_EINVAL, "non-finite parameter");
-    abi_to_internal(n, h.data(), w);
-    NCK(n, cudaMemcpyAsync(n->w, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice, n->stream));
-    NCK(n, refresh_weights(n));
+    const float *v = on_device ? h.data() : a;
+    for (int64_t i = 0; i < n->nabi; i++)
+        if (!std::isfinite(v[i])) return nfail(n, LBM_EINVAL, "non-finite parameter");
+    NCK(n, cudaMemcpyAsync(n->abi, v, n->nabi * sizeof(float), cudaMemcpyHostToDevice, n->stream));
+    NCK(n, (nn::k_from_abi<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->tab, n->abi, n->w, n->nparam),
+            cudaGetLastError()));
     NCK(n, cudaMemsetAsync(n->m, 0, n->nparam * sizeof(float), n->stream));
     NCK(n, cudaMemsetAsync(n->v, 0, n->nparam * sizeof(float), n->stream));
     n->adam_t = 0;
@@ -1532,13 +1550,11 @@ lbm_status lbm_unet_forward(lbm_unet *n, const float *in, float *out, int32_t B,
     NCK(n, cudaSetDevice(n->cfg.device));
     const float *din = nullptr;
     lbm_status st = stage_inputs(n, in, nullptr, nullptr, B, on_device, &din, nullptr, nullptr);
-    if (st == LBM_OK) st = forward(n, din, B);
-    if (st != LBM_OK) return st;
+    if (st == LBM_OK) st = forward(n, din, on_device ? out : n->out, B);
+    if (st != LBM_OK || on_device) return st;
     const size_t bytes = (size_t)B * 3 * n->cfg.height * n->cfg.width * sizeof(float);
-    NCK(n, cudaMemcpyAsync(out, n->out, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                           n->stream));
-    if (!on_device) return check_err(n);
-    return LBM_OK;
+    NCK(n, cudaMemcpyAsync(out, n->out, bytes, cudaMemcpyDeviceToHost, n->stream));
+    return check_err(n);
 }
 
 lbm_status lbm_unet_gradients(lbm_unet *n, const float *in, const float *tgt, const float *fl,
@@ -1547,23 +1563,15 @@ lbm_status lbm_unet_gradients(lbm_unet *n, const float *in, const float *tgt, co
     NCK(n, cudaSetDevice(n->cfg.device));
     const float *din, *dt, *df;
     lbm_status st = stage_inputs(n, in, tgt, fl, B, on_device, &din, &dt, &df);
-    if (st == LBM_OK) st = forward(n, din, B);
+    if (st == LBM_OK) st = forward(n, din, n->out, B);
     if (st == LBM_OK) st = backward(n, dt, df, B);
     if (st != LBM_OK) return st;
-    std::vector<float> g(n->nparam), h(lbm_unet_param_count(n));
     double l = 0.0;
-    NCK(n, cudaMemcpyAsync(g.data(), n->g, g.size() * sizeof(float), cudaMemcpyDeviceToHost, n->stream));
     NCK(n, cudaMemcpyAsync(&l, n->loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
     NCK(n, cudaStreamSynchronize(n->stream));
     st = check_err(n);
+    if (st == LBM_OK) st = export_abi(n, n->g, grads, on_device);
     if (st != LBM_OK) return st;
-    internal_to_abi(n, g.data(), h.data());
-    if (on_device) {
-        NCK(n, cudaMemcpyAsync(grads, h.data(), h.size() * sizeof(float), cudaMemcpyHostToDevice, n->stream));
-        NCK(n, cudaStreamSynchronize(n->stream));
-    } else {
-        std::memcpy(grads, h.data(), h.size() * sizeof(float));
-    }
     if (loss) *loss = l;
     return LBM_OK;
 }
@@ -1574,21 +1582,15 @@ lbm_status lbm_unet_train_step(lbm_unet *n, const float *in, const float *tgt, c
     NCK(n, cudaSetDevice(n->cfg.device));
     const float *din, *dt, *df;
     lbm_status st = stage_inputs(n, in, tgt, fl, B, on_device, &din, &dt, &df);
-    if (st == LBM_OK) st = forward(n, din, B);
+    if (st == LBM_OK) st = forward(n, din, n->out, B);
     if (st == LBM_OK) st = backward(n, dt, df, B);
     if (st != LBM_OK) return st;
     n->adam_t++;
     const float c1 = (float)(1.0 - std::pow(0.9, (double)n->adam_t));
     const float c2 = (float)(1.0 - std::pow(0.999, (double)n->adam_t));
-    NCK(n, (nn::k_adam<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->w, n->g, n->m, n->v, n->wb,
+    NCK(n, (nn::k_adam<<<nn::blocks(n->nparam), nn::EW, 0, n->stream>>>(n->tab, n->w, n->g, n->m, n->v,
                                                                        n->nparam, lr, c1, c2),
            cudaGetLastError()));
-    for (const Conv &cv : n->convs) {
-        const long long cnt = (long long)cv.co * cv.k * cv.k * cv.ci;
-        NCK(n, (nn::k_transpose_w<<<nn::blocks(cnt), nn::EW, 0, n->stream>>>(n->wb + cv.w_off, cv.wt, cv.co,
-                                                                          cv.k * cv.k, cv.ci),
-               cudaGetLastError()));
-    }
     if (loss) {
         NCK(n, cudaMemcpyAsync(loss, n->loss, sizeof(double), cudaMemcpyDeviceToHost, n->stream));
         return check_err(n);
