@@ -101,8 +101,10 @@ __device__ __forceinline__ uint4 pack8(const float (&f)[8]) {
 
 // ------------------------------------------------ tcgen05 convolution
 
-constexpr int TC_M = 128, TC_THREADS = 192;  // producer warp, MMA warp, four epilogue warps
-constexpr int TC_MAX_STAGES = 10, TC_MAX_A = 4;
+constexpr int TC_M = 128;
+constexpr int TC_THREADS = 224;  // warps: A, MMA, four for the epilogue, B
+constexpr int WG_THREADS = 192;  // copies, MMA, four for the bias gradient and the epilogue
+constexpr int TC_MAX_STAGES = 10, TC_MAX_A = 12;
 constexpr int TC_KB = 16;                // K groups of 8 channels per stage of B, at most
 constexpr long long TC_SPIN = 1 << 24;
 
@@ -286,23 +288,26 @@ struct ConvOp {
     long long sstr, ostr;
     Geo geo, fine;
     int B, G, N, Ge, KG, sign, relu, up;
-    // A in shared memory: a tile's pixels with their neighbours, once for all taps
-    // (nseg row segments of segpx pixels per plane, rowpx between rows), na buffers; or
-    // nseg = 0: too large, each stage brings its taps' A along
-    int nseg, segpx, rowpx, na;
-    int stages;  // of kb K groups of B (kb divides Ge); 0: all of B stays in shared memory
-    int kb;
+    // Shared memory, either (stages = 0) all of B and na tiles of A: a tile's pixels with
+    // their neighbours for all taps, nseg row segments of segpx pixels per group, rowpx
+    // between rows; or stages of gb K groups of B (gb divides Ge) and na units of A: gb
+    // groups of one of the three rows of taps, 130 pixels each, for that row's taps.
+    int nseg, segpx, rowpx, gb, na, stages;
     int ntile;   // tiles of 128 padded pixels
 };
 
-// Persistent CTAs, tiles of 128 consecutive padded pixels x BN outputs.  Warp 0 copies
-// (a tile's A once for all taps; the weights once, where they fit beside it, else in
-// stages), a thread of warp 1 issues the MMAs in the order of K (tap by tap, channels
-// ascending) into one of two accumulators, warps 2 to 5 store the other.  What bounds
-// it: the operands' shared-memory reads at N = 32 and 64 (4 KB of A for 16 or 32 cycles
-// of tensor work), the streamed weights' way through L2 on the coarse levels.  One CTA
-// per tile, with everything in turn, left each CTA waiting for its own copies (8 to 14
-// us per tile, tensor pipe 6 to 17% active).
+// Persistent CTAs, tiles of 128 consecutive padded pixels x BN outputs.  Warp 0 copies A
+// (once for all taps, or once for the three taps of a row), warp 6 the weights (once,
+// where they fit beside two tiles of A, else in stages), warp 1 issues the MMAs in the
+// order of K (tap by tap, channels ascending) into one of two accumulators, warps 2 to 5
+// store the other.  What bounds it: the operands' shared-memory reads at N = 32 and 64
+// (4 KB of A for 16 or 32 cycles of tensor work), the streamed weights' way through L2
+// on the coarse levels.  One CTA per tile, with everything in turn, left each CTA
+// waiting for its own copies (8 to 14 us per tile, tensor pipe 6 to 17% active).  At 4
+// levels of 32 to 256 channels, 16 images of 128 x 256: 1297 us a forward pass then, 303
+// now; with all of a tile's A in one buffer (or, where two do not fit, each tap's A
+// beside its weights) instead of units of a row, 330; with units of a row throughout,
+// 437 (the waits of each row and tap are longer than the few MMAs between them).
 template <int BN>
 __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long long limit, int *err) {
     extern __shared__ __align__(1024) unsigned char smem[];
@@ -311,70 +316,69 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
     constexpr uint32_t HI = desc_hi(128);
     constexpr int ACC = BN <= 32 ? 32 : (BN <= 64 ? 64 : 128), NCOLS = 2 * ACC;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockIdx.y;
-    const bool resident = op.nseg > 0, bstays = op.stages == 0;
-    const int S = op.stages, nkb = bstays ? 0 : op.KG / op.kb;
-    const uint32_t gs = resident ? (uint32_t)(op.nseg * op.segpx * 16) : TC_M * 16;  // K group stride
-    const uint32_t abytes = resident ? op.Ge * gs : 0;
-    const uint32_t a0 = smem_u32(smem), b0 = a0 + op.na * abytes;
-    const uint32_t stage = op.kb * (BN + (resident ? 0 : TC_M)) * 16;  // B, then A
+    const bool bstays = op.stages == 0;
+    const int S = op.stages, nblk = bstays ? 1 : op.Ge / op.gb;
+    constexpr int SEG = TC_M + 2;                                                // pixels of a unit's group
+    const uint32_t gs = (bstays ? (uint32_t)(op.nseg * op.segpx) : SEG) * 16;    // K group stride
+    const uint32_t unit = (bstays ? op.Ge : op.gb) * gs;
+    const uint32_t a0 = smem_u32(smem), b0 = a0 + op.na * unit, stage = op.gb * BN * 16;
     const bf16 *w = op.w + (long long)nt * op.KG * BN * 8;
-    // displacement of tap t in pixels of the padded image
-    auto shift = [&](int t, int row) { return op.sign * ((t / 3 - 1) * row + t % 3 - 1); };
     if (tid < BN) bias[tid] = op.bias && nt * BN + tid < op.N ? op.bias[nt * BN + tid] : 0.f;
     pipe_init(pp, 1, NCOLS, warp, tid);
     const uint32_t tmem = pp.tmem;
     if (warp == 0) {
-        int fills = 0, afills = 0;
-        Ring br, ar;  // an empty[] of an earlier use: the other parity
+        int fills = 0;
+        Ring ar;  // an empty[] of an earlier use: the other parity
         bool go = true;
-        if (bstays && lane == 0) {
+        for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x) {
+            const long long q0 = op.geo.Wp + (long long)tile * TC_M - 1;
+            for (int u = 0; u < (bstays ? 1 : 3 * nblk); u++) {
+                if (!ar.first) go = pipe_wait_warp(pp, pp.aempty[ar.s], ar.phase ^ 1, limit);
+                if (!go) break;
+                const uint32_t bar = smem_u32(&pp.afull[ar.s]), to = a0 + ar.s * unit;
+                if (lane == 0) mbar_expect(bar, unit);
+                __syncwarp();
+                if (bstays) {
+                    for (int c = lane; c < op.Ge * op.nseg; c += 32) {
+                        const int g = op.nseg == 3 ? c / 3 : c, row = op.nseg == 3 ? c - 3 * g - 1 : -1;
+                        bulk_copy(to + c * op.segpx * 16,
+                                  op.src + ((g < op.G ? g : 0) * op.sstr + q0 + row * op.geo.Wp) * 8, op.segpx * 16, bar);
+                    }
+                } else if (lane < op.gb) {
+                    const int row = u / nblk - 1, g = u % nblk * op.gb + lane;
+                    bulk_copy(to + lane * SEG * 16,
+                              op.src + ((g < op.G ? g : 0) * op.sstr + q0 + op.sign * row * op.geo.Wp) * 8, SEG * 16, bar);
+                }
+                ar.next(op.na);
+                fills++;
+            }
+        }
+        __syncwarp();
+        if (lane == 0 && *(volatile int *)&pp.abort) drain_fills(pp.afull, op.na, fills);
+    } else if (warp == 6) {
+        int fills = 0;
+        if (lane == 0 && bstays) {
             mbar_expect(smem_u32(&pp.once), op.KG * BN * 16);
             for (int k = 0; k < op.KG; k += TC_KB)
                 bulk_copy(b0 + k * BN * 16, w + (long long)k * BN * 8, min(TC_KB, op.KG - k) * BN * 16,
                           smem_u32(&pp.once));
-        }
-        const int ncopy = op.Ge * op.nseg;
-        for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x) {
-            const int q0 = op.geo.Wp + tile * TC_M;
-            if (resident) {
-                if (!ar.first) go = pipe_wait_warp(pp, pp.aempty[ar.s], ar.phase ^ 1, limit);
-                if (!go) break;
-                const uint32_t bar = smem_u32(&pp.afull[ar.s]), to = a0 + ar.s * abytes;
-                if (lane == 0) mbar_expect(bar, abytes);
-                __syncwarp();
-                for (int c = lane; c < ncopy; c += 32) {
-                    const int g = op.nseg == 3 ? c / 3 : c, sg = c - g * op.nseg;
-                    const long long from =
-                        (g < op.G ? g : 0) * op.sstr + q0 - 1 + (op.nseg == 3 ? (sg - 1) * op.geo.Wp : -op.geo.Wp);
-                    bulk_copy(to + c * op.segpx * 16, op.src + from * 8, op.segpx * 16, bar);
+        } else if (lane == 0) {
+            Ring br;
+            bool go = true;
+            for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x)
+                for (int k = 0; k < 9 * nblk; k++) {
+                    if (!br.first && !(go = pipe_wait(pp, pp.empty[br.s], br.phase ^ 1, limit))) break;
+                    const uint32_t bar = smem_u32(&pp.full[br.s]);
+                    mbar_expect(bar, stage);
+                    bulk_copy(b0 + br.s * stage, w + (long long)k * op.gb * BN * 8, stage, bar);
+                    br.next(S);
+                    fills++;
                 }
-                ar.next(op.na);
-                afills++;
-            }
-            for (int kb = 0; kb < nkb; kb++) {
-                const int n = op.kb;
-                if (!br.first) go = pipe_wait_warp(pp, pp.empty[br.s], br.phase ^ 1, limit);
-                if (!go) break;
-                const uint32_t at = b0 + br.s * stage, bar = smem_u32(&pp.full[br.s]);
-                if (lane == 0) {
-                    mbar_expect(bar, n * (BN + (resident ? 0 : TC_M)) * 16);
-                    bulk_copy(at, w + (long long)kb * n * BN * 8, n * BN * 16, bar);
-                }
-                __syncwarp();
-                if (!resident && lane < n) {
-                    const int kg = kb * n + lane, t = kg / op.Ge, g = kg % op.Ge;
-                    bulk_copy(at + n * BN * 16 + lane * TC_M * 16,
-                              op.src + ((g < op.G ? g : 0) * op.sstr + q0 + shift(t, op.geo.Wp)) * 8, TC_M * 16, bar);
-                }
-                br.next(S);
-                fills++;
-            }
         }
         __syncwarp();
         if (lane == 0 && *(volatile int *)&pp.abort) {
             if (bstays) tc_wait(smem_u32(&pp.once), 0, TC_SPIN);
             else drain_fills(pp.full, S, fills);
-            drain_fills(pp.afull, op.na, afills);
         }
     } else if (warp == 1) {
         // kind::f16: D FP32, A and B BF16, both K-major, M = 128, N = BN
@@ -382,83 +386,77 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
                                    ((uint32_t)(TC_M >> 4) << 24);
         const bool leader = elect_one();
         bool go = !bstays || pipe_wait_warp(pp, pp.once, 0, limit), issued = false;
-        Ring br, ar, acr;  // stages, tiles of A, accumulators
+        Ring br, ar, acr;  // stages of B, units of A, accumulators
         for (int tile = blockIdx.x; tile < op.ntile && go; tile += gridDim.x) {
             if (!acr.first) go = pipe_wait_warp(pp, pp.tempty[acr.s], acr.phase ^ 1, limit);
-            if (go && resident) go = pipe_wait_warp(pp, pp.afull[ar.s], ar.phase, limit);
             if (!go) break;
-            asm volatile("tcgen05.fence::after_thread_sync;\n");
-            const uint32_t d = tmem + acr.s * ACC, abuf = a0 + ar.s * abytes;
+            const uint32_t d = tmem + acr.s * ACC;
             uint32_t blo = desc_lo(b0, BN * 16), acc = 0;
-            if (op.Ge == 1) {
-                // one group (all of B stays): two taps each, the distance between them
-                // the stride of K groups; the last one's partner (the next pixel) has
-                // zero weights
+            issued = true;
+            if (bstays) {
+                if (!(go = pipe_wait_warp(pp, pp.afull[ar.s], ar.phase, limit))) break;
+                asm volatile("tcgen05.fence::after_thread_sync;\n");
+                const uint32_t abuf = a0 + ar.s * unit;
+                if (op.Ge == 1) {
+                    // two taps each, the distance between them the stride of K groups; the
+                    // last one's partner (the next pixel) has zero weights
 #pragma unroll
-                for (int t = 0; t < 10; t += 2) {
-                    const uint32_t o0 = t / 3 * op.rowpx + t % 3, o1 = t < 8 ? (t + 1) / 3 * op.rowpx + (t + 1) % 3 : o0 + 1;
-                    if (leader) tc_mma(d, desc_lo(abuf, (o1 - o0) * 16) + o0, HI, blo, HI, idesc, t > 0);
-                    blo += 2 * BN;
-                }
-            } else if (bstays) {
-                const uint32_t alo = desc_lo(abuf, gs) + (op.sign > 0 ? 0 : 2 * op.rowpx + 2);
-                for (int dy = 0; dy < 3; dy++)
-                    for (int dx = 0; dx < 3; dx++) {
-                        uint32_t an = alo + op.sign * (dy * op.rowpx + dx);
-#pragma unroll 2
-                        for (int g = 0; g < op.Ge; g += 2) {
-                            if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
-                            acc = 1;
-                            an += gs >> 3;
-                            blo += 2 * BN;
-                        }
+                    for (int t = 0; t < 10; t += 2) {
+                        const uint32_t o0 = t / 3 * op.rowpx + t % 3, o1 = t < 8 ? (t + 1) / 3 * op.rowpx + (t + 1) % 3 : o0 + 1;
+                        if (leader) tc_mma(d, desc_lo(abuf, (o1 - o0) * 16) + o0, HI, blo, HI, idesc, t > 0);
+                        blo += 2 * BN;
                     }
-            } else if (resident) {
-                const uint32_t alo = desc_lo(abuf, gs) + (op.sign > 0 ? 0 : 2 * op.rowpx + 2);
-                for (int dy = 0; dy < 3 && go; dy++)
-                    for (int dx = 0; dx < 3 && go; dx++) {
-                        uint32_t an = alo + op.sign * (dy * op.rowpx + dx);
-                        for (int g0 = 0; g0 < op.Ge; g0 += op.kb) {  // a stage each
-                            if (!(go = pipe_wait_warp(pp, pp.full[br.s], br.phase, limit))) break;
-                            asm volatile("tcgen05.fence::after_thread_sync;\n");
-                            blo = desc_lo(b0 + br.s * stage, BN * 16);
+                } else {
+                    const uint32_t alo = desc_lo(abuf, gs) + (op.sign > 0 ? 0 : 2 * op.rowpx + 2);
+                    for (int dy = 0; dy < 3; dy++)
+                        for (int dx = 0; dx < 3; dx++) {
+                            uint32_t an = alo + op.sign * (dy * op.rowpx + dx);
 #pragma unroll 2
-                            for (int k = 0; k < op.kb; k += 2) {
+                            for (int g = 0; g < op.Ge; g += 2) {
                                 if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
                                 acc = 1;
                                 an += gs >> 3;
                                 blo += 2 * BN;
                             }
-                            issued = true;
-                            if (leader) tc_commit(smem_u32(&pp.empty[br.s]));
+                        }
+                }
+                if (leader) tc_commit(smem_u32(&pp.aempty[ar.s]));
+                ar.next(op.na);
+            } else {
+                // no way out of these loops: a branch on a wait's outcome would make their
+                // values non-uniform.  After a wait that gave up the MMAs left read what
+                // is there, and nothing is stored.
+                for (int row = 0; row < 3; row++) {
+                    const int as0 = ar.s;
+                    const uint32_t ap0 = ar.phase;
+                    for (int dx = 0; dx < 3; dx++) {
+                        ar.s = as0;
+                        ar.phase = ap0;
+                        for (int blk = 0; blk < nblk; blk++) {
+                            if (dx == 0) pipe_wait_warp(pp, pp.afull[ar.s], ar.phase, limit);
+                            pipe_wait_warp(pp, pp.full[br.s], br.phase, limit);
+                            asm volatile("tcgen05.fence::after_thread_sync;\n");
+                            uint32_t an = desc_lo(a0 + ar.s * unit, SEG * 16) + (op.sign > 0 ? dx : 2 - dx);
+                            blo = desc_lo(b0 + br.s * stage, BN * 16);
+#pragma unroll 2
+                            for (int k = 0; k < op.gb; k += 2) {
+                                if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
+                                acc = 1;
+                                an += 2 * SEG;
+                                blo += 2 * BN;
+                            }
+                            if (leader) {
+                                tc_commit(smem_u32(&pp.empty[br.s]));
+                                if (dx == 2) tc_commit(smem_u32(&pp.aempty[ar.s]));
+                            }
                             br.next(S);
+                            ar.next(op.na);
                         }
                     }
-            } else {
-                for (int kb = 0; kb < nkb; kb++) {
-                    if (!(go = pipe_wait_warp(pp, pp.full[br.s], br.phase, limit))) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;\n");
-                    const uint32_t at = b0 + br.s * stage;
-                    uint32_t an = desc_lo(at + op.kb * BN * 16, TC_M * 16);
-                    blo = desc_lo(at, BN * 16);
-#pragma unroll 2
-                    for (int k = 0; k < op.kb; k += 2) {
-                        if (leader) tc_mma(d, an, HI, blo, HI, idesc, acc);
-                        acc = 1;
-                        an += 2 * TC_M;
-                        blo += 2 * BN;
-                    }
-                    issued = true;
-                    if (leader) tc_commit(smem_u32(&pp.empty[br.s]));
-                    br.next(S);
                 }
+                go = __all_sync(0xffffffffu, *(volatile int *)&pp.abort == 0);
             }
-            issued = true;
-            if (go && leader) {
-                if (resident) tc_commit(smem_u32(&pp.aempty[ar.s]));
-                tc_commit(smem_u32(&pp.tfull[acr.s]));
-            }
-            ar.next(op.na);
+            if (go && leader) tc_commit(smem_u32(&pp.tfull[acr.s]));
             acr.next(2);
         }
         if (issued && leader && *(volatile int *)&pp.abort) drain_mmas(pp);
@@ -550,7 +548,7 @@ struct WgradOp {
 constexpr int WG_PX = 128, WG_APX = WG_PX + 2;
 
 template <int BN>
-__global__ void __launch_bounds__(TC_THREADS) k_wgrad_tc(const WgradOp op, long long limit, int *err) {
+__global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long long limit, int *err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) Pipe pp;
     __shared__ float bsum[BN];
@@ -1096,33 +1094,30 @@ cudaError_t launch_tc(lbm_unet *n, nn::ConvOp &op) {
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    // A once for all taps: three row segments where a tile is shorter than a row, else
-    // the run of pixels from the row above to the row below; in the stages, tap by tap,
-    // where it does not fit beside two stages of weights
-    op.kb = op.Ge < TC_KB ? op.Ge : TC_KB;
-    while (op.Ge % op.kb) op.kb -= 2;
-    const int wstage = op.kb * BN * 16, wall = op.KG * BN * 16;
+    // A tile of A once for all taps: three row segments where a tile is shorter than a
+    // row, else the run of pixels from the row above to the row below (pairs of taps: a
+    // pixel more, for the partner of the last tap)
     op.nseg = op.geo.Wp >= TC_M + 2 ? 3 : 1;
-    // (pairs of taps: a pixel more, for the partner of the last tap)
     op.segpx = (op.nseg == 3 ? TC_M + 2 : TC_M + 2 * op.geo.Wp + 2) + (op.Ge == 1);
     op.rowpx = op.nseg == 3 ? op.segpx : op.geo.Wp;
-    int a = op.Ge * op.nseg * op.segpx * 16, smem = 0;
-    if (2 * a + wall <= SMEM_MAX) {  // all weights
+    const int a = op.Ge * op.nseg * op.segpx * 16, wall = op.KG * BN * 16;
+    int smem = 0;
+    if (2 * a + wall <= SMEM_MAX) {  // all weights beside two tiles or more, two CTAs if they fit
         op.stages = 0;
-        op.na = 2 * a + wall <= SMEM_TWO ? (SMEM_TWO - wall) / a : (SMEM_MAX - wall) / a;
-        if (op.na > TC_MAX_A) op.na = TC_MAX_A;
+        op.na = (2 * a + wall <= SMEM_TWO ? SMEM_TWO - wall : SMEM_MAX - wall) / a;
+        if (op.na > 4) op.na = 4;
         smem = op.na * a + wall;
-    } else if (a + 2 * wstage <= SMEM_MAX) {
-        op.na = 2 * a + 3 * wstage <= SMEM_MAX ? 2 : 1;
-        op.stages = (SMEM_MAX - op.na * a) / wstage;
-        if (op.stages > TC_MAX_STAGES) op.stages = TC_MAX_STAGES;
-        smem = op.na * a + op.stages * wstage;
     } else {
-        op.nseg = 0;
-        op.na = 1;
-        const int both = wstage + op.kb * nn::TC_M * 16;
-        op.stages = SMEM_MAX / both < TC_MAX_STAGES ? SMEM_MAX / both : TC_MAX_STAGES;
-        smem = op.stages * both;
+        // the units of a row and two to come, and stages of weights (a copy is 2000 to
+        // 3000 cycles on its way, a stage of 16 groups 400 to 512 of MMAs)
+        op.gb = op.Ge < TC_KB ? op.Ge : TC_KB;
+        while (op.Ge % op.gb) op.gb -= 2;
+        const int unit = op.gb * (TC_M + 2) * 16, wstage = op.gb * BN * 16;
+        op.na = op.Ge / op.gb + 2;
+        if (op.na * unit + 3 * wstage > SMEM_MAX) op.na--;
+        op.stages = (SMEM_MAX - op.na * unit) / wstage;
+        if (op.stages > TC_MAX_STAGES) op.stages = TC_MAX_STAGES;
+        smem = op.na * unit + op.stages * wstage;
     }
     const long long rows = (long long)op.B * op.geo.PSI - op.geo.Wp;
     op.ntile = (int)((rows + TC_M - 1) / TC_M);
@@ -1198,7 +1193,7 @@ cudaError_t launch_wg(lbm_unet *n, nn::WgradOp &op) {
     if (z > op.nchunk) z = op.nchunk;
     op.perz = (op.nchunk + z - 1) / z;
     z = (op.nchunk + op.perz - 1) / op.perz;
-    k_wgrad_tc<BN><<<dim3(gx, gy, z), TC_THREADS, op.stages * stage, n->stream>>>(op, n->wait_limit, n->err_d);
+    k_wgrad_tc<BN><<<dim3(gx, gy, z), WG_THREADS, op.stages * stage, n->stream>>>(op, n->wait_limit, n->err_d);
     return cudaGetLastError();
 }
 
