@@ -28,6 +28,7 @@ pytestmark = pytest.mark.gpu
     (2, 8, 6, 128, 2),    # padded rows of 130: three segments of a full tile
     (2, 8, 10, 130, 2),   # rows and tiles out of step; 3 groups and a zero one
     (3, 16, 12, 260, 1),  # 6 and 12 groups; N of 96 backward
+    (3, 16, 12, 192, 2),  # weight gradient: rows in two runs, one, two rows to a run of three
     (4, 32, 64, 128, 5),  # streamed weights; more tiles than resident blocks
 ])
 def test_tile_edges(levels, base, H, W, B, monkeypatch):
