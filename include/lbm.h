@@ -387,8 +387,9 @@ lbm_status lbm_batch_state(lbm_batch *b, int32_t *state, int64_t *steps, double 
  * nothing changed.  The drag history restarts. */
 lbm_status lbm_batch_retire(lbm_batch *b, const int32_t *ids, int32_t n);
 
-/* Launch policy.  Tiles of the fused kernel are tile_rows rows (1..64) of
- * 128 threads x the nodes per thread of `variant` (as for
+/* Launch policy.  Tiles of the fused kernel are runs of row segments, rows
+ * in order, tile_rows segments (1..64) for each of the block's 4 warps; a
+ * segment is 32 threads x the nodes per thread of `variant` (as for
  * lbm_set_kernel_variant).  persistent = 1 runs the fused kernel as resident
  * blocks walking the tile list, 0 as one block per tile (default).  graph = 1
  * captures the `every` steps between two tests (and the test) into one CUDA

@@ -1432,7 +1432,7 @@ constexpr int CV_BLOCK = 1024;
 __global__ void __launch_bounds__(CV_BLOCK)
     k_batch_converge(BatchLaunch b, int ncase, double tol, long long max_steps, int window,
                      int mode, int *state, double *drag, int *calm, double *anchor,
-                     long long *steps, int *toff, int *ioff, int tile_w, int tile_h) {
+                     long long *steps, int *toff, int *ioff, int seg_w, int tile_n) {
     __shared__ int changed;
     __shared__ int wsum[3][CV_BLOCK / 32];
     __shared__ int carry[3];
@@ -1488,7 +1488,7 @@ __global__ void __launch_bounds__(CV_BLOCK)
         if (c < ncase && state[c] == 0) {
             const Lattice &L = b.cases[c].L;
             v[0] = 1;
-            v[1] = (L.nx + tile_w - 1) / tile_w * ((L.ny + tile_h - 1) / tile_h);
+            v[1] = ((L.nx + seg_w - 1) / seg_w * L.ny + tile_n - 1) / tile_n;
             v[2] = b.cases[c].nsolid;
         }
         int inc[3];
@@ -1540,10 +1540,10 @@ __global__ void __launch_bounds__(CV_BLOCK)
     for (int a = 0; a < na; a++) {
         const int c = b.active[a];
         const Lattice &L = b.cases[c].L;
-        const int nbx = (L.nx + tile_w - 1) / tile_w, nby = (L.ny + tile_h - 1) / tile_h;
-        const int nt = nbx * nby, o = toff[c];
+        const int nseg = (L.nx + seg_w - 1) / seg_w;
+        const int nt = (nseg * L.ny + tile_n - 1) / tile_n, o = toff[c];
         for (int k = tid; k < nt; k += CV_BLOCK)
-            tiles[o + k] = make_int4(c, k % nbx, (k / nbx) * tile_h, 0);
+            tiles[o + k] = make_int4(c, k * tile_n % nseg, k * tile_n / nseg, nseg);
         const int ns = b.cases[c].nsolid, oi = ioff[c];
         for (int s = tid; s < ns; s += CV_BLOCK) items[oi + s] = make_int2(c, s);
     }
@@ -1563,8 +1563,8 @@ cudaError_t launch_batch_converge(const BatchLaunch &b, const BatchState &s, int
                                   cudaStream_t st) {
     k_batch_converge<<<1, CV_BLOCK, 0, st>>>(b, s.ncase, s.tol, s.max_steps, s.window, mode,
                                              s.state, s.drag, s.calm, s.anchor, s.steps, s.toff,
-                                             s.ioff, tile_nodes(b.precision, b.variant),
-                                             b.tile_h);
+                                             s.ioff, segment_nodes(b.precision, b.variant),
+                                             tile_segments(b.tile_h));
     return cudaGetLastError();
 }
 

@@ -1,29 +1,41 @@
-// The fused kernel over a batch of independent domains (cases): the tiles
-// {case, x block, first row} of every active case in one launch, each tile
-// with its own case's parameters and step counter; open-channel columns are
-// computed by the per-node path.  The device code is in k_stream_collide.cuh.
+// The fused kernel over a batch of independent domains (cases): the tiles of every
+// active case in one launch, each with its own case's parameters.  A tile is a run of
+// row segments (32 lanes x V nodes, rows in order), one per warp, tile_h per warp: a
+// block works on as many rows as its warps need.  With tiles of one row and 128 threads
+// half of a block had no nodes on rows of 256 (V = 4), and part of the last block of
+// every row elsewhere: 96 open channels of 256 x 128, FP32, one launch 58 us, now 47
+// (its bytes at the copy rate: 34); 512 channels of 128 to 1024 x 64 to 512, 1125 us,
+// now 1099 (972).  What is left between a launch and its bytes: the two dependent loads
+// (tile, case) before a block's populations.  The device code is in
+// k_stream_collide.cuh.
 #include "k_stream_collide.cuh"
 
 namespace gbm {
 
 namespace {
 
-// One row of one tile.  The force kernel of the step has swapped the buffers: f1
-// holds the current populations, f0 takes the next.
+constexpr int SC_WARPS = SC_BLOCK_X / 32;
+
+// This warp's row segments of one tile {case, first segment, its row, segments per row}.
+// The force kernel of the step has swapped the buffers: f1 holds the current populations,
+// f0 takes the next.
 template <int P, int V, bool FORCE, bool LOCAL>
-__device__ __forceinline__ void tile_row(const StepParams &p, int bx, int y) {
+__device__ __forceinline__ void tile_segments(const StepParams &p, const int4 &tl, int tile_h) {
     using R = typename Raw<P>::R;
-    const R *fin = static_cast<const R *>(p.f1);
-    R *fout = static_cast<R *>(p.f0);
-    const int x0 = (bx * SC_BLOCK_X + threadIdx.x) * V;
-    if constexpr (P == LBM_FP16_DEV) sc_tile<P, V, FORCE, LOCAL, true>(p, fin, fout, x0, y);
-    else if (p.L.bc_x == LBM_OPEN) sc_row<P, V, FORCE, true, 0>(p, fin, fout, x0, y);
-    else sc_row<P, V, FORCE, false, 0>(p, fin, fout, x0, y);
+    int seg = tl.y + (threadIdx.x >> 5), y = tl.z;
+    for (int h = 0; h < tile_h; h++, seg += SC_WARPS) {
+        for (; seg >= tl.w; seg -= tl.w) y++;
+        if (y >= p.L.ny) return;
+        const R *fin = static_cast<const R *>(p.f1);
+        R *fout = static_cast<R *>(p.f0);
+        const int x0 = (seg * 32 + (threadIdx.x & 31)) * V;
+        if constexpr (P == LBM_FP16_DEV) sc_tile<P, V, FORCE, LOCAL, true>(p, fin, fout, x0, y);
+        else if (p.L.bc_x == LBM_OPEN) sc_row<P, V, FORCE, true, 0>(p, fin, fout, x0, y);
+        else sc_row<P, V, FORCE, false, 0>(p, fin, fout, x0, y);
+    }
 }
 
-// Batch of independent domains: persistent blocks walk the list of active
-// tiles {case, x block, first row} of all cases (case-major), each tile
-// (tile_h rows of SC_BLOCK_X * V nodes) with its own case's parameters.
+// Persistent blocks walk the list of the active tiles of all cases (case-major).
 template <int P, int V, bool FORCE, bool LOCAL>
 __global__ void __launch_bounds__(SC_BLOCK_X, 6)
     k_stream_collide_batch(const StepParams *__restrict__ cases, const int4 *__restrict__ tiles,
@@ -31,9 +43,7 @@ __global__ void __launch_bounds__(SC_BLOCK_X, 6)
     const int n = *ntiles;
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         const int4 tl = tiles[k];
-        const StepParams &p = cases[tl.x];
-        const int y1 = min(tl.z + tile_h, p.L.ny);
-        for (int y = tl.z; y < y1; y++) tile_row<P, V, FORCE, LOCAL>(p, tl.y, y);
+        tile_segments<P, V, FORCE, LOCAL>(cases[tl.x], tl, tile_h);
     }
 }
 
@@ -49,13 +59,7 @@ __global__ void __launch_bounds__(SC_BLOCK_X, (tiles_min_blocks<P, V>()))
                            const int *__restrict__ ntiles, int tile_h) {
     if ((int)blockIdx.x >= *ntiles) return;
     const int4 tl = tiles[blockIdx.x];
-    const StepParams &p = cases[tl.x];
-    if (!ROWS) {
-        tile_row<P, V, FORCE, LOCAL>(p, tl.y, tl.z);
-        return;
-    }
-    const int y1 = min(tl.z + tile_h, p.L.ny);
-    for (int y = tl.z; y < y1; y++) tile_row<P, V, FORCE, LOCAL>(p, tl.y, y);
+    tile_segments<P, V, FORCE, LOCAL>(cases[tl.x], tl, ROWS ? tile_h : 1);
 }
 
 template <int P, int V, bool FORCE, bool LOCAL>
@@ -103,11 +107,13 @@ cudaError_t launch_scb_p(const BatchLaunch &b, cudaStream_t st) {
 
 }  // namespace
 
-int tile_nodes(int precision, int variant) {
+int segment_nodes(int precision, int variant) {
     const int v16 = precision == LBM_FP64 ? 2 : (precision == LBM_FP32_DEV ? 4 : 8);
     const int v = variant == 1 ? v16 / 2 : (variant == 2 ? (v16 / 4 > 0 ? v16 / 4 : 1) : v16);
-    return SC_BLOCK_X * v;
+    return 32 * v;
 }
+
+int tile_segments(int tile_h) { return SC_WARPS * tile_h; }
 
 cudaError_t launch_stream_collide_batch(const BatchLaunch &b, cudaStream_t st) {
     switch (b.precision) {

@@ -1203,7 +1203,7 @@ struct lbm_batch {
     bool force = false;
     // launch policy
     int variant = 0;
-    int tile_h = 1;  // rows per tile of the fused kernel
+    int tile_h = 1;  // row segments per warp of the fused kernel
     bool persistent = false, graph = true;
     // convergence test
     int every = 100;
@@ -1341,14 +1341,15 @@ lbm_status bprepare(lbm_batch *b) {
         BCK(b, cudaStreamSynchronize(b->stream));
         for (size_t k = 0; k < n; k++) b->cases[k]->t = b->steps[k];
     }
-    const int w = gbm::tile_nodes(b->precision, b->variant);
-    const int wmin = gbm::tile_nodes(b->precision, 2);
+    const int w = gbm::segment_nodes(b->precision, b->variant);
+    const int wmin = gbm::segment_nodes(b->precision, 2);
+    const int per = gbm::tile_segments(b->tile_h), permin = gbm::tile_segments(1);
     long long tiles = 0, tiles_min = 0, items = 0;
     std::vector<StepParams> hp(b->cases.size());
     for (size_t k = 0; k < b->cases.size(); k++) {
         const lbm_ctx *c = b->cases[k];
-        tiles += (long long)((c->cfg.nx + w - 1) / w) * ((c->cfg.ny + b->tile_h - 1) / b->tile_h);
-        tiles_min += (long long)((c->cfg.nx + wmin - 1) / wmin) * c->cfg.ny;
+        tiles += ((long long)((c->cfg.nx + w - 1) / w) * c->cfg.ny + per - 1) / per;
+        tiles_min += ((long long)((c->cfg.nx + wmin - 1) / wmin) * c->cfg.ny + permin - 1) / permin;
         items += c->nsolid;
         hp[k] = params(c);
         hp[k].sc_variant = b->variant;

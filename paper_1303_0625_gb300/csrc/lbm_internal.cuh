@@ -387,7 +387,7 @@ __device__ __forceinline__ float reciprocal(float r) { return 1.f / r; }
 // k_solid_step.cu).
 struct BatchLaunch {
     StepParams *cases;        // [ncase], device; f0 = populations of the case's time t
-    int4 *tiles;              // active tiles {case, x block, row, 0}, device
+    int4 *tiles;              // active tiles {case, segment, row, segments per row}, device
     int *ntiles;              // device
     int2 *items;              // active (case, local solid) pairs, device
     int *nitems;              // device
@@ -398,7 +398,7 @@ struct BatchLaunch {
     bool force, local;
     int max_items;            // capacity of items (all solids of all cases)
     int max_tiles;            // tiles of all cases at the current tile shape
-    int tile_h;               // rows per tile
+    int tile_h;               // row segments per warp of a tile
     bool persistent;          // fused kernel: persistent blocks, else one block per tile
 };
 
@@ -434,7 +434,8 @@ cudaError_t launch_open_columns(const StepParams &p, cudaStream_t st);
 
 // k_stream_collide_batch.cu
 cudaError_t launch_stream_collide_batch(const BatchLaunch &b, cudaStream_t st);
-int tile_nodes(int precision, int variant);  // nodes along x of one tile
+int segment_nodes(int precision, int variant);  // nodes of a warp's row segment
+int tile_segments(int tile_h);                  // row segments of a tile
 // k_solid_step.cu: per-solid work of a step t -> t+1.  launch_forces, before the
 // advection-collision kernel (FP16: before or beside it): force record of time t
 // and motion t -> t+1 of every solid, and in FP64 and FP32 the populations that
