@@ -3,6 +3,8 @@
 // work of the solids lives in k_solid_step.cu.
 #include "lbm_internal.cuh"
 
+#include <cmath>
+
 namespace gbm {
 
 namespace {
@@ -247,33 +249,87 @@ __global__ void k_export_owner(const StepParams p, int32_t *out) {
     out[(long long)y * L.nx + x] = s == FLUID ? -1 : (int32_t)s;
 }
 
-// Sums of the deviation modes' populations for k_fields, exact: each d_i = f_i - w_i
-// as a 64-bit integer in units of 2^-60 (bits below that, 1e-18, are cut off, less
-// than the rounding of one FP64 addition of a weight), so that sums cost integer
-// additions.  GB300 issues about two FP64 lanes per clock and SM: the FP64 sums of
-// nine populations were 66 operations a node, and k_fields took 3.79 ms on
-// 8192 x 4096 nodes, twelve times what its memory traffic does.
-__device__ __forceinline__ long long fixed60(float d) {  // |d| < 1/2
-    const int b = __float_as_int(d), sh = ((b >> 23) & 0xFF) - 90;
-    const unsigned m = (b & 0x7FFFFF) | 0x800000;  // subnormals and zeros: shifted out
-    const unsigned long long v =
-        sh >= 0 ? (unsigned long long)m << sh : (unsigned long long)(m >> min(-sh, 31));
-    return b < 0 ? -(long long)v : (long long)v;
+// Density and velocity: r = sum f_i, u = (sum e_i f_i - F / 2) / r, in 64 bits without
+// FP64 arithmetic, of which GB300 issues about two lanes per clock and SM: one FP64
+// operation of a warp takes as long as 32 or more of its integer operations.  Sums: the
+// populations (in the deviation modes d_i = f_i - w_i) as 64-bit integers in units of
+// 2^-60 (FP64: 2^-58; bits below, 1e-18, are cut off, less than an FP64 addition
+// rounds), so exact.  Division: a fixed-point reciprocal of r and one product each,
+// rounded once, 0.55 units in the last place at most.  8192 x 4096 nodes, FP32 and
+// FP16: 0.50 ms (its bytes at the copy rate: 0.30 and 0.21; the integer units bound it);
+// with the sums alone in integers 1.01, all in FP64 3.79.  FP64, 2048 x 1024: 42 us (28),
+// before 172.
+template <int P> struct Fixed;
+template <> struct Fixed<LBM_FP32_DEV> {
+    static constexpr int BITS = 60;
+    static constexpr long long ONE = 1ll << BITS;  // added to the sum of the d_i
+    // false: |d| >= 1/2 or not a number
+    static __device__ __forceinline__ bool from(float d, long long &q) {
+        const int b = __float_as_int(d), e = (b >> 23) & 0xFF, sh = e - 90;
+        const unsigned m = (b & 0x7FFFFF) | 0x800000;  // subnormals and zeros: shifted out
+        const unsigned long long v =
+            sh >= 0 ? (unsigned long long)m << sh : (unsigned long long)(m >> min(-sh, 31));
+        q = b < 0 ? -(long long)v : (long long)v;
+        return e < 126;
+    }
+};
+template <> struct Fixed<LBM_FP16_DEV> : Fixed<LBM_FP32_DEV> {};
+template <> struct Fixed<LBM_FP64> {
+    static constexpr int BITS = 58;
+    static constexpr long long ONE = 0;
+    // false: |f| >= 1 or not a number
+    static __device__ __forceinline__ bool from(double f, long long &q) {
+        const long long b = __double_as_longlong(f);
+        const int e = (int)(b >> 52) & 0x7FF, sh = e - 1017;
+        const unsigned long long m = (b & 0xFFFFFFFFFFFFFll) | 0x10000000000000ll;
+        const unsigned long long v = sh >= 0 ? m << min(sh, 5) : m >> min(-sh, 63);
+        q = b < 0 ? -(long long)v : (long long)v;
+        return e < 1023;
+    }
+};
+
+// p 2^(e - 64), p > 0, rounded to nearest (the exponent far from the ends of its range).
+__device__ __forceinline__ double packed64(unsigned long long p, int e, bool negative) {
+    const int n = __clzll((long long)p);
+    p <<= n;
+    const long long m = (long long)(p >> 11) + (long long)(p >> 10 & 1);
+    const long long b = ((long long)(e - n + 1021) << 52) + m;
+    return __longlong_as_double(negative ? b | 0x8000000000000000ll : b);
 }
 
-// q 2^-60 + add (add a small whole number), rounded once: the two halves of q in the
-// low mantissa bits of two doubles (ulps 2^-28 and 2^-60) whose offsets cancel.
-__device__ __forceinline__ double from60(long long q, double add) {
-    const int hi = (int)(q >> 32) ^ (int)0x80000000, lo = (int)q;
-    const double h = __hiloint2double(0x41700000, hi);  // 2^24 + (q_hi + 2^31) 2^-28
-    const double l = __hiloint2double(0x3F700000, lo);  // 2^-8 + q_lo 2^-60
-    return (h - (16777216.0 + 8.0 + 0.00390625 - add)) + l;
+// 2^122 / r for r in [2^59, 2^61), to 2^-57 of it: FP32's approximation of 1 / r to about
+// 22 bits, y, then y (1 + e + e^2) with e = 1 - r y in fixed point.
+__device__ __forceinline__ unsigned long long reciprocal62(unsigned long long r) {
+    const unsigned rh = (unsigned)(r >> 32), rl = (unsigned)r;
+    const unsigned y = (unsigned)(__fdividef(1.f, (float)rh * 0x1p-28f) * 0x1p30f);
+    const long long ry = (long long)((unsigned long long)rh * y + ((unsigned long long)rl * y >> 32));
+    const long long e = (1ll << 58) - ry;  // below 2^37
+    const int es = (int)(e >> 22);
+    const long long t = e + (long long)(es * es >> 14);
+    return ((unsigned long long)y << 32) + ((unsigned long long)y * (unsigned)t >> 26) +
+           (unsigned long long)(((long long)y * (int)(t >> 32)) * 64);
 }
 
-// Density and velocity: r = sum f_i, u = (sum e_i f_i - F / 2) / r.
+// j / r from y = reciprocal62(r): j in units of 2^-BITS.
+template <int BITS>
+__device__ __forceinline__ double quotient62(long long j, unsigned long long y) {
+    if (j == 0) return 0.0;
+    unsigned long long a = j < 0 ? -(unsigned long long)j : (unsigned long long)j;
+    const int n = __clzll((long long)a);
+    a <<= n;
+    const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a, yh = (unsigned)(y >> 32), yl = (unsigned)y;
+    const unsigned long long q = (unsigned long long)ah * yh + ((unsigned long long)ah * yl >> 32) +
+                                 ((unsigned long long)al * yh >> 32);
+    return packed64(q, 66 - n - BITS, j < 0);
+}
+
+// half_x, half_y: F / 2 in units of 2^-BITS, or fixed = false.  Nodes outside the range
+// of the fixed-point form (1/2 <= r < 2) take FP64 arithmetic.
 template <int P>
-__global__ void k_fields(const StepParams p, double *rho, double *ux, double *uy) {
+__global__ void k_fields(const StepParams p, bool fixed, long long half_x, long long half_y, double *rho, double *ux,
+                         double *uy) {
     using S = typename Prec<P>::S;
+    using X = Fixed<P>;
     const Lattice &L = p.L;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= L.nx) return;
@@ -287,43 +343,27 @@ __global__ void k_fields(const StepParams p, double *rho, double *ux, double *uy
     typename Prec<P>::C d[9];
 #pragma unroll
     for (int i = 0; i < 9; i++) d[i] = ldc(f + i * L.plane + k);
-    double r, jx, jy;
-    bool plain = !Prec<P>::dev;
-    if constexpr (Prec<P>::dev) {
+    long long q[9];
 #pragma unroll
-        for (int i = 0; i < 9; i++) plain |= !(fabsf(d[i]) < 0.5f);  // NaN too
-        if (!plain) {
-            long long q[9];
-#pragma unroll
-            for (int i = 0; i < 9; i++) q[i] = fixed60(d[i]);
-            const long long a = q[5] - q[7], b = q[6] - q[8];
-            r = from60(((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])) + q[8], 1.0);
-            jx = from60(q[1] - q[3] + a - b, 0.0);
-            jy = from60(q[2] - q[4] + a + b, 0.0);
-        }
-    }
-    if (plain) {
-        double v[9];
-#pragma unroll
-        for (int i = 0; i < 9; i++) v[i] = Prec<P>::dev ? (double)d[i] + wgt<double>(i) : (double)d[i];
-        const double a = v[5] - v[7], b = v[6] - v[8];
-        r = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])) + v[8];
-        jx = (v[1] - v[3]) + (a - b);
-        jy = (v[2] - v[4]) + (a + b);
-    }
-    if (p.body_x != 0.0 || p.body_y != 0.0) {
-        jx -= 0.5 * p.body_x;
-        jy -= 0.5 * p.body_y;
-    }
-    rho[o] = r;
-    if ((unsigned)(((__double2hiint(r) >> 20) & 0x7FF) - 923) > 200u) {  // not within 2^-100 .. 2^100
-        ux[o] = jx / r;
-        uy[o] = jy / r;
+    for (int i = 0; i < 9; i++) fixed &= X::from(d[i], q[i]);
+    const long long a = q[5] - q[7], b = q[6] - q[8];
+    const long long r60 = (((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7])) + q[8] + X::ONE)
+                          << (60 - X::BITS);
+    if (fixed && r60 >= 1ll << 59 && r60 < 1ll << 61) {
+        const unsigned long long inv = reciprocal62((unsigned long long)r60);
+        rho[o] = packed64((unsigned long long)r60, 4, false);
+        ux[o] = quotient62<X::BITS>(q[1] - q[3] + a - b - half_x, inv);
+        uy[o] = quotient62<X::BITS>(q[2] - q[4] + a + b - half_y, inv);
         return;
     }
-    const double inv = reciprocal(r);
-    ux[o] = jx * inv;
-    uy[o] = jy * inv;
+    double v[9];
+#pragma unroll
+    for (int i = 0; i < 9; i++) v[i] = Prec<P>::dev ? (double)d[i] + wgt<double>(i) : (double)d[i];
+    const double c = v[5] - v[7], e = v[6] - v[8];
+    const double r = ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7])) + v[8];
+    rho[o] = r;
+    ux[o] = ((v[1] - v[3]) + (c - e) - 0.5 * p.body_x) / r;
+    uy[o] = ((v[2] - v[4]) + (c + e) - 0.5 * p.body_y) / r;
 }
 
 // bit i of mask[y][x]: fluid node x has a link along e_i (x + e_i solid).
@@ -421,14 +461,21 @@ cudaError_t launch_export_owner(const StepParams &p, int32_t *out, cudaStream_t 
     return cudaGetLastError();
 }
 
+template <int P>
+cudaError_t launch_fields_p(const StepParams &p, double *rho, double *ux, double *uy, cudaStream_t st) {
+    const bool fixed = std::fabs(p.body_x) < 0.5 && std::fabs(p.body_y) < 0.5;
+    auto half = [&](double f) { return fixed ? std::llrint(std::ldexp(0.5 * f, Fixed<P>::BITS)) : 0ll; };
+    k_fields<P><<<cell_grid(p.L), 128, 0, st>>>(p, fixed, half(p.body_x), half(p.body_y), rho, ux, uy);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_fields(const StepParams &p, double *rho, double *ux, double *uy,
                           cudaStream_t st) {
     switch (p.precision) {
-        case LBM_FP64: k_fields<LBM_FP64><<<cell_grid(p.L), 128, 0, st>>>(p, rho, ux, uy); break;
-        case LBM_FP32_DEV: k_fields<LBM_FP32_DEV><<<cell_grid(p.L), 128, 0, st>>>(p, rho, ux, uy); break;
-        default: k_fields<LBM_FP16_DEV><<<cell_grid(p.L), 128, 0, st>>>(p, rho, ux, uy);
+        case LBM_FP64: return launch_fields_p<LBM_FP64>(p, rho, ux, uy, st);
+        case LBM_FP32_DEV: return launch_fields_p<LBM_FP32_DEV>(p, rho, ux, uy, st);
+        default: return launch_fields_p<LBM_FP16_DEV>(p, rho, ux, uy, st);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_link_masks(const StepParams &p, uint8_t *mask, cudaStream_t st) {
