@@ -98,9 +98,20 @@ lbm_status fail(lbm_ctx *c, lbm_status st, const char *fmt, ...) {
 size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DEV ? 4 : 2); }
 
 // Does work go to the side stream, beside the advection-collision kernel?
+// On a small FP32 domain that kernel is shorter than the hand-over between the streams,
+// and with few moving solids the ring goes into the re-rasterisation's launch: 128 x 64
+// nodes, 1 disk: 36.0 us a step against 41.5 with the side stream; at 768 x 512 59 and
+// 57, so up to 2^18 nodes (in FP64, whose kernel takes longer, the side stream is faster
+// from the smallest domain on).
+bool few_moving(const lbm_ctx *c) {
+    return !c->moving.empty() && c->moving.size() <= gbm::FEW_MOVING && c->cfg.boundary == LBM_HALFWAY;
+}
+constexpr long long FORK_NODES = 1 << 18;
 bool forks(const lbm_ctx *c) {
     if (!c->overlap || c->nsolid == 0) return false;
-    return c->cfg.precision == LBM_FP16_DEV || !c->moving.empty();
+    if (c->cfg.precision == LBM_FP16_DEV) return true;
+    if (c->cfg.precision == LBM_FP32_DEV && few_moving(c) && (long long)c->cfg.nx * c->cfg.ny <= FORK_NODES) return false;
+    return !c->moving.empty();
 }
 
 // Blocks per solid of the link kernel, or 0 for links, record and motion in one
@@ -276,7 +287,7 @@ lbm_status upload_moving(lbm_ctx *c) {
 // changes applied, refill), which advances t (or a clock tick when no solid
 // moves).  FP16: the links too are the side stream's.
 lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
-    const bool half = p.precision == LBM_FP16_DEV, fork = forks(c);
+    const bool half = p.precision == LBM_FP16_DEV, fork = forks(c), tail = !fork && few_moving(c);
     if (!(half && fork)) CK(c, gbm::launch_forces(p, c->stream));
     cudaStream_t rest = c->stream;
     if (fork) {
@@ -286,9 +297,9 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
         if (half) CK(c, gbm::launch_forces(p, rest));
     }
     CK(c, gbm::launch_record(p, rest));
-    CK(c, gbm::launch_ring(p, rest));
+    if (!tail) CK(c, gbm::launch_ring(p, rest));
     if (fork) CK(c, cudaEventRecord(c->join, rest));
-    c->launches += (p.nsolid > 0 ? (p.link_parts ? 2 : 1) : 0) + (p.nmoving > 0 ? 1 : 0);
+    c->launches += (p.nsolid > 0 ? (p.link_parts ? 2 : 1) : 0) + (p.nmoving > 0 && !tail ? 1 : 0);
     if (timed) {
         if (c->ev_used + 2 > c->ev.size()) {
             for (int k = 0; k < 2; k++) {
@@ -313,7 +324,7 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
         c->launches++;
     }
     if (fork && !p.list_by_forces) CK(c, cudaStreamWaitEvent(c->stream, c->join, 0));
-    if (p.nmoving > 0) CK(c, gbm::launch_remask(p, c->stream));
+    if (p.nmoving > 0) CK(c, gbm::launch_remask(p, tail, c->stream));
     else CK(c, gbm::launch_tick(p, c->stream));
     c->launches += gbm::stream_collide_launches(p) + 1;
     return LBM_OK;

@@ -448,7 +448,9 @@ int tile_segments(int tile_h);                  // row segments of a tile
 cudaError_t launch_forces(const StepParams &p, cudaStream_t st);
 cudaError_t launch_record(const StepParams &p, cudaStream_t st);
 cudaError_t launch_ring(const StepParams &p, cudaStream_t st);
-cudaError_t launch_remask(const StepParams &p, cudaStream_t st);
+// ring: launch_ring's work too (no more than FEW_MOVING moving solids)
+cudaError_t launch_remask(const StepParams &p, bool ring, cudaStream_t st);
+constexpr int FEW_MOVING = 16;
 // batch: force record of every resting solid of every active case, t += 1
 cudaError_t launch_solids_batch(const BatchLaunch &b, cudaStream_t st);
 // batch: BATCH_TEST retires the active cases whose drag (Eq. 5 Fx summed

@@ -12,7 +12,7 @@ import numpy as np
 import pytest
 
 import workloads as W
-from _pairs import force_rel, run_pair
+from _pairs import force_rel, make_gpu, make_oracle, run_pair, seeded_f
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +66,25 @@ def test_links_of_a_disk_match_oracle(solids, boundary, precision):
              wall_ux=(0.0, 0.0), body_force=(0.0, 0.0), rho_w_mode=W.RHOW_LOCAL if boundary else
              W.RHOW_CONST, refill=1, boundary=boundary, solids=disks)
     _check(w, 30, precision)
+
+
+@pytest.mark.parametrize("overlap", [0, 1])
+@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("nmoving", [1, 2, 16, 17])
+def test_few_moving_solids_match_oracle(nmoving, precision, overlap):
+    """Up to 16 moving solids are re-rasterised by one cluster of blocks, with the ring
+    in the same launch where nothing runs beside it; 17 by a cooperative grid."""
+    disks = [_disk(10.3 + 18.0 * (k % 6), 10.1 + 17.0 * (k // 6), 5.2 + 0.13 * k, 0.05 - 0.005 * k, 0.03, 0.002 * k)
+             for k in range(nmoving)] + [_disk(100.0, 61.0, 4.4)]
+    w = dict(nx=111, ny=71, tau=0.8, rho0=1.0, bc_x=W.PERIODIC, bc_y=W.PERIODIC, u0=(0.0, 0.0),
+             wall_ux=(0.0, 0.0), body_force=(0.0, 0.0), rho_w_mode=W.RHOW_CONST, refill=1, solids=disks)
+    o, g = make_oracle(w), make_gpu(w, precision, ring=40)
+    g.set_force_overlap(bool(overlap))
+    f0 = seeded_f(w, 1)
+    o.set_f(f0)
+    g.set_f(f0)
+    ref, got = o.step(40), g.step_record(40)
+    assert np.array_equal(o.owner(), g.owner())
+    assert force_rel(got, ref, [s["r"] for s in disks]) <= (1e-12 if precision == "fp64" else 1e-5)
+    fl = o.owner() < 0
+    assert np.abs(g.get_f()[:, fl] - o.get_f()[:, fl]).max() <= (1e-12 if precision == "fp64" else 2e-6)
