@@ -241,12 +241,25 @@ __global__ void k_case_features(const StepParams p, float re, float *in) {
     in[7 * n + o] = yy / h - 0.5f;
 }
 
+// Four nodes a thread: rows of 8192 nodes, 4096 of them: 38 us, with one 134.
 __global__ void k_export_owner(const StepParams p, int32_t *out) {
     const Lattice &L = p.L;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+    const int x = 4 * (blockIdx.x * blockDim.x + threadIdx.x), y = blockIdx.y;
     if (x >= L.nx) return;
-    const uint16_t s = p.owner[cell_of(L, x, y)];
-    out[(long long)y * L.nx + x] = s == FLUID ? -1 : (int32_t)s;
+    // the pitch is a multiple of 64; out is the caller's, its rows not padded
+    const ushort4 s = *reinterpret_cast<const ushort4 *>(p.owner + cell_of(L, x, y));
+    const uint16_t v[4] = {s.x, s.y, s.z, s.w};
+    int32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; j++) o[j] = v[j] == FLUID ? -1 : (int32_t)v[j];
+    int32_t *to = out + (long long)y * L.nx + x;
+    if ((reinterpret_cast<uintptr_t>(to) & 15) == 0 && x + 4 <= L.nx) {
+        *reinterpret_cast<int4 *>(to) = make_int4(o[0], o[1], o[2], o[3]);
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+        if (x + j < L.nx) to[j] = o[j];
 }
 
 // Density and velocity: r = sum f_i, u = (sum e_i f_i - F / 2) / r, in 64 bits without
@@ -457,7 +470,7 @@ cudaError_t launch_case_features(const StepParams &p, double re, float *in, cuda
 }
 
 cudaError_t launch_export_owner(const StepParams &p, int32_t *out, cudaStream_t st) {
-    k_export_owner<<<cell_grid(p.L), 128, 0, st>>>(p, out);
+    k_export_owner<<<dim3((p.L.nx + 511) / 512, p.L.ny), 128, 0, st>>>(p, out);
     return cudaGetLastError();
 }
 
