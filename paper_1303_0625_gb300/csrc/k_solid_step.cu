@@ -779,9 +779,9 @@ __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
 
 // The same in two kernels: k_links, after which the advection-collision kernel can
 // run, and k_record (records and motion), beside it.  A solid's links go to
-// gridDim.y blocks: one, or LINK_PARTS that take its candidates 32 at a time in
-// turn, each the share of one warp of the single block, so that the sums are the
-// same bit for bit.  (With the interpolated boundary one 30-node disk in FP64 took
+// gridDim.y blocks: one, or several that take its candidates 32 at a time in turn
+// (LINK_PARTS: each the share of one warp of the single block, so that the sums are
+// the same bit for bit).  (With the interpolated boundary one 30-node disk in FP64 took
 // 68 us in one block with a thread per candidate: one SM's FP64 unit.)
 constexpr int LINK_CHUNK = FB / LINK_PARTS;
 
@@ -801,7 +801,7 @@ __global__ void __launch_bounds__(FB) k_links(const StepParams p) {
         double acc[6];
         block_sums(lacc, sh, acc);
         if (threadIdx.x == 0)
-            for (int q = 0; q < 6; q++) p.part[((long long)s * LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
+            for (int q = 0; q < 6; q++) p.part[((long long)s * MAX_LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
         __syncthreads();
     }
 }
@@ -822,7 +822,8 @@ __global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
     }
     double aq = 0.0, acc[6], booked[6];
     if (lane < 6)
-        for (int c = 0; c < p.link_parts; c++) aq += p.part[((long long)s * LINK_PARTS + c) * 6 + lane];
+#pragma unroll 4
+        for (int c = 0; c < p.link_parts; c++) aq += p.part[((long long)s * MAX_LINK_PARTS + c) * 6 + lane];
 #pragma unroll
     for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
     booked_events(p, b, t, lane, booked);

@@ -82,8 +82,8 @@ constexpr int NEAR_CAP = 32;
 constexpr float NEAR_REACH = 4.5f;
 constexpr float NEAR_MARGIN = 4.0f;
 
-// blocks that can share one solid's links
-constexpr int LINK_PARTS = 4;
+// blocks that share one solid's links: the warps of a single block, or in FP64 more
+constexpr int LINK_PARTS = 4, MAX_LINK_PARTS = 16;
 
 // covered/fresh nodes one solid can queue per step
 constexpr int SOLID_EVENTS = 256;
@@ -136,7 +136,7 @@ struct StepParams {
     int chg_cap;
     int *bnd;                 // deferred per-node path: {length at even t, at odd t, list...}
     int bnd_cap;              // capacity of the list
-    double *part;             // [nsolid][LINK_PARTS][6] link sums of a solid's blocks
+    double *part;             // [nsolid][MAX_LINK_PARTS][6] link sums of a solid's blocks
     int link_parts;           // blocks per solid of k_links, which k_record follows; 0: k_forces
     int list_by_forces;       // FP16: the force kernel fills the deferred list; the fused pass
                               // leaves the update to launch_deferred_update
