@@ -158,7 +158,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /* Wait for all enqueued work.  The status a step's kernels raised:
  * LBM_EUNSTABLE for a non-finite or non-positive density or a non-finite
- * solid state; LBM_ETIMEOUT when a grid barrier of the per-solid kernel gave
+ * solid state; LBM_ETIMEOUT when the re-rasterisation gave
  * up; LBM_ESTATE when a solid covered or uncovered more than 256 nodes in one
  * step (its event queue), the step's owner changes overflowed their list
  * (twice the event lists' room), or the deferred list of nodes next to
@@ -260,12 +260,12 @@ int32_t lbm_nsolid(const lbm_ctx *ctx);
 const char *lbm_last_error(const lbm_ctx *ctx);
 const char *lbm_status_string(lbm_status st);
 
-/* Bounded device waits: a grid-wide barrier of the re-rasterisation kernel
- * gives up after `polls` polls of about 64 ns (default 2^24, about one
- * second); the launch then stops, and the next call that waits returns
+/* Limit of the device waits of the re-rasterisation of moving solids, in
+ * polls.  Its waits are the hardware's (kernel order, a cluster's barrier) and
+ * cannot run out, so that any limit above 0 (default 2^24) lets them pass; 0
+ * gives up at once: the launch stops, and the next call that waits returns
  * LBM_ETIMEOUT (the step's per-solid work is incomplete: restore a state
- * saved by lbm_save before stepping on).  0 gives up at once, so that every
- * step with moving solids times out: the time-out path can be exercised
+ * saved by lbm_save before stepping on), which exercises the time-out path
  * without a stalled device.  LBM_EINVAL for polls < 0. */
 lbm_status lbm_set_wait_limit(lbm_ctx *ctx, int64_t polls);
 

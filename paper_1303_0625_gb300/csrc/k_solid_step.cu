@@ -21,15 +21,14 @@
 //      owner changes goes to the step's change list; covered and fresh nodes
 //      are queued per warp in lane order and published as the solid's
 //      segment of the step's event list.
-// k_remask follows all three, in one cooperative launch:
+// k_changes and k_events follow all three (few moving solids: k_remask_few, one launch):
 //   A  the change list into the owner map and the node flags (a node on the
 //      rings of several solids is listed by each with the same owner; flag
-//      bits are set and cleared atomically)
-//   E  after a grid-wide barrier whose wait is bounded: every warp of the grid
-//      takes events from the list: a fresh node is refilled by extrapolation
-//      (Sec. IV.B) from nodes fluid at t and at t+1; each event's momentum and
-//      torque go to its own slot; the moving solids' state becomes t+1; the
-//      clock advances.
+//      bits are set and cleared atomically); the clock advances
+//   E  after that: every warp of the grid takes events from the list: a fresh
+//      node is refilled by extrapolation (Sec. IV.B) from nodes fluid at t and
+//      at t+1; each event's momentum and torque go to its own slot; the moving
+//      solids' state becomes t+1.
 //
 // Work per solid follows its perimeter: the nodes near the ends of the disk's
 // chord in every row (FP32 bounds with a one-node margin) are dealt out to the
@@ -43,6 +42,8 @@
 // about 100 us per step on 2000 disks.)
 #include "lbm_internal.cuh"
 
+#include <algorithm>
+
 namespace gbm {
 
 namespace {
@@ -54,44 +55,9 @@ constexpr unsigned FULL = 0xffffffffu;
 
 // ------------------------------------------------------------- barrier
 
-// Grid-wide barrier for a cooperative launch.  Returns false (and raises
-// status bit 2) if the other blocks did not arrive within p.spin_limit polls;
-// the caller's block then returns, and so does every block at its next
-// barrier.  A limit of 0 gives up at once: the barrier never completes (the
-// time-out path's test).  The arrival count is left as it stands; the host
-// clears it when it reads bit 2.
-__device__ bool grid_sync(const StepParams &p) {
-    __shared__ int ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned int *gen = p.bar + 1;
-        const unsigned int g = *gen;
-        __threadfence();
-        const unsigned int arrived = atomicAdd(p.bar, 1u) + 1u;
-        ok = 1;
-        if (arrived == gridDim.x && p.spin_limit > 0) {
-            atomicExch(p.bar, 0u);
-            __threadfence();
-            atomicAdd(p.bar + 1, 1u);
-        } else {
-            long long spins = 0;
-            while (*gen == g) {
-                if (++spins > p.spin_limit) {
-                    atomicOr(p.status, 4);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-    }
-    __syncthreads();
-    return ok != 0;
-}
-
-// The same for a grid that is one cluster (few moving solids): the hardware's barrier,
-// which no block can fail to reach; a limit of 0 gives up as above.
+// Barrier of a grid that is one cluster (few moving solids): the hardware's, which no
+// block can fail to reach.  A limit of 0 polls gives up at once (the time-out path's
+// test): false, and status bit 2 raised; the caller's block then returns.
 __device__ bool cluster_sync(const StepParams &p) {
     if (p.spin_limit <= 0) {
         if (threadIdx.x == 0) atomicOr(p.status, 4);
@@ -1296,33 +1262,45 @@ __device__ __forceinline__ void changes(const StepParams &p) {
     }
 }
 
-// E: the step's covered and fresh nodes, dealt to every warp of the grid.
+// The clock, and the pair test's control words, once nothing of the step t reads them.
+__device__ __forceinline__ void advance_clock(const StepParams &p, long long t) {
+    *p.t = t + 1;
+    volatile unsigned int *ctl = p.bar;
+    if (ctl[3] != 0u || __uint_as_float(ctl[2]) >= 0.5f * NEAR_MARGIN) {
+        ctl[2] = 0u;  // the pair test of this step has run
+        ctl[3] = 0u;
+    }
+}
+
+// E: the covered and fresh nodes of step t, dealt to every warp of the grid.
 template <int P>
 __device__ __forceinline__ void events(const StepParams &p, long long t) {
     const int gt = blockIdx.x * SW_BLOCK + threadIdx.x, nt = gridDim.x * SW_BLOCK;
     void *fnew = ((t + 1) & 1) ? p.f1 : p.f0;  // populations of time t+1
-    if (gt == 0) {
-        *p.t = t + 1;  // every block has read t
-        volatile unsigned int *ctl = p.bar;
-        if (ctl[3] != 0u || __uint_as_float(ctl[2]) >= 0.5f * NEAR_MARGIN) {
-            ctl[2] = 0u;  // the pair test of this step has run
-            ctl[3] = 0u;
-        }
-    }
     const int nev = min(*(volatile int *)p.ev_len, p.ev_cap);
     for (int e = gt >> 5; e < nev; e += nt >> 5) phase_event<P>(p, e, threadIdx.x & 31, fnew);
     for (int m = gt; m < p.nmoving; m += nt) advance_solid(p.L, p.S[p.moving[m]]);
 }
 
-// A and E (after the advection-collision kernel and k_ring), one cooperative
-// launch.
-template <int P>
-__global__ void __launch_bounds__(SW_BLOCK, 4) k_remask(const StepParams p) {
+// A and E (after the advection-collision kernel and k_ring).  Two launches, the second
+// set up while the first runs: as one, with a barrier across the grid, it had to be
+// launched cooperatively, which waits for an idle GPU.  A step of 2048 x 1024 nodes with
+// 125 disks, FP64: 13 us less; 8192 x 4096, 2000 disks, FP32: 3.4; 500 disks on a
+// quarter of that: 1.5.  (Without the early start of the second: 1.8 us more there.)
+__global__ void __launch_bounds__(SW_BLOCK) k_changes(const StepParams p) {
+    // k_events' blocks may take their places; they wait for the end of this launch
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (*(volatile int *)p.status & 4) return;
-    const long long t = *p.t;
     changes(p);
-    if (!grid_sync(p)) return;
-    events<P>(p, t);
+    if (blockIdx.x != 0 || threadIdx.x != 0) return;
+    if (p.spin_limit <= 0) atomicOr(p.status, 4);  // as cluster_sync
+    else advance_clock(p, *p.t);
+}
+template <int P>
+__global__ void __launch_bounds__(SW_BLOCK, 4) k_events(const StepParams p) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (*(volatile int *)p.status & 4) return;
+    events<P>(p, *p.t - 1);
 }
 
 // The same for few moving solids, in one cluster; RING: after P and R in the same
@@ -1338,6 +1316,7 @@ __global__ void __launch_bounds__(SW_BLOCK, 4) k_remask_few(const StepParams p) 
     }
     changes(p);
     if (!cluster_sync(p)) return;
+    if (blockIdx.x == 0 && threadIdx.x == 0) advance_clock(p, t);  // every block has read t
     events<P>(p, t);
 }
 
@@ -1395,19 +1374,25 @@ cudaError_t launch_r(const StepParams &p, bool ring, cudaStream_t st) {
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_remask<P>, SW_BLOCK, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_events<P>, SW_BLOCK, 0);
         if (e != cudaSuccess) return e;
     }
-    // the changes go to every thread, the events to every warp: up to every
-    // resident block, but not many more warps than a step has events (tens per
-    // moving solid), for the barrier waits for all of them
-    int blocks = per_sm * sms;
-    if (blocks > 4LL * p.nmoving) blocks = 4 * p.nmoving;
-    if (blocks < 1) blocks = 1;
-    StepParams pp = p;
-    void *args[] = {&pp};
-    return cudaLaunchCooperativeKernel((const void *)k_remask<P>, dim3(blocks), dim3(SW_BLOCK),
-                                       args, 0, st);
+    // the changes go to every thread, the events to every warp: not many more than a
+    // step has of them (tens per moving solid), up to every resident block
+    const int blocks = std::min(per_sm * sms, 4 * p.nmoving);
+    k_changes<<<std::min(2 * sms, p.nmoving), SW_BLOCK, 0, st>>>(p);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(SW_BLOCK);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_events<P>, p);
 }
 
 // ------------------------------------------------------------- batch

@@ -40,7 +40,7 @@ struct lbm_ctx {
     int ring_cap = 0;      // solids the ring was laid out for
     long long *t_d = nullptr;
     int *status_d = nullptr;
-    unsigned int *bar_d = nullptr;  // per-solid control words (barrier, displacement, pair test)
+    unsigned int *bar_d = nullptr;  // per-solid control words (displacement, pair test)
     uint16_t *near_d = nullptr;     // near lists, [solid_cap][NEAR_CAP]
     double *part_d = nullptr;       // link sums by block, [solid_cap][MAX_LINK_PARTS][6]
     long long spin_limit = 1ll << 24;  // polls of a bounded device wait (about one second)
@@ -332,7 +332,7 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
     if (fork && !p.list_by_forces) CK(c, cudaStreamWaitEvent(c->stream, c->join, 0));
     if (p.nmoving > 0) CK(c, gbm::launch_remask(p, tail, c->stream));
     else CK(c, gbm::launch_tick(p, c->stream));
-    c->launches += gbm::stream_collide_launches(p) + 1;
+    c->launches += gbm::stream_collide_launches(p) + (p.nmoving > gbm::FEW_MOVING ? 2 : 1);
     return LBM_OK;
 }
 
@@ -353,13 +353,10 @@ lbm_status check_status(lbm_ctx *c) {
     int st = 0;
     CK(c, cudaMemcpyAsync(&st, c->status_d, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));
-    // a grid barrier that gave up leaves its arrival count behind: clear it
-    // whatever else was raised, so that a restored state steps cleanly
-    if (st & 4) CK(c, cudaMemsetAsync(c->bar_d, 0, 2 * sizeof(unsigned int), c->stream));
     if (st & 1) return fail(c, LBM_EUNSTABLE, "non-finite or non-positive density produced");
     if (st & 2) return fail(c, LBM_EUNSTABLE, "a solid reached a non-finite state");
     if (st & 4)
-        return fail(c, LBM_ETIMEOUT, "a grid-wide barrier of the re-rasterisation kernel gave up");
+        return fail(c, LBM_ETIMEOUT, "the re-rasterisation gave up waiting");
     if (st & 8)
         return fail(c, LBM_ESTATE,
                     "a solid covered or uncovered more nodes in one step than its event queue "

@@ -120,10 +120,9 @@ struct StepParams {
     int sc_variant;           // node width per thread of the advection-collision kernel
     float omega_f, body_xf, body_yf, rho0_f;  // FP32 copies for the FP32 kernels
     float wall_ux0_f, wall_ux1_f, umax_f;
-    unsigned int *bar;        // per-solid control words: grid barrier {count, generation},
-                              // largest displacement since the pair test (FP32 bits), pair
-                              // test requested
-    long long spin_limit;     // polls of a bounded device wait (0: give up at once)
+    unsigned int *bar;        // control words: two unused, largest displacement since the
+                              // pair test (FP32 bits), pair test requested
+    long long spin_limit;     // 0: the re-rasterisation gives up (LBM_ETIMEOUT)
     uint16_t *near_id;        // [nsolid][NEAR_CAP] near lists
     int4 *ev;                 // covered/fresh events of the step: {node code (cell << 1 |
                               // fresh), solid, unwrapped x, y in the solid's frame}
@@ -444,7 +443,7 @@ int tile_segments(int tile_h);                  // row segments of a tile
 // lists when due, the moving solids' owner changes and covered/fresh nodes, listed
 // (it writes nothing that the advection-collision kernel reads, so it may run
 // beside it); launch_remask, after all three: the owner changes applied, refill,
-// t += 1 (one cooperative launch).
+// t += 1 (one launch with few moving solids, else two).
 cudaError_t launch_forces(const StepParams &p, cudaStream_t st);
 cudaError_t launch_record(const StepParams &p, cudaStream_t st);
 cudaError_t launch_ring(const StepParams &p, cudaStream_t st);
