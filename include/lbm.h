@@ -158,7 +158,7 @@ lbm_status lbm_step(lbm_ctx *ctx, int64_t nsteps);
 
 /* Wait for all enqueued work.  The status a step's kernels raised:
  * LBM_EUNSTABLE for a non-finite or non-positive density or a non-finite
- * solid state; LBM_ETIMEOUT when the re-rasterisation gave
+ * solid state; LBM_ETIMEOUT when the re-rasterisation of solids gave
  * up; LBM_ESTATE when a solid covered or uncovered more than 256 nodes in one
  * step (its event queue), the step's owner changes overflowed their list
  * (twice the event lists' room), or the deferred list of nodes next to
