@@ -409,26 +409,25 @@ __device__ void record_forces(const StepParams &p, int s, int lane, long long t,
 // arithmetic precision of the storage mode, then across the block's warps in
 // FP64, in warp order.  (A force is a small difference of large link terms, so
 // another order of the FP32 sums would change it in the fifth digit.)
-constexpr int FB = 128;                  // threads per solid
-constexpr int FW = FB / 32;
+constexpr int FB = 128;                  // threads per solid (batches: or twice as many)
 constexpr int LU = 2;                    // links a thread loads before it works on them
 constexpr float ANN_EPS = 0.05f;         // above the FP32 rounding of a chord end
 
-template <int P> struct LinkShared {
+template <int P, int NT = FB> struct LinkShared {
     using C = typename Prec<P>::C;
-    int wsum[FW];
-    int cnt[FB];                  // the chunk's rows: exclusive prefix of their candidates
-    int lo[FB], i0[FB], i1[FB];   // row: [lo, hi] minus the inner chord [i0, i1]
-    int4 cand[FB];                // candidate: {cell, x - floor X, y - floor Y, flags}
-    uint16_t link[8 * FB];        // direction | candidate << 4
-    C rho[FB];                    // local density of the candidates (rho_w local)
-    C term[6][LU * FB];           // the terms of the links in hand
-    double part[FW][6];
+    int wsum[NT / 32];
+    int cnt[NT];                  // the chunk's rows: exclusive prefix of their candidates
+    int lo[NT], i0[NT], i1[NT];   // row: [lo, hi] minus the inner chord [i0, i1]
+    int4 cand[NT];                // candidate: {cell, x - floor X, y - floor Y, flags}
+    uint16_t link[8 * NT];        // direction | candidate << 4
+    C rho[NT];                    // local density of the candidates (rho_w local)
+    C term[6][LU * NT];           // the terms of the links in hand
+    double part[NT / 32][6];
 };
 
 // Exclusive prefix of n over the block, and its total (whole blocks call it).
-template <int P>
-__device__ __forceinline__ int block_scan(int n, LinkShared<P> &sh, int &total) {
+template <int P, int NT>
+__device__ __forceinline__ int block_scan(int n, LinkShared<P, NT> &sh, int &total) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     int inc = n;
 #pragma unroll
@@ -442,7 +441,7 @@ __device__ __forceinline__ int block_scan(int n, LinkShared<P> &sh, int &total) 
     int before = 0;
     total = 0;
 #pragma unroll
-    for (int w = 0; w < FW; w++) {
+    for (int w = 0; w < NT / 32; w++) {
         if (w < wib) before += sh.wsum[w];
         total += sh.wsum[w];
     }
@@ -452,16 +451,16 @@ __device__ __forceinline__ int block_scan(int n, LinkShared<P> &sh, int &total) 
 // The links of solid s: their sums into lacc (this thread's share; Eq. 4 force
 // and torque, then Eq. 5) and, with GHOST, the returned populations into the solid
 // nodes' slots of fs.  The solid's candidates are taken chunk by chunk of `chunk`
-// <= FB; this block takes the chunks part, part + nparts ...
+// <= NT; this block takes the chunks part, part + nparts ...
 //   per link  f_i = f~_i(x_f), the returned f_bb = f_i - 6 w_i rho_w (e_i . v) with
 //   v the solid's velocity at x_s = x_f + e_i / 2 (BND: interpolated from the cut
 //   of the link, v and the lever there); Eq. 4 = e_i f_i - e_opp f_bb, Eq. 5 =
 //   (e_i - v) f_i - (e_opp - v) f_bb, torque (x_s - R) x F (Eq. 7).
-template <int P, bool LOCAL, bool BND, bool GHOST>
+template <int P, bool LOCAL, bool BND, bool GHOST, int NT>
 __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b, int s,
                                             typename Prec<P>::S *fs, bool owners, bool list,
                                             long long t, int chunk, int part, int nparts,
-                                            LinkShared<P> &sh, typename Prec<P>::C (&lacc)[6]) {
+                                            LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6]) {
     using C = typename Prec<P>::C;
     using S = typename Prec<P>::S;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -474,7 +473,7 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
     const C rho0 = pick<C>(p.rho0, p.rho0_f);
     int j0, j1;
     rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
-    for (int jc = j0; jc <= j1; jc += FB) {  // rows in chunks of FB
+    for (int jc = j0; jc <= j1; jc += NT) {  // rows in chunks of NT
         // candidates of row jc + tid
         int lo = 1, hi = 0, i0 = 1, i1 = 0, n = 0;
         const int j = jc + tid;
@@ -494,8 +493,8 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
             const int e = base + tid;
             int q = 0;
 #pragma unroll
-            for (int step = FB / 2; step > 0; step >>= 1)
-                if (q + step < FB && sh.cnt[q + step] <= e) q += step;
+            for (int step = NT / 2; step > 0; step >>= 1)
+                if (q + step < NT && sh.cnt[q + step] <= e) q += step;
             const int jj = jc + q;
             int iu = sh.lo[q] + (e - sh.cnt[q]);
             const int a = sh.i0[q], bb = sh.i1[q];
@@ -537,7 +536,7 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
             for (int at = mine0; dirs; dirs &= dirs - 1)
                 sh.link[at++] = (uint16_t)((__ffs(dirs) - 1) | tid << 4);
             __syncthreads();
-            for (int l0 = 0; l0 < nlink; l0 += LU * FB) {
+            for (int l0 = 0; l0 < nlink; l0 += LU * NT) {
                 int4 cd[LU];
                 int kb[LU], dir[LU];
                 S fi_s[LU], fo_s[LU], fn_s[LU];
@@ -547,7 +546,7 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
 #pragma unroll
                 for (int u = 0; u < LU; u++) {
                     kb[u] = -1;
-                    const int l = l0 + u * FB + tid;
+                    const int l = l0 + u * NT + tid;
                     if (l >= nlink) continue;
                     const int lk = sh.link[l], i = lk & 15;
                     const int4 cc = cd[u] = sh.cand[lk >> 4];
@@ -632,11 +631,11 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
                         v[5] = dx * gmy - dy * gmx;
                     }
 #pragma unroll
-                    for (int q6 = 0; q6 < 6; q6++) sh.term[q6][u * FB + tid] = v[q6];
+                    for (int q6 = 0; q6 < 6; q6++) sh.term[q6][u * NT + tid] = v[q6];
                 }
                 __syncthreads();
                 // the candidate's thread adds its links' terms
-                for (int l = max(mine0, l0); l < min(mine1, l0 + LU * FB); l++)
+                for (int l = max(mine0, l0); l < min(mine1, l0 + LU * NT); l++)
 #pragma unroll
                     for (int q6 = 0; q6 < 6; q6++) lacc[q6] += sh.term[q6][l - l0];
                 __syncthreads();  // the terms (and the list) are reused
@@ -647,8 +646,8 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
 
 // Lane 0's sums over the block of every thread's lacc, in warp order, plus one
 // term per component (acc[q] of lane q < 6), to all lanes of warp 0.
-template <int P>
-__device__ __forceinline__ void block_sums(typename Prec<P>::C (&lacc)[6], LinkShared<P> &sh,
+template <int P, int NT>
+__device__ __forceinline__ void block_sums(LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
                                            double (&acc)[6]) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     warp_sum(lacc);
@@ -658,7 +657,7 @@ __device__ __forceinline__ void block_sums(typename Prec<P>::C (&lacc)[6], LinkS
     if (wib != 0) return;
     double aq = 0.0;
     if (lane < 6)
-        for (int w = 0; w < FW; w++) aq += sh.part[w][lane];
+        for (int w = 0; w < NT / 32; w++) aq += sh.part[w][lane];
 #pragma unroll
     for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
 }
@@ -730,7 +729,7 @@ __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
         solid_links<P, LOCAL, false, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
                                                  FB, 0, 1, sh, lacc);
         double acc[6];
-        block_sums(lacc, sh, acc);
+        block_sums(sh, lacc, acc);
         if (tid < 32) {
             double booked[6];
             booked_events(p, b, t, lane, booked);
@@ -765,7 +764,7 @@ __global__ void __launch_bounds__(FB) k_links(const StepParams p) {
                                                 gridDim.y > 1 ? LINK_CHUNK : FB, blockIdx.y,
                                                 gridDim.y, sh, lacc);
         double acc[6];
-        block_sums(lacc, sh, acc);
+        block_sums(sh, lacc, acc);
         if (threadIdx.x == 0)
             for (int q = 0; q < 6; q++) p.part[((long long)s * MAX_LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
         __syncthreads();
@@ -1404,14 +1403,14 @@ cudaError_t launch_r(const StepParams &p, bool ring, cudaStream_t st) {
 // buffers, after every block has read them.  Batch convention: between steps f0
 // holds the current populations; the fused kernel, which comes after this swap,
 // reads f1 and writes f0.
-template <int P, bool LOCAL>
-__global__ void __launch_bounds__(FB, 8)
+template <int P, bool LOCAL, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     k_solids_batch(StepParams *cases, const int2 *__restrict__ items,
                    const int *__restrict__ nitems, const int *__restrict__ active,
                    const int *__restrict__ nactive, unsigned int *ticket) {
     using S = typename Prec<P>::S;
     __shared__ bool last;
-    __shared__ LinkShared<P> sh;
+    __shared__ LinkShared<P, NT> sh;
     const int n = *nitems;
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         const int2 it = items[k];
@@ -1423,10 +1422,10 @@ __global__ void __launch_bounds__(FB, 8)
             continue;
         }
         typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
-        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, FB,
+        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, NT,
                                                  0, 1, sh, lacc);
         double acc[6];
-        block_sums(lacc, sh, acc);
+        block_sums(sh, lacc, acc);
         if (threadIdx.x < 32) {
             const double none[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // resting: no node changes type
             record_forces(p, it.y, threadIdx.x, t, acc, none);
@@ -1452,24 +1451,41 @@ __global__ void __launch_bounds__(FB, 8)
     if (threadIdx.x == 0) *ticket = 0;
 }
 
-template <int P, bool LOCAL>
-cudaError_t launch_sb(const BatchLaunch &b, cudaStream_t st) {
+template <int P, bool LOCAL, int NT>
+cudaError_t launch_sb_n(const BatchLaunch &b, cudaStream_t st) {
     static int per_sm = -1, sms = 0;
     if (per_sm < 0) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solids_batch<P, LOCAL>,
-                                                              FB, 0);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solids_batch<P, LOCAL, NT>,
+                                                              NT, 0);
         if (e != cudaSuccess) return e;
     }
     int blocks = b.max_items;
     if (blocks > per_sm * sms) blocks = per_sm * sms;
     if (blocks < 1) blocks = 1;
-    k_solids_batch<P, LOCAL><<<blocks, FB, 0, st>>>(b.cases, b.items, b.nitems, b.active,
+    k_solids_batch<P, LOCAL, NT><<<blocks, NT, 0, st>>>(b.cases, b.items, b.nitems, b.active,
                                                           b.nactive, b.ticket);
     return cudaGetLastError();
+}
+
+// A disk has about 9.5 r + 7 candidates.  Up to 128, one turn of 128 threads; more take
+// another turn, a chain of loads, where 256 threads need one: 96 open channels of 256 x
+// 128 with disks of up to 16, 68.1 -> 65.9 us a step; two of 1024 x 512, r 51, 34.3 ->
+// 28.0; but 8 of 64 x 48, r 4.8, 13.9 -> 14.5.  More items than find room at 256 threads
+// go to 128.
+template <int P, bool LOCAL>
+cudaError_t launch_sb(const BatchLaunch &b, cudaStream_t st) {
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+    }
+    return b.rmax > 12.5 && b.max_items <= 4 * sms ? launch_sb_n<P, LOCAL, 256>(b, st) : launch_sb_n<P, LOCAL, FB>(b, st);
 }
 
 // Convergence test and list rebuild, one block.  Case states: 0 active,

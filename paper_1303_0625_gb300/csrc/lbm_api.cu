@@ -1,6 +1,7 @@
 // Host side of the C ABI declared in include/lbm.h: context lifetime, solid
 // table, step scheduling (direct launches or a captured CUDA graph), force
 // history, field export and kernel timing.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -27,6 +28,7 @@ struct lbm_ctx {
     DSolid *solids = nullptr;
     int solid_cap = 0;
     int nsolid = 0;
+    double rmax = 0.0;  // largest radius of a solid added
     int *moving_d = nullptr;
     int moving_cap = 0;
     void *ev_d = nullptr;  // covered/fresh events: {length, pad}, int4 list, 6 doubles each
@@ -563,6 +565,7 @@ lbm_status lbm_add_solid(lbm_ctx *c, const lbm_disk *d, int32_t *id_out) {
     const int id = c->nsolid;
     CK(c, cudaMemcpyAsync(c->solids + id, &s, sizeof s, cudaMemcpyHostToDevice, c->stream));
     c->nsolid++;
+    c->rmax = std::max(c->rmax, d->r);
     c->is_moving.push_back(translates(s) ? 1 : 0);
     lbm_status st = upload_moving(c);
     if (st != LBM_OK) return st;
@@ -1242,6 +1245,7 @@ struct lbm_batch {
     int *toff_d = nullptr, *ioff_d = nullptr;
     long long tile_cap = 0, item_cap = 0;
     int max_tiles = 0, max_items = 0;
+    double rmax = 0.0;  // largest radius of a solid
     int *nactive_h = nullptr;  // pinned
     // host copies of the per-case results
     std::vector<int32_t> state;
@@ -1295,6 +1299,7 @@ gbm::BatchLaunch blaunch(const lbm_batch *b) {
     l.force = b->force;
     l.local = b->rho_w_mode == LBM_RHOW_LOCAL;
     l.max_items = b->max_items;
+    l.rmax = b->rmax;
     l.max_tiles = b->max_tiles;
     l.tile_h = b->tile_h;
     l.persistent = b->persistent;
@@ -1390,6 +1395,8 @@ lbm_status bprepare(lbm_batch *b) {
         BCK(b, cudaMalloc(&b->items_d, (size_t)cap * sizeof(int2)));
         b->item_cap = cap;
     }
+    b->rmax = 0.0;
+    for (const lbm_ctx *c : b->cases) b->rmax = std::max(b->rmax, c->rmax);
     b->max_tiles = (int)tiles;
     b->max_items = (int)items;
     BCK(b, cudaMemcpyAsync(b->cases_d, hp.data(), hp.size() * sizeof(StepParams),

@@ -396,6 +396,7 @@ struct BatchLaunch {
     int precision, variant;
     bool force, local;
     int max_items;            // capacity of items (all solids of all cases)
+    double rmax;              // largest radius of a solid
     int max_tiles;            // tiles of all cases at the current tile shape
     int tile_h;               // row segments per warp of a tile
     bool persistent;          // fused kernel: persistent blocks, else one block per tile
