@@ -707,6 +707,7 @@ __device__ __forceinline__ bool need_owners(const StepParams &p, const DSolid &b
 // The half-way boundary: links, record and motion of one solid per block.
 template <int P, bool LOCAL>
 __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
+    early_start();
     using S = typename Prec<P>::S;
     __shared__ LinkShared<P> sh;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -752,6 +753,7 @@ constexpr int LINK_CHUNK = FB / LINK_PARTS;
 
 template <int P, bool LOCAL, bool BND>
 __global__ void __launch_bounds__(FB) k_links(const StepParams p) {
+    early_start();
     using S = typename Prec<P>::S;
     __shared__ LinkShared<P> sh;
     const long long t = *p.t;
@@ -772,6 +774,7 @@ __global__ void __launch_bounds__(FB) k_links(const StepParams p) {
 }
 
 __global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
+    early_start();
     const int lane = threadIdx.x & 31;
     const long long t = *p.t;
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.ev_len) {
@@ -1306,6 +1309,7 @@ __global__ void __launch_bounds__(SW_BLOCK, 4) k_events(const StepParams p) {
 // launch, where they do not run beside the advection-collision kernel.
 template <int P, bool RING>
 __global__ void __launch_bounds__(SW_BLOCK, 4) k_remask_few(const StepParams p) {
+    early_start();
     __shared__ RingShared sh;
     if (*(volatile int *)p.status & 4) return;
     const long long t = *p.t;
@@ -1334,13 +1338,11 @@ cudaError_t launch_f(const StepParams &p, cudaStream_t st) {
     if (blocks > 8 * per_sm * sms) blocks = 8 * per_sm * sms;
     if (blocks < 1) blocks = 1;
     if (!p.link_parts) {
-        k_forces<P, LOCAL><<<blocks, FB, 0, st>>>(p);
-        return cudaGetLastError();
+        return launch_step(p, k_forces<P, LOCAL>, dim3(blocks), FB, st, p);
     }
     const dim3 grid(blocks, p.link_parts);
-    if (p.boundary == LBM_INTERPOLATED) k_links<P, LOCAL, true><<<grid, FB, 0, st>>>(p);
-    else k_links<P, LOCAL, false><<<grid, FB, 0, st>>>(p);
-    return cudaGetLastError();
+    return p.boundary == LBM_INTERPOLATED ? launch_step(p, k_links<P, LOCAL, true>, grid, FB, st, p)
+                                          : launch_step(p, k_links<P, LOCAL, false>, grid, FB, st, p);
 }
 
 // Re-rasterisation of up to FEW_MOVING solids: one cluster of 8 blocks (one solid: 4)
@@ -1355,12 +1357,14 @@ cudaError_t launch_few(const StepParams &p, bool ring, cudaStream_t st) {
     cfg.gridDim = dim3(p.nmoving > 1 ? 8 : 4);
     cfg.blockDim = dim3(SW_BLOCK);
     cfg.stream = st;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cfg.gridDim.x;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cfg.gridDim.x;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = p.early ? 2 : 1;
     return ring ? cudaLaunchKernelEx(&cfg, k_remask_few<P, true>, p) : cudaLaunchKernelEx(&cfg, k_remask_few<P, false>, p);
 }
 
@@ -1649,8 +1653,7 @@ cudaError_t launch_forces(const StepParams &p, cudaStream_t st) {
 
 cudaError_t launch_record(const StepParams &p, cudaStream_t st) {
     if (p.nsolid == 0 || !p.link_parts) return cudaSuccess;
-    k_record<<<(p.nsolid + WARPS - 1) / WARPS, SW_BLOCK, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_step(p, k_record, dim3((p.nsolid + WARPS - 1) / WARPS), SW_BLOCK, st, p);
 }
 
 cudaError_t launch_ring(const StepParams &p, cudaStream_t st) {

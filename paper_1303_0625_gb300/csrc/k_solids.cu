@@ -36,7 +36,7 @@ __device__ __forceinline__ void stamp(const StepParams &p, int s, double X, doub
     }
 }
 
-__global__ void k_tick(const StepParams p) { *p.t += 1; }
+__global__ void k_tick(const StepParams p) { early_start(); *p.t += 1; }
 
 // --------------------------------------------------------- initialisation
 
@@ -403,8 +403,7 @@ dim3 cell_grid(const Lattice &L) { return dim3((L.nx + 127) / 128, L.ny); }
 // ------------------------------------------------------------ launchers
 
 cudaError_t launch_tick(const StepParams &p, cudaStream_t st) {
-    k_tick<<<1, 1, 0, st>>>(p);
-    return cudaGetLastError();
+    return launch_step(p, k_tick, dim3(1), 1, st, p);
 }
 
 cudaError_t launch_init_populations(const StepParams &p, cudaStream_t st) {

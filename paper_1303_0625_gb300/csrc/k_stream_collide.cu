@@ -11,6 +11,7 @@ namespace {
 // One block per SC_BLOCK_X * V nodes of a row.
 template <int P, int V, bool FORCE, bool OPEN, int COLL>
 __global__ void __launch_bounds__(SC_BLOCK_X) k_stream_collide(const StepParams p) {
+    early_start();
     using R = typename Raw<P>::R;
     const long long t = *p.t;
     sc_row<P, V, FORCE, OPEN, COLL>(p, static_cast<const R *>((t & 1) ? p.f1 : p.f0),
@@ -96,10 +97,8 @@ template <int P, int V, bool FORCE, int COLL>
 cudaError_t launch_row(const StepParams &p, cudaStream_t st) {
     const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
     if (p.L.bc_x == LBM_OPEN)
-        k_stream_collide<P, V, FORCE, true, COLL><<<grid, SC_BLOCK_X, 0, st>>>(p);
-    else
-        k_stream_collide<P, V, FORCE, false, COLL><<<grid, SC_BLOCK_X, 0, st>>>(p);
-    return cudaGetLastError();
+        return launch_step(p, k_stream_collide<P, V, FORCE, true, COLL>, grid, SC_BLOCK_X, st, p);
+    return launch_step(p, k_stream_collide<P, V, FORCE, false, COLL>, grid, SC_BLOCK_X, st, p);
 }
 
 template <int P, int V>

@@ -845,8 +845,8 @@ __device__ __noinline__ void inner_update(const StepParams &p, const typename Ra
 //          open columns (OPEN): the collided inner neighbour extrapolated
 //          (extrapolate_open), from this lane's registers or the lane before.
 template <int P, int V, bool FORCE, bool OPEN, int COLL>
-__device__ __forceinline__ void sc_row(const StepParams &p, const typename Raw<P>::R *__restrict__ fin,
-                                       typename Raw<P>::R *__restrict__ fout, int x0, int y) {
+__device__ __forceinline__ void sc_row(const StepParams &p, const typename Raw<P>::R *fin,
+                                       typename Raw<P>::R *fout, int x0, int y) {
     using R = typename Raw<P>::R;
     using C = typename Prec<P>::C;
     using W = typename Word<sizeof(R) * V>::T;
@@ -864,7 +864,7 @@ __device__ __forceinline__ void sc_row(const StepParams &p, const typename Raw<P
     Pack<R, V> raw[9];
 #pragma unroll
     for (int i = 0; i < 9; i++)
-        raw[i].u = __ldg(reinterpret_cast<const W *>(fin + i * plane + SROW(i) + xl));
+        raw[i].u = *reinterpret_cast<const W *>(fin + i * plane + SROW(i) + xl);
     FlagPack<V> fl;
     fl.u = *reinterpret_cast<const typename Word<2 * V>::T *>(p.flags + r0 + xl);
     R hl[3] = {R(0), R(0), R(0)};
@@ -940,7 +940,7 @@ __device__ __forceinline__ void sc_row(const StepParams &p, const typename Raw<P
         for (int i = 0; i < 9; i++) {
             own[i].u = W{};
             if (p.rho_w_mode == LBM_RHOW_LOCAL || cy(i) == (lo ? -1 : 1))
-                own[i].u = __ldg(reinterpret_cast<const W *>(fin + i * plane + r0 + xl));
+                own[i].u = *reinterpret_cast<const W *>(fin + i * plane + r0 + xl);
         }
 #pragma unroll
         for (int j = 0; j < V; j++) {

@@ -100,36 +100,34 @@ lbm_status fail(lbm_ctx *c, lbm_status st, const char *fmt, ...) {
 size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DEV ? 4 : 2); }
 
 // Does work go to the side stream, beside the advection-collision kernel?
-// On a small FP32 domain that kernel is shorter than the hand-over between the streams,
-// and with few moving solids the ring goes into the re-rasterisation's launch: 128 x 64
-// nodes, 1 disk: 36.0 us a step against 41.5 with the side stream; at 768 x 512 59 and
-// 57, so up to 2^18 nodes (in FP64, whose kernel takes longer, the side stream is faster
-// from the smallest domain on).
+// On a small FP32 domain that kernel is shorter than the hand-over between the streams:
+// with few moving solids, whose rings then go into the re-rasterisation's launch, or
+// with none that moves, the step stays on one stream (FILL_NOFORK).  In FP64, whose
+// kernels take longer, the side stream is faster from the smallest domain on.
 bool few_moving(const lbm_ctx *c) {
     return !c->moving.empty() && c->moving.size() <= gbm::FEW_MOVING && c->cfg.boundary == LBM_HALFWAY;
 }
 constexpr long long FORK_NODES = 1 << 18;
 bool forks(const lbm_ctx *c) {
     if (!c->overlap || c->nsolid == 0) return false;
-    if (c->cfg.precision == LBM_FP16_DEV) return true;
-    if (c->cfg.precision == LBM_FP32_DEV && few_moving(c) && (long long)c->cfg.nx * c->cfg.ny <= FORK_NODES) return false;
-    return !c->moving.empty();
+    if (c->cfg.precision != LBM_FP32_DEV || (long long)c->cfg.nx * c->cfg.ny > FORK_NODES) return true;
+    return !few_moving(c) && !(c->moving.empty() && c->cfg.boundary == LBM_HALFWAY);
 }
 
 // Blocks per solid of the link kernel, or 0 for links, record and motion in one
 // kernel.  The record and the motion are a kernel of their own where they can run
-// beside the advection-collision kernel, and with the interpolated boundary, whose
-// links are worth several blocks where the solids alone would not fill the SMs.
-// LINK_PARTS blocks give the sums of one bit for bit.  FP64, whose unit is what one
-// block waits for, takes them with either boundary, and with few solids as many blocks
-// as most disks have chunks of candidates (other partial sums, 1e-16 apart).  A step of
-// 256 x 128 nodes with one disk: 34.5 -> 31 us (one block before), of 1200 x 120 with an
-// interpolated one 47 -> 41 (four before).
+// beside the advection-collision kernel, and with the interpolated boundary.  Below 256
+// solids, which alone would not fill the SMs, LINK_PARTS blocks take a solid's links;
+// they give the sums of one bit for bit.  FP64, whose unit is what a block waits for,
+// takes with few solids as many blocks as most disks have chunks of candidates (other
+// partial sums, 1e-16 apart).  A step of 256 x 128 nodes with one disk, FP64: 34.5 -> 31
+// us (one block before), of 1200 x 120 with an interpolated one 47 -> 41 (four before);
+// 768 x 512 with six of r 51, FP32: 55 -> 50 (one before).
 int link_parts(const lbm_ctx *c) {
     const bool cut = c->cfg.boundary == LBM_INTERPOLATED, fp64 = c->cfg.precision == LBM_FP64;
     if (!cut && (c->cfg.precision == LBM_FP16_DEV || !forks(c))) return 0;
     if (fp64 && c->nsolid <= 32) return gbm::MAX_LINK_PARTS;
-    return (cut || fp64) && c->nsolid < 256 ? gbm::LINK_PARTS : 1;
+    return c->nsolid < 256 ? gbm::LINK_PARTS : 1;
 }
 
 StepParams params(const lbm_ctx *c) {
@@ -203,6 +201,8 @@ StepParams params(const lbm_ctx *c) {
     p.near_id = c->near_d;
     p.part = c->part_d;
     p.link_parts = link_parts(c);
+    // one stream, nothing between its kernels but (with many moving solids) the ring's
+    p.early = c->cfg.precision == LBM_FP32_DEV && !forks(c) && !c->timing && (c->moving.empty() || few_moving(c));
     return p;
 }
 

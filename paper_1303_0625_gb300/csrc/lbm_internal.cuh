@@ -137,6 +137,7 @@ struct StepParams {
     int bnd_cap;              // capacity of the list
     double *part;             // [nsolid][MAX_LINK_PARTS][6] link sums of a solid's blocks
     int link_parts;           // blocks per solid of k_links, which k_record follows; 0: k_forces
+    int early;                // this step's kernels are launched early
     int list_by_forces;       // FP16: the force kernel fills the deferred list; the fused pass
                               // leaves the update to launch_deferred_update
 };
@@ -168,6 +169,15 @@ template <> struct Prec<LBM_FP16_DEV> {
     using C = float;
     static constexpr bool dev = true;
 };
+
+// Steps on one stream (StepParams::early): each kernel is launched early, set up while
+// the one ahead still runs, and waits here before it reads or writes anything of the
+// step; then lets the next one be set up.  Every thread calls it first (in a kernel that
+// was launched as usual it does nothing).
+__device__ __forceinline__ void early_start() {
+    asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 
 __device__ __forceinline__ double ld(const double *p) { return __ldg(p); }
 __device__ __forceinline__ float ld(const float *p) { return __ldg(p); }
@@ -415,6 +425,21 @@ struct BatchState {
     long long *steps;         // step counter of each case at the last test
     int *toff, *ioff;         // offsets of each active case in the tile and item lists
 };
+
+// A kernel whose first statement is early_start().
+template <class... K, class... A>
+cudaError_t launch_step(const StepParams &p, void (*kernel)(K...), dim3 grid, int threads, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = p.early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
 
 // k_stream_collide.cu
 // the fused advection-collision kernel, and in FP16 with variants 3-5 the pass
