@@ -245,7 +245,7 @@ def captured_traffic(precision, nx, ny, variant):
         return None
     if not rec or rec.get("kernel_sha256_16") != kernel_source_hash():
         return None
-    if bool(rec.get("deferred", False)) != (variant >= 3):
+    if bool(rec.get("deferred", False)) != (precision == "fp16" and variant >= 3):
         return None
     # captured on a smaller domain: traffic scales with the node count
     return rec["dram_bytes_per_launch"] * (nx * ny) / (rec["nx"] * rec["ny"])
@@ -326,7 +326,7 @@ def run_ours(a, ws, rank, local):
     peak = float(peaks.get("hbm_gbs", FALLBACK_HBM_GBS))
     traffic = (None if a.collision == "mrt" or interp  # the record is the half-way BGK pass's
                else captured_traffic(a.precision, a.nx, a.ny, main["variant"]))
-    kernels = ("k_stream_collide + k_boundary_update" if main["variant"] >= 3 or interp
+    kernels = ("k_stream_collide + k_boundary_update" if a.precision == "fp16" and (main["variant"] >= 3 or interp)
                else "k_stream_collide")
     if a.collision == "mrt":
         kernels = "k_stream_collide (MRT)"
