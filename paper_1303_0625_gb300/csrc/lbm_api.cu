@@ -102,8 +102,11 @@ size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DE
 // Does work go to the side stream, beside the advection-collision kernel?
 // On a small FP32 domain that kernel is shorter than the hand-over between the streams:
 // with few moving solids, whose rings then go into the re-rasterisation's launch, or
-// with none that moves, the step stays on one stream (FILL_NOFORK).  In FP64, whose
-// kernels take longer, the side stream is faster from the smallest domain on.
+// with none that moves, the step stays on one stream and its kernels are launched early
+// (StepParams::early): 128 x 64 nodes with one moving disk 24.8 us a step, launched one by
+// one (41.5 with the side stream), 300 x 200 with four at rest 14.3 (22.5).  Larger: with
+// the side stream 768 x 512 and six moving disks take 39.7 in a graph against 46.3.  In
+// FP64, whose kernels take longer, it is faster from the smallest domain on.
 bool few_moving(const lbm_ctx *c) {
     return !c->moving.empty() && c->moving.size() <= gbm::FEW_MOVING && c->cfg.boundary == LBM_HALFWAY;
 }
