@@ -57,10 +57,9 @@ const char *lbm_unet_last_error(const lbm_unet *net);
 
 /* Polls of an mbarrier before a wait of the tensor-core convolutions gives
  * up (default 2^24; 0 gives up at the first wait).  A CTA whose wait gave up
- * issues no further copies or MMAs, waits (at most 2^24 polls each) for those
- * it issued, frees its tensor memory and stores nothing more (it may have
- * stored earlier tiles); the next call that
- * synchronises (a host-array forward, lbm_unet_gradients,
+ * takes no further tile, waits (at most 2^24 polls each) for the copies and
+ * MMAs it issued, frees its tensor memory and stores nothing more (it may
+ * have stored earlier tiles); the next call that synchronises (a host-array forward, lbm_unet_gradients,
  * lbm_unet_train_step with a loss) returns LBM_ETIMEOUT once and clears the
  * flag.  The outputs and parameters of the calls since are then undefined:
  * set them again.  LBM_EINVAL for polls < 0. */
