@@ -148,6 +148,13 @@ cudaError_t launch_update(const StepParams &p, cudaStream_t st) {
 template <int V, bool FORCE, bool LOCAL, bool DEFER>
 cudaError_t launch_sc(const StepParams &p, cudaStream_t st) {
     const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
+    // An SM changes its split of L1 and shared memory only when it is empty: with the
+    // split that this kernel would get by itself the force kernel (13 KB a block) beside
+    // it waited for SMs to drain (768 x 512 nodes, six disks of r 51: 59 us a step, now 50;
+    // 2000 x 1500, 180 of r 18: 91 and 87).
+    static const cudaError_t split = cudaFuncSetAttribute(
+        k_stream_collide16<V, FORCE, LOCAL, DEFER>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
+    if (split != cudaSuccess) return split;
     k_stream_collide16<V, FORCE, LOCAL, DEFER><<<grid, SC_BLOCK_X, 0, st>>>(p);
     cudaError_t e = cudaGetLastError();
     // with solids, the force kernel lists the nodes next to them and the
