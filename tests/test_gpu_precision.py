@@ -1,0 +1,82 @@
+"""What the arithmetic of the kernels loses to rounding.
+
+Mass and momentum: advection and collision conserve both; what the constants' rounding
+lets drift is systematic.  Bound: what weights rounded to nearest would give, 9 fl(1/9) - 1
+= 2^-27 of the deviation (3 w_i over e_i e_i: of the momentum), times omega, a step.  Omega
+times weight rounded one by one lets them drift by up to ten times as much.
+
+Force records, relative 2-norm over 100 steps of eight seeded boxes with two disks against
+the FP64 oracle.  Bound: the geometric mean of the errors that nine separate FP32 equilibria
+relaxed as g - omega (g - eq) gave next to the disks, measured on the same boxes, plus 10%.
+"""
+import math
+
+import numpy as np
+import pytest
+
+import workloads as W
+from _pairs import make_gpu, make_oracle, seeded_f
+
+pytestmark = pytest.mark.gpu
+
+CX = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1])[:, None, None]
+CY = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1])[:, None, None]
+WT = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+
+
+def _box(tau, nx=96, ny=64, **kw):
+    w = dict(nx=nx, ny=ny, tau=tau, rho0=1.0, bc_x=W.PERIODIC, bc_y=W.PERIODIC, u0=(0.0, 0.0),
+             wall_ux=(0.0, 0.0), body_force=(0.0, 0.0), rho_w_mode=W.RHOW_CONST, refill=1, solids=[])
+    w.update(kw)
+    return w
+
+
+@pytest.mark.parametrize("variant", [0, 1])
+@pytest.mark.parametrize("tau", [0.55, 0.8, 0.85])
+def test_fp32_mass_and_momentum_do_not_drift(tau, variant):
+    w = _box(tau, u0=(0.1, -0.1))
+    g = make_gpu(w, "fp32")
+    g.set_kernel_variant(variant)
+    g.set_f(1.1 * seeded_f(w, 2))
+
+    def sums():
+        d = g.get_f() - WT
+        return np.array([math.fsum((c * d).ravel()) for c in (1.0, CX, CY)])
+
+    before = sums()
+    g.step(200)
+    assert (np.abs(sums() - before) <= 200 / tau * 2.0 ** -27 * np.abs(before)).all()
+
+
+def _flow(w, seed):
+    """Equilibrium of a smooth velocity field, a few waves each way."""
+    rng = np.random.default_rng(seed)
+    x, y = (np.arange(n) / n * 2 * np.pi for n in (w["nx"], w["ny"]))
+    ux, uy, rho = np.zeros((w["ny"], w["nx"])), np.zeros((w["ny"], w["nx"])), np.ones((w["ny"], w["nx"]))
+    for _ in range(3):
+        k, m = rng.integers(1, 4, 2)
+        a, b, c = rng.uniform(0, 2 * np.pi, 3)
+        ux += 0.006 * np.sin(m * y + a)[:, None] * np.cos(k * x + b)[None]
+        uy += 0.006 * np.sin(k * x + c)[None] * np.cos(m * y + a)[:, None]
+        rho += 0.001 * np.cos(m * y + c)[:, None] * np.sin(k * x + a)[None]
+    e = CX * ux + CY * uy
+    return rho * WT * (1 + 3 * e + 4.5 * e * e - 1.5 * (ux * ux + uy * uy))
+
+
+@pytest.mark.parametrize("boundary,motion,bound", [
+    (0, "rest", 6.868e-6), (0, "spin", 7.795e-7), (0, "move", 1.439e-6),
+    (1, "rest", 8.847e-6), (1, "spin", 8.448e-7), (1, "move", 1.502e-6)])
+def test_fp32_force_records(boundary, motion, bound):
+    errors = []
+    for seed in range(8):
+        rng = np.random.default_rng([seed, 7])
+        vx, vy, om = dict(rest=(0.0, 0.0, 0.0), spin=(0.0, 0.0, 0.002), move=(0.03, 0.02, 0.001))[motion]
+        disks = [dict(cx=24 + 48 * k + rng.uniform(-2, 2), cy=40 + rng.uniform(-10, 10), r=rng.uniform(7, 14),
+                      vx=vx, vy=vy, omega=om, rho_s=1.5, motion=0) for k in range(2)]
+        w = _box(rng.uniform(0.7, 0.95), ny=80, boundary=boundary, solids=disks)
+        o, g, f = make_oracle(w), make_gpu(w, "fp32", ring=100), _flow(w, seed)
+        o.set_f(f)
+        g.set_f(f)
+        ref = o.step(100)
+        errors.append(np.linalg.norm(g.step_record(100) - ref) / np.linalg.norm(ref))
+    assert np.exp(np.mean(np.log(errors))) <= 1.1 * bound, errors
