@@ -36,10 +36,11 @@
 //
 // Precision: per-link products and each lane's running sum over its links
 // (a handful) are in the arithmetic precision of the storage mode (FP32 in the
-// deviation modes); the sums across lanes, the booked momenta and the motion
-// are FP64, in a fixed order.  (GB300 runs FP64 at about two fused
-// multiply-adds per clock per SM: FP64 lane sums would cost the force kernel
-// about 100 us per step on 2000 disks.)
+// deviation modes), and so are the sums across the lanes of a warp (in a batch:
+// FP64); the sums across warps, the booked momenta and the motion are FP64, in a
+// fixed order.  (GB300 runs FP64 at about two fused multiply-adds per clock per
+// SM: FP64 lane sums would cost the force kernel about 100 us per step on 2000
+// disks.)
 #include "lbm_internal.cuh"
 
 #include <algorithm>
@@ -75,6 +76,25 @@ __device__ __forceinline__ void warp_sum(T (&v)[N]) {
 #pragma unroll
     for (int k = 0; k < N; k++)
         for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(FULL, v[k], o);
+}
+
+// The warp's sums of six FP64 values: component sum_of(lane) < 6 in each lane.  Halves of
+// the values go to the other lane of a pair at each step, so that a warp issues 9 FP64
+// additions (two lanes per clock and SM) instead of 30.
+__device__ __forceinline__ int sum_of(int lane) { return lane >> 2 & 4 | lane >> 2 & 2 | lane >> 2 & 1; }
+__device__ __forceinline__ double warp_sum6(const double (&v)[6], int lane) {
+    const bool a = lane & 16, b = lane & 8, c = lane & 4;
+    double h[4], q[2];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const double up = k < 2 ? v[4 + (k & 1)] : 0.0;
+        h[k] = (a ? up : v[k]) + __shfl_xor_sync(FULL, a ? v[k] : up, 16);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; k++) q[k] = (b ? h[k + 2] : h[k]) + __shfl_xor_sync(FULL, b ? h[k] : h[k + 2], 8);
+    double s = (c ? q[1] : q[0]) + __shfl_xor_sync(FULL, c ? q[0] : q[1], 4);
+    s += __shfl_xor_sync(FULL, s, 2);
+    return s + __shfl_xor_sync(FULL, s, 1);
 }
 
 // Set or clear one bit of a 16-bit flags word atomically.
@@ -644,15 +664,28 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
     }
 }
 
-// Lane 0's sums over the block of every thread's lacc, in warp order, plus one
-// term per component (acc[q] of lane q < 6), to all lanes of warp 0.
-template <int P, int NT>
+// Sums over the block of every thread's lacc, over each warp's lanes (WIDE: in FP64) and
+// then over the warps in FP64, in order, to all lanes of warp 0.
+template <int P, int NT, bool WIDE = false>
 __device__ __forceinline__ void block_sums(LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
                                            double (&acc)[6]) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    warp_sum(lacc);
-    if (lane == 0)
-        for (int q = 0; q < 6; q++) sh.part[wib][q] = (double)lacc[q];
+    if constexpr (WIDE) {
+        double v[6], t = 0.0;
+        bool any = false;  // half of a batch's warps have no link
+#pragma unroll
+        for (int q = 0; q < 6; q++) any |= lacc[q] != 0;
+        if (__any_sync(FULL, any)) {
+#pragma unroll
+            for (int q = 0; q < 6; q++) v[q] = (double)lacc[q];
+            t = warp_sum6(v, lane);
+        }
+        if (!(lane & 3) && sum_of(lane) < 6) sh.part[wib][sum_of(lane)] = t;
+    } else {
+        warp_sum(lacc);
+        if (lane == 0)
+            for (int q = 0; q < 6; q++) sh.part[wib][q] = (double)lacc[q];
+    }
     __syncthreads();
     if (wib != 0) return;
     double aq = 0.0;
@@ -1429,7 +1462,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
         solid_links<P, LOCAL, false, ghosts<P>()>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, NT,
                                                  0, 1, sh, lacc);
         double acc[6];
-        block_sums(sh, lacc, acc);
+        block_sums<P, NT, true>(sh, lacc, acc);  // the drags decide when a case has converged
         if (threadIdx.x < 32) {
             const double none[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // resting: no node changes type
             record_forces(p, it.y, threadIdx.x, t, acc, none);

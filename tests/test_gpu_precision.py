@@ -8,14 +8,19 @@ times weight rounded one by one lets them drift by up to ten times as much.
 Force records, relative 2-norm over 100 steps of eight seeded boxes with two disks against
 the FP64 oracle.  Bound: the geometric mean of the errors that nine separate FP32 equilibria
 relaxed as g - omega (g - eq) gave next to the disks, measured on the same boxes, plus 10%.
+
+Batches: first force records of 24 channels (nothing but the links' terms and their sums),
+in units of rho0 r.  Bound: rms errors that FP64 sums over the lanes gave, measured on the
+same channels, plus 10% (FP32 sums: 1.3 to 2.2 times as much).
 """
 import math
 
 import numpy as np
 import pytest
 
+import paper_1303_0625_gb300 as G
 import workloads as W
-from _pairs import make_gpu, make_oracle, seeded_f
+from _pairs import PREC, make_gpu, make_oracle, seeded_f
 
 pytestmark = pytest.mark.gpu
 
@@ -80,3 +85,15 @@ def test_fp32_force_records(boundary, motion, bound):
         ref = o.step(100)
         errors.append(np.linalg.norm(g.step_record(100) - ref) / np.linalg.norm(ref))
     assert np.exp(np.mean(np.log(errors))) <= 1.1 * bound, errors
+
+
+@pytest.mark.parametrize("seed,nx,ny,bound", [
+    (47, (40, 150), (24, 64), 1.953e-8), (47, (200, 400), (100, 200), 1.250e-8),
+    (48, (40, 150), (24, 64), 1.903e-8), (49, (200, 400), (100, 200), 8.852e-9)])
+def test_fp32_batch_sums_of_links(seed, nx, ny, bound):
+    ws = W.cylinder_sweep(24, seed_offset=seed, nx_range=nx, ny_range=ny)
+    b = G.Batch.from_workloads(ws, precision=PREC["fp32"], force_ring=8)
+    b.run(1)
+    off = [(b.case(k).forces(0, 1) - make_oracle(w).step(1))[0, 0, 1, :2] / w["solids"][0]["r"]
+           for k, w in enumerate(ws)]
+    assert np.sqrt(np.mean(np.square(off))) <= 1.1 * bound
