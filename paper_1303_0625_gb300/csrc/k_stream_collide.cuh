@@ -680,12 +680,17 @@ __device__ __forceinline__ bool unphysical(double r, double vx, double vy) {
 
 // BGK collision of one FP64 node, no body force.  GB300 issues about two FP64
 // lanes per clock and SM, so the number of FP64 operations is the kernel's time:
-// about 60 here, against about 154 with nine separate equilibria and a division
-// (2048 x 1024 nodes: 259 us a launch against 550).
-// With h_i = (f_i + f_opp) / 2 and d_i = (f_i - f_opp) / 2 the even and the odd
-// part of the equilibrium relax on their own:
+// about 57 here, against about 154 with nine separate equilibria and a division
+// (2048 x 1024 nodes: 246 us a step against 484).
+// The even and the odd part of two opposite populations relax on their own, each by
+// omega times its distance from equilibrium, so that what is rounded is small:
 //   E_i = rho - 1.5 j.u + 4.5 (e_i.j)(e_i.u)   (rho u = j)
-//   f_i, f_opp  <-  [(1 - omega) h_i + omega w_i E_i] +- [(1 - omega) d_i + 3 omega w_i (e_i.j)]
+//   s = 2 w_i E_i - (f_i + f_opp),  m = 6 w_i (e_i.j) - (f_i - f_opp)
+//   f_i, f_opp  +=  omega / 2 (s +- m)
+// (As (1 - omega) f + omega (...) it took 60 operations, 263 us, and the error against
+// 64-bit arithmetic in another order was 1.1 times that of nine equilibria, in the density
+// of a channel after 100 steps up to 4.8 times: mass drifted by up to 1.2 times the
+// weights' own rounding, 9 fl(1/9) - 1.)
 __device__ __forceinline__ void bgk64(double om, double (&g)[9], double &rho, double &ux,
                                       double &uy) {
     const double a1 = g[1] + g[3], d1 = g[1] - g[3], a2 = g[2] + g[4], d2 = g[2] - g[4];
@@ -696,21 +701,18 @@ __device__ __forceinline__ void bgk64(double om, double (&g)[9], double &rho, do
     ux = jx * inv;
     uy = jy * inv;
     const double pxx = jx * ux, pyy = jy * uy, pxy = jx * uy, t = pxx + pyy;
-    // omega E_i: omega goes into rho, not into the weights, whose sum is then as
-    // close to one as 9 fl(1/9) is (omega w_i rounded one by one let the mass drift)
-    const double o4 = 4.5 * om, A = fma(-1.5 * om, t, om * rho), B = fma(o4, t, A);
-    const double c = 1.0 - om, ch = 0.5 * c;  // uniform over the launch
-    g[0] = fma(wgt<double>(0), A, c * g[0]);
+    const double A = fma(-1.5, t, rho), B = fma(4.5, t, A);
+    const double oh = 0.5 * om;  // uniform over the launch
+    g[0] = fma(om, fma(wgt<double>(0), A, -g[0]), g[0]);
     auto pair = [&](int i, int k, double E, double ej, double a, double d) {
-        const double hs = fma(wgt<double>(i), E, ch * a);
-        const double hd = fma(3.0 * wgt<double>(i) * om, ej, ch * d);
-        g[i] = hs + hd;
-        g[k] = hs - hd;
+        const double s = fma(2.0 * wgt<double>(i), E, -a), m = fma(6.0 * wgt<double>(i), ej, -d);
+        g[i] = fma(oh, s + m, g[i]);
+        g[k] = fma(oh, s - m, g[k]);
     };
-    pair(1, 3, fma(o4, pxx, A), jx, a1, d1);
-    pair(2, 4, fma(o4, pyy, A), jy, a2, d2);
-    pair(5, 7, fma(2.0 * o4, pxy, B), jx + jy, a5, d5);
-    pair(6, 8, fma(-2.0 * o4, pxy, B), jy - jx, a6, d6);
+    pair(1, 3, fma(4.5, pxx, A), jx, a1, d1);
+    pair(2, 4, fma(4.5, pyy, A), jy, a2, d2);
+    pair(5, 7, fma(9.0, pxy, B), jx + jy, a5, d5);
+    pair(6, 8, fma(-9.0, pxy, B), jy - jx, a6, d6);
 }
 
 // Two FP32 nodes per instruction: BGK in deviation form, j = rho u,
