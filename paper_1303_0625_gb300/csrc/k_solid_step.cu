@@ -428,7 +428,8 @@ __device__ void record_forces(const StepParams &p, int s, int lane, long long t,
 // them in the order of the directions; then over each warp's tree, both in the
 // arithmetic precision of the storage mode, then across the block's warps in
 // FP64, in warp order.  (A force is a small difference of large link terms, so
-// another order of the FP32 sums would change it in the fifth digit.)
+// another order of the FP32 sums would change it in the fifth digit.)  FP64: a tree
+// for each 32 candidates, so that a warp's candidates may go to several blocks.
 constexpr int FB = 128;                  // threads per solid (batches: or twice as many)
 constexpr int LU = 2;                    // links a thread loads before it works on them
 constexpr float ANN_EPS = 0.05f;         // above the FP32 rounding of a chord end
@@ -468,10 +469,13 @@ __device__ __forceinline__ int block_scan(int n, LinkShared<P, NT> &sh, int &tot
     return before + inc - n;
 }
 
-// The links of solid s: their sums into lacc (this thread's share; Eq. 4 force
-// and torque, then Eq. 5) and, with GHOST, the returned populations into the solid
+// The links of solid s: their sums into lacc (this thread's share; in FP64 its warp's, of
+// which lane l has component sum_of(l) in lacc[0]; Eq. 4 force and torque, then Eq. 5) and, with GHOST, the returned populations into the solid
 // nodes' slots of fs.  The solid's candidates are taken chunk by chunk of `chunk`
-// <= NT; this block takes the chunks part, part + nparts ...
+// <= NT; this block takes the chunks part, part + nparts ...  With slots (FP64, chunks of
+// a warp) each chunk's sums are left there, six to a slot, with slots of zeros after the
+// chunks of each turn of rows up to a multiple of LINK_PARTS and to MAX_LINK_PARTS, and
+// their number in the last slot.
 //   per link  f_i = f~_i(x_f), the returned f_bb = f_i - 6 w_i rho_w (e_i . v) with
 //   v the solid's velocity at x_s = x_f + e_i / 2 (BND: interpolated from the cut
 //   of the link, v and the lever there); Eq. 4 = e_i f_i - e_opp f_bb, Eq. 5 =
@@ -480,7 +484,8 @@ template <int P, bool LOCAL, bool BND, bool GHOST, int NT>
 __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b, int s,
                                             typename Prec<P>::S *fs, bool owners, bool list,
                                             long long t, int chunk, int part, int nparts,
-                                            LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6]) {
+                                            LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
+                                            double *slots = nullptr) {
     using C = typename Prec<P>::C;
     using S = typename Prec<P>::S;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -491,7 +496,7 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
     const float r = sqrtf(b.r2f);
     const C vx = pick<C>(b.vx, b.vxf), vy = pick<C>(b.vy, b.vyf), om = pick<C>(b.om, b.omf);
     const C rho0 = pick<C>(p.rho0, p.rho0_f);
-    int j0, j1;
+    int j0, j1, nslot = 0;
     rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
     for (int jc = j0; jc <= j1; jc += NT) {  // rows in chunks of NT
         // candidates of row jc + tid
@@ -553,6 +558,7 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
                 sh.rho[tid] = Prec<P>::dev ? (C)1 + a9 : a9;
             }
             sh.cand[tid] = make_int4(k, iu - c.xi, jj - c.yi, (int)m);
+            C sum[6] = {0, 0, 0, 0, 0, 0};  // FP64: of this candidate's links
             for (int at = mine0; dirs; dirs &= dirs - 1)
                 sh.link[at++] = (uint16_t)((__ffs(dirs) - 1) | tid << 4);
             __syncthreads();
@@ -657,20 +663,36 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
                 // the candidate's thread adds its links' terms
                 for (int l = max(mine0, l0); l < min(mine1, l0 + LU * NT); l++)
 #pragma unroll
-                    for (int q6 = 0; q6 < 6; q6++) lacc[q6] += sh.term[q6][l - l0];
+                    for (int q6 = 0; q6 < 6; q6++) (P == LBM_FP64 ? sum : lacc)[q6] += sh.term[q6][l - l0];
                 __syncthreads();  // the terms (and the list) are reused
             }
+            if constexpr (P == LBM_FP64)
+                if ((tid & ~31) < chunk && base + (tid & ~31) < total) {
+                    const double v = warp_sum6(sum, lane);
+                    lacc[0] += v;
+                    if (slots && !(lane & 3) && sum_of(lane) < 6) slots[(nslot + base / 32) * 6 + sum_of(lane)] = v;
+                }
+        }
+        if (P == LBM_FP64 && slots) {
+            int k = (total + 31) / 32;
+            for (; k % LINK_PARTS || nslot + k < MAX_LINK_PARTS; k++)
+                if (k % nparts == part && tid < 6) slots[(nslot + k) * 6 + tid] = 0.0;
+            nslot += k;
+            if (part == 0 && tid == 0) slots[(LINK_SLOTS - 1) * 6] = (double)nslot;
         }
     }
 }
 
-// Sums over the block of every thread's lacc, over each warp's lanes (WIDE: in FP64) and
-// then over the warps in FP64, in order, to all lanes of warp 0.
+// Sums over the block of every thread's lacc, over each warp's lanes (WIDE: in FP64; FP64:
+// solid_links has done that) and then over the warps in FP64, in order, to all lanes of
+// warp 0.
 template <int P, int NT, bool WIDE = false>
 __device__ __forceinline__ void block_sums(LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
                                            double (&acc)[6]) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    if constexpr (WIDE) {
+    if constexpr (P == LBM_FP64) {
+        if (!(lane & 3) && sum_of(lane) < 6) sh.part[wib][sum_of(lane)] = lacc[0];
+    } else if constexpr (WIDE) {
         double v[6], t = 0.0;
         bool any = false;  // half of a batch's warps have no link
 #pragma unroll
@@ -778,9 +800,10 @@ __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
 
 // The same in two kernels: k_links, after which the advection-collision kernel can
 // run, and k_record (records and motion), beside it.  A solid's links go to
-// gridDim.y blocks: one, or several that take its candidates 32 at a time in turn
-// (LINK_PARTS: each the share of one warp of the single block, so that the sums are
-// the same bit for bit).  (With the interpolated boundary one 30-node disk in FP64 took
+// gridDim.y blocks: one, or several that take its candidates 32 at a time in turn:
+// LINK_PARTS, each the share of one warp of the single block, or in FP64
+// MAX_LINK_PARTS, each what a warp takes in one turn: they leave every turn's sums to
+// k_record.  The sums are the same bit for bit, whichever way.  (With the interpolated boundary one 30-node disk in FP64 took
 // 68 us in one block with a thread per candidate: one SM's FP64 unit.)
 constexpr int LINK_CHUNK = FB / LINK_PARTS;
 
@@ -795,13 +818,15 @@ __global__ void __launch_bounds__(FB) k_links(const StepParams p) {
         const DSolid &b = p.S[s];
         if (!solid_ok(b)) continue;  // k_record reports it
         typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
+        double *slots = P == LBM_FP64 && gridDim.y > LINK_PARTS ? p.part + (long long)s * LINK_SLOTS * 6 : nullptr;
         solid_links<P, LOCAL, BND, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
                                                 gridDim.y > 1 ? LINK_CHUNK : FB, blockIdx.y,
-                                                gridDim.y, sh, lacc);
+                                                gridDim.y, sh, lacc, slots);
+        if (slots) continue;
         double acc[6];
         block_sums(sh, lacc, acc);
         if (threadIdx.x == 0)
-            for (int q = 0; q < 6; q++) p.part[((long long)s * MAX_LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
+            for (int q = 0; q < 6; q++) p.part[((long long)s * LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
         __syncthreads();
     }
 }
@@ -822,9 +847,21 @@ __global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
         return;
     }
     double aq = 0.0, acc[6], booked[6];
-    if (lane < 6)
-#pragma unroll 4
-        for (int c = 0; c < p.link_parts; c++) aq += p.part[((long long)s * MAX_LINK_PARTS + c) * 6 + lane];
+    if (p.link_parts > LINK_PARTS) {  // as the warps of one block have added them
+        const double *part = p.part + (long long)s * LINK_SLOTS * 6 + lane;
+        if (lane < 6) {
+            double a[LINK_PARTS] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+            for (int c = 0; c < MAX_LINK_PARTS; c++) a[c % LINK_PARTS] += part[c * 6];
+            const int n = (int)part[(LINK_SLOTS - 1) * 6 - lane];
+            for (int c = MAX_LINK_PARTS; c < n; c += LINK_PARTS)
+#pragma unroll
+                for (int w = 0; w < LINK_PARTS; w++) a[w] += part[(c + w) * 6];
+            aq = ((a[0] + a[1]) + a[2]) + a[3];
+        }
+    } else if (lane < 6) {
+        for (int c = 0; c < p.link_parts; c++) aq += p.part[((long long)s * LINK_PARTS + c) * 6 + lane];
+    }
 #pragma unroll
     for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
     booked_events(p, b, t, lane, booked);

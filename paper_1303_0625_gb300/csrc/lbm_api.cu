@@ -44,7 +44,7 @@ struct lbm_ctx {
     int *status_d = nullptr;
     unsigned int *bar_d = nullptr;  // per-solid control words (displacement, pair test)
     uint16_t *near_d = nullptr;     // near lists, [solid_cap][NEAR_CAP]
-    double *part_d = nullptr;       // link sums by block, [solid_cap][MAX_LINK_PARTS][6]
+    double *part_d = nullptr;       // link sums by block or chunk (StepParams::part)
     long long spin_limit = 1ll << 24;  // polls of a bounded device wait (about one second)
     // the force kernel runs on a second stream beside the advection-collision
     // kernel: fork after the previous step, join before the re-rasterisation
@@ -120,16 +120,16 @@ bool forks(const lbm_ctx *c) {
 // Blocks per solid of the link kernel, or 0 for links, record and motion in one
 // kernel.  The record and the motion are a kernel of their own where they can run
 // beside the advection-collision kernel, and with the interpolated boundary.  Below 256
-// solids, which alone would not fill the SMs, LINK_PARTS blocks take a solid's links;
-// they give the sums of one bit for bit.  FP64, whose unit is what a block waits for,
-// takes with few solids as many blocks as most disks have chunks of candidates (other
-// partial sums, 1e-16 apart).  A step of 256 x 128 nodes with one disk, FP64: 34.5 -> 31
-// us (one block before), of 1200 x 120 with an interpolated one 47 -> 41 (four before);
-// 768 x 512 with six of r 51, FP32: 55 -> 50 (one before).
+// solids, which alone would not fill the SMs, LINK_PARTS blocks take a solid's links.
+// FP64, whose unit is what a block waits for, takes with few solids as many blocks as
+// most disks have chunks of candidates.  The sums are those of one block bit for bit,
+// whichever way.  A step of 256 x 128 nodes with one disk, FP64: 34.5 -> 31 us (one block
+// before), of 1200 x 120 with an interpolated one 47 -> 41 (four before); 768 x 512 with
+// six of r 51, FP32: 55 -> 50 (one before).
 int link_parts(const lbm_ctx *c) {
     const bool cut = c->cfg.boundary == LBM_INTERPOLATED, fp64 = c->cfg.precision == LBM_FP64;
     if (!cut && (c->cfg.precision == LBM_FP16_DEV || !forks(c))) return 0;
-    if (fp64 && c->nsolid <= 32) return gbm::MAX_LINK_PARTS;
+    if (fp64 && c->nsolid <= gbm::MAX_PARTS_SOLIDS && c->rmax <= gbm::MAX_PARTS_RADIUS) return gbm::MAX_LINK_PARTS;
     return c->nsolid < 256 ? gbm::LINK_PARTS : 1;
 }
 
@@ -523,7 +523,8 @@ lbm_status lbm_add_solid(lbm_ctx *c, const lbm_disk *d, int32_t *id_out) {
         CK(c, cudaMalloc(&c->near_d, (size_t)cap * gbm::NEAR_CAP * sizeof(uint16_t)));
         if (c->part_d) CK(c, cudaFree(c->part_d));
         c->part_d = nullptr;
-        CK(c, cudaMalloc(&c->part_d, (size_t)cap * gbm::MAX_LINK_PARTS * 6 * sizeof(double)));
+        const int slots = std::max(cap * gbm::LINK_PARTS, gbm::MAX_PARTS_SOLIDS * gbm::LINK_SLOTS);
+        CK(c, cudaMalloc(&c->part_d, (size_t)slots * 6 * sizeof(double)));
         c->solid_cap = cap;
     }
     if (c->nsolid + 1 > c->ring_cap) {

@@ -82,8 +82,13 @@ constexpr int NEAR_CAP = 32;
 constexpr float NEAR_REACH = 4.5f;
 constexpr float NEAR_MARGIN = 4.0f;
 
-// blocks that share one solid's links: the warps of a single block, or in FP64 more
-constexpr int LINK_PARTS = 4, MAX_LINK_PARTS = 16;
+// Blocks that share one solid's links: the warps of a single block, or in FP64 more, which
+// leave the sums of every 32 candidates.  A disk has up to 4.76 (2 r + 1.42) candidates on
+// its annulus and two more in each of its 2 r + 9 rows, taken 128 rows at a time: up to
+// r = 150, 65 chunks, and 12 to fill up three turns.
+constexpr int LINK_PARTS = 4, MAX_LINK_PARTS = 16, LINK_SLOTS = 80;
+constexpr double MAX_PARTS_RADIUS = 150.0;
+constexpr int MAX_PARTS_SOLIDS = 32;
 
 // covered/fresh nodes one solid can queue per step
 constexpr int SOLID_EVENTS = 256;
@@ -135,7 +140,8 @@ struct StepParams {
     int chg_cap;
     int *bnd;                 // deferred per-node path: {length at even t, at odd t, list...}
     int bnd_cap;              // capacity of the list
-    double *part;             // [nsolid][MAX_LINK_PARTS][6] link sums of a solid's blocks
+    double *part;             // [nsolid][LINK_PARTS][6] link sums of a solid's blocks, or with
+                              // more blocks [nsolid][LINK_SLOTS][6] of its chunks
     int link_parts;           // blocks per solid of k_links, which k_record follows; 0: k_forces
     int early;                // this step's kernels are launched early
     int list_by_forces;       // FP16: the force kernel fills the deferred list; the fused pass

@@ -112,3 +112,48 @@ def test_fp32_batch_sums_of_links(seed, nx, ny, bound):
     off = [(b.case(k).forces(0, 1) - make_oracle(w).step(1))[0, 0, 1, :2] / w["solids"][0]["r"]
            for k, w in enumerate(ws)]
     assert np.sqrt(np.mean(np.square(off))) <= 1.1 * bound
+
+
+def _records(w, precision, overlap, steps, save=None, load=None):
+    g = make_gpu(w, precision, ring=40)
+    g.set_force_overlap(overlap)
+    if load is None:
+        g.set_f(seeded_f(w, 3))
+    else:
+        g.load(load)
+    rec = g.step_record(steps)
+    return rec, g.get_f(), g.solids(), g.save() if save else None
+
+
+@pytest.mark.parametrize("boundary", [0, 1])
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+@pytest.mark.parametrize("r", [15.0, 30.0, 51.0, 70.0, 151.0])  # FP64 parts: 5, 10, 16 chunks; two turns of rows; none
+def test_forces_do_not_depend_on_where_they_are_summed(r, precision, boundary):
+    """The link sums of a disk come out bit for bit whether one block takes them or several,
+    with the per-solid work beside the advection-collision kernel and before it, and a free
+    disk's path with them; a state saved one way goes on the other."""
+    n = int(4 * r + 30)
+    disks = [dict(cx=n / 4, cy=n / 4 + 3.3, r=r / 2, vx=0.02, vy=0.01, omega=0.001, rho_s=1.5, motion=0),
+             dict(cx=5 * n / 8, cy=5 * n / 8, r=r, vx=0.01, vy=-0.02, omega=0.0, rho_s=1.2, motion=1)]
+    w = _box(0.8, n, n, gravity=(0.0, -1e-5), boundary=boundary, solids=disks)
+    beside, before = (_records(w, precision, on, 30, save=True) for on in (True, False))
+    for a, b in zip(beside[:3], before[:3]):
+        assert np.array_equal(a, b)
+    again = [_records(w, precision, on, 10, load=beside[3]) for on in (True, False)]
+    for a, b in zip(*again):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,few", [("fp64", 32), ("fp64", 255), ("fp32", 255)])
+def test_forces_do_not_depend_on_the_number_of_solids(precision, few):
+    """Another disk, far from the first, changes the number of blocks that share a disk's links."""
+    one = dict(cx=40.2, cy=41.7, r=22.0, vx=0.02, vy=0.01, omega=0.002, rho_s=1.5, motion=0)
+    small = [dict(cx=100.0 + 16 * (k % 32), cy=20.0 + 16 * (k // 32), r=4.0, vx=0.0, vy=0.0, omega=0.0, rho_s=1.0, motion=0)
+             for k in range(few)]
+    first = []
+    for k in (few - 1, few):
+        w = _box(0.8, 640, 180, solids=[one] + small[:k])
+        g = make_gpu(w, precision, ring=4)
+        g.set_f(seeded_f(w, 4))
+        first.append(g.step_record(1)[:, 0])
+    assert np.array_equal(*first)
