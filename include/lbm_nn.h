@@ -86,7 +86,8 @@ lbm_status lbm_unet_gradients(lbm_unet *net, const float *in, const float *targe
 
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8, bias-corrected) on the
  * loss of one mini-batch; *loss (when not NULL) receives the loss before
- * the step. */
+ * the step.  Gradients and losses are summed in a fixed order: the same steps
+ * on the same kind of device give the same parameters bit for bit. */
 lbm_status lbm_unet_train_step(lbm_unet *net, const float *in, const float *target,
                                const float *fluid, int32_t batch, float lr, double *loss,
                                int32_t on_device);

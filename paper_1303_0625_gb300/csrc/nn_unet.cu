@@ -20,8 +20,10 @@
 //   forward      out[Q][co]  = sum_{tap,ci} x[Q + s(tap)][ci] w[co][tap][ci]      M=Q  N=Cout K=9 Cin
 //   data grad    dx[Q][ci]   = sum_{tap,co} dz[Q - s(tap)][co] w[co][tap][ci]     M=Q  N=Cin  K=9 Cout
 //   weight grad  dw[tap][ci][co] = sum_Q x[Q + s(tap)][ci] dz[Q][co]  M=(dy, ci)  N=Cout K=Q, one per dx
-// s(tap) = (tap / 3 - 1, tap % 3 - 1).  The weight gradient splits K over blocks and
-// adds FP32 partial sums atomically.
+// s(tap) = (tap / 3 - 1, tap % 3 - 1).  The weight gradient splits K over blocks, whose
+// FP32 partial sums are added in a fixed order (k_sum_parts): nothing in a training step
+// depends on the order in which blocks come to an end, so that it can be repeated bit
+// for bit.
 //
 // Weights: FP32 masters, gradients and Adam moments [tap][Cin][Cout]; BF16 copies
 // packed as the B operands of the forward and data-gradient convolutions (packed_at).
@@ -549,12 +551,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
 // MN-major (8 consecutive channels of a pixel are a core-matrix row), so the planes are
 // copied as they are: 8-channel groups (dy, g) of a run of pixels, from (dy, -1) on, and
 // dz's groups.  dx shifts A's start address by a pixel.  A CTA takes 16 groups (128
-// rows) x BN outputs and a range of pixels, in runs of up to 128 (Runs); the result goes
-// to dw with FP32 atomics, four outputs at a time.  The bias gradient, the sum of dz, is
-// taken from the staged dz by the epilogue warps.
+// rows) x BN outputs and a range of pixels, in runs of up to 128 (Runs); its sums go to
+// the range's partial result, four outputs at a time.  The bias gradient, the sum of dz,
+// is taken from the staged dz by the epilogue warps.
 struct WgradOp {
     const bf16 *x, *dz;  // planes, xstr and zstr pixels each
-    float *dw, *db;      // [tap][Ci][Co], [Co]
+    float *part;         // of every range of pixels: [tap][Ci][Co], then [Co] for the bias
     long long xstr, zstr;
     int Wp, Ci, Co, G, stages;
     // the sum over pixels: rows of W pixels, H of them PSI apart, the first at q0; npix
@@ -604,7 +606,6 @@ template <int BN>
 __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long long limit, int *err) {
     extern __shared__ __align__(1024) unsigned char smem[];
     __shared__ __align__(8) Pipe pp;
-    __shared__ float bsum[BN];
     constexpr int COLS = 3 * BN, NCOLS = COLS <= 128 ? 128 : (COLS <= 256 ? 256 : 512);
     const uint32_t AG = (op.runpx + 2) * 16, ZG = op.runpx * 16;  // bytes of a group of A, of dz
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -615,7 +616,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long 
     const uint32_t base = smem_u32(smem), stage = 16 * AG + BN / 8 * ZG;
     const bool bias = blockIdx.x == 0;
     Runs run(op);
-    if (tid < BN) bsum[tid] = 0.f;
+    float *sum = op.part + (long long)blockIdx.z * (9 * op.Ci + 1) * op.Co;  // of this range
     pipe_init(pp, bias ? 5 : 1, NCOLS, warp, tid);
     const uint32_t tmem = pp.tmem;
     if (warp == 0) {
@@ -671,10 +672,10 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long 
         if (issued && leader && *(volatile int *)&pp.abort) drain_mmas(pp);
         __syncwarp();
     } else {
+        // 128 threads: channel group g, every np-th pixel
+        const int t = tid - 64, g = t % zg, np = 128 / zg, p0 = t / zg;
+        float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (bias) {
-            // 128 threads: channel group g, every np-th pixel
-            const int t = tid - 64, g = t % zg, np = 128 / zg, p0 = t / zg;
-            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             Ring r;
             for (; run.next(op); run.advance(op), r.next(S)) {
                 if (!pipe_wait_warp(pp, pp.full[r.s], r.phase, limit)) break;
@@ -694,11 +695,25 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long 
                 __syncwarp();
                 if (lane == 0) mbar_arrive(smem_u32(&pp.empty[r.s]));
             }
-            if (p0 < np)
-#pragma unroll
-                for (int j = 0; j < 8; j++) atomicAdd(&bsum[g * 8 + j], a[j]);
         }
-        if (pipe_wait_warp(pp, pp.tfull[0], 0, limit)) {
+        const bool done = pipe_wait_warp(pp, pp.tfull[0], 0, limit);
+        if (bias) {
+            // every MMA has read its stages, and after the barrier every thread its dz:
+            // the first stage takes the threads' sums, added in the order of the pixels
+            // (the four warps come to the barriers whatever their waits' outcome)
+            float *sums = reinterpret_cast<float *>(smem);
+            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            if (done && p0 < np)
+#pragma unroll
+                for (int j = 0; j < 8; j++) sums[t * 8 + j] = a[j];
+            asm volatile("bar.sync 1, 128;\n" ::: "memory");
+            if (done && t < zg * 8) {
+                float b = 0.f;
+                for (int p = 0; p < np; p++) b += sums[(p * zg + (t >> 3)) * 8 + (t & 7)];
+                sum[(long long)9 * op.Ci * op.Co + n0 + t] = b;
+            }
+        }
+        if (done) {
             asm volatile("tcgen05.fence::after_thread_sync;\n");
             const int part = warp & 3;
             const int m = m0 + part * 4 + (lane >> 3);  // this lane's (dy, g)
@@ -706,7 +721,7 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long 
             const int dy = m / op.G, ci = (m - dy * op.G) * 8 + (lane & 7);
 #pragma unroll
             for (int dx = 0; dx < 3; dx++) {
-                float *row = op.dw + ((long long)(dy * 3 + dx) * op.Ci + ci) * op.Co + n0;
+                float *row = sum + ((long long)(dy * 3 + dx) * op.Ci + ci) * op.Co + n0;
 #pragma unroll
                 for (int c0 = 0; c0 < BN; c0 += 32) {
                     float f[32];
@@ -715,19 +730,57 @@ __global__ void __launch_bounds__(WG_THREADS) k_wgrad_tc(const WgradOp op, long 
 #pragma unroll
                     for (int j = 0; j < 32; j += 4)
                         if (mine && n0 + c0 + j < op.Co)
-                            atomicAdd(reinterpret_cast<float4 *>(row + c0 + j),
-                                      make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]));
+                            *reinterpret_cast<float4 *>(row + c0 + j) =
+                                make_float4(f[j], f[j + 1], f[j + 2], f[j + 3]);
                 }
             }
         }
     }
     __syncthreads();
-    if (pp.abort) {
-        if (tid == 0) atomicOr(err, 1);
-    } else if (bias && tid < BN && n0 + tid < op.Co) {
-        atomicAdd(op.db + n0 + tid, bsum[tid]);
-    }
+    if (tid == 0 && pp.abort) atomicOr(err, 1);
     tc_free(tmem, NCOLS, warp);
+}
+
+// s + c, c the rounding errors, plus x (Knuth's two-sum)
+__device__ __forceinline__ void add_comp(float &s, float &c, float x) {
+    const float t = s + x, b = t - s;
+    c += (s - (t - b)) + (x - b);
+    s = t;
+}
+
+// The sum of nz partial results of n4 + m4 float4 each, into dst and dst2 (m4 of them): a
+// thread of SP_Z takes every SP_Z-th, in order, and the first thread adds theirs, in
+// order; the additions' rounding errors are added up beside them, so that the sum is
+// rounded once.  What bounds it is the reads, from L2 (up to 40 MB a layer).
+constexpr int SP_X = 32, SP_Z = 8;
+__global__ void __launch_bounds__(SP_X *SP_Z) k_sum_parts(const float4 *part, int nz, int n4, int m4, float4 *dst,
+                                                          float4 *dst2) {
+    __shared__ float4 ss[SP_Z][SP_X], sc[SP_Z][SP_X];
+    const int x = threadIdx.x % SP_X, z0 = threadIdx.x / SP_X, i = blockIdx.x * SP_X + x;
+    const long long str = n4 + m4;
+    float4 s = make_float4(0.f, 0.f, 0.f, 0.f), c = s;
+    if (i < str)
+#pragma unroll 4
+        for (int z = z0; z < nz; z += SP_Z) {
+            const float4 v = part[z * str + i];
+            add_comp(s.x, c.x, v.x);
+            add_comp(s.y, c.y, v.y);
+            add_comp(s.z, c.z, v.z);
+            add_comp(s.w, c.w, v.w);
+        }
+    ss[z0][x] = s;
+    sc[z0][x] = c;
+    __syncthreads();
+    if (z0 != 0 || i >= str) return;
+    for (int z = 1; z < SP_Z; z++) {
+        const float4 v = ss[z][x], d = sc[z][x];
+        add_comp(s.x, c.x, v.x);
+        add_comp(s.y, c.y, v.y);
+        add_comp(s.z, c.z, v.z);
+        add_comp(s.w, c.w, v.w);
+        c = make_float4(c.x + d.x, c.y + d.y, c.z + d.z, c.w + d.w);
+    }
+    (i < n4 ? dst[i] : dst2[i - n4]) = make_float4(s.x + c.x, s.y + c.y, s.z + c.z, s.w + c.w);
 }
 
 // ------------------------------------------------------ other layers
@@ -836,27 +889,35 @@ __global__ void k_head(const bf16 *d, long long dstr, const float *w, const floa
     for (int o = 0; o < 3; o++) out[(n * 3 + o) * HW + r] = acc[o];
 }
 
-// fluid-node count (for the loss normalisation)
-__global__ void k_count(const float *fluid, long long n, float *cnt) {
-    __shared__ float s[EW];
-    float a = 0.f;
-    for (long long i = (long long)blockIdx.x * EW + threadIdx.x; i < n; i += (long long)gridDim.x * EW)
-        a += fluid[i];
+// a block's sum of one value per thread, in a fixed order, in thread 0
+__device__ __forceinline__ float block_sum(float (&s)[EW], float a) {
     s[threadIdx.x] = a;
     __syncthreads();
     for (int o = EW / 2; o > 0; o >>= 1) {
         if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
         __syncthreads();
     }
-    if (threadIdx.x == 0) atomicAdd(cnt, s[0]);
+    return s[0];
 }
 
-// loss = sum (out - t)^2 m / (3 count); dout = 2 (out - t) m / (3 count)
+// fluid-node count (for the loss normalisation), a part per block
+__global__ void k_count(const float *fluid, long long n, float *cnt) {
+    __shared__ float s[EW];
+    float a = 0.f;
+    for (long long i = (long long)blockIdx.x * EW + threadIdx.x; i < n; i += (long long)gridDim.x * EW)
+        a += fluid[i];
+    a = block_sum(s, a);
+    if (threadIdx.x == 0) cnt[blockIdx.x] = a;
+}
+
+// loss = sum (out - t)^2 m / (3 count), a part per block; dout = 2 (out - t) m / (3 count)
 __global__ void k_loss(const float *out, const float *tgt, const float *fluid, const float *cnt,
                        float *dout, double *loss, int B, int HW) {
     __shared__ float s[EW];
     const long long n3 = (long long)B * 3 * HW;
-    const float inv = 1.f / (3.f * fmaxf(*cnt, 1.f));
+    const float count = block_sum(s, cnt[threadIdx.x]);
+    __syncthreads();
+    const float inv = 1.f / (3.f * fmaxf(count, 1.f));
     float a = 0.f;
     for (long long i = (long long)blockIdx.x * EW + threadIdx.x; i < n3; i += (long long)gridDim.x * EW) {
         const long long n = i / (3 * HW), r = i % HW;
@@ -865,26 +926,28 @@ __global__ void k_loss(const float *out, const float *tgt, const float *fluid, c
         a += d * d;
         dout[i] = 2.f * d * inv;
     }
-    s[threadIdx.x] = a;
-    __syncthreads();
-    for (int o = EW / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) s[threadIdx.x] += s[threadIdx.x + o];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) atomicAdd(loss, (double)(s[0] * inv));
+    a = block_sum(s, a);
+    if (threadIdx.x == 0) loss[1 + blockIdx.x] = (double)(a * inv);
+}
+constexpr int CNT_BLOCKS = EW, LOSS_BLOCKS = 1024;
+
+// the loss's parts, in order
+__global__ void __launch_bounds__(32) k_loss_sum(double *loss) {
+    double a = 0.0;
+    for (int i = threadIdx.x; i < LOSS_BLOCKS; i += 32) a += loss[1 + i];
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_down_sync(0xffffffffu, a, o);
+    if (threadIdx.x == 0) loss[0] = a;
 }
 
-// head backward: dd[c] = (d[c] > 0) sum_o dout[o] w[o][c]; dw[o][c] += sum over the
-// pixels of dout[o] d[c]; db[o] += sum of dout[o].  A thread takes every
+// head backward: dd[c] = (d[c] > 0) sum_o dout[o] w[o][c]; of the block's pixels, into
+// its partial result: dw[o][c] = sum of dout[o] d[c], db[o] = sum of dout[o].  A thread takes every
 // gridDim.x EW-th pixel of one group of 8 channels and keeps its 24 sums in registers
 // to the end (one pixel per thread and 96 warp sums for it took 220 us at 0.5 M
 // pixels, the memory traffic 12).
 __global__ void __launch_bounds__(EW) k_head_back(const float *dout, const bf16 *d, long long dstr,
-                                                  const float *w, bf16 *dd, float *dw, float *db, int B,
-                                                  Geo geo, int C) {
-    __shared__ float red[27];
-    if (threadIdx.x < 27) red[threadIdx.x] = 0.f;
-    __syncthreads();
+                                                  const float *w, bf16 *dd, float *part, int B, Geo geo,
+                                                  int C) {
+    __shared__ float red[EW / 32][28];
     const int c0 = blockIdx.y * 8;
     const long long HW = (long long)geo.H * geo.W;
     float wv[3][8], s[3][8], sb[3] = {0.f, 0.f, 0.f};
@@ -916,7 +979,7 @@ __global__ void __launch_bounds__(EW) k_head_back(const float *dout, const bf16 
     }
     auto sum = [&](float v, int k) {
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if ((threadIdx.x & 31) == 0) atomicAdd(&red[k], v);
+        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
     };
 #pragma unroll
     for (int o = 0; o < 3; o++) {
@@ -925,8 +988,13 @@ __global__ void __launch_bounds__(EW) k_head_back(const float *dout, const bf16 
         sum(sb[o], 24 + o);
     }
     __syncthreads();
-    if (threadIdx.x < 24) atomicAdd(dw + (threadIdx.x >> 3) * C + c0 + (threadIdx.x & 7), red[threadIdx.x]);
-    if (blockIdx.y == 0 && threadIdx.x >= 24 && threadIdx.x < 27) atomicAdd(db + threadIdx.x - 24, red[threadIdx.x]);
+    if (threadIdx.x >= 28) return;
+    float v = 0.f;  // the last of the four for the bias stays zero
+    if (threadIdx.x < 27)
+        for (int k = 0; k < EW / 32; k++) v += red[k][threadIdx.x];
+    float *p = part + (long long)blockIdx.x * (3 * C + 4);
+    if (threadIdx.x < 24) p[(threadIdx.x >> 3) * C + c0 + (threadIdx.x & 7)] = v;
+    else if (blockIdx.y == 0) p[3 * C + threadIdx.x - 24] = v;
 }
 
 // Where a parameter sits: the vector of all convolutions, weights [tap][Cin][Cout] (the
@@ -1055,8 +1123,9 @@ struct lbm_unet {
     lbm_unet_config cfg{};
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    cudaStream_t side = nullptr;  // weight gradients (backward)
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t side[2] = {};    // weight gradients (backward), in turn
+    cudaEvent_t fork = nullptr, join[2] = {};
+    int turn = 0;
     std::vector<Conv> convs;  // parameter order
     std::vector<Level> lv;
     nn::ConvTab tab{};
@@ -1066,8 +1135,9 @@ struct lbm_unet {
     float *out = nullptr, *dout = nullptr;
     float *io_in = nullptr, *io_tgt = nullptr, *io_fl = nullptr;  // staging
     float *abi = nullptr;    // parameters or gradients in the caller's order
-    float *cnt = nullptr;
-    double *loss = nullptr;
+    float *part[2] = {};     // partial sums of a layer's gradient, one for each side stream
+    float *cnt = nullptr;    // fluid nodes, by block
+    double *loss = nullptr;  // the loss, then its parts by block
     int *err_d = nullptr;    // bit 0: a bounded wait of a tensor-core kernel ran out
     long long wait_limit = nn::TC_SPIN;  // polls of an mbarrier before a wait gives up
     int sms = 0;             // streaming multiprocessors of the device
@@ -1151,9 +1221,11 @@ cudaError_t palloc(lbm_unet *n, Planes *q, const nn::Geo &geo, int C) {
 void nrelease(lbm_unet *n) {
     if (!n) return;
     for (void *p : n->allocs) cudaFree(p);
-    if (n->side) cudaStreamDestroy(n->side);
+    for (cudaStream_t s : n->side)
+        if (s) cudaStreamDestroy(s);
     if (n->fork) cudaEventDestroy(n->fork);
-    if (n->join) cudaEventDestroy(n->join);
+    for (cudaEvent_t v : n->join)
+        if (v) cudaEventDestroy(v);
     if (n->own_stream && n->stream) cudaStreamDestroy(n->stream);
     delete n;
 }
@@ -1258,8 +1330,48 @@ cudaError_t conv_dgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Plan
     return conv(n, cv.bwd, cv.co, cv.ci, -1, nullptr, false, dz, mask, dx, geo, nullptr, B);
 }
 
+// K splits of a weight gradient: four per SM and tile of 128 (tap, ci) rows, at most one
+// per 64 pixels (`blocks`).  An accumulator adds one split's pixels in series, each
+// addition rounded towards zero in the tensor core, so the length of a split is part of
+// the gradient's rounding, not only of its time.
+int wg_splits(const lbm_unet *n, int ci, int co, long long blocks) {
+    const int bn = co <= 32 ? 32 : (co <= 64 ? 64 : 128);
+    const int z = 4 * n->sms / ((9 * ci + 127) / 128 * ((co + bn - 1) / bn));
+    return z < 1 ? 1 : (z > blocks ? (int)blocks : z);
+}
+
+// Floats of the partial sums of any layer's gradient.
+size_t part_size(const lbm_unet *n) {
+    const nn::Geo g(n->cfg.height, n->cfg.width);
+    const long long blocks = ((long long)n->cfg.max_batch * g.PSI + nn::WG_SPLIT - 1) / nn::WG_SPLIT;
+    size_t most = (size_t)2 * n->sms * (3 * n->cfg.base + 4);  // the head
+    for (const Conv &c : n->convs) {
+        const size_t s = c.k == 1 ? 0 : (size_t)wg_splits(n, c.ci, c.co, blocks) * (9 * c.ci + 1) * c.co;
+        if (s > most) most = s;
+    }
+    return most;
+}
+
+// dst = the sum of nz partial results' first cnt floats, dst2 that of the rest (cnt2)
+cudaError_t sum_parts(const float *part, int nz, int cnt, int cnt2, float *dst, float *dst2, cudaStream_t st) {
+    const int n4 = cnt / 4, m4 = cnt2 / 4;
+    nn::k_sum_parts<<<(n4 + m4 + nn::SP_X - 1) / nn::SP_X, nn::SP_X * nn::SP_Z, 0, st>>>(
+        reinterpret_cast<const float4 *>(part), nz, n4, m4, reinterpret_cast<float4 *>(dst),
+        reinterpret_cast<float4 *>(dst2));
+    return cudaGetLastError();
+}
+
+// The next side stream and its partial sums, once what the main stream has so far is done.
+cudaError_t next_side(lbm_unet *n, cudaStream_t *st, float **part) {
+    *st = n->side[n->turn];
+    *part = n->part[n->turn];
+    n->turn ^= 1;
+    const cudaError_t e = cudaEventRecord(n->fork, n->stream);
+    return e == cudaSuccess ? cudaStreamWaitEvent(*st, n->fork, 0) : e;
+}
+
 template <int BN>
-cudaError_t launch_wg(lbm_unet *n, nn::WgradOp &op, cudaStream_t st) {
+cudaError_t launch_wg(lbm_unet *n, nn::WgradOp &op, float *dw, float *db, cudaStream_t st) {
     using namespace nn;
     static bool attr = false;
     if (!attr) {
@@ -1272,17 +1384,13 @@ cudaError_t launch_wg(lbm_unet *n, nn::WgradOp &op, cudaStream_t st) {
     op.stages = (two ? SMEM_TWO : SMEM_MAX) / stage;
     if (op.stages > 4) op.stages = 4;
     const int gx = (3 * op.G + 15) / 16, gy = (op.Co + BN - 1) / BN;
-    // K splits: four per SM and tile of 128 (tap, ci) rows.  An accumulator adds one
-    // split's pixels in series, each addition rounded towards zero in the tensor core,
-    // so the length of a split is part of the gradient's rounding, not only of its time
-    int z = 4 * n->sms / ((9 * op.Ci + 127) / 128 * gy);
     const long long blocks = (op.npix + WG_SPLIT - 1) / WG_SPLIT;
-    if (z < 1) z = 1;
-    if (z > blocks) z = (int)blocks;
+    int z = wg_splits(n, op.Ci, op.Co, blocks);
     op.perz = (blocks + z - 1) / z * WG_SPLIT;
     z = (int)((op.npix + op.perz - 1) / op.perz);
     k_wgrad_tc<BN><<<dim3(gx, gy, z), WG_THREADS, op.stages * stage, st>>>(op, n->wait_limit, n->err_d);
-    return cudaGetLastError();
+    cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? sum_parts(op.part, z, 9 * op.Ci * op.Co, op.Co, dw, db, st) : e;
 }
 
 cudaError_t conv_wgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Planes &x, const nn::Geo &geo, int B) {
@@ -1291,8 +1399,7 @@ cudaError_t conv_wgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Plan
     op.xstr = x.str;
     op.dz = dz.p;
     op.zstr = dz.str;
-    op.dw = n->g + cv.w_off;
-    op.db = n->g + cv.b_off;
+    float *dw = n->g + cv.w_off, *db = n->g + cv.b_off;
     op.Wp = geo.Wp;
     op.PSI = geo.PSI;
     if (geo.W % 16 == 0) {
@@ -1314,12 +1421,11 @@ cudaError_t conv_wgrad(lbm_unet *n, const Conv &cv, const Planes &dz, const Plan
     op.Ci = cv.ci;
     op.Co = cv.co;
     op.G = cv.ci / 8;
-    // beside the main stream, once dz is complete
-    cudaError_t e = cudaEventRecord(n->fork, n->stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(n->side, n->fork, 0);
+    cudaStream_t st;
+    cudaError_t e = next_side(n, &st, &op.part);
     if (e != cudaSuccess) return e;
-    return cv.co <= 32 ? launch_wg<32>(n, op, n->side)
-                       : (cv.co <= 64 ? launch_wg<64>(n, op, n->side) : launch_wg<128>(n, op, n->side));
+    return cv.co <= 32 ? launch_wg<32>(n, op, dw, db, st)
+                       : (cv.co <= 64 ? launch_wg<64>(n, op, dw, db, st) : launch_wg<128>(n, op, dw, db, st));
 }
 
 lbm_status forward_chain(lbm_unet *n, const float *in_dev, float *out_dev, int B) {
@@ -1364,26 +1470,28 @@ lbm_status forward(lbm_unet *n, const float *in_dev, float *out_dev, int B) {
 
 // The main stream waits for the weight gradients so far.
 cudaError_t join_side(lbm_unet *n) {
-    cudaError_t e = cudaEventRecord(n->join, n->side);
-    return e == cudaSuccess ? cudaStreamWaitEvent(n->stream, n->join, 0) : e;
+    for (int k = 0; k < 2; k++) {
+        cudaError_t e = cudaEventRecord(n->join[k], n->side[k]);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(n->stream, n->join[k], 0);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
-// The weight gradients run on a stream of their own, each from the dz it sums on:
+// The weight gradients run on two streams of their own in turn, each from the dz it sums
+// on, so that the sums over one layer's splits are not in the way of the next layer:
 // nothing before the optimizer needs them, and neither they nor the convolutions that
 // carry the gradient on fill the chip (four training steps of 16 images of 128 x 256:
-// 6.15 ms in one stream, 5.32 so).  A level's g1 and g2 are written twice,
-// by the decoder's and by the encoder's half: the second writes wait for the first half's
-// weight gradients.
+// 6.15 ms in one stream, 5.32 with one beside it, when the splits were added atomically).
+// A level's g1 and g2 are written twice, by the decoder's and by the encoder's half: the
+// second writes wait for the first half's weight gradients.
 lbm_status backward_side(lbm_unet *n, const float *tgt_dev, const float *fl_dev, int B) {
     const int L = n->cfg.levels;
     const nn::Geo &g0 = n->lv[0].geo;
     const long long HW = (long long)g0.H * g0.W;
-    NCK(n, cudaMemsetAsync(n->g, 0, n->nparam * sizeof(float), n->stream));
-    NCK(n, cudaMemsetAsync(n->cnt, 0, sizeof(float), n->stream));
-    NCK(n, cudaMemsetAsync(n->loss, 0, sizeof(double), n->stream));
-    NCK(n, (nn::k_count<<<256, nn::EW, 0, n->stream>>>(fl_dev, B * HW, n->cnt), cudaGetLastError()));
-    NCK(n, (nn::k_loss<<<1024, nn::EW, 0, n->stream>>>(n->out, tgt_dev, fl_dev, n->cnt, n->dout,
-                                                       n->loss, B, (int)HW),
+    NCK(n, (nn::k_count<<<nn::CNT_BLOCKS, nn::EW, 0, n->stream>>>(fl_dev, B * HW, n->cnt), cudaGetLastError()));
+    NCK(n, (nn::k_loss<<<nn::LOSS_BLOCKS, nn::EW, 0, n->stream>>>(n->out, tgt_dev, fl_dev, n->cnt, n->dout,
+                                                                  n->loss, B, (int)HW),
            cudaGetLastError()));
     // head: gradient of d0 (masked by d0 > 0) into lv[0].g1
     Level &v0 = n->lv[0];
@@ -1391,8 +1499,13 @@ lbm_status backward_side(lbm_unet *n, const float *tgt_dev, const float *fl_dev,
     unsigned hb = nn::blocks(B * HW);
     if (hb > 2u * n->sms) hb = 2u * n->sms;
     NCK(n, (nn::k_head_back<<<dim3(hb, v0.C / 8), nn::EW, 0, n->stream>>>(
-               n->dout, v0.d.p, v0.d.str, n->w + hd.w_off, v0.g1.p, n->g + hd.w_off, n->g + hd.b_off, B, g0, v0.C),
+               n->dout, v0.d.p, v0.d.str, n->w + hd.w_off, v0.g1.p, n->part[n->turn], B, g0, v0.C),
             cudaGetLastError()));
+    cudaStream_t st;
+    float *part;
+    NCK(n, next_side(n, &st, &part));
+    NCK(n, (nn::k_loss_sum<<<1, 32, 0, st>>>(n->loss), cudaGetLastError()));
+    NCK(n, sum_parts(part, (int)hb, 3 * v0.C, 4, n->g + hd.w_off, n->g + hd.b_off, st));
     // decoder: g1 of level l holds d(d_l) (masked)
     for (int l = 0; l < L - 1; l++) {
         Level &v = n->lv[l];
@@ -1550,9 +1663,11 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
         t.bwd = cv.bwd;
     }
     const size_t HW = (size_t)c.height * c.width;
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n->fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n->join, cudaEventDisableTiming);
+    for (int k = 0; k < 2 && e == cudaSuccess; k++) {
+        e = cudaStreamCreateWithFlags(&n->side[k], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n->join[k], cudaEventDisableTiming);
+    }
     if (e == cudaSuccess) e = palloc(n, &n->x, nn::Geo(c.height, c.width), 8);
     if (e == cudaSuccess) e = nalloc(n, &n->abi, (size_t)n->nabi);
     if (e == cudaSuccess) e = nalloc(n, &n->out, B * HW * 3);
@@ -1560,8 +1675,9 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
     if (e == cudaSuccess) e = nalloc(n, &n->io_in, B * HW * 8);
     if (e == cudaSuccess) e = nalloc(n, &n->io_tgt, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->io_fl, B * HW);
-    if (e == cudaSuccess) e = nalloc(n, &n->cnt, 1);
-    if (e == cudaSuccess) e = nalloc(n, &n->loss, 1);
+    for (int k = 0; k < 2 && e == cudaSuccess; k++) e = nalloc(n, &n->part[k], part_size(n));
+    if (e == cudaSuccess) e = nalloc(n, &n->cnt, nn::CNT_BLOCKS);
+    if (e == cudaSuccess) e = nalloc(n, &n->loss, 1 + nn::LOSS_BLOCKS);
     if (e == cudaSuccess) e = nalloc(n, &n->err_d, 1);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->err_d, 0, sizeof(int), n->stream);
     n->lv.resize(L);
@@ -1583,6 +1699,7 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
         if (e == cudaSuccess) e = palloc(n, &v.g2, v.geo, v.C);
         if (e == cudaSuccess && l > 0) e = palloc(n, &v.gin, v.geo, cprev);
     }
+    if (e == cudaSuccess) e = cudaMemsetAsync(n->g, 0, off * sizeof(float), n->stream);  // the padding
     if (e == cudaSuccess) e = cudaMemsetAsync(n->m, 0, off * sizeof(float), n->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(n->v, 0, off * sizeof(float), n->stream);
     if (e != cudaSuccess) {
