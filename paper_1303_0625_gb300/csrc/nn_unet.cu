@@ -67,8 +67,9 @@ struct Geo {
 };
 
 // 8-channel groups of the K axis of a convolution with G source groups: taps come in
-// pairs of groups (K = 16 an instruction), so an odd G gets one more group of zero
-// weights, unless one group is all (the input layer): there two taps share a pair.
+// pairs of groups (K = 16 an instruction), so an odd G gets one more group of zeros,
+// unless one group is all (the input layer): there two taps share a pair, the last with
+// zeros.  Zeros on both sides: an infinity times a zero weight is not a number.
 __host__ __device__ inline int k_groups(int G, bool pair_taps) {
     return pair_taps ? 10 : 9 * (G + (G & 1));
 }
@@ -294,6 +295,7 @@ __device__ __forceinline__ void drain_mmas(Pipe &pp) {
 // given; with up, stored to the 2 x 2 pixels of the next finer level.
 struct ConvOp {
     const bf16 *src;    // planes, sstr pixels each
+    const bf16 *zero;   // zeros, as many pixels as a copy takes: the group after an odd G
     const bf16 *w;      // packed, [N tile][KG][BN][8]
     const float *bias;  // [N] or null
     const bf16 *mask;   // planes as out, or null
@@ -335,8 +337,13 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
     const uint32_t gs = (bstays ? (uint32_t)(op.nseg * op.segpx) : SEG) * 16;    // K group stride
     const uint32_t unit = (bstays ? op.Ge : op.gb) * gs;
     const uint32_t a0 = smem_u32(smem), b0 = a0 + op.na * unit, stage = op.gb * BN * 16;
+    const uint32_t none = b0 + op.KG * BN * 16;  // the input layer: a tile of zeros
     const bf16 *w = op.w + (long long)nt * op.KG * BN * 8;
     if (tid < BN) bias[tid] = op.bias && nt * BN + tid < op.N ? op.bias[nt * BN + tid] : 0.f;
+    if (op.Ge == 1 && tid < TC_M) {
+        *reinterpret_cast<uint4 *>(smem + (none - a0) + tid * 16) = make_uint4(0, 0, 0, 0);
+        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
     pipe_init(pp, 1, NCOLS, warp, tid);
     const uint32_t tmem = pp.tmem;
     if (warp == 0) {
@@ -356,12 +363,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
                     for (int c = lane; c < op.Ge * op.nseg; c += 32) {
                         const int g = op.nseg == 3 ? c / 3 : c, row = op.nseg == 3 ? c - 3 * g - 1 : -1;
                         bulk_copy(to + c * op.segpx * 16,
-                                  op.src + ((g < op.G ? g : 0) * op.sstr + q0 + row * op.geo.Wp) * 8, op.segpx * 16, bar);
+                                  g < op.G ? op.src + (g * op.sstr + q0 + row * op.geo.Wp) * 8 : op.zero, op.segpx * 16, bar);
                     }
                 } else if (lane < op.gb) {
                     const int row = u / nblk - 1, g = u % nblk * op.gb + lane;
                     bulk_copy(to + lane * SEG * 16,
-                              op.src + ((g < op.G ? g : 0) * op.sstr + q0 + op.sign * row * op.geo.Wp) * 8, SEG * 16, bar);
+                              g < op.G ? op.src + (g * op.sstr + q0 + op.sign * row * op.geo.Wp) * 8 : op.zero, SEG * 16, bar);
                 }
                 ar.next(op.na);
                 fills++;
@@ -414,11 +421,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_conv_tc(const ConvOp op, long lo
                 const uint32_t abuf = a0 + ar.s * unit;
                 if (op.Ge == 1) {
                     // two taps each, the distance between them the stride of K groups; the
-                    // last one's partner (the next pixel) has zero weights
+                    // last one's partner is the tile of zeros
 #pragma unroll
                     for (int t = 0; t < 10; t += 2) {
-                        const uint32_t o0 = t / 3 * op.rowpx + t % 3, o1 = t < 8 ? (t + 1) / 3 * op.rowpx + (t + 1) % 3 : o0 + 1;
-                        if (leader) tc_mma(d, desc_lo(abuf, (o1 - o0) * 16) + o0, HI, blo, HI, idesc, t > 0);
+                        const uint32_t o0 = abuf + (t / 3 * op.rowpx + t % 3) * 16;
+                        const uint32_t o1 = t < 8 ? abuf + ((t + 1) / 3 * op.rowpx + (t + 1) % 3) * 16 : none;
+                        if (leader) tc_mma(d, desc_lo(o0, o1 - o0), HI, blo, HI, idesc, t > 0);
                         blo += 2 * BN;
                     }
                 } else {
@@ -1132,6 +1140,7 @@ struct lbm_unet {
     long long nparam = 0, nabi = 0;
     float *w = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;
     Planes x;                // packed input
+    bf16 *zero = nullptr;    // ConvOp::zero
     float *out = nullptr, *dout = nullptr;
     float *io_in = nullptr, *io_tgt = nullptr, *io_fl = nullptr;  // staging
     float *abi = nullptr;    // parameters or gradients in the caller's order
@@ -1190,8 +1199,6 @@ cudaError_t nalloc(lbm_unet *n, T **p, size_t count) {
     return e;
 }
 
-// C channels of planes for max_batch images, all zero, with room before and after
-// them that the convolutions' halos may read (zero as well)
 template <class... K, class... A>
 cudaError_t launch(lbm_unet *n, bool early, void (*kernel)(K...), dim3 grid, int threads, int smem, A... args) {
     cudaLaunchConfig_t cfg{};
@@ -1207,6 +1214,8 @@ cudaError_t launch(lbm_unet *n, bool early, void (*kernel)(K...), dim3 grid, int
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
 
+// C channels of planes for max_batch images, all zero, with room before and after
+// them that the convolutions' halos may read (zero as well)
 cudaError_t palloc(lbm_unet *n, Planes *q, const nn::Geo &geo, int C) {
     const size_t front = (size_t)(geo.Wp + 16) / 8 * 8 + 8, back = nn::TC_M + geo.Wp + 32;
     q->str = (long long)n->cfg.max_batch * geo.PSI;
@@ -1250,12 +1259,12 @@ cudaError_t launch_tc(lbm_unet *n, nn::ConvOp &op) {
         attr = true;
     }
     // A tile of A once for all taps: three row segments where a tile is shorter than a
-    // row, else the run of pixels from the row above to the row below (pairs of taps: a
-    // pixel more, for the partner of the last tap)
+    // row, else the run of pixels from the row above to the row below
     op.nseg = op.geo.Wp >= TC_M + 2 ? 3 : 1;
-    op.segpx = (op.nseg == 3 ? TC_M + 2 : TC_M + 2 * op.geo.Wp + 2) + (op.Ge == 1);
+    op.segpx = op.nseg == 3 ? TC_M + 2 : TC_M + 2 * op.geo.Wp + 2;
     op.rowpx = op.nseg == 3 ? op.segpx : op.geo.Wp;
-    const int a = op.Ge * op.nseg * op.segpx * 16, wall = op.KG * BN * 16;
+    const int a = op.Ge * op.nseg * op.segpx * 16;
+    const int wall = op.KG * BN * 16 + (op.Ge == 1 ? TC_M * 16 : 0);  // and the tile of zeros
     int smem = 0;
     if (2 * a + wall <= SMEM_MAX) {  // all weights beside two tiles or more, two CTAs if they fit
         op.stages = 0;
@@ -1295,6 +1304,7 @@ cudaError_t conv(lbm_unet *n, const bf16 *w, int Cs, int N, int sign, const floa
     nn::ConvOp op{};
     op.src = src.p;
     op.sstr = src.str;
+    op.zero = n->zero;
     op.w = w;
     op.bias = bias;
     op.mask = mask ? mask->p : nullptr;
@@ -1669,6 +1679,9 @@ lbm_status lbm_unet_create(const lbm_unet_config *cfg, lbm_unet **out) {
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&n->join[k], cudaEventDisableTiming);
     }
     if (e == cudaSuccess) e = palloc(n, &n->x, nn::Geo(c.height, c.width), 8);
+    const size_t zeros = (nn::TC_M + 2 * (c.width + 2) + 2) * 8;  // the longest copy of a convolution
+    if (e == cudaSuccess) e = nalloc(n, &n->zero, zeros);
+    if (e == cudaSuccess) e = cudaMemsetAsync(n->zero, 0, zeros * sizeof(bf16), n->stream);
     if (e == cudaSuccess) e = nalloc(n, &n->abi, (size_t)n->nabi);
     if (e == cudaSuccess) e = nalloc(n, &n->out, B * HW * 3);
     if (e == cudaSuccess) e = nalloc(n, &n->dout, B * HW * 3);
