@@ -34,16 +34,14 @@
 // chord in every row (FP32 bounds with a one-node margin) are dealt out to the
 // threads; every decision is taken by the exact test.
 //
-// Precision: per-link products and each lane's running sum over its links
-// (a handful) are in the arithmetic precision of the storage mode (FP32 in the
-// deviation modes), and so are the sums across the lanes of a warp (in a batch:
-// FP64); the sums across warps, the booked momenta and the motion are FP64, in a
-// fixed order.  (GB300 runs FP64 at about two fused multiply-adds per clock per
-// SM: FP64 lane sums would cost the force kernel about 100 us per step on 2000
-// disks.)
+// Precision: per-link products and a candidate's sum over its links (up to eight) are in
+// the arithmetic precision of the storage mode (FP32 in the deviation modes), and so is
+// the sum over the 32 candidates that a warp takes at once (in a batch: FP64); the sums
+// of these, the booked momenta and the motion are FP64, in a fixed order.
 #include "lbm_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 namespace gbm {
 
@@ -78,23 +76,32 @@ __device__ __forceinline__ void warp_sum(T (&v)[N]) {
         for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(FULL, v[k], o);
 }
 
-// The warp's sums of six FP64 values: component sum_of(lane) < 6 in each lane.  Halves of
-// the values go to the other lane of a pair at each step, so that a warp issues 9 FP64
-// additions (two lanes per clock and SM) instead of 30.
-__device__ __forceinline__ int sum_of(int lane) { return lane >> 2 & 4 | lane >> 2 & 2 | lane >> 2 & 1; }
-__device__ __forceinline__ double warp_sum6(const double (&v)[6], int lane) {
+// The warp's sums of the lanes' six values: component sum_of(lane) in each lane whose
+// sum_of is below 6.  Halves of the values go to the other lane of a pair at each step, so
+// that a warp issues 9 additions instead of 30, over the same tree (FP64: two lanes per
+// clock and SM).
+__device__ __forceinline__ int sum_of(int lane) { return lane & 3 ? 6 : lane >> 2; }
+template <class T>
+__device__ __forceinline__ T warp_sum6(const T (&v)[6], int lane) {
     const bool a = lane & 16, b = lane & 8, c = lane & 4;
-    double h[4], q[2];
+    T h[4], q[2];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        const double up = k < 2 ? v[4 + (k & 1)] : 0.0;
+        const T up = k < 2 ? v[4 + (k & 1)] : T(0);
         h[k] = (a ? up : v[k]) + __shfl_xor_sync(FULL, a ? v[k] : up, 16);
     }
 #pragma unroll
     for (int k = 0; k < 2; k++) q[k] = (b ? h[k + 2] : h[k]) + __shfl_xor_sync(FULL, b ? h[k] : h[k + 2], 8);
-    double s = (c ? q[1] : q[0]) + __shfl_xor_sync(FULL, c ? q[0] : q[1], 4);
+    T s = (c ? q[1] : q[0]) + __shfl_xor_sync(FULL, c ? q[0] : q[1], 4);
     s += __shfl_xor_sync(FULL, s, 2);
     return s + __shfl_xor_sync(FULL, s, 1);
+}
+// The same, WIDE: added in FP64, else in the type they come in.
+template <bool WIDE, class T>
+__device__ __forceinline__ double chunk_sum(const T (&v)[6], int lane) {
+    if constexpr (!WIDE) return (double)warp_sum6(v, lane);
+    const double w[6] = {(double)v[0], (double)v[1], (double)v[2], (double)v[3], (double)v[4], (double)v[5]};
+    return warp_sum6(w, lane);
 }
 
 // Set or clear one bit of a 16-bit flags word atomically.
@@ -413,42 +420,53 @@ __device__ void record_forces(const StepParams &p, int s, int lane, long long t,
 
 // ------------------------------------------------- fluid-solid links
 
-// A block of FB threads walks the links of one solid in two stages.  Candidates:
-// a node x_f can have a link into the disk when r - eps < |x_f - R| <= r +
-// sqrt 2 + eps, between the outer chord of each row and the inner one; thread t
-// reads the flags of candidate t, t + FB ... and lists its links (direction i
-// with x_f + e_i solid) in shared memory, in candidate order.  Links: every thread
-// takes links t, t + FB ... of that list, so that all lanes work: with a thread
-// per candidate, the lanes of a warp had one to five links each in different
-// directions, and the warp went through the link's arithmetic up to eight times
-// (which in FP64, two lanes per clock and SM, was most of the kernel's time).
+// A block of FB threads walks the links of one solid.  Candidates: a node x_f can have a
+// link into the disk when r - eps < |x_f - R| <= r + sqrt 2 + eps, between the outer chord
+// of each row and the inner one; thread t reads the flags of candidate t, t + FB ...
+// FP32 arithmetic, half-way: a candidate's thread takes its links itself (direction i with
+// x_f + e_i solid).  FP64, and with the interpolated boundary: it lists them in shared
+// memory, in candidate order, and every thread takes links t, t + FB ... of that list, so
+// that all lanes work: with a thread per candidate, the lanes of a warp have one to five
+// links each in different directions, and the warp goes through the link's arithmetic up
+// to eight times, which in FP64 (two lanes per clock and SM) was most of the kernel's
+// time.  In FP32 the list costs more than it saves (a step of 768 x 512 nodes with six
+// disks of r 51, FP16, the links before the fused kernel: 46.4 us with it, 43.5 without),
+// and with its 11 KB of shared memory a block, SMs beside FP16's fused kernel had to
+// change their split of L1 and shared memory, which they do only when empty.
 // A link reads its own population, its solid's owner only when the near list is
 // not empty, and with the interpolated boundary one population more.  Sums: a
-// link's six terms go through shared memory to its candidate's thread, which adds
-// them in the order of the directions; then over each warp's tree, both in the
-// arithmetic precision of the storage mode, then across the block's warps in
-// FP64, in warp order.  (A force is a small difference of large link terms, so
-// another order of the FP32 sums would change it in the fifth digit.)  FP64: a tree
-// for each 32 candidates, so that a warp's candidates may go to several blocks.
+// candidate's links in the order of the directions (the list's terms go through shared
+// memory to the candidate's thread); then over the tree of its warp's 32, both in the
+// arithmetic precision of the storage mode; then in FP64 over the turns of each of four
+// warps (one block of 128 threads) and over these four, in order, so that a solid's
+// candidates may go to several blocks.  (A force is a small difference of large link
+// terms, so another order of the FP32 sums would change it in the fifth digit.)
 constexpr int FB = 128;                  // threads per solid (batches: or twice as many)
 constexpr int LU = 2;                    // links a thread loads before it works on them
 constexpr float ANN_EPS = 0.05f;         // above the FP32 rounding of a chord end
 
-template <int P, int NT = FB> struct LinkShared {
+// Do candidates' own threads take their links (above)?
+template <int P, bool BND>
+__host__ __device__ constexpr bool direct() {
+    return P != LBM_FP64 && !BND;
+}
+
+template <int P, bool BND, int NT = FB> struct LinkShared {
     using C = typename Prec<P>::C;
+    static constexpr int LIST = direct<P, BND>() ? 0 : 1;
     int wsum[NT / 32];
-    int cnt[NT];                  // the chunk's rows: exclusive prefix of their candidates
+    int cnt[NT];                  // the turn's rows: exclusive prefix of their candidates
     int lo[NT], i0[NT], i1[NT];   // row: [lo, hi] minus the inner chord [i0, i1]
-    int4 cand[NT];                // candidate: {cell, x - floor X, y - floor Y, flags}
-    uint16_t link[8 * NT];        // direction | candidate << 4
-    C rho[NT];                    // local density of the candidates (rho_w local)
-    C term[6][LU * NT];           // the terms of the links in hand
-    double part[NT / 32][6];
+    double part[NT / 32][6];      // the warps' sums
+    int4 cand[LIST * NT + 1];     // candidate: {cell, x - floor X, y - floor Y, flags}
+    uint16_t link[LIST * 8 * NT + 1];  // direction | candidate << 4
+    C rho[LIST * NT + 1];         // local density of the candidates (rho_w local)
+    C term[6][LIST * LU * NT + 1];     // the terms of the links in hand
 };
 
 // Exclusive prefix of n over the block, and its total (whole blocks call it).
-template <int P, int NT>
-__device__ __forceinline__ int block_scan(int n, LinkShared<P, NT> &sh, int &total) {
+template <int P, bool BND, int NT>
+__device__ __forceinline__ int block_scan(int n, LinkShared<P, BND, NT> &sh, int &total) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     int inc = n;
 #pragma unroll
@@ -469,22 +487,37 @@ __device__ __forceinline__ int block_scan(int n, LinkShared<P, NT> &sh, int &tot
     return before + inc - n;
 }
 
-// The links of solid s: their sums into lacc (this thread's share; in FP64 its warp's, of
-// which lane l has component sum_of(l) in lacc[0]; Eq. 4 force and torque, then Eq. 5) and, with GHOST, the returned populations into the solid
-// nodes' slots of fs.  The solid's candidates are taken chunk by chunk of `chunk`
-// <= NT; this block takes the chunks part, part + nparts ...  With slots (FP64, chunks of
-// a warp) each chunk's sums are left there, six to a slot, with slots of zeros after the
-// chunks of each turn of rows up to a multiple of LINK_PARTS and to MAX_LINK_PARTS, and
-// their number in the last slot.
+// Terms of a link along e_i whose middle is (dx, dy) from R: Eq. 4 force and torque, then
+// Eq. 5, from f_i and the returned f_bb, at the solid's velocity (ux, uy) there.
+template <class C>
+__device__ __forceinline__ void link_terms(C ex, C ey, C dx, C dy, C ux, C uy, C fi, C fbb, C (&v)[6]) {
+    const C cmx = ex * fi + ex * fbb, cmy = ey * fi + ey * fbb;
+    const C gmx = (ex - ux) * fi - (-ex - ux) * fbb;
+    const C gmy = (ey - uy) * fi - (-ey - uy) * fbb;
+    v[0] = cmx;
+    v[1] = cmy;
+    v[2] = dx * cmy - dy * cmx;
+    v[3] = gmx;
+    v[4] = gmy;
+    v[5] = dx * gmy - dy * gmx;
+}
+
+// The links of solid s: their sums added to acc (its warp's: component sum_of(l) of the
+// Eq. 4 force and torque, then of Eq. 5, in lane l), and with GHOST the returned
+// populations into the solid nodes' slots of fs.
+// The solid's candidates are taken chunk by chunk of `chunk` <= NT; this block takes the chunks part, part + nparts ...  With
+// slots (chunks of a warp) each chunk's sums are left there instead, six to a slot, with
+// slots of zeros after the chunks of each turn of rows up to a multiple of LINK_PARTS and
+// to LEAD_SLOTS, and their number in the last slot.
 //   per link  f_i = f~_i(x_f), the returned f_bb = f_i - 6 w_i rho_w (e_i . v) with
 //   v the solid's velocity at x_s = x_f + e_i / 2 (BND: interpolated from the cut
 //   of the link, v and the lever there); Eq. 4 = e_i f_i - e_opp f_bb, Eq. 5 =
 //   (e_i - v) f_i - (e_opp - v) f_bb, torque (x_s - R) x F (Eq. 7).
-template <int P, bool LOCAL, bool BND, bool GHOST, int NT>
+template <int P, bool LOCAL, bool BND, bool GHOST, bool WIDE, int NT>
 __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b, int s,
                                             typename Prec<P>::S *fs, bool owners, bool list,
                                             long long t, int chunk, int part, int nparts,
-                                            LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
+                                            LinkShared<P, BND, NT> &sh, double &acc,
                                             double *slots = nullptr) {
     using C = typename Prec<P>::C;
     using S = typename Prec<P>::S;
@@ -498,11 +531,11 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
     const C rho0 = pick<C>(p.rho0, p.rho0_f);
     int j0, j1, nslot = 0;
     rows_of_i(b.iy0, b.iy0, b.rc, 3, j0, j1);
-    for (int jc = j0; jc <= j1; jc += NT) {  // rows in chunks of NT
+    for (int jc = j0; jc <= j1; jc += FB) {  // rows in turns of FB
         // candidates of row jc + tid
         int lo = 1, hi = 0, i0 = 1, i1 = 0, n = 0;
         const int j = jc + tid;
-        if (j <= j1 && c.chord(j, r + 1.4143f + ANN_EPS, lo, hi) && lo <= hi) {
+        if (tid < FB && j <= j1 && c.chord(j, r + 1.4143f + ANN_EPS, lo, hi) && lo <= hi) {
             n = hi - lo + 1;
             if (c.chord(j, r - ANN_EPS, i0, i1) && i0 <= i1) n -= i1 - i0 + 1;
         }
@@ -544,175 +577,194 @@ __device__ __forceinline__ void solid_links(const StepParams &p, const DSolid &b
             }
             // bit i: x_f + e_i is solid or beyond a wall (bit opp(i) of the flags)
             unsigned dirs = bounced_node ? ((m & 0x66u) << 2 | (m >> 2 & 0x66u)) : 0u;
-            int nlink;
-            const int mine0 = block_scan(__popc(dirs), sh, nlink), mine1 = mine0 + __popc(dirs);
-            if (LOCAL) {
-                C a9 = 0;
-                if (dirs) {
-                    S fv[9];
+            C sum[6] = {0, 0, 0, 0, 0, 0};  // of this candidate's links
+            const bool any = dirs != 0;
+            if constexpr (direct<P, BND>()) {
+                S fv[9];
+                int kb[9];
+                uint16_t own[9];
 #pragma unroll
-                    for (int q9 = 0; q9 < 9; q9++) fv[q9] = fs[q9 * plane + k];
-#pragma unroll
-                    for (int q9 = 0; q9 < 9; q9++) a9 += (C)cvt_s(fv[q9]);
-                }
-                sh.rho[tid] = Prec<P>::dev ? (C)1 + a9 : a9;
-            }
-            sh.cand[tid] = make_int4(k, iu - c.xi, jj - c.yi, (int)m);
-            C sum[6] = {0, 0, 0, 0, 0, 0};  // FP64: of this candidate's links
-            for (int at = mine0; dirs; dirs &= dirs - 1)
-                sh.link[at++] = (uint16_t)((__ffs(dirs) - 1) | tid << 4);
-            __syncthreads();
-            for (int l0 = 0; l0 < nlink; l0 += LU * NT) {
-                int4 cd[LU];
-                int kb[LU], dir[LU];
-                S fi_s[LU], fo_s[LU], fn_s[LU];
-                C rho_w[LU];
-                uint16_t own[LU];
-                bool inner[LU];  // BND: x_f - e_i is a fluid node of the domain
-#pragma unroll
-                for (int u = 0; u < LU; u++) {
-                    kb[u] = -1;
-                    const int l = l0 + u * NT + tid;
-                    if (l >= nlink) continue;
-                    const int lk = sh.link[l], i = lk & 15;
-                    const int4 cc = cd[u] = sh.cand[lk >> 4];
-                    dir[u] = i;
-                    rho_w[u] = LOCAL ? sh.rho[lk >> 4] : rho0;
+                for (int i = 1; i < 9; i++) {
+                    kb[i] = -1;
                     int xb, yb;
-                    if (!wrap(c.xi + cc.y + cx(i), c.yi + cc.z + cy(i), xb, yb)) continue;
-                    kb[u] = (int)cell_of(L, xb, yb);  // else beyond a wall
-                    fi_s[u] = fs[i * plane + cc.x];
-                    if (owners) own[u] = p.owner[kb[u]];
-                    if (BND) {
-                        inner[u] = !((cc.w >> i) & 1);
-                        fo_s[u] = fs[opp(i) * plane + cc.x];
-                        fn_s[u] = fi_s[u];
-                        int xn, yn;
-                        if (inner[u] && wrap(c.xi + cc.y - cx(i), c.yi + cc.z - cy(i), xn, yn))
-                            fn_s[u] = fs[i * plane + (int)cell_of(L, xn, yn)];
-                    }
+                    if (!(dirs >> i & 1u) || !wrap(iu + cx(i), jj + cy(i), xb, yb)) continue;
+                    kb[i] = (int)cell_of(L, xb, yb);  // else beyond a wall
+                    fv[i] = fs[i * plane + k];
+                    if (owners) own[i] = p.owner[kb[i]];
                 }
+                C rho_w = rho0;
+                if (LOCAL && any) {
+                    C a9 = 0;
 #pragma unroll
-                for (int u = 0; u < LU; u++) {
-                    C v[6] = {0, 0, 0, 0, 0, 0};
-                    if (kb[u] >= 0 && !(owners && own[u] != (uint16_t)s)) {
-                        const int i = dir[u], di = cd[u].y, dj = cd[u].z;
-                        const C ex = (C)cx(i), ey = (C)cy(i), w = wgt<C>(i);
-                        const C back = (C)cvt_s(fi_s[u]);  // as stored
-                        const C fi = Prec<P>::dev ? back + w : back;
-                        C dx, dy, ux, uy, fbb, ret = 0;  // ret: f_bb as stored
-                        if (BND) {
-                            C q;  // the link is cut at this fraction
-                            if (Prec<P>::dev) {
-                                q = (C)link_fraction_split(di, dj, c.fx, c.fy, b.r, cx(i), cy(i));
-                                dx = ((C)di - (C)c.fx) + q * ex;
-                                dy = ((C)dj - (C)c.fy) + q * ey;
-                            } else {
-                                // the unwrapped node is at the centre's nearest image
-                                const double px = (double)(c.xi + di) - b.x;
-                                const double py = (double)(c.yi + dj) - b.y;
-                                q = (C)link_fraction_at(px, py, b.r, cx(i), cy(i));
-                                dx = (C)px + q * ex;
-                                dy = (C)py + q * ey;
-                            }
-                            ux = vx - om * dy;
-                            uy = vy + om * dx;
-                            const C mw = -(C)6 * w * rho_w[u] * (ex * ux + ey * uy);
-                            const C q2 = (C)2 * q;
-                            const C fo = (C)cvt_s(fo_s[u]), fn = (C)cvt_s(fn_s[u]);
-                            auto returned = [&](C f, C o, C nb) {
-                                if (q2 >= (C)1) return (f + mw) / q2 + ((q2 - (C)1) / q2) * o;
-                                if (inner[u]) return q2 * f + ((C)1 - q2) * nb + mw;
-                                return f + mw;
-                            };
-                            // full populations for the force; as stored for the pull
-                            // (the interpolation's weights sum to one)
-                            if (Prec<P>::dev) fbb = returned(fi, fo + w, fn + w);
-                            if (GHOST || !Prec<P>::dev) ret = returned(back, fo, fn);
-                            if (!Prec<P>::dev) fbb = ret;
-                        } else {
-                            // x_s = x_f + e_i / 2 relative to R, from the unwrapped coordinate
-                            if (Prec<P>::dev) {
-                                dx = (C)di + (C)0.5 * ex - (C)c.fx;
-                                dy = (C)dj + (C)0.5 * ey - (C)c.fy;
-                            } else {
-                                dx = (C)(((double)(c.xi + di) + 0.5 * (double)ex) - b.x);
-                                dy = (C)(((double)(c.yi + dj) + 0.5 * (double)ey) - b.y);
-                            }
-                            ux = vx - om * dy;
-                            uy = vy + om * dx;
-                            const C a6 = (C)6 * w * rho_w[u], eu = ex * ux + ey * uy;
-                            fbb = fma(-a6, eu, fi);
-                            ret = fma(-a6, eu, back);
-                        }
-                        if (GHOST) st(fs + opp(i) * plane + kb[u], ret);
-                        const C cmx = ex * fi + ex * fbb, cmy = ey * fi + ey * fbb;
-                        const C gmx = (ex - ux) * fi - (-ex - ux) * fbb;
-                        const C gmy = (ey - uy) * fi - (-ey - uy) * fbb;
-                        v[0] = cmx;
-                        v[1] = cmy;
-                        v[2] = dx * cmy - dy * cmx;
-                        v[3] = gmx;
-                        v[4] = gmy;
-                        v[5] = dx * gmy - dy * gmx;
-                    }
-#pragma unroll
-                    for (int q6 = 0; q6 < 6; q6++) sh.term[q6][u * NT + tid] = v[q6];
+                    for (int q9 = 0; q9 < 9; q9++) a9 += (C)cvt_s(fs[q9 * plane + k]);
+                    rho_w = (C)1 + a9;
                 }
+                const C px = (C)(iu - c.xi), py = (C)(jj - c.yi);
+#pragma unroll
+                for (int i = 1; i < 9; i++) {
+                    if (kb[i] < 0 || (owners && own[i] != (uint16_t)s)) continue;
+                    const C ex = (C)cx(i), ey = (C)cy(i), w = wgt<C>(i);
+                    const C back = (C)cvt_s(fv[i]), fi = back + w;
+                    const C dx = px + (C)0.5 * ex - (C)c.fx, dy = py + (C)0.5 * ey - (C)c.fy;
+                    const C ux = vx - om * dy, uy = vy + om * dx;
+                    const C a6 = (C)6 * w * rho_w, eu = ex * ux + ey * uy;
+                    C v[6];
+                    if (GHOST) st(fs + opp(i) * plane + kb[i], fma(-a6, eu, back));
+                    link_terms(ex, ey, dx, dy, ux, uy, fi, fma(-a6, eu, fi), v);
+#pragma unroll
+                    for (int q6 = 0; q6 < 6; q6++) sum[q6] += v[q6];
+                }
+            } else {
+                int nlink;
+                const int mine0 = block_scan(__popc(dirs), sh, nlink), mine1 = mine0 + __popc(dirs);
+                if (LOCAL) {
+                    C a9 = 0;
+                    if (dirs) {
+                        S fv[9];
+#pragma unroll
+                        for (int q9 = 0; q9 < 9; q9++) fv[q9] = fs[q9 * plane + k];
+#pragma unroll
+                        for (int q9 = 0; q9 < 9; q9++) a9 += (C)cvt_s(fv[q9]);
+                    }
+                    sh.rho[tid] = Prec<P>::dev ? (C)1 + a9 : a9;
+                }
+                sh.cand[tid] = make_int4(k, iu - c.xi, jj - c.yi, (int)m);
+                for (int at = mine0; dirs; dirs &= dirs - 1)
+                    sh.link[at++] = (uint16_t)((__ffs(dirs) - 1) | tid << 4);
                 __syncthreads();
-                // the candidate's thread adds its links' terms
-                for (int l = max(mine0, l0); l < min(mine1, l0 + LU * NT); l++)
+                for (int l0 = 0; l0 < nlink; l0 += LU * NT) {
+                    int4 cd[LU];
+                    int kb[LU], dir[LU];
+                    S fi_s[LU], fo_s[LU], fn_s[LU];
+                    C rho_w[LU];
+                    uint16_t own[LU];
+                    bool inner[LU];  // BND: x_f - e_i is a fluid node of the domain
 #pragma unroll
-                    for (int q6 = 0; q6 < 6; q6++) (P == LBM_FP64 ? sum : lacc)[q6] += sh.term[q6][l - l0];
-                __syncthreads();  // the terms (and the list) are reused
-            }
-            if constexpr (P == LBM_FP64)
-                if ((tid & ~31) < chunk && base + (tid & ~31) < total) {
-                    const double v = warp_sum6(sum, lane);
-                    lacc[0] += v;
-                    if (slots && !(lane & 3) && sum_of(lane) < 6) slots[(nslot + base / 32) * 6 + sum_of(lane)] = v;
+                    for (int u = 0; u < LU; u++) {
+                        kb[u] = -1;
+                        const int l = l0 + u * NT + tid;
+                        if (l >= nlink) continue;
+                        const int lk = sh.link[l], i = lk & 15;
+                        const int4 cc = cd[u] = sh.cand[lk >> 4];
+                        dir[u] = i;
+                        rho_w[u] = LOCAL ? sh.rho[lk >> 4] : rho0;
+                        int xb, yb;
+                        if (!wrap(c.xi + cc.y + cx(i), c.yi + cc.z + cy(i), xb, yb)) continue;
+                        kb[u] = (int)cell_of(L, xb, yb);  // else beyond a wall
+                        fi_s[u] = fs[i * plane + cc.x];
+                        if (owners) own[u] = p.owner[kb[u]];
+                        if (BND) {
+                            inner[u] = !((cc.w >> i) & 1);
+                            fo_s[u] = fs[opp(i) * plane + cc.x];
+                            fn_s[u] = fi_s[u];
+                            int xn, yn;
+                            if (inner[u] && wrap(c.xi + cc.y - cx(i), c.yi + cc.z - cy(i), xn, yn))
+                                fn_s[u] = fs[i * plane + (int)cell_of(L, xn, yn)];
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < LU; u++) {
+                        C v[6] = {0, 0, 0, 0, 0, 0};
+                        if (kb[u] >= 0 && !(owners && own[u] != (uint16_t)s)) {
+                            const int i = dir[u], di = cd[u].y, dj = cd[u].z;
+                            const C ex = (C)cx(i), ey = (C)cy(i), w = wgt<C>(i);
+                            const C back = (C)cvt_s(fi_s[u]);  // as stored
+                            const C fi = Prec<P>::dev ? back + w : back;
+                            C dx, dy, ux, uy, fbb, ret = 0;  // ret: f_bb as stored
+                            if (BND) {
+                                C q;  // the link is cut at this fraction
+                                if (Prec<P>::dev) {
+                                    q = (C)link_fraction_split(di, dj, c.fx, c.fy, b.r, cx(i), cy(i));
+                                    dx = ((C)di - (C)c.fx) + q * ex;
+                                    dy = ((C)dj - (C)c.fy) + q * ey;
+                                } else {
+                                    // the unwrapped node is at the centre's nearest image
+                                    const double px = (double)(c.xi + di) - b.x;
+                                    const double py = (double)(c.yi + dj) - b.y;
+                                    q = (C)link_fraction_at(px, py, b.r, cx(i), cy(i));
+                                    dx = (C)px + q * ex;
+                                    dy = (C)py + q * ey;
+                                }
+                                ux = vx - om * dy;
+                                uy = vy + om * dx;
+                                const C mw = -(C)6 * w * rho_w[u] * (ex * ux + ey * uy);
+                                const C q2 = (C)2 * q;
+                                const C fo = (C)cvt_s(fo_s[u]), fn = (C)cvt_s(fn_s[u]);
+                                auto returned = [&](C f, C o, C nb) {
+                                    if (q2 >= (C)1) return (f + mw) / q2 + ((q2 - (C)1) / q2) * o;
+                                    if (inner[u]) return q2 * f + ((C)1 - q2) * nb + mw;
+                                    return f + mw;
+                                };
+                                // full populations for the force; as stored for the pull
+                                // (the interpolation's weights sum to one)
+                                if (Prec<P>::dev) fbb = returned(fi, fo + w, fn + w);
+                                if (GHOST || !Prec<P>::dev) ret = returned(back, fo, fn);
+                                if (!Prec<P>::dev) fbb = ret;
+                            } else {
+                                // x_s = x_f + e_i / 2 relative to R, from the unwrapped coordinate
+                                if (Prec<P>::dev) {
+                                    dx = (C)di + (C)0.5 * ex - (C)c.fx;
+                                    dy = (C)dj + (C)0.5 * ey - (C)c.fy;
+                                } else {
+                                    dx = (C)(((double)(c.xi + di) + 0.5 * (double)ex) - b.x);
+                                    dy = (C)(((double)(c.yi + dj) + 0.5 * (double)ey) - b.y);
+                                }
+                                ux = vx - om * dy;
+                                uy = vy + om * dx;
+                                const C a6 = (C)6 * w * rho_w[u], eu = ex * ux + ey * uy;
+                                fbb = fma(-a6, eu, fi);
+                                ret = fma(-a6, eu, back);
+                            }
+                            if (GHOST) st(fs + opp(i) * plane + kb[u], ret);
+                            link_terms(ex, ey, dx, dy, ux, uy, fi, fbb, v);
+                        }
+#pragma unroll
+                        for (int q6 = 0; q6 < 6; q6++) sh.term[q6][u * NT + tid] = v[q6];
+                    }
+                    __syncthreads();
+                    // the candidate's thread adds its links' terms
+                    for (int l = max(mine0, l0); l < min(mine1, l0 + LU * NT); l++)
+#pragma unroll
+                        for (int q6 = 0; q6 < 6; q6++) sum[q6] += sh.term[q6][l - l0];
+                    __syncthreads();  // the terms (and the list) are reused
                 }
+            }
+            const int e32 = base + (tid & ~31);  // this warp's first candidate
+            if ((tid & ~31) < chunk && e32 < total) {
+                double v = 0.0;
+                if (__any_sync(FULL, any)) v = chunk_sum<WIDE>(sum, lane);
+                if (!slots) acc += v;
+                else if (sum_of(lane) < 6 && nslot + e32 / 32 < p.link_slots - 1)
+                    slots[(nslot + e32 / 32) * 6 + sum_of(lane)] = v;
+            }
         }
-        if (P == LBM_FP64 && slots) {
+        if (slots) {
             int k = (total + 31) / 32;
-            for (; k % LINK_PARTS || nslot + k < MAX_LINK_PARTS; k++)
-                if (k % nparts == part && tid < 6) slots[(nslot + k) * 6 + tid] = 0.0;
+            for (; k % LINK_PARTS || nslot + k < LEAD_SLOTS; k++)
+                if (k % nparts == part && tid < 6 && nslot + k < p.link_slots - 1) slots[(nslot + k) * 6 + tid] = 0.0;
             nslot += k;
-            if (part == 0 && tid == 0) slots[(LINK_SLOTS - 1) * 6] = (double)nslot;
+            if (part == 0 && tid == 0) slots[(p.link_slots - 1) * 6] = (double)nslot;
         }
     }
 }
 
-// Sums over the block of every thread's lacc, over each warp's lanes (WIDE: in FP64; FP64:
-// solid_links has done that) and then over the warps in FP64, in order, to all lanes of
-// warp 0.
-template <int P, int NT, bool WIDE = false>
-__device__ __forceinline__ void block_sums(LinkShared<P, NT> &sh, typename Prec<P>::C (&lacc)[6],
-                                           double (&acc)[6]) {
+// Sums over the block's warps (whose sums solid_links has left in w), in order, to all
+// lanes of warp 0: warps LINK_PARTS apart first, as one that takes their chunks in turn.
+template <int P, bool BND, int NT>
+__device__ __forceinline__ void block_sums(LinkShared<P, BND, NT> &sh, double w, double (&acc)[6]) {
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    if constexpr (P == LBM_FP64) {
-        if (!(lane & 3) && sum_of(lane) < 6) sh.part[wib][sum_of(lane)] = lacc[0];
-    } else if constexpr (WIDE) {
-        double v[6], t = 0.0;
-        bool any = false;  // half of a batch's warps have no link
-#pragma unroll
-        for (int q = 0; q < 6; q++) any |= lacc[q] != 0;
-        if (__any_sync(FULL, any)) {
-#pragma unroll
-            for (int q = 0; q < 6; q++) v[q] = (double)lacc[q];
-            t = warp_sum6(v, lane);
-        }
-        if (!(lane & 3) && sum_of(lane) < 6) sh.part[wib][sum_of(lane)] = t;
-    } else {
-        warp_sum(lacc);
-        if (lane == 0)
-            for (int q = 0; q < 6; q++) sh.part[wib][q] = (double)lacc[q];
-    }
+    if (sum_of(lane) < 6) sh.part[wib][sum_of(lane)] = w;
     __syncthreads();
     if (wib != 0) return;
     double aq = 0.0;
     if (lane < 6)
-        for (int w = 0; w < NT / 32; w++) aq += sh.part[w][lane];
+#pragma unroll
+        for (int c = 0; c < LINK_PARTS; c++) {
+            double a = sh.part[c][lane];
+#pragma unroll
+            for (int k = c + LINK_PARTS; k < NT / 32; k += LINK_PARTS) a += sh.part[k][lane];
+            aq += a;
+        }
 #pragma unroll
     for (int q = 0; q < 6; q++) acc[q] = __shfl_sync(FULL, aq, q);
 }
@@ -746,6 +798,14 @@ __device__ __forceinline__ float displacement(const DSolid &b) {
     return fmaxf(d0, d1) + 1e-3f;
 }
 
+// FP64 sums over a warp's lanes: in FP64, and in batches.  (In FP32 they would cost the
+// force kernel of 2000 disks tens of microseconds: GB300 issues FP64 for about two lanes
+// per clock and SM.)
+template <int P>
+__host__ __device__ constexpr bool wide() {
+    return P == LBM_FP64;
+}
+
 // FP16 rounds a returned population: it stays in registers there (sc_tile).
 template <int P>
 __host__ __device__ constexpr bool ghosts() {
@@ -760,11 +820,11 @@ __device__ __forceinline__ bool need_owners(const StepParams &p, const DSolid &b
 }
 
 // The half-way boundary: links, record and motion of one solid per block.
-template <int P, bool LOCAL>
-__global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
+template <int P, bool LOCAL, int NT>
+__global__ void __launch_bounds__(NT, 896 / NT) k_forces(const StepParams p) {
     early_start();
     using S = typename Prec<P>::S;
-    __shared__ LinkShared<P> sh;
+    __shared__ LinkShared<P, false, NT> sh;
     const int tid = threadIdx.x, lane = tid & 31;
     const long long t = *p.t;
     S *fs = static_cast<S *>((t & 1) ? p.f1 : p.f0);  // populations of time t
@@ -781,11 +841,10 @@ __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
             if (tid == 0) atomicOr(p.status, 2);
             continue;
         }
-        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
-        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
-                                                 FB, 0, 1, sh, lacc);
-        double acc[6];
-        block_sums(sh, lacc, acc);
+        double sum = 0.0, acc[6];
+        solid_links<P, LOCAL, false, ghosts<P>(), wide<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
+                                                             NT, 0, 1, sh, sum);
+        block_sums(sh, sum, acc);
         if (tid < 32) {
             double booked[6];
             booked_events(p, b, t, lane, booked);
@@ -799,62 +858,53 @@ __global__ void __launch_bounds__(FB, 8) k_forces(const StepParams p) {
 }
 
 // The same in two kernels: k_links, after which the advection-collision kernel can
-// run, and k_record (records and motion), beside it.  A solid's links go to
+// run, and k_record (records and motion), beside it, or after it as the step's last.  A solid's links go to
 // gridDim.y blocks: one, or several that take its candidates 32 at a time in turn:
-// LINK_PARTS, each the share of one warp of the single block, or in FP64
-// MAX_LINK_PARTS, each what a warp takes in one turn: they leave every turn's sums to
-// k_record.  The sums are the same bit for bit, whichever way.  (With the interpolated boundary one 30-node disk in FP64 took
+// LINK_PARTS, each the share of one warp of the single block, or more, which leave every
+// turn's sums to k_record.  The sums are the same bit for bit, whichever way.  (With the interpolated boundary one 30-node disk in FP64 took
 // 68 us in one block with a thread per candidate: one SM's FP64 unit.)
 constexpr int LINK_CHUNK = FB / LINK_PARTS;
 
-template <int P, bool LOCAL, bool BND>
-__global__ void __launch_bounds__(FB) k_links(const StepParams p) {
+// BLOCKS: registers for so many blocks on an SM, at the cost of a few bytes of spills.
+template <int P, bool LOCAL, bool BND, int BLOCKS>
+__global__ void __launch_bounds__(FB, BLOCKS) k_links(const StepParams p) {
     early_start();
     using S = typename Prec<P>::S;
-    __shared__ LinkShared<P> sh;
+    __shared__ LinkShared<P, BND> sh;
     const long long t = *p.t;
     S *fs = static_cast<S *>((t & 1) ? p.f1 : p.f0);
     for (int s = blockIdx.x; s < p.nsolid; s += gridDim.x) {
         const DSolid &b = p.S[s];
         if (!solid_ok(b)) continue;  // k_record reports it
-        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
-        double *slots = P == LBM_FP64 && gridDim.y > LINK_PARTS ? p.part + (long long)s * LINK_SLOTS * 6 : nullptr;
-        solid_links<P, LOCAL, BND, ghosts<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
-                                                gridDim.y > 1 ? LINK_CHUNK : FB, blockIdx.y,
-                                                gridDim.y, sh, lacc, slots);
+        double *slots = p.link_slots ? p.part + (long long)s * p.link_slots * 6 : nullptr;
+        double sum = 0.0, acc[6];
+        solid_links<P, LOCAL, BND, ghosts<P>(), wide<P>()>(p, b, s, fs, need_owners(p, b), p.list_by_forces, t,
+                                                           gridDim.y > 1 ? LINK_CHUNK : FB, blockIdx.y, gridDim.y,
+                                                           sh, sum, slots);
         if (slots) continue;
-        double acc[6];
-        block_sums(sh, lacc, acc);
+        block_sums(sh, sum, acc);
         if (threadIdx.x == 0)
             for (int q = 0; q < 6; q++) p.part[((long long)s * LINK_PARTS + blockIdx.y) * 6 + q] = acc[q];
-        __syncthreads();
+        __syncthreads();  // sh.part is reused
     }
 }
 
-__global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
-    early_start();
-    const int lane = threadIdx.x & 31;
-    const long long t = *p.t;
-    if (blockIdx.x == 0 && threadIdx.x == 0 && p.ev_len) {
-        *p.ev_len = 0;
-        *p.chg_len = 0;
-    }
-    const int s = blockIdx.x * WARPS + (threadIdx.x >> 5);
-    if (s >= p.nsolid) return;
+// Record and motion of solid s, by one warp.
+__device__ __forceinline__ void record_solid(const StepParams &p, int s, int lane, long long t) {
     DSolid &b = p.S[s];
     if (!solid_ok(b)) {
         if (lane == 0) atomicOr(p.status, 2);
         return;
     }
     double aq = 0.0, acc[6], booked[6];
-    if (p.link_parts > LINK_PARTS) {  // as the warps of one block have added them
-        const double *part = p.part + (long long)s * LINK_SLOTS * 6 + lane;
+    if (p.link_slots) {  // as the warps of one block would have added them
+        const double *part = p.part + (long long)s * p.link_slots * 6 + lane;
         if (lane < 6) {
             double a[LINK_PARTS] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-            for (int c = 0; c < MAX_LINK_PARTS; c++) a[c % LINK_PARTS] += part[c * 6];
-            const int n = (int)part[(LINK_SLOTS - 1) * 6 - lane];
-            for (int c = MAX_LINK_PARTS; c < n; c += LINK_PARTS)
+            for (int c = 0; c < LEAD_SLOTS; c++) a[c % LINK_PARTS] += part[c * 6];
+            const int n = min((int)part[(p.link_slots - 1) * 6 - lane], p.link_slots - LINK_PARTS);
+            for (int c = LEAD_SLOTS; c < n; c += LINK_PARTS)
 #pragma unroll
                 for (int w = 0; w < LINK_PARTS; w++) a[w] += part[(c + w) * 6];
             aq = ((a[0] + a[1]) + a[2]) + a[3];
@@ -867,6 +917,19 @@ __global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
     booked_events(p, b, t, lane, booked);
     record_forces(p, s, lane, t, acc, booked);
     if (lane == 0) atomicMax(p.bar + 2, __float_as_uint(displacement(b)));
+}
+
+__global__ void __launch_bounds__(SW_BLOCK) k_record(const StepParams p) {
+    early_start();
+    const int lane = threadIdx.x & 31;
+    const long long t = *p.t;
+    if (blockIdx.x == 0 && threadIdx.x == 0 && p.ev_len) {
+        *p.ev_len = 0;
+        *p.chg_len = 0;
+    }
+    const int s = blockIdx.x * WARPS + (threadIdx.x >> 5);
+    if (s < p.nsolid) record_solid(p, s, lane, t);
+    if (p.record_last) end_of_step(p, t, gridDim.x);
 }
 
 // ----------------------------------------------------- re-rasterisation
@@ -1393,26 +1456,45 @@ __global__ void __launch_bounds__(SW_BLOCK, 4) k_remask_few(const StepParams p) 
     events<P>(p, t);
 }
 
-template <int P, bool LOCAL>
-cudaError_t launch_f(const StepParams &p, cudaStream_t st) {
-    static int per_sm = -1, sms = 0;
-    if (per_sm < 0) {
+cudaError_t sm_count(int &sms) {
+    static std::atomic<int> known{0};
+    cudaError_t e = cudaSuccess;
+    if (!(sms = known.load())) {
         int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
+        e = cudaGetDevice(&dev);
         if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forces<P, LOCAL>, FB, 0);
+        if (e == cudaSuccess) known = sms;
+    }
+    return e;
+}
+
+template <int P, bool LOCAL, int NT>
+cudaError_t launch_f_n(const StepParams &p, cudaStream_t st, int sms) {
+    static int per_sm = -1;
+    if (per_sm < 0) {
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_forces<P, LOCAL, NT>, NT, 0);
         if (e != cudaSuccess) return e;
     }
-    int blocks = p.nsolid;  // one solid per block, looped beyond the resident blocks
-    if (blocks > 8 * per_sm * sms) blocks = 8 * per_sm * sms;
-    if (blocks < 1) blocks = 1;
-    if (!p.link_parts) {
-        return launch_step(p, k_forces<P, LOCAL>, dim3(blocks), FB, st, p);
-    }
-    const dim3 grid(blocks, p.link_parts);
-    return p.boundary == LBM_INTERPOLATED ? launch_step(p, k_links<P, LOCAL, true>, grid, FB, st, p)
-                                          : launch_step(p, k_links<P, LOCAL, false>, grid, FB, st, p);
+    // one solid per block, looped beyond the resident blocks
+    return launch_step(p, k_forces<P, LOCAL, NT>, dim3(std::min(p.nsolid, 8 * per_sm * sms)), NT, st, p);
+}
+
+// k_links with the interpolated boundary: 96 registers in FP32, five blocks on an SM; seven
+// with 72 are 1.5 us slower at 500 disks of r 20 (115 us a step), but take 1000 in one
+// wave instead of two (228 -> 216).
+template <int P, bool LOCAL>
+cudaError_t launch_f(const StepParams &p, cudaStream_t st) {
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
+    if (!p.link_parts)
+        return launch_f_n<P, LOCAL, FB>(p, st, sms);
+    const dim3 grid(std::min(p.nsolid, 64 * sms), p.link_parts);
+    constexpr bool fp64 = P == LBM_FP64;
+    if (p.boundary != LBM_INTERPOLATED) return launch_step(p, k_links<P, LOCAL, false, fp64 ? 5 : 7>, grid, FB, st, p);
+    if (!fp64 && p.nsolid * p.link_parts > 5 * sms)
+        return launch_step(p, k_links<P, LOCAL, true, fp64 ? 4 : 7>, grid, FB, st, p);
+    return launch_step(p, k_links<P, LOCAL, true, fp64 ? 4 : 5>, grid, FB, st, p);
 }
 
 // Re-rasterisation of up to FEW_MOVING solids: one cluster of 8 blocks (one solid: 4)
@@ -1477,14 +1559,15 @@ cudaError_t launch_r(const StepParams &p, bool ring, cudaStream_t st) {
 // buffers, after every block has read them.  Batch convention: between steps f0
 // holds the current populations; the fused kernel, which comes after this swap,
 // reads f1 and writes f0.
-template <int P, bool LOCAL, int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT)
+// BLOCKS: on an SM.
+template <int P, bool LOCAL, int NT, int BLOCKS>
+__global__ void __launch_bounds__(NT, BLOCKS)
     k_solids_batch(StepParams *cases, const int2 *__restrict__ items,
                    const int *__restrict__ nitems, const int *__restrict__ active,
                    const int *__restrict__ nactive, unsigned int *ticket) {
     using S = typename Prec<P>::S;
     __shared__ bool last;
-    __shared__ LinkShared<P, NT> sh;
+    __shared__ LinkShared<P, false, NT> sh;
     const int n = *nitems;
     for (int k = blockIdx.x; k < n; k += gridDim.x) {
         const int2 it = items[k];
@@ -1495,11 +1578,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
             if (threadIdx.x == 0) atomicOr(p.status, 2);
             continue;
         }
-        typename Prec<P>::C lacc[6] = {0, 0, 0, 0, 0, 0};
-        solid_links<P, LOCAL, false, ghosts<P>()>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, NT,
-                                                 0, 1, sh, lacc);
-        double acc[6];
-        block_sums<P, NT, true>(sh, lacc, acc);  // the drags decide when a case has converged
+        // FP64 sums throughout: the drags decide when a case has converged
+        double sum = 0.0, acc[6];
+        solid_links<P, LOCAL, false, ghosts<P>(), true>(p, b, it.y, static_cast<S *>(p.f0), true, false, t, NT, 0,
+                                                        1, sh, sum);
+        block_sums(sh, sum, acc);
         if (threadIdx.x < 32) {
             const double none[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // resting: no node changes type
             record_forces(p, it.y, threadIdx.x, t, acc, none);
@@ -1525,24 +1608,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     if (threadIdx.x == 0) *ticket = 0;
 }
 
-template <int P, bool LOCAL, int NT>
-cudaError_t launch_sb_n(const BatchLaunch &b, cudaStream_t st) {
-    static int per_sm = -1, sms = 0;
-    if (per_sm < 0) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e == cudaSuccess)
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_solids_batch<P, LOCAL, NT>,
-                                                              NT, 0);
-        if (e != cudaSuccess) return e;
-    }
-    int blocks = b.max_items;
-    if (blocks > per_sm * sms) blocks = per_sm * sms;
-    if (blocks < 1) blocks = 1;
-    k_solids_batch<P, LOCAL, NT><<<blocks, NT, 0, st>>>(b.cases, b.items, b.nitems, b.active,
-                                                          b.nactive, b.ticket);
+template <int P, bool LOCAL, int NT, int BLOCKS>
+cudaError_t launch_sb_b(const BatchLaunch &b, cudaStream_t st, int sms) {
+    const int blocks = std::max(1, std::min(b.max_items, BLOCKS * sms));
+    k_solids_batch<P, LOCAL, NT, BLOCKS><<<blocks, NT, 0, st>>>(b.cases, b.items, b.nitems, b.active,
+                                                                b.nactive, b.ticket);
     return cudaGetLastError();
+}
+
+// 80 registers a thread, or 64 and some spills where that makes room for all items at once
+// (96 channels of 256 x 128: 58.8 us a step with 80, 59.8 with 64; 512 of 128 to 1024 x 64
+// to 512, in two waves with 80: 1130, with 64 1115).
+template <int P, bool LOCAL, int NT>
+cudaError_t launch_sb_n(const BatchLaunch &b, cudaStream_t st, int sms) {
+    return b.max_items <= 768 / NT * sms ? launch_sb_b<P, LOCAL, NT, 768 / NT>(b, st, sms)
+                                         : launch_sb_b<P, LOCAL, NT, 1024 / NT>(b, st, sms);
 }
 
 // A disk has about 9.5 r + 7 candidates.  Up to 128, one turn of 128 threads; more take
@@ -1552,14 +1632,11 @@ cudaError_t launch_sb_n(const BatchLaunch &b, cudaStream_t st) {
 // go to 128.
 template <int P, bool LOCAL>
 cudaError_t launch_sb(const BatchLaunch &b, cudaStream_t st) {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-    }
-    return b.rmax > 12.5 && b.max_items <= 4 * sms ? launch_sb_n<P, LOCAL, 256>(b, st) : launch_sb_n<P, LOCAL, FB>(b, st);
+    int sms = 0;
+    const cudaError_t e = sm_count(sms);
+    if (e != cudaSuccess) return e;
+    return b.rmax > 12.5 && b.max_items <= 4 * sms ? launch_sb_n<P, LOCAL, 256>(b, st, sms)
+                                                   : launch_sb_n<P, LOCAL, FB>(b, st, sms);
 }
 
 // Convergence test and list rebuild, one block.  Case states: 0 active,

@@ -8,15 +8,26 @@ namespace gbm {
 
 namespace {
 
+// Blocks on an SM, of BGK without a body force: for at most 80 registers a thread with
+// 16-byte words, 56 (FP64) or 48 with 8, 32 with 4.  (With 84 and 94, one block less: a
+// step of the FP64 channel of 1200 x 120 nodes 38.1 us, now 35.2; 2048 x 1024 nodes in
+// FP32 24.7, now 23.5.)
+template <int P, int V, bool FORCE, bool OPEN, int COLL>
+constexpr int row_blocks() {
+    constexpr int bytes = V * (int)sizeof(typename Raw<P>::R);
+    return FORCE || OPEN || COLL ? 0 : (bytes == 16 ? 6 : (bytes == 4 ? 16 : (P == LBM_FP64 ? 9 : 10)));
+}
+
 // One block per SC_BLOCK_X * V nodes of a row.
 template <int P, int V, bool FORCE, bool OPEN, int COLL>
-__global__ void __launch_bounds__(SC_BLOCK_X) k_stream_collide(const StepParams p) {
+__global__ void __launch_bounds__(SC_BLOCK_X, (row_blocks<P, V, FORCE, OPEN, COLL>())) k_stream_collide(const StepParams p) {
     early_start();
     using R = typename Raw<P>::R;
     const long long t = *p.t;
     sc_row<P, V, FORCE, OPEN, COLL>(p, static_cast<const R *>((t & 1) ? p.f1 : p.f0),
                                     static_cast<R *>((t & 1) ? p.f0 : p.f1),
                                     (blockIdx.x * SC_BLOCK_X + threadIdx.x) * V, blockIdx.y);
+    if (P == LBM_FP32_DEV && p.sc_last) end_of_step(p, t, gridDim.x * gridDim.y);
 }
 
 template <int V, bool FORCE, bool LOCAL, bool DEFER, int COLL = 0, bool BND = false>
@@ -148,13 +159,6 @@ cudaError_t launch_update(const StepParams &p, cudaStream_t st) {
 template <int V, bool FORCE, bool LOCAL, bool DEFER>
 cudaError_t launch_sc(const StepParams &p, cudaStream_t st) {
     const dim3 grid((p.L.nx + SC_BLOCK_X * V - 1) / (SC_BLOCK_X * V), p.L.ny);
-    // An SM changes its split of L1 and shared memory only when it is empty: with the
-    // split that this kernel would get by itself the force kernel (13 KB a block) beside
-    // it waited for SMs to drain (768 x 512 nodes, six disks of r 51: 59 us a step, now 50;
-    // 2000 x 1500, 180 of r 18: 91 and 87).
-    static const cudaError_t split = cudaFuncSetAttribute(
-        k_stream_collide16<V, FORCE, LOCAL, DEFER>, cudaFuncAttributePreferredSharedMemoryCarveout, 50);
-    if (split != cudaSuccess) return split;
     k_stream_collide16<V, FORCE, LOCAL, DEFER><<<grid, SC_BLOCK_X, 0, st>>>(p);
     cudaError_t e = cudaGetLastError();
     // with solids, the force kernel lists the nodes next to them and the

@@ -28,7 +28,7 @@ struct lbm_ctx {
     DSolid *solids = nullptr;
     int solid_cap = 0;
     int nsolid = 0;
-    double rmax = 0.0;  // largest radius of a solid added
+    double rmax = 0.0;  // largest radius of a solid
     int *moving_d = nullptr;
     int moving_cap = 0;
     void *ev_d = nullptr;  // covered/fresh events: {length, pad}, int4 list, 6 doubles each
@@ -45,6 +45,7 @@ struct lbm_ctx {
     unsigned int *bar_d = nullptr;  // per-solid control words (displacement, pair test)
     uint16_t *near_d = nullptr;     // near lists, [solid_cap][NEAR_CAP]
     double *part_d = nullptr;       // link sums by block or chunk (StepParams::part)
+    size_t part_cap = 0;            // of six each
     long long spin_limit = 1ll << 24;  // polls of a bounded device wait (about one second)
     // the force kernel runs on a second stream beside the advection-collision
     // kernel: fork after the previous step, join before the re-rasterisation
@@ -97,6 +98,8 @@ lbm_status fail(lbm_ctx *c, lbm_status st, const char *fmt, ...) {
                         "%s failed: %s", #call, cudaGetErrorString(e_));                   \
     } while (0)
 
+constexpr int FEW_SOLIDS = 32;  // whose links may go to more than LINK_PARTS blocks each
+
 size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DEV ? 4 : 2); }
 
 // Does work go to the side stream, beside the advection-collision kernel?
@@ -104,33 +107,62 @@ size_t elem_bytes(int prec) { return prec == LBM_FP64 ? 8 : (prec == LBM_FP32_DE
 // with few moving solids, whose rings then go into the re-rasterisation's launch, or
 // with none that moves, the step stays on one stream and its kernels are launched early
 // (StepParams::early): 128 x 64 nodes with one moving disk 24.8 us a step, launched one by
-// one (41.5 with the side stream), 300 x 200 with four at rest 14.3 (22.5).  Larger: with
+// one (41.5 with the side stream), 300 x 200 with four at rest 13.1 (22.5).  Larger: with
 // the side stream 768 x 512 and six moving disks take 39.7 in a graph against 46.3.  In
 // FP64, whose kernels take longer, it is faster from the smallest domain on.
 bool few_moving(const lbm_ctx *c) {
     return !c->moving.empty() && c->moving.size() <= gbm::FEW_MOVING && c->cfg.boundary == LBM_HALFWAY;
 }
 constexpr long long FORK_NODES = 1 << 18;
+bool small(const lbm_ctx *c) {
+    return c->cfg.precision == LBM_FP32_DEV && (long long)c->cfg.nx * c->cfg.ny <= FORK_NODES;
+}
 bool forks(const lbm_ctx *c) {
     if (!c->overlap || c->nsolid == 0) return false;
-    if (c->cfg.precision != LBM_FP32_DEV || (long long)c->cfg.nx * c->cfg.ny > FORK_NODES) return true;
-    return !few_moving(c) && !(c->moving.empty() && c->cfg.boundary == LBM_HALFWAY);
+    return !small(c) || !(few_moving(c) || (c->moving.empty() && c->cfg.boundary == LBM_HALFWAY));
 }
 
 // Blocks per solid of the link kernel, or 0 for links, record and motion in one
 // kernel.  The record and the motion are a kernel of their own where they can run
-// beside the advection-collision kernel, and with the interpolated boundary.  Below 256
+// beside the advection-collision kernel, with the interpolated boundary, and with large
+// solids at rest, where that kernel takes the place of the clock's tick.  Below 256
 // solids, which alone would not fill the SMs, LINK_PARTS blocks take a solid's links.
-// FP64, whose unit is what a block waits for, takes with few solids as many blocks as
-// most disks have chunks of candidates.  The sums are those of one block bit for bit,
-// whichever way.  A step of 256 x 128 nodes with one disk, FP64: 34.5 -> 31 us (one block
-// before), of 1200 x 120 with an interpolated one 47 -> 41 (four before); 768 x 512 with
-// six of r 51, FP32: 55 -> 50 (one before).
+// Few solids, if they are large (or in FP64, whose unit is what a block waits for), get
+// as many blocks as a disk has chunks of candidates.  FP16's links run beside the
+// advection-collision kernel as it is: several blocks and a second kernel are worth it for
+// large disks only.  The sums are those of one block bit for bit, whichever way.
+// A step, FP32, disks at rest: 300 x 200 nodes, one of r 70: 16.7 us in a graph (one block
+// 30.4), 768 x 512, six of r 51: 14.5 (four blocks 20.6), 2000 x 1500, two of r 200: 54
+// (92); FP16, 768 x 512, six of r 51, MRT: 19.4 (one block 24.1); FP64, 256 x 128 with one
+// disk: 31 (34.5), 1200 x 120 with an interpolated one 41 (four blocks 47).
 int link_parts(const lbm_ctx *c) {
     const bool cut = c->cfg.boundary == LBM_INTERPOLATED, fp64 = c->cfg.precision == LBM_FP64;
-    if (!cut && (c->cfg.precision == LBM_FP16_DEV || !forks(c))) return 0;
-    if (fp64 && c->nsolid <= gbm::MAX_PARTS_SOLIDS && c->rmax <= gbm::MAX_PARTS_RADIUS) return gbm::MAX_LINK_PARTS;
+    const bool few = c->nsolid <= FEW_SOLIDS, still = c->moving.empty();
+    if (c->cfg.precision == LBM_FP16_DEV) {
+        const bool mrt = c->cfg.collision == LBM_MRT;
+        if (!cut && !(few && c->rmax > (mrt || !still ? 40.0 : 60.0))) return 0;
+    } else if (!cut && !forks(c)) {
+        if (!small(c) || !still || c->rmax <= 25.0) return 0;
+    }
+    if (few && (fp64 || c->rmax > 12.5)) {
+        const int chunks = (int)(9.5 * c->rmax + 7.0) / 32 + 1;  // about
+        return std::min((chunks + 15) / 16 * 16, gbm::MAX_LINK_PARTS);
+    }
     return c->nsolid < 256 ? gbm::LINK_PARTS : 1;
+}
+
+// Room for the link sums of solids of radius r: by block for every solid, or by chunk for
+// a few (the sums of earlier steps are of no use any more).
+lbm_status room_for_links(lbm_ctx *c, double r) {
+    const size_t sums = std::max((size_t)c->solid_cap * gbm::LINK_PARTS, (size_t)FEW_SOLIDS * gbm::slots_of(r));
+    if (sums <= c->part_cap) return LBM_OK;
+    double *part = nullptr;
+    CK(c, cudaMalloc(&part, sums * 6 * sizeof(double)));
+    CK(c, cudaStreamSynchronize(c->stream));
+    if (c->part_d) CK(c, cudaFree(c->part_d));
+    c->part_d = part;
+    c->part_cap = sums;
+    return LBM_OK;
 }
 
 StepParams params(const lbm_ctx *c) {
@@ -203,7 +235,13 @@ StepParams params(const lbm_ctx *c) {
     p.spin_limit = c->spin_limit;
     p.near_id = c->near_d;
     p.part = c->part_d;
+    p.rmax = c->rmax;
     p.link_parts = link_parts(c);
+    p.link_slots = p.link_parts > gbm::LINK_PARTS ? gbm::slots_of(c->rmax) : 0;
+    // at rest on one stream the clock needs no launch of its own
+    const bool rest = small(c) && !forks(c) && c->moving.empty();
+    p.record_last = rest && p.link_parts;
+    p.sc_last = rest && !p.link_parts;
     // one stream, nothing between its kernels but (with many moving solids) the ring's
     p.early = c->cfg.precision == LBM_FP32_DEV && !forks(c) && !c->timing && (c->moving.empty() || few_moving(c));
     return p;
@@ -307,7 +345,7 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
         rest = c->side;
         if (half) CK(c, gbm::launch_forces(p, rest));
     }
-    CK(c, gbm::launch_record(p, rest));
+    if (!p.record_last) CK(c, gbm::launch_record(p, rest));
     if (!tail) CK(c, gbm::launch_ring(p, rest));
     if (fork) CK(c, cudaEventRecord(c->join, rest));
     c->launches += (p.nsolid > 0 ? (p.link_parts ? 2 : 1) : 0) + (p.nmoving > 0 && !tail ? 1 : 0);
@@ -335,9 +373,10 @@ lbm_status enqueue_step(lbm_ctx *c, const StepParams &p, bool timed) {
         c->launches++;
     }
     if (fork && !p.list_by_forces) CK(c, cudaStreamWaitEvent(c->stream, c->join, 0));
-    if (p.nmoving > 0) CK(c, gbm::launch_remask(p, tail, c->stream));
-    else CK(c, gbm::launch_tick(p, c->stream));
-    c->launches += gbm::stream_collide_launches(p) + (p.nmoving > gbm::FEW_MOVING ? 2 : 1);
+    if (p.record_last) CK(c, gbm::launch_record(p, c->stream));
+    else if (p.nmoving > 0) CK(c, gbm::launch_remask(p, tail, c->stream));
+    else if (!p.sc_last) CK(c, gbm::launch_tick(p, c->stream));
+    c->launches += gbm::stream_collide_launches(p) + (p.nmoving > gbm::FEW_MOVING ? 2 : (p.record_last || p.sc_last ? 0 : 1));
     return LBM_OK;
 }
 
@@ -521,12 +560,10 @@ lbm_status lbm_add_solid(lbm_ctx *c, const lbm_disk *d, int32_t *id_out) {
         if (c->near_d) CK(c, cudaFree(c->near_d));  // rebuilt by the next pair test
         c->near_d = nullptr;
         CK(c, cudaMalloc(&c->near_d, (size_t)cap * gbm::NEAR_CAP * sizeof(uint16_t)));
-        if (c->part_d) CK(c, cudaFree(c->part_d));
-        c->part_d = nullptr;
-        const int slots = std::max(cap * gbm::LINK_PARTS, gbm::MAX_PARTS_SOLIDS * gbm::LINK_SLOTS);
-        CK(c, cudaMalloc(&c->part_d, (size_t)slots * 6 * sizeof(double)));
         c->solid_cap = cap;
     }
+    lbm_status ps = room_for_links(c, std::max(c->rmax, d->r));
+    if (ps != LBM_OK) return ps;
     if (c->nsolid + 1 > c->ring_cap) {
         int cap = c->ring_cap ? c->ring_cap : 64;
         while (cap < c->nsolid + 1) cap *= 2;
@@ -882,6 +919,20 @@ lbm_status lbm_load(lbm_ctx *c, const void *buf, int64_t bytes) {
     lbm_status st = harvest_timing(c);
     if (st != LBM_OK) return st;
     const char *base = static_cast<const char *>(buf);
+    // the state's disks need not be as large as those added here
+    const char *sv = base + sizeof h + 9 * ((size_t)c->cfg.ny * c->pitch) * c->elem +
+                     2 * ((size_t)c->cfg.ny * c->pitch) * sizeof(uint16_t);
+    double rmax = 0.0;
+    for (int s = 0; s < c->nsolid; s++) {
+        DSolid d;
+        std::memcpy(&d, sv + s * sizeof d, sizeof d);
+        if (!(d.r > 0.0) || !(d.r < c->cfg.nx) || !(d.r < c->cfg.ny))
+            return fail(c, LBM_EINVAL, "the state's solid %d has radius %g", s, d.r);
+        rmax = std::max(rmax, d.r);
+    }
+    st = room_for_links(c, rmax);
+    if (st != LBM_OK) return st;
+    c->rmax = rmax;
     const char *mv = base + state_bytes(c, h.ev_len) - c->nsolid;
     for (int s = 0; s < c->nsolid; s++) c->is_moving[s] = mv[s] ? 1 : 0;
     st = upload_moving(c);  // also sizes the event list

@@ -82,13 +82,20 @@ constexpr int NEAR_CAP = 32;
 constexpr float NEAR_REACH = 4.5f;
 constexpr float NEAR_MARGIN = 4.0f;
 
-// Blocks that share one solid's links: the warps of a single block, or in FP64 more, which
-// leave the sums of every 32 candidates.  A disk has up to 4.76 (2 r + 1.42) candidates on
-// its annulus and two more in each of its 2 r + 9 rows, taken 128 rows at a time: up to
-// r = 150, 65 chunks, and 12 to fill up three turns.
-constexpr int LINK_PARTS = 4, MAX_LINK_PARTS = 16, LINK_SLOTS = 80;
-constexpr double MAX_PARTS_RADIUS = 150.0;
-constexpr int MAX_PARTS_SOLIDS = 32;
+// Blocks that share one solid's links: the warps of a single block, or up to
+// MAX_LINK_PARTS, which leave the sums of every 32 candidates in slots.
+constexpr int LINK_PARTS = 4, MAX_LINK_PARTS = 64;
+constexpr int LEAD_SLOTS = 16;  // slots that are written, and read, however few chunks there are
+
+// Candidates for links of a disk: the nodes of an annulus 1.52 wide, at most two more in
+// each of its rows.
+__host__ __device__ inline int link_candidates(double r) { return (int)(4.76 * (2.0 * r + 1.42) + 2.0 * (2.0 * r + 10.0)); }
+
+// Slots for a disk: its chunks of 32, taken 128 rows at a time and filled up to LINK_PARTS
+// for each of these turns, LEAD_SLOTS at least, and one for their number.
+__host__ __device__ inline int slots_of(double r) {
+    return link_candidates(r) / 32 + 1 + LINK_PARTS * ((int)(2.0 * r + 12.0) / 128 + 1) + LEAD_SLOTS + 1;
+}
 
 // covered/fresh nodes one solid can queue per step
 constexpr int SOLID_EVENTS = 256;
@@ -125,8 +132,8 @@ struct StepParams {
     int sc_variant;           // node width per thread of the advection-collision kernel
     float omega_f, body_xf, body_yf, rho0_f;  // FP32 copies for the FP32 kernels
     float wall_ux0_f, wall_ux1_f, umax_f;
-    unsigned int *bar;        // control words: two unused, largest displacement since the
-                              // pair test (FP32 bits), pair test requested
+    unsigned int *bar;        // control words: ticket of a step's last kernel, one unused, largest
+                              // displacement since the pair test (FP32 bits), pair test requested
     long long spin_limit;     // 0: the re-rasterisation gives up (LBM_ETIMEOUT)
     uint16_t *near_id;        // [nsolid][NEAR_CAP] near lists
     int4 *ev;                 // covered/fresh events of the step: {node code (cell << 1 |
@@ -140,9 +147,12 @@ struct StepParams {
     int chg_cap;
     int *bnd;                 // deferred per-node path: {length at even t, at odd t, list...}
     int bnd_cap;              // capacity of the list
-    double *part;             // [nsolid][LINK_PARTS][6] link sums of a solid's blocks, or with
-                              // more blocks [nsolid][LINK_SLOTS][6] of its chunks
     int link_parts;           // blocks per solid of k_links, which k_record follows; 0: k_forces
+    double rmax;              // largest radius of a solid
+    int link_slots;           // slots per solid for the sums of chunks; 0: sums of blocks
+    double *part;             // [nsolid][link_slots or LINK_PARTS][6] link sums
+    int sc_last, record_last; // the step's last kernel, which advances t: the advection-collision
+                              // kernel; k_record, which then comes after it; neither: another
     int early;                // this step's kernels are launched early
     int list_by_forces;       // FP16: the force kernel fills the deferred list; the fused pass
                               // leaves the update to launch_deferred_update
@@ -184,6 +194,15 @@ __device__ __forceinline__ void early_start() {
     asm volatile("griddepcontrol.wait;\ngriddepcontrol.launch_dependents;" ::: "memory");
 }
 
+
+// At the end of a step's last kernel, which started at t, by all threads: the clock
+// advances once every block has read it (a ticket, no waiting).
+__device__ __forceinline__ void end_of_step(const StepParams &p, long long t, unsigned int blocks) {
+    __syncthreads();
+    if (threadIdx.x != 0 || (blocks > 1 && atomicAdd(p.bar, 1u) != blocks - 1)) return;
+    p.bar[0] = 0u;
+    *p.t = t + 1;
+}
 
 __device__ __forceinline__ double ld(const double *p) { return __ldg(p); }
 __device__ __forceinline__ float ld(const float *p) { return __ldg(p); }

@@ -157,3 +157,18 @@ def test_forces_do_not_depend_on_the_number_of_solids(precision, few):
         g.set_f(seeded_f(w, 4))
         first.append(g.step_record(1)[:, 0])
     assert np.array_equal(*first)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32", "fp16"])
+def test_a_state_may_hold_larger_disks_than_its_context(precision):
+    def box(r):
+        return _box(0.8, 420, 410, solids=[dict(cx=210.3, cy=205.1, r=r, vx=0.01, vy=0.02, omega=0.0, rho_s=1.5, motion=0)])
+
+    g = make_gpu(box(190.0), precision, ring=40)
+    g.set_f(seeded_f(box(190.0), 5))
+    g.step(5)
+    state = g.save()
+    h = make_gpu(box(3.0), precision, ring=40)
+    h.load(state)
+    assert np.array_equal(g.step_record(10), h.step_record(10))
+    assert np.array_equal(g.get_f(), h.get_f())
