@@ -305,9 +305,11 @@ int32_t lbm_force_overlap(const lbm_ctx *ctx);
 /* Autotuner: run 1 + steps real steps with each of the 6 variants of the
  * advection-collision kernel, with the per-solid work beside it and before it,
  * timing whole steps with CUDA events, and keep the fastest pair (the variant
- * stored in *best when not NULL; lbm_force_overlap tells the other).  The
- * simulation advances by 12 (1 + steps) steps; results do not depend on the
- * choice.  Waits for the stream. */
+ * stored in *best when not NULL; lbm_force_overlap tells the other).  Pairs
+ * that come to the same launches (FP64 and FP32: variants 3-5 as 0-2; MRT: all
+ * six; small FP32 domains: either overlap) are repeats of one measurement, of
+ * which the first is kept.  The simulation advances by 12 (1 + steps) steps;
+ * results do not depend on the choice.  Waits for the stream. */
 lbm_status lbm_autotune(lbm_ctx *ctx, int32_t steps, int32_t *best);
 
 /* ------------------------------------------------------------------ batches

@@ -3,6 +3,7 @@
 // history, field export and kernel timing.
 #include <algorithm>
 #include <cmath>
+#include <iterator>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -1205,6 +1206,23 @@ lbm_status lbm_set_force_overlap(lbm_ctx *c, int32_t on) {
 
 int32_t lbm_force_overlap(const lbm_ctx *c) { return c ? (c->overlap ? 1 : 0) : -1; }
 
+// The first of the variants and overlap settings that launch the same kernels in the same
+// way as variant v with overlap o does: there is nothing to choose between them.
+static int launch_shape(lbm_ctx *c, int v, bool o) {
+    const lbm_config &g = c->cfg;
+    const bool deferred = g.precision == LBM_FP16_DEV && v >= 3;
+    int first = v % 3 + (deferred ? 3 : 0);
+    if (g.precision == LBM_FP16_DEV && g.boundary == LBM_INTERPOLATED) first = v % 3;  // always deferred
+    if (g.collision == LBM_MRT) first = 0;
+    const bool keep = c->overlap;
+    c->overlap = true;
+    const bool beside = forks(c);
+    c->overlap = false;
+    const bool same = beside == forks(c);
+    c->overlap = keep;
+    return first + (o || same ? 0 : gbm::KERNEL_VARIANTS);
+}
+
 lbm_status lbm_autotune(lbm_ctx *c, int32_t steps, int32_t *best) {
     if (!c || steps < 1) return LBM_EINVAL;
     if (c->batch) return fail(c, LBM_EINVAL, "a case of a batch is tuned by lbm_batch_autotune");
@@ -1218,9 +1236,10 @@ lbm_status lbm_autotune(lbm_ctx *c, int32_t steps, int32_t *best) {
     CK(c, cudaEventCreate(&e1));
     c->timing = false;
     c->graph_steps = 0;
-    double best_ms = 0.0;
-    int best_v = 0;
-    bool best_o = true;
+    // the shortest time of each launch shape, at its first setting; settings that come to
+    // the same shape are repeats of its measurement
+    float shape_ms[2 * gbm::KERNEL_VARIANTS];
+    std::fill(std::begin(shape_ms), std::end(shape_ms), INFINITY);
     for (int o = 1; o >= 0 && st == LBM_OK; o--) {
         for (int v = 0; v < gbm::KERNEL_VARIANTS && st == LBM_OK; v++) {
             c->sc_variant = v;
@@ -1234,13 +1253,13 @@ lbm_status lbm_autotune(lbm_ctx *c, int32_t steps, int32_t *best) {
             if (st == LBM_OK) st = lbm_sync(c);
             float ms = 0.f;
             if (st == LBM_OK && cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess) st = LBM_ECUDA;
-            if (st == LBM_OK && ((o == 1 && v == 0) || ms < best_ms)) {
-                best_ms = ms;
-                best_v = v;
-                best_o = o != 0;
-            }
+            float &shape = shape_ms[launch_shape(c, v, o != 0)];
+            if (st == LBM_OK) shape = std::min(shape, ms);
         }
     }
+    const int chosen = (int)(std::min_element(std::begin(shape_ms), std::end(shape_ms)) - std::begin(shape_ms));
+    const int best_v = chosen % gbm::KERNEL_VARIANTS;
+    const bool best_o = chosen < gbm::KERNEL_VARIANTS;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     c->sc_variant = best_v;
