@@ -268,7 +268,8 @@ __global__ void k_export_owner(const StepParams p, int32_t *out) {
 // populations (in the deviation modes d_i = f_i - w_i) as 64-bit integers in units of
 // 2^-60 (FP64: 2^-58; bits below, 1e-18, are cut off, less than an FP64 addition
 // rounds), so exact.  Division: a fixed-point reciprocal of r and one product each,
-// rounded once, 0.55 units in the last place at most.  8192 x 4096 nodes, FP32 and
+// rounded once: 0.63 units in the last place at most, half of one and the reciprocal's
+// 2^-56, an eighth of one for a mantissa close to 2.  8192 x 4096 nodes, FP32 and
 // FP16: 0.50 ms (its bytes at the copy rate: 0.30 and 0.21; the integer units bound it);
 // with the sums alone in integers 1.01, all in FP64 3.79.  FP64, 2048 x 1024: 42 us (28),
 // before 172.
@@ -310,8 +311,10 @@ __device__ __forceinline__ double packed64(unsigned long long p, int e, bool neg
     return __longlong_as_double(negative ? b | 0x8000000000000000ll : b);
 }
 
-// 2^122 / r for r in [2^59, 2^61), to 2^-57 of it: FP32's approximation of 1 / r to about
-// 22 bits, y, then y (1 + e + e^2) with e = 1 - r y in fixed point.
+// 2^122 / r for r in [2^59, 2^61), to 2^-56 of it: FP32's approximation of 1 / r to about
+// 22 bits, y, then y (1 + e + e^2) with e = 1 - r y in fixed point.  (Two units in the last
+// place of y, the bound of __fdividef, leave |e| below 2^-21; the square from e's upper 16
+// bits is then within 2^-56.3.)
 __device__ __forceinline__ unsigned long long reciprocal62(unsigned long long r) {
     const unsigned rh = (unsigned)(r >> 32), rl = (unsigned)r;
     const unsigned y = (unsigned)(__fdividef(1.f, (float)rh * 0x1p-28f) * 0x1p30f);
