@@ -214,10 +214,22 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
     }
 }
 
-// BGK collision (with Guo forcing when FORCE) of one node in place.  CHECK:
-// flag a non-physical state (sc_row checks its fluid nodes itself).
-template <int P, bool FORCE, bool CHECK = true>
-__device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C (&g)[9]) {
+// Is (rho, ux, uy) not a physical state?  FP64: from the high words (the FP64
+// unit is what bounds the FP64 kernel, and a comparison occupies it too).
+__device__ __forceinline__ bool unphysical(float r, float vx, float vy) {
+    return !(r > 0.f) || !(fabsf(vx) < 1e30f) || !(fabsf(vy) < 1e30f);
+}
+__device__ __forceinline__ bool unphysical(double r, double vx, double vy) {
+    constexpr int BIG = 0x46293E59;  // high word of 1e30
+    const int h = __double2hiint(r);
+    return h <= 0 || h >= 0x7FF00000 || (__double2hiint(vx) & 0x7FFFFFFF) > BIG ||
+           (__double2hiint(vy) & 0x7FFFFFFF) > BIG;
+}
+
+// BGK collision (with Guo forcing when FORCE) of one node in place; check(rho, ux, uy)
+// sees its density and velocity.
+template <int P, bool FORCE, class Check>
+__device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C (&g)[9], Check &&check) {
     using C = typename Prec<P>::C;
     C s0 = 0, jx = 0, jy = 0;
 #pragma unroll
@@ -228,13 +240,12 @@ __device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C
     }
     const C rho = Prec<P>::dev ? (C)1 + s0 : s0;
     const C Fx = pick<C>(p.body_x, p.body_xf), Fy = pick<C>(p.body_y, p.body_yf);
-    const C inv = (C)1 / rho;
+    const C inv = reciprocal(rho);
     const C ux = FORCE ? (jx + (C)0.5 * Fx) * inv : jx * inv;
     const C uy = FORCE ? (jy + (C)0.5 * Fy) * inv : jy * inv;
     const C uu = ux * ux + uy * uy;
     const C om = pick<C>(p.omega, p.omega_f);
-    if (CHECK && (!(rho > (C)0) || !(fabs(ux) < (C)1e30) || !(fabs(uy) < (C)1e30)))
-        atomicOr(p.status, 1);
+    check(rho, ux, uy);
 #pragma unroll
     for (int i = 0; i < 9; i++) {
         const C eu = (C)cx(i) * ux + (C)cy(i) * uy;
@@ -259,11 +270,10 @@ __device__ __forceinline__ void collide(const StepParams &p, typename Prec<P>::C
 // (j_x^2 - j_y^2) / rho and j_x j_y / rho (in the deviation modes minus the
 // moments of the weights, which are 1, -2, 1 and zeros), and the change goes
 // back to the populations through the transposed basis over the squared row
-// norms (36, 36, 12, 12, 4, 4).  No body force.  CHECK: flag a non-physical
-// state (the vector path checks its fluid nodes itself; solid nodes there
-// hold no state).
-template <int P, bool CHECK>
-__device__ __forceinline__ void collide_mrt(const StepParams &p, typename Prec<P>::C (&g)[9]) {
+// norms (36, 36, 12, 12, 4, 4).  No body force.  check(rho, ux, uy) sees the
+// node's density and velocity.
+template <int P, class Check>
+__device__ __forceinline__ void collide_mrt(const StepParams &p, typename Prec<P>::C (&g)[9], Check &&check) {
     using C = typename Prec<P>::C;
     const C ax = g[1] + g[2] + g[3] + g[4], dg = g[5] + g[6] + g[7] + g[8];
     const C s0 = g[0] + ax + dg;
@@ -271,8 +281,7 @@ __device__ __forceinline__ void collide_mrt(const StepParams &p, typename Prec<P
     const C jy = g[2] - g[4] + g[5] + g[6] - g[7] - g[8];
     const C rho = Prec<P>::dev ? (C)1 + s0 : s0;
     const C inv = reciprocal(rho);
-    if (CHECK && (!(rho > (C)0) || !(fabs(jx * inv) < (C)1e30) || !(fabs(jy * inv) < (C)1e30)))
-        atomicOr(p.status, 1);
+    check(rho, jx * inv, jy * inv);
     const C jj = (jx * jx + jy * jy) * inv;
     const C e = (C)-4 * g[0] - ax + (C)2 * dg;
     const C eps = (C)4 * g[0] - (C)2 * ax + dg;
@@ -413,8 +422,11 @@ __device__ __noinline__ void update_node(const StepParams &p, const typename Raw
         g[i] = cvt(fin[i * plane + ys * L.pitch + xs]);
     }
     if (flu & 0x1FEu) bounce<P, LOCAL, BND>(p, fin, xu, y, flu, g);
-    if constexpr (COLL == 1) collide_mrt<P, true>(p, g);
-    else collide<P, FORCE>(p, g);
+    auto check = [&](C rho, C ux, C uy) {
+        if (unphysical(rho, ux, uy)) atomicOr(p.status, 1);
+    };
+    if constexpr (COLL == 1) collide_mrt<P>(p, g, check);
+    else collide<P, FORCE>(p, g, check);
     if (OPEN && open) extrapolate_open<P, FORCE>(p, x == 0, u_in, g);
 #pragma unroll
     for (int i = 0; i < 9; i++) {
@@ -517,7 +529,7 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
             }
             const C r = Prec<P>::dev ? (C)1 + a : a;
             classify(j, r, jx / r, jy / r);
-            collide_mrt<P, false>(p, g);
+            collide_mrt<P>(p, g, [](C, C, C) {});
 #pragma unroll
             for (int i = 0; i < 9; i++) put(o[i].r[j], (fl.f[j] & 1u) ? (C)0 : g[i]);
         }
@@ -666,18 +678,6 @@ __device__ __forceinline__ void open_row(const StepParams &p, typename Raw<P>::R
 
 // ------------------------------------------------ FP64 and FP32: sc_row
 
-// Is (rho, ux, uy) not a physical state?  FP64: from the high words (the FP64
-// unit is what bounds the FP64 kernel, and a comparison occupies it too).
-__device__ __forceinline__ bool unphysical(float r, float vx, float vy) {
-    return !(r > 0.f) || !(fabsf(vx) < 1e30f) || !(fabsf(vy) < 1e30f);
-}
-__device__ __forceinline__ bool unphysical(double r, double vx, double vy) {
-    constexpr int BIG = 0x46293E59;  // high word of 1e30
-    const int h = __double2hiint(r);
-    return h <= 0 || h >= 0x7FF00000 || (__double2hiint(vx) & 0x7FFFFFFF) > BIG ||
-           (__double2hiint(vy) & 0x7FFFFFFF) > BIG;
-}
-
 // BGK collision of one FP64 node, no body force.  GB300 issues about two FP64
 // lanes per clock and SM, so the number of FP64 operations is the kernel's time:
 // about 57 here, against about 154 with nine separate equilibria and a division
@@ -751,25 +751,6 @@ __device__ __forceinline__ void bgk32x2(float om, float2 (&g)[9], float2 &rho, f
     pair(6, 8, fma2(dup2(-9.f), xy, B), sub2(jy, jx));
 }
 
-// Density and velocity of one node from its pulled populations.
-template <int P, bool FORCE>
-__device__ __forceinline__ void node_state(const StepParams &p, const typename Prec<P>::C (&g)[9],
-                                           typename Prec<P>::C &rho, typename Prec<P>::C &ux,
-                                           typename Prec<P>::C &uy) {
-    using C = typename Prec<P>::C;
-    C s0 = 0, jx = 0, jy = 0;
-#pragma unroll
-    for (int i = 0; i < 9; i++) {
-        s0 += g[i];
-        jx += (C)cx(i) * g[i];
-        jy += (C)cy(i) * g[i];
-    }
-    rho = Prec<P>::dev ? (C)1 + s0 : s0;
-    const C inv = reciprocal(rho);
-    ux = FORCE ? (jx + (C)0.5 * pick<C>(p.body_x, p.body_xf)) * inv : jx * inv;
-    uy = FORCE ? (jy + (C)0.5 * pick<C>(p.body_y, p.body_yf)) * inv : jy * inv;
-}
-
 // Collision of V nodes in place; check(j, rho, ux, uy) for each of them.
 template <int P, int V, bool FORCE, int COLL, class Check>
 __device__ __forceinline__ void collide_nodes(const StepParams &p, typename Prec<P>::C (&g)[V][9],
@@ -793,15 +774,15 @@ __device__ __forceinline__ void collide_nodes(const StepParams &p, typename Prec
     } else {
 #pragma unroll
         for (int j = 0; j < V; j++) {
-            C rho, ux, uy;
-            if constexpr (COLL == 0 && !FORCE && P == LBM_FP64) {
+            auto check_j = [&](C rho, C ux, C uy) { check(j, rho, ux, uy); };
+            if constexpr (COLL == 1) {
+                collide_mrt<P>(p, g[j], check_j);
+            } else if constexpr (!FORCE && P == LBM_FP64) {
+                C rho, ux, uy;
                 bgk64(p.omega, g[j], rho, ux, uy);
-                check(j, rho, ux, uy);
+                check_j(rho, ux, uy);
             } else {
-                node_state<P, FORCE>(p, g[j], rho, ux, uy);
-                check(j, rho, ux, uy);
-                if constexpr (COLL == 1) collide_mrt<P, false>(p, g[j]);
-                else collide<P, FORCE, false>(p, g[j]);
+                collide<P, FORCE>(p, g[j], check_j);
             }
         }
     }
@@ -834,8 +815,9 @@ __device__ __noinline__ void inner_update(const StepParams &p, const typename Ra
             g[i] = cvt(fin[i * plane + ys * L.pitch + x - cx(i)]);
         }
     }
-    if constexpr (COLL == 1) collide_mrt<P, false>(p, g);
-    else collide<P, FORCE, false>(p, g);
+    auto unchecked = [](C, C, C) {};  // the node's own lane checks it
+    if constexpr (COLL == 1) collide_mrt<P>(p, g, unchecked);
+    else collide<P, FORCE>(p, g, unchecked);
 }
 
 // One row segment: nodes x0 .. x0 + V - 1 of row y in each lane, x0 = 32 V times
