@@ -245,28 +245,18 @@ __device__ __forceinline__ void rows_of_i(int iy0, int iy1, int rc, int g, int &
 }
 
 // Deals the nodes of rows j0..j1 (the ranges that rng(j, R) gives for each
-// row) to the lanes of the warp, U nodes per lane at a time: fetch(i, j, u)
-// is called for all U nodes of a lane first (to issue their loads together),
-// then mid(ok) once (loads that depend on what fetch loaded, for all U nodes
-// together), then process(u, ok) for each, on every lane of the warp together
-// (ok is false for items past the end and for nodes fetch rejected).  Rows come in
-// blocks of RB <= 32 (lane l < RB takes row l of a block); with nw > 1 warps
-// sharing the rows, this warp (wi) takes the blocks wi, wi + nw ...
-struct NoMid {
-    template <int NB>
-    __device__ __forceinline__ void operator()(const bool (&)[NB]) const {}
-};
-
-template <int NB, int RB = 32, class RF, class FF, class PF, class MF = NoMid>
-__device__ __forceinline__ void warp_nodes_n(int j0, int j1, int lane, RF &&rng, FF &&fetch,
-                                             PF &&process, int wi = 0, int nw = 1,
-                                             MF &&mid = MF()) {
-    for (int jb = j0 + RB * wi; jb <= j1; jb += RB * nw) {
+// row) to the lanes of the warp, NB nodes per lane at a time: fetch(i, j, u)
+// is called for all NB nodes of a lane first, then process(u, ok) for each, on
+// every lane of the warp together (ok is false for items past the end and for
+// nodes fetch rejected).  Rows come in blocks of 32, one to a lane.
+template <int NB, class RF, class FF, class PF>
+__device__ __forceinline__ void warp_nodes_n(int j0, int j1, int lane, RF &&rng, FF &&fetch, PF &&process) {
+    for (int jb = j0; jb <= j1; jb += 32) {
         const int j = jb + lane;
         Ranges R;
         R.a0 = R.a1 = 0;
         int n0 = 0, n1 = 0;
-        if (lane < RB && j <= j1 && rng(j, R)) {
+        if (j <= j1 && rng(j, R)) {
             n0 = R.b0 >= R.a0 ? R.b0 - R.a0 + 1 : 0;
             n1 = R.b1 >= R.a1 ? R.b1 - R.a1 + 1 : 0;
         }
@@ -297,7 +287,6 @@ __device__ __forceinline__ void warp_nodes_n(int j0, int j1, int lane, RF &&rng,
                 const int i = tt < qn0 ? qa0 + tt : qa1 + (tt - qn0);
                 ok[u] = e < total && fetch(i, jb + q, u);
             }
-            mid(ok);
 #pragma unroll
             for (int u = 0; u < NB; u++) process(u, ok[u]);
         }

@@ -32,10 +32,9 @@ __global__ void __launch_bounds__(SC_BLOCK_X, (row_blocks<P, V, FORCE, OPEN, COL
 
 template <int V, bool FORCE, bool LOCAL, bool DEFER, int COLL = 0, bool BND = false>
 __global__ void __launch_bounds__(SC_BLOCK_X) k_stream_collide16(const StepParams p) {
-    constexpr int P = LBM_FP16_DEV;
-    using R = Raw<P>::R;
+    using R = Raw<LBM_FP16_DEV>::R;
     const long long t = *p.t;
-    sc_tile<P, V, FORCE, LOCAL, false, DEFER, COLL, BND>(
+    sc_tile<V, FORCE, LOCAL, false, DEFER, COLL, BND>(
         p, static_cast<const R *>((t & 1) ? p.f1 : p.f0), static_cast<R *>((t & 1) ? p.f0 : p.f1),
         (blockIdx.x * SC_BLOCK_X + threadIdx.x) * V, blockIdx.y);
 }
@@ -61,8 +60,7 @@ __host__ __device__ inline long long boundary_edge_nodes(const Lattice &L) {
 
 template <bool FORCE, bool LOCAL, bool BND>
 __global__ void __launch_bounds__(BN_BLOCK) k_boundary_update(const StepParams p) {
-    constexpr int P = LBM_FP16_DEV;
-    using R = Raw<P>::R;
+    using R = Raw<LBM_FP16_DEV>::R;
     const Lattice &L = p.L;
     const long long t = *p.t;
     const R *fin = static_cast<const R *>((t & 1) ? p.f1 : p.f0);
@@ -87,7 +85,7 @@ __global__ void __launch_bounds__(BN_BLOCK) k_boundary_update(const StepParams p
             x = 1 + (c < w ? c : c - w);
         }
         if (!(p.flags[cell_of(L, x, y)] & 1u))
-            update_node<P, FORCE, LOCAL, false, 0, BND>(p, fin, fout, x, y);
+            update_node<FORCE, LOCAL, false, 0, BND>(p, fin, fout, x, y);
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && p.bnd) p.bnd[(t + 1) & 1] = 0;
 }
@@ -99,7 +97,7 @@ __global__ void k_open_columns(const StepParams p) {
     const int y = blockIdx.x * blockDim.x + threadIdx.x;
     if (y >= p.L.ny) return;
     const long long t = *p.t;
-    open_row<LBM_FP16_DEV, FORCE>(p, static_cast<R *>((t & 1) ? p.f0 : p.f1), y);
+    open_row<FORCE>(p, static_cast<R *>((t & 1) ? p.f0 : p.f1), y);
 }
 
 // ------------------------------------------------------------ FP64, FP32

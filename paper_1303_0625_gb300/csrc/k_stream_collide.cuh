@@ -72,11 +72,7 @@ __device__ __forceinline__ void put(unsigned short &d, float v) {
     d = __half_as_ushort(__float2half_rn(v));
 }
 
-// two adjacent values of a population plane at once (FP16: one half2)
-__device__ __forceinline__ void put2(float *d, float a, float b) {
-    d[0] = a;
-    d[1] = b;
-}
+// two adjacent values of a population plane at once
 __device__ __forceinline__ void put2(unsigned short *d, float a, float b) {
     *reinterpret_cast<__half2 *>(d) = __floats2half2_rn(a, b);
 }
@@ -101,25 +97,25 @@ __device__ __forceinline__ unsigned short shfl_dn1(unsigned short v) {
     return (unsigned short)__shfl_down_sync(0xffffffffu, (int)v, 1);
 }
 
-// Replace the bounced populations of node (x, y) (rare path): population i,
+// FP16: replace the bounced populations of node (x, y) (rare path): population i,
 // whose source x - e_i is a wall or a solid, becomes f~_opp(x) + 6 w_i rho_w
 // (e_i . v) with v the wall's or solid's velocity at x - e_i / 2 (Sec. III.A;
 // the moving-wall term).
 // BND: disks with the interpolated boundary (LBM_INTERPOLATED), compiled only
 // into the kernels that run the per-node path outside the vector path.
-template <int P, bool LOCAL, bool BND = false>
-__device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P>::R *fin, int x,
-                                       int y, uint16_t fl, typename Prec<P>::C (&g)[9]) {
-    using C = typename Prec<P>::C;
+template <bool LOCAL, bool BND = false>
+__device__ __forceinline__ void bounce(const StepParams &p, const Raw<LBM_FP16_DEV>::R *fin, int x,
+                                       int y, uint16_t fl, float (&g)[9]) {
+    using C = float;
     const Lattice &L = p.L;
     const int k = y * L.pitch + x;
     const int plane = (int)L.plane;
-    C rho_w = pick<C>(p.rho0, p.rho0_f);
+    C rho_w = p.rho0_f;
     if (LOCAL) {
         C s = 0;
 #pragma unroll
         for (int j = 0; j < 9; j++) s += cvt(fin[j * plane + k]);
-        rho_w = Prec<P>::dev ? (C)1 + s : s;
+        rho_w = 1.f + s;
     }
 #pragma unroll
     for (int i = 1; i < 9; i++) {
@@ -128,7 +124,7 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
         C vx = 0, vy = 0;
         int xs, ys;
         if (L.bc_y == LBM_WALL && (sy < 0 || sy >= L.ny)) {
-            vx = sy < 0 ? pick<C>(p.wall_ux0, p.wall_ux0_f) : pick<C>(p.wall_ux1, p.wall_ux1_f);
+            vx = sy < 0 ? p.wall_ux0_f : p.wall_ux1_f;
         } else if (locate(L, sx, sy, xs, ys)) {
             const uint16_t o = p.owner[cell_of(L, xs, ys)];
             if (BND && o != FLUID) {
@@ -140,32 +136,20 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
                 // M = 6 w_i rho_w (e_i . v), v at the cut x - q e_i; half-way
                 // value where x + e_i is not a fluid node
                 const DSolid &b = p.S[o];
-                C q, ux, uy;
-                if (Prec<P>::dev) {
-                    // FP32: the offset from the centre's nearest image, split
-                    int di = x - b.xwi, dj = y - b.ywi;
-                    if (L.bc_x == LBM_PERIODIC) {
-                        if (2 * di > L.nx) di -= L.nx;
-                        else if (2 * di < -L.nx) di += L.nx;
-                    }
-                    if (L.bc_y == LBM_PERIODIC) {
-                        if (2 * dj > L.ny) dj -= L.ny;
-                        else if (2 * dj < -L.ny) dj += L.ny;
-                    }
-                    q = (C)link_fraction_split(di, dj, b.xwr, b.ywr, b.r, -cx(i), -cy(i));
-                    const C ddx = ((C)di - (C)b.xwr) - q * (C)cx(i);
-                    const C ddy = ((C)dj - (C)b.ywr) - q * (C)cy(i);
-                    ux = (C)b.vxf - (C)b.omf * ddy;
-                    uy = (C)b.vyf + (C)b.omf * ddx;
-                } else {
-                    const double qd = link_fraction(L, b, x, y, opp(i));
-                    double vxd, vyd, ddx, ddy;
-                    point_velocity(L, b.x, b.y, b.vx, b.vy, b.om, (double)x - qd * cx(i),
-                                   (double)y - qd * cy(i), vxd, vyd, ddx, ddy);
-                    q = (C)qd;
-                    ux = (C)vxd;
-                    uy = (C)vyd;
+                // the offset from the centre's nearest image, split
+                int di = x - b.xwi, dj = y - b.ywi;
+                if (L.bc_x == LBM_PERIODIC) {
+                    if (2 * di > L.nx) di -= L.nx;
+                    else if (2 * di < -L.nx) di += L.nx;
                 }
+                if (L.bc_y == LBM_PERIODIC) {
+                    if (2 * dj > L.ny) dj -= L.ny;
+                    else if (2 * dj < -L.ny) dj += L.ny;
+                }
+                const C q = (C)link_fraction_split(di, dj, b.xwr, b.ywr, b.r, -cx(i), -cy(i));
+                const C ddx = ((C)di - (C)b.xwr) - q * (C)cx(i);
+                const C ddy = ((C)dj - (C)b.ywr) - q * (C)cy(i);
+                const C ux = (C)b.vxf - (C)b.omf * ddy, uy = (C)b.vyf + (C)b.omf * ddx;
                 const C m = (C)6 * wgt<C>(i) * rho_w * ((C)cx(i) * ux + (C)cy(i) * uy);
                 const C back = cvt(fin[opp(i) * plane + k]);
                 const C q2 = (C)2 * q;
@@ -183,18 +167,12 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
             }
             if (o != FLUID) {
                 const DSolid &b = p.S[o];
-                vx = pick<C>(b.vx, b.vxf);
-                vy = pick<C>(b.vy, b.vyf);
+                vx = b.vxf;
+                vy = b.vyf;
                 if (b.omf != 0.0f) {
                     // x - e_i / 2 relative to R, nearest periodic image
-                    C dx, dy;
-                    if (Prec<P>::dev) {
-                        dx = (C)(x - b.xwi) - (C)(0.5f * cx(i)) - (C)b.xwr;
-                        dy = (C)(y - b.ywi) - (C)(0.5f * cy(i)) - (C)b.ywr;
-                    } else {
-                        dx = (C)((double)x - 0.5 * cx(i) - b.xw);
-                        dy = (C)((double)y - 0.5 * cy(i) - b.yw);
-                    }
+                    C dx = (C)(x - b.xwi) - (C)(0.5f * cx(i)) - (C)b.xwr;
+                    C dy = (C)(y - b.ywi) - (C)(0.5f * cy(i)) - (C)b.ywr;
                     if (L.bc_x == LBM_PERIODIC) {
                         if (dx > (C)(0.5 * L.nx)) dx -= (C)L.nx;
                         else if (dx < (C)(-0.5 * L.nx)) dx += (C)L.nx;
@@ -203,7 +181,7 @@ __device__ __forceinline__ void bounce(const StepParams &p, const typename Raw<P
                         if (dy > (C)(0.5 * L.ny)) dy -= (C)L.ny;
                         else if (dy < (C)(-0.5 * L.ny)) dy += (C)L.ny;
                     }
-                    const C om = pick<C>(b.om, b.omf);
+                    const C om = b.omf;
                     vx -= om * dy;
                     vy += om * dx;
                 }
@@ -368,7 +346,7 @@ __device__ __forceinline__ void extrapolate_open(const StepParams &p, bool inlet
     }
 }
 
-// Complete update of one node, with periodic wrap, bounce-back and walls
+// FP16: complete update of one node, with periodic wrap, bounce-back and walls
 // (beyond a non-periodic edge: a resting wall): used for the nodes the vector
 // path leaves out (fluid nodes next to a solid or wall, the first and last
 // column).  With OPEN, the columns of an open channel are computed here too:
@@ -377,11 +355,12 @@ __device__ __forceinline__ void extrapolate_open(const StepParams &p, bool inlet
 // the inlet is feq(rho0, u_in) and the outlet updates as a walled node.
 // Without OPEN they update as walled nodes and a later pass (open_col)
 // replaces them.
-template <int P, bool FORCE, bool LOCAL, bool OPEN, int COLL = 0, bool BND = false>
-__device__ __noinline__ void update_node(const StepParams &p, const typename Raw<P>::R *fin,
-                                         typename Raw<P>::R *fout, int x, int y) {
-    using C = typename Prec<P>::C;
-    using R = typename Raw<P>::R;
+template <bool FORCE, bool LOCAL, bool OPEN, int COLL = 0, bool BND = false>
+__device__ __noinline__ void update_node(const StepParams &p, const Raw<LBM_FP16_DEV>::R *fin,
+                                         Raw<LBM_FP16_DEV>::R *fout, int x, int y) {
+    constexpr int P = LBM_FP16_DEV;
+    using C = float;
+    using R = Raw<P>::R;
     const Lattice &L = p.L;
     const int plane = (int)L.plane;
     const int k = y * L.pitch + x;
@@ -421,7 +400,7 @@ __device__ __noinline__ void update_node(const StepParams &p, const typename Raw
         if (ys >= L.ny) ys = per_y ? ys - L.ny : L.ny - 1;
         g[i] = cvt(fin[i * plane + ys * L.pitch + xs]);
     }
-    if (flu & 0x1FEu) bounce<P, LOCAL, BND>(p, fin, xu, y, flu, g);
+    if (flu & 0x1FEu) bounce<LOCAL, BND>(p, fin, xu, y, flu, g);
     auto check = [&](C rho, C ux, C uy) {
         if (unphysical(rho, ux, uy)) atomicOr(p.status, 1);
     };
@@ -442,13 +421,12 @@ __device__ __noinline__ void update_node(const StepParams &p, const typename Raw
 // DEFER: the per-node path is a later pass over those nodes (k_boundary_update);
 // otherwise each thread runs it for its own nodes at the end of the segment.
 // COLL: 0 = BGK, 1 = MRT (no body force, slow nodes inline).
-template <int P, int V, bool FORCE, bool LOCAL, bool OPEN, bool DEFER = false, int COLL = 0,
-          bool BND = false>
-__device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<P>::R *__restrict__ fin,
-                                        typename Raw<P>::R *__restrict__ fout, int x0, int y) {
-    static_assert(P == LBM_FP16_DEV, "FP64 and FP32 take sc_row");
-    using R = typename Raw<P>::R;
-    using C = typename Prec<P>::C;
+template <int V, bool FORCE, bool LOCAL, bool OPEN, bool DEFER = false, int COLL = 0, bool BND = false>
+__device__ __forceinline__ void sc_tile(const StepParams &p, const Raw<LBM_FP16_DEV>::R *__restrict__ fin,
+                                        Raw<LBM_FP16_DEV>::R *__restrict__ fout, int x0, int y) {
+    constexpr int P = LBM_FP16_DEV;
+    using R = Raw<P>::R;
+    using C = float;
     const Lattice &L = p.L;
     const int lane = threadIdx.x & 31;
     const int plane = (int)L.plane;
@@ -527,7 +505,7 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
                 jx += (C)cx(i) * g[i];
                 jy += (C)cy(i) * g[i];
             }
-            const C r = Prec<P>::dev ? (C)1 + a : a;
+            const C r = (C)1 + a;
             classify(j, r, jx / r, jy / r);
             collide_mrt<P>(p, g, [](C, C, C) {});
 #pragma unroll
@@ -536,13 +514,15 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
 #pragma unroll
         for (int i = 0; i < 9; i++)
             *reinterpret_cast<typename Word<sizeof(R) * V>::T *>(fout + i * plane + r0 + x0) = o[i].u;
-    } else if constexpr (Prec<P>::dev && !FORCE && V % 2 == 0) {
+    } else if constexpr (!FORCE) {
         // Deviation form, two nodes per instruction (FADD2 / FMUL2 / FFMA2).
         // With E_i = s0 + rho (3 e_i.u + 4.5 (e_i.u)^2 - 1.5 u.u) the
         // equilibrium deviation is w_i E_i, and BGK gives
         // (1 - omega) g_i + omega w_i E_i.  Opposite populations share
         // A = s0 - 1.5 rho u.u and the even part 4.5 rho (e.u)^2; the odd part
-        // 3 rho e.u changes sign.
+        // 3 rho e.u changes sign.  (bgk32x2 is exact to FP32's rounding, which the
+        // storage rounds ten thousand times as much.)
+        static_assert(V % 2 == 0, "two nodes at a time");
         const float om = p.omega_f;
         const float2 omc = dup2(1.f - om);
         Pack<R, V> o[9];
@@ -596,16 +576,15 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
             jx += (C)cx(i) * g;
             jy += (C)cy(i) * g;
         }
-        const C r = Prec<P>::dev ? (C)1 + a : a;
-        const C inv = (C)1 / r;
+        const C r = (C)1 + a, inv = (C)1 / r;
         s0[j] = a;
         rho[j] = r;
-        ux[j] = FORCE ? (jx + (C)0.5 * pick<C>(p.body_x, p.body_xf)) * inv : jx * inv;
-        uy[j] = FORCE ? (jy + (C)0.5 * pick<C>(p.body_y, p.body_yf)) * inv : jy * inv;
+        ux[j] = (jx + 0.5f * p.body_xf) * inv;
+        uy[j] = (jy + 0.5f * p.body_yf) * inv;
         classify(j, r, ux[j], uy[j]);
     }
     // relax towards equilibrium, one population plane at a time
-    const C om = pick<C>(p.omega, p.omega_f);
+    const C om = p.omega_f;
 #pragma unroll
     for (int i = 0; i < 9; i++) {
         Pack<R, V> o;
@@ -615,15 +594,12 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
             const C eu = (C)cx(i) * ux[j] + (C)cy(i) * uy[j];
             const C uu = ux[j] * ux[j] + uy[j] * uy[j];
             const C poly = (C)3 * eu + (C)4.5 * eu * eu - (C)1.5 * uu;
-            const C eq = Prec<P>::dev ? wgt<C>(i) * (s0[j] + rho[j] * poly)
-                                      : rho[j] * wgt<C>(i) * ((C)1 + poly);
+            const C eq = wgt<C>(i) * (s0[j] + rho[j] * poly);
             C v = g - (g - eq) * om;
-            if (FORCE) {
-                const C Fx = pick<C>(p.body_x, p.body_xf), Fy = pick<C>(p.body_y, p.body_yf);
-                v += ((C)1 - (C)0.5 * om) * wgt<C>(i) *
-                     ((C)3 * (((C)cx(i) - ux[j]) * Fx + ((C)cy(i) - uy[j]) * Fy) +
-                      (C)9 * eu * ((C)cx(i) * Fx + (C)cy(i) * Fy));
-            }
+            const C Fx = p.body_xf, Fy = p.body_yf;
+            v += ((C)1 - (C)0.5 * om) * wgt<C>(i) *
+                 ((C)3 * (((C)cx(i) - ux[j]) * Fx + ((C)cy(i) - uy[j]) * Fy) +
+                  (C)9 * eu * ((C)cx(i) * Fx + (C)cy(i) * Fy));
             put(o.r[j], (fl.f[j] & 1u) ? (C)0 : v);  // solid nodes store zeros
         }
         *reinterpret_cast<typename Word<sizeof(R) * V>::T *>(fout + i * plane + r0 + x0) = o.u;
@@ -635,21 +611,21 @@ __device__ __forceinline__ void sc_tile(const StepParams &p, const typename Raw<
         while (slow) {
             const int j = __ffs(slow) - 1;
             slow &= slow - 1;
-            update_node<P, FORCE, LOCAL, OPEN, COLL, BND>(p, fin, fout, x0 + j, y);
+            update_node<FORCE, LOCAL, OPEN, COLL, BND>(p, fin, fout, x0 + j, y);
         }
     }
 }
 
-// Open channel (bc_x = LBM_OPEN), after the fused kernel of step t has
+// FP16 open channel (bc_x = LBM_OPEN), after the fused kernel of step t has
 // written the populations of t+1 into f: column x = 0 (inlet) or x = nx - 1
 // (outlet) of row y takes the non-equilibrium extrapolation of its inner
 // neighbour's post-collision populations (extrapolate_open); next to a solid
 // neighbour the inlet takes feq(rho0, u_in) and the outlet keeps its own
 // update (a resting wall beyond the edge).  open_row does both columns.
-template <int P, bool FORCE>
-__device__ __forceinline__ void open_col(const StepParams &p, typename Raw<P>::R *f, int y,
-                                         bool inlet) {
-    using C = typename Prec<P>::C;
+template <bool FORCE>
+__device__ __forceinline__ void open_col(const StepParams &p, Raw<LBM_FP16_DEV>::R *f, int y, bool inlet) {
+    constexpr int P = LBM_FP16_DEV;
+    using C = float;
     const Lattice &L = p.L;
     const int plane = (int)L.plane;
     const int x = inlet ? 0 : L.nx - 1;
@@ -669,10 +645,10 @@ __device__ __forceinline__ void open_col(const StepParams &p, typename Raw<P>::R
     for (int i = 0; i < 9; i++) put(f[i * plane + k], g[i]);
 }
 
-template <int P, bool FORCE>
-__device__ __forceinline__ void open_row(const StepParams &p, typename Raw<P>::R *f, int y) {
-    open_col<P, FORCE>(p, f, y, true);
-    open_col<P, FORCE>(p, f, y, false);
+template <bool FORCE>
+__device__ __forceinline__ void open_row(const StepParams &p, Raw<LBM_FP16_DEV>::R *f, int y) {
+    open_col<FORCE>(p, f, y, true);
+    open_col<FORCE>(p, f, y, false);
 }
 
 

@@ -29,7 +29,7 @@ __device__ __forceinline__ void tile_segments(const StepParams &p, const int4 &t
         const R *fin = static_cast<const R *>(p.f1);
         R *fout = static_cast<R *>(p.f0);
         const int x0 = (seg * 32 + (threadIdx.x & 31)) * V;
-        if constexpr (P == LBM_FP16_DEV) sc_tile<P, V, FORCE, LOCAL, true>(p, fin, fout, x0, y);
+        if constexpr (P == LBM_FP16_DEV) sc_tile<V, FORCE, LOCAL, true>(p, fin, fout, x0, y);
         else if (p.L.bc_x == LBM_OPEN) sc_row<P, V, FORCE, true, 0>(p, fin, fout, x0, y);
         else sc_row<P, V, FORCE, false, 0>(p, fin, fout, x0, y);
     }

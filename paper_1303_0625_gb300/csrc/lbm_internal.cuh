@@ -346,25 +346,10 @@ __device__ __forceinline__ void point_velocity(const Lattice &L, const double X,
 }
 
 // Interpolated boundary (the disks' boundary condition of the paper's
-// simulations, ref. [40]): fraction q in (0, 1] of the link from the fluid
-// node (x, y) along e_i at which it meets the circle of disk b, the smaller
-// root of |p + q e_i - R|^2 = r^2 with p - R at the nearest periodic image.
-__device__ __forceinline__ double link_fraction(const Lattice &L, const DSolid &b, int x, int y,
-                                                int i) {
-    const double px = min_image(__dsub_rn((double)x, b.x), L.nx, L.bc_x == LBM_PERIODIC);
-    const double py = min_image(__dsub_rn((double)y, b.y), L.ny, L.bc_y == LBM_PERIODIC);
-    const double ex = cx(i), ey = cy(i);
-    const double a = ex * ex + ey * ey, h = px * ex + py * ey;
-    const double cc = px * px + py * py - b.r * b.r;  // > 0: the node is outside
-    const double disc = h * h - a * cc;
-    double q = disc > 0.0 ? (-h - sqrt(disc)) / a : 0.5;
-    if (!(q > 0.0)) q = 0.0;
-    if (q > 1.0) q = 1.0;
-    return q;
-}
-
-// The same from the node's offset (px, py) from the centre's nearest image, known
-// already (a is 1 or 2: the division by it is exact).
+// simulations, ref. [40]): fraction q in (0, 1] of the link from a fluid node
+// along (ex, ey) at which it meets the circle, the smaller root of
+// |p + q e - R|^2 = r^2, from the node's offset p - R = (px, py) from the centre's
+// nearest image (a = e.e is 1 or 2: the division by it is exact).
 __device__ __forceinline__ double link_fraction_at(double px, double py, double r, int ex, int ey) {
     const double a = (double)(ex * ex + ey * ey), h = px * ex + py * ey;
     const double disc = h * h - a * (px * px + py * py - r * r);
