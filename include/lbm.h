@@ -222,7 +222,7 @@ lbm_status lbm_set_populations(lbm_ctx *ctx, const double *f, int32_t on_device)
  * steps taken (a state after LBM_EUNSTABLE or LBM_ETIMEOUT is not saved).
  * lbm_load restores a state into a context created with the same
  * configuration (stream and device aside) and holding the same solids (the
- * same lbm_add_solid calls): the status word and the bounded waits' counters
+ * same lbm_add_solid calls): the status word and the control words
  * are cleared, and the steps that follow give the same results, bit for bit,
  * as those that followed the save.  Errors: LBM_EINVAL for a buffer that is
  * too small, not a saved state, or from another configuration or solid

@@ -1,7 +1,8 @@
 // Per-solid work of one step t -> t+1.
 //
 // k_forces, one block per solid (or k_links, one or several blocks per solid, and
-// k_record, one warp per solid), comes first:
+// k_record, one warp per solid, which may run beside the advection-collision kernel or
+// after it), comes first:
 //   the link sums of Eq. 4 and Eq. 5 over every fluid-solid link of time t (Eq. 6
 //   and Eq. 7), and in the FP64 and FP32 modes the population each link returns,
 //   left in the solid node's slot for the advection-collision kernel to pull;
@@ -1357,7 +1358,7 @@ __device__ __forceinline__ void rings(const StepParams &p, RingShared &sh) {
 // Beside the advection-collision kernel.
 __global__ void __launch_bounds__(SW_BLOCK, 4) k_ring(const StepParams p) {
     __shared__ RingShared sh;
-    // a barrier of an earlier launch gave up: the state is not the method's
+    // the re-rasterisation of an earlier step gave up: the state is not the method's
     // any more, and this launch does nothing (the host reports the time-out)
     if (*(volatile int *)p.status & 4) return;
     rings(p, sh);

@@ -43,11 +43,11 @@ struct lbm_ctx {
     int ring_cap = 0;      // solids the ring was laid out for
     long long *t_d = nullptr;
     int *status_d = nullptr;
-    unsigned int *bar_d = nullptr;  // per-solid control words (displacement, pair test)
+    unsigned int *bar_d = nullptr;  // control words (ticket, displacement, pair test)
     uint16_t *near_d = nullptr;     // near lists, [solid_cap][NEAR_CAP]
     double *part_d = nullptr;       // link sums by block or chunk (StepParams::part)
     size_t part_cap = 0;            // of six each
-    long long spin_limit = 1ll << 24;  // polls of a bounded device wait (about one second)
+    long long spin_limit = 1ll << 24;  // lbm_set_wait_limit: only 0 makes a difference
     // the force kernel runs on a second stream beside the advection-collision
     // kernel: fork after the previous step, join before the re-rasterisation
     cudaStream_t side = nullptr;
@@ -947,7 +947,7 @@ lbm_status lbm_load(lbm_ctx *c, const void *buf, int64_t bytes) {
     const long long t = h.t;
     CK(c, cudaMemcpyAsync(c->t_d, &t, sizeof t, cudaMemcpyHostToDevice, c->stream));
     if (c->ev_d) CK(c, cudaMemcpyAsync(c->ev_d, &h.ev_len, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-    // clean control words: status, barrier, displacement; a pair test first
+    // clean control words: status, ticket, displacement; a pair test first
     const unsigned int ctl[4] = {0u, 0u, 0u, 1u};
     CK(c, cudaMemcpyAsync(c->bar_d, ctl, sizeof ctl, cudaMemcpyHostToDevice, c->stream));
     CK(c, cudaMemsetAsync(c->status_d, 0, sizeof(int), c->stream));
