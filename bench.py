@@ -867,13 +867,18 @@ def run_e2e(a, w, local, stream):
     torch.cuda.synchronize()
     t0 = time.perf_counter()
     L.lbm_set_populations(lat.handle, f0.numpy())
+    lat.sync()
+    upload = time.perf_counter() - t0
     t_start = lat.t
-    done = 0
+    done, reads = 0, 0.0
     while done < steps:
         n = min(block, steps - done)
         lat.step(n)
+        lat.sync()
+        t1 = time.perf_counter()
         for form in (L.LBM_CME, L.LBM_GME):
             L.lbm_forces(lat.handle, form, t_start + done, n, out[form].numpy())
+        reads += time.perf_counter() - t1
         done += n
     lat.sync()
     dt = time.perf_counter() - t0
@@ -883,6 +888,8 @@ def run_e2e(a, w, local, stream):
     return {"value": round(nx * ny * steps / dt / 1e6, 1), "unit": "MLUPS",
             "h2d_bytes_per_step": int(h2d / steps), "d2h_bytes_per_step": int(d2h / steps),
             "seconds": round(dt, 4), "steps": steps,
+            "parts": {"upload_s": round(upload, 4), "steps_s": round(dt - upload - reads, 4),
+                      "reads_s": round(reads, 4)},
             "what": "C ABI with host buffers: FP64 initial populations uploaded from pinned host "
                     "memory once per job of max(steps, 400) steps, both force forms copied to "
                     "the host every 50 steps"}
